@@ -3,9 +3,11 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "fda_internal.h"
+#include "fda_rows.cuh"
 
 namespace {
 
@@ -13,15 +15,15 @@ constexpr uint64_t kP61 = (1ull << 61) - 1;
 
 struct DeviceGuard {
     int prev = -1;
-    bool ok = true;
+    bool ok = true, changed = false;
     explicit DeviceGuard(int dev)
     {
         if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; prev = -1; return; }
-        if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+        if (prev != dev) { changed = true; ok = cudaSetDevice(dev) == cudaSuccess; }
     }
     ~DeviceGuard()
     {
-        if (prev >= 0) cudaSetDevice(prev);
+        if (changed) cudaSetDevice(prev);
     }
 };
 
@@ -40,6 +42,42 @@ fda_status fail_cuda(fda_ctx *ctx, cudaError_t e, const char *where)
     return e == cudaErrorMemoryAllocation ? FDA_ERR_NOMEM : FDA_ERR_CUDA;
 }
 
+// Mapped host memory for the estimates that callers read at once: one page per process (allocating
+// and freeing it with every context would add milliseconds to fda_create and fda_destroy), a slot
+// per context, given back when the context goes.  Contexts beyond the page's slots copy instead.
+struct EstimateSlots {
+    static constexpr int kSlots = 64, kBytes = 128;
+    std::mutex mutex;
+    unsigned char *page = nullptr;
+    uint64_t used = 0;
+    fda_estimate *take()
+    {
+        static_assert(sizeof(fda_estimate) <= kBytes, "a slot holds an estimate");
+        std::lock_guard<std::mutex> lock(mutex);
+        if (!page) {
+            void *ptr = nullptr;
+            if (cudaHostAlloc(&ptr, kSlots * kBytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+                cudaGetLastError();
+                return nullptr;
+            }
+            page = static_cast<unsigned char *>(ptr);
+        }
+        for (int i = 0; i < kSlots; ++i)
+            if (!((used >> i) & 1u)) {
+                used |= (uint64_t)1 << i;
+                return reinterpret_cast<fda_estimate *>(page + i * kBytes);
+            }
+        return nullptr;
+    }
+    void give_back(fda_estimate *slot)
+    {
+        if (!slot) return;
+        std::lock_guard<std::mutex> lock(mutex);
+        used &= ~((uint64_t)1 << ((reinterpret_cast<unsigned char *>(slot) - page) / kBytes));
+    }
+};
+EstimateSlots g_estimates;
+
 void free_device(fda_ctx *ctx)
 {
     cudaFree(ctx->coeffs_dev);
@@ -50,6 +88,8 @@ void free_device(fda_ctx *ctx)
     cudaFree(ctx->part_np);
     cudaFree(ctx->combine_scratch);
     cudaFree(ctx->combine_ticket);
+    cudaFree(ctx->row_tickets);
+    g_estimates.give_back(ctx->est_pinned);
     cudaFree(ctx->mean_model);
     cudaFree(ctx->stage_w);
     cudaFree(ctx->stage_w_t0);
@@ -126,6 +166,7 @@ fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uin
             ctx->sched_build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
         if (e == cudaSuccess) e = cudaMalloc(&ctx->part_sk, sizeof(float) * ctx->part_sk_floats);
+        if (e == cudaSuccess && ctx->sched) e = fda_setup_local_state_gather(ctx);
         if (e == cudaSuccess && ctx->sched) {
             e = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
@@ -134,9 +175,13 @@ fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uin
     }
     ctx->part_np_doubles = (size_t)ctx->max_blocks * (size_t)(K_max > 32 ? K_max : 32) * 2;
     if (e == cudaSuccess) e = cudaMalloc(&ctx->part_np, sizeof(double) * ctx->part_np_doubles);
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->combine_scratch, sizeof(double) * (2 + FDA_MAX_ROWS));
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->combine_scratch, sizeof(double) * fda_combine_scratch_doubles(ctx->l, ctx->m));
     if (e == cudaSuccess) e = cudaMalloc(&ctx->combine_ticket, sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMemset(ctx->combine_ticket, 0, sizeof(unsigned int));
+    ctx->est_pinned = g_estimates.take();
+    ctx->n_row_tickets = (K_max + fda_rows::kRows - 1) / fda_rows::kRows;
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->row_tickets, sizeof(unsigned int) * ctx->n_row_tickets);
+    if (e == cudaSuccess) e = cudaMemset(ctx->row_tickets, 0, sizeof(unsigned int) * ctx->n_row_tickets);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         const fda_status st = e == cudaErrorMemoryAllocation ? FDA_ERR_NOMEM : FDA_ERR_CUDA;
@@ -225,10 +270,13 @@ fda_status fda_combine_estimate(fda_ctx *ctx, const float *states, int K, int va
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return fail(ctx, FDA_ERR_CUDA, "fda_combine_estimate: cannot select device");
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = fda_launch_combine(ctx, states, K, variant, epsilon, theta, est_dev, s);
+    // the kernel writes the estimate to mapped host memory as well: no copy stands between it and the host
+    cudaError_t e = fda_launch_combine(ctx, states, K, variant, epsilon, theta, est_dev,
+                                       est_host ? ctx->est_pinned : nullptr, s);
     if (e == cudaSuccess && est_host) {
-        e = cudaMemcpyAsync(est_host, est_dev, sizeof(fda_estimate), cudaMemcpyDeviceToHost, s);
+        if (!ctx->est_pinned) e = cudaMemcpyAsync(est_host, est_dev, sizeof(fda_estimate), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess && ctx->est_pinned) std::memcpy(est_host, ctx->est_pinned, sizeof(fda_estimate));
     }
     if (e != cudaSuccess) return fail_cuda(ctx, e, "fda_combine_estimate");
     return FDA_OK;
@@ -385,7 +433,7 @@ fda_status fda_context_info(const fda_ctx *ctx, int64_t *info)
     const int64_t table = ctx->tab ? (int64_t)(sizeof(uint16_t) * (size_t)ctx->l * ctx->tab_stride) : 0;
     const int64_t sched = ctx->sched ? (int64_t)(ctx->sched_bytes + sizeof(uint64_t) * (size_t)(ctx->sched_tiles + 1)) : 0;
     const int64_t partial = (int64_t)(sizeof(float) * ctx->part_sk_floats + sizeof(double) * ctx->part_np_doubles +
-                                      sizeof(double) * (2 + FDA_MAX_ROWS) + sizeof(unsigned int)) +
+                                      sizeof(double) * fda_combine_scratch_doubles(ctx->l, ctx->m) + sizeof(unsigned int) * (1 + ctx->n_row_tickets)) +
                             (ctx->coeffs_dev ? (int64_t)sizeof(uint64_t) * 6 * ctx->l : 0);
     const int64_t mean = ctx->mean_model ? (int64_t)sizeof(float) * ((ctx->d_max + 3) / 4 * 4) : 0;
     int64_t stage = 0;

@@ -16,6 +16,7 @@ __global__ void __launch_bounds__(256)
 k_average(float *w, int64_t row_stride, int K, int64_t d, float *__restrict__ w_t0,
           const fda_estimate *est, int broadcast, float *__restrict__ xi_out, double *__restrict__ part)
 {
+    fda_grid_wait();
     if (est != nullptr && est->trigger == 0) return;
     double dsq = 0.0;
     const float inv_k = 1.0f / (float)K;
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(256)
 k_scale_xi(float *__restrict__ xi_out, int64_t d, const double *__restrict__ part, int nparts,
            const fda_estimate *est)
 {
+    fda_grid_wait();
     if (est != nullptr && est->trigger == 0) return;
     __shared__ float scale_s;
     if (threadIdx.x == 0) {
@@ -111,14 +113,11 @@ cudaError_t fda_launch_average(const fda_ctx *ctx, float *w, int64_t row_stride,
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     if (xi_out) {
-        if (vec) k_average<true, true><<<(unsigned)blocks, threads, 0, s>>>(w, row_stride, K, d, w_t0, gate, broadcast, xi_out, ctx->part_np);
-        else     k_average<false, true><<<(unsigned)blocks, threads, 0, s>>>(w, row_stride, K, d, w_t0, gate, broadcast, xi_out, ctx->part_np);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = fda_launch_dependent(vec ? k_average<true, true> : k_average<false, true>, (int)blocks, threads, 0, s,
+                                             w, row_stride, K, d, w_t0, gate, broadcast, xi_out, ctx->part_np);
         if (e != cudaSuccess) return e;
-        k_scale_xi<<<(unsigned)blocks, threads, 0, s>>>(xi_out, d, ctx->part_np, (int)blocks, gate);
-        return cudaGetLastError();
+        return fda_launch_dependent(k_scale_xi, (int)blocks, threads, 0, s, xi_out, d, ctx->part_np, (int)blocks, gate);
     }
-    if (vec) k_average<true, false><<<(unsigned)blocks, threads, 0, s>>>(w, row_stride, K, d, w_t0, gate, broadcast, nullptr, nullptr);
-    else     k_average<false, false><<<(unsigned)blocks, threads, 0, s>>>(w, row_stride, K, d, w_t0, gate, broadcast, nullptr, nullptr);
-    return cudaGetLastError();
+    return fda_launch_dependent(vec ? k_average<true, false> : k_average<false, false>, (int)blocks, threads, 0, s,
+                                w, row_stride, K, d, w_t0, gate, broadcast, (float *)nullptr, (double *)nullptr);
 }

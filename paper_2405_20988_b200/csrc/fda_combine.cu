@@ -1,135 +1,185 @@
 // Combine step: average state, row norms of the averaged sketch, median, H, trigger
 // (Algorithm 1: the state average and the variance test; Theorem 1 for SketchFDA, Theorem 2 for LinearFDA).
 //
-// One block per sketch row plus one for the two scalar entries, so that the K x (2 + l*m) reads
-// of a large state table are spread over several SMs; the block that finishes last (a ticket
-// counter, no waiting) takes the median and writes the estimate.  fp64 accumulation in a fixed
-// order, so the result is reproducible.
+// Bound: latency.  The K x (2 + l*m) floats are a few kilobytes to a megabyte; what takes time is
+// the chain launch - loads - reductions - (meeting of the blocks) - median - result.  So a thread
+// asks for sixteen workers' values of a column before it adds any, and a warp meets the others once.
+// Tables of up to kOneBlock floats are taken by one block (a ticket and a second trip to L2 cost more
+// than reading them on one SM); larger ones by one block per 64 columns of a row, its threads
+// splitting the workers four ways, and the block that finishes last (a ticket counter, no waiting)
+// takes the median.  The median comes from the ranks of the row norms, all rows at once.
+// fp64 accumulation in a fixed order, so the result is reproducible.
 #include "fda_internal.h"
 
 namespace {
 
-constexpr int kCombineThreads = 1024;
+constexpr int kThreads = 1024;             // of the block that takes everything
+constexpr int kUnitColumns = 64;           // columns of a block that takes a part of a row,
+constexpr int kUnitSlices = 4;             // and the slices of workers its threads split into
+constexpr int kUnitThreads = kUnitColumns * kUnitSlices;
+constexpr int64_t kOneBlock = 12 * 1024;   // states (floats) one block reads in about the time of a meeting
 
-__device__ double block_sum(double v, double *scratch)
+struct CombineParams {
+    const float *states;
+    int K, l, m, chunks;                   // chunks: blocks per sketch row (several blocks only)
+    int variant;
+    float epsilon, theta;
+    double *scratch;                       // [0..1] S-bar[0..1], then one partial per block
+    unsigned int *ticket;                  // 0 between launches
+    fda_estimate *est, *est_host;          // est_host: mapped host memory or null
+};
+
+__device__ __forceinline__ double warp_sum(double v)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    __syncthreads();                       // scratch may still be read from the last call
-    if (lane == 0) scratch[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int wv = 0; wv < nwarps; ++wv) t += scratch[wv];
-    return t;                              // valid in thread 0
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
 }
 
-// scratch (device, owned by the context): [0..1] S-bar[0..1], [2 .. 2+l) row norms; *ticket is 0
-// between launches.
-__global__ void __launch_bounds__(kCombineThreads, 1)
-k_combine(const float *__restrict__ states, int K, int l, int m, int cw /* pow2 >= min(m, threads) */,
-          int variant, float epsilon, float theta, double *scratch_out, unsigned int *ticket,
-          fda_estimate *__restrict__ est)
+// sum over the workers first, first + step, ... of one column, in order, sixteen loads in flight
+__device__ __forceinline__ double column_sum(const float *col, int first, int step, int K, size_t slen)
 {
-    __shared__ double scratch[32];
-    __shared__ double part_s[kCombineThreads];
-    __shared__ bool last_s;
-    const size_t slen = 2 + (size_t)l * (size_t)m;
-    const double inv_k = 1.0 / (double)K;
-    const int tid = threadIdx.x;
-    const int i = blockIdx.x;              // sketch row; block l handles the two scalars
-
-    if (i == l) {
-        if (tid < 2) {                     // S-bar[0] and S-bar[1]
-            double acc = 0.0;
-            for (int k = 0; k < K; ++k) acc += (double)states[(size_t)k * slen + tid];
-            scratch_out[tid] = acc * inv_k;
-            __threadfence();
-        }
-    } else {                               // ||row i of the averaged sketch||^2
-        // thread (kp, cl): workers kp, kp + ks, ... of column c0 + cl; then the ks partial sums
-        // of a column are added in order
-        const int ks = blockDim.x / cw, cl = tid % cw, kp = tid / cw;
-        double part = 0.0;
-        for (int c0 = 0; c0 < m; c0 += cw) {
-            const int c = c0 + cl;
-            double acc = 0.0;
-            if (c < m && kp < ks) {
-                const float *col = states + 2 + (size_t)i * m + c;
-                int k = kp;
-                for (; k + 3 * ks < K; k += 4 * ks) {
-                    const float v0 = col[(size_t)k * slen], v1 = col[(size_t)(k + ks) * slen],
-                                v2 = col[(size_t)(k + 2 * ks) * slen], v3 = col[(size_t)(k + 3 * ks) * slen];
-                    acc += (double)v0; acc += (double)v1; acc += (double)v2; acc += (double)v3;
-                }
-                for (; k < K; k += ks) acc += (double)col[(size_t)k * slen];
-            }
-            __syncthreads();               // part_s of the previous chunk has been read
-            part_s[tid] = acc;
-            __syncthreads();
-            if (kp == 0 && c < m) {
-                double t = 0.0;
-                for (int q = 0; q < ks; ++q) t += part_s[q * cw + cl];
-                t *= inv_k;
-                part += t * t;
-            }
-        }
-        const double r = block_sum(part, scratch);
-        if (tid == 0) scratch_out[2 + i] = r;
+    constexpr int kBatch = 16;
+    double acc = 0.0;
+    for (int k = first; k < K; k += kBatch * step) {
+        float v[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) v[u] = k + u * step < K ? __ldcg(col + (size_t)(k + u * step) * slen) : 0.f;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) acc += (double)v[u];
     }
+    return acc;
+}
 
-    // ---- the last block to arrive finishes the estimate ----
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        const unsigned int t = atomicAdd(ticket, 1u);
-        last_s = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!last_s || tid != 0) return;
-    __threadfence();
-    const volatile double *res = scratch_out;
-    double rows[FDA_MAX_ROWS];
-    for (int r = 0; r < l; ++r) rows[r] = res[2 + r];
-    const double head0 = res[0], head1 = res[1];
-    double est_sq;
-    if (variant == FDA_VARIANT_SKETCH) {
-        double srt[FDA_MAX_ROWS];
-        for (int r = 0; r < l; ++r) {              // insertion sort, l <= 16
-            double v = rows[r];
-            int q = r;
-            while (q > 0 && srt[q - 1] > v) { srt[q] = srt[q - 1]; --q; }
-            srt[q] = v;
+// S-bar[e] (e = 0, 1): lanes stride the workers, fixed shuffle tree
+__device__ __forceinline__ double scalar_mean(const float *states, int K, size_t slen, int e, int lane)
+{
+    double acc = 0.0;
+    for (int k = lane; k < K; k += 32) acc += (double)__ldcg(states + (size_t)k * slen + e);
+    return warp_sum(acc) / (double)K;
+}
+
+// One warp: lane r < l holds ||row r of the averaged sketch||^2; writes the estimate.
+__device__ __forceinline__ void finish(const CombineParams &p, double row, double head0, double head1, int lane)
+{
+    double est_sq = head1 * head1;
+    if (p.variant == FDA_VARIANT_SKETCH) {
+        int rank = 0;                      // of this lane's row, ties by row number
+        for (int q = 0; q < p.l; ++q) {
+            const double o = __shfl_sync(0xffffffffu, row, q);
+            rank += (o < row || (o == row && q < lane)) ? 1 : 0;
         }
-        const double med = (l & 1) ? srt[l / 2] : 0.5 * (srt[l / 2 - 1] + srt[l / 2]);
-        est_sq = med / (1.0 + (double)epsilon);
-    } else {
-        est_sq = head1 * head1;
+        const unsigned lo = __ballot_sync(0xffffffffu, lane < p.l && rank == (p.l - 1) / 2);
+        const unsigned hi = __ballot_sync(0xffffffffu, lane < p.l && rank == p.l / 2);
+        const double a = __shfl_sync(0xffffffffu, row, lo ? __ffs(lo) - 1 : 0);
+        const double b = __shfl_sync(0xffffffffu, row, hi ? __ffs(hi) - 1 : 0);
+        est_sq = ((p.l & 1) ? a : 0.5 * (a + b)) / (1.0 + (double)p.epsilon);
     }
     const double H = head0 - est_sq;
-    est->mean_sq_norm = (float)head0;
-    est->est_sq_norm_of_mean = (float)est_sq;
-    est->H = (float)H;
-    est->theta = theta;
-    est->trigger = (H > (double)theta) ? 1 : 0;    // decided in fp64, strict '>'
-    est->l = l;
-    for (int r = 0; r < FDA_MAX_ROWS; ++r) est->row_sq_norm[r] = r < l ? (float)rows[r] : 0.f;
-    *ticket = 0u;                                  // ready for the next launch on this context
+    const int trigger = (H > (double)p.theta) ? 1 : 0;    // decided in fp64, strict '>'
+    for (int t = 0; t < 2; ++t) {
+        fda_estimate *est = t == 0 ? p.est : p.est_host;
+        if (!est) continue;
+        if (lane == 0) {
+            est->mean_sq_norm = (float)head0;
+            est->est_sq_norm_of_mean = (float)est_sq;
+            est->H = (float)H;
+            est->theta = p.theta;
+            est->trigger = trigger;
+            est->l = p.l;
+        }
+        if (lane < FDA_MAX_ROWS) est->row_sq_norm[lane] = lane < p.l ? (float)row : 0.f;
+    }
+}
+
+// One block: warp w takes the columns stripe*32 + lane, + 32*stripes, ... of row w % l.
+__global__ void __launch_bounds__(kThreads, 1) k_combine_small(const CombineParams p)
+{
+    __shared__ double part_s[32], head_s[2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t slen = 2 + (size_t)p.l * (size_t)p.m;
+    const int stripes = p.l > 0 ? 30 / p.l : 0;            // warps per row; the last two warps take the scalars
+    fda_grid_wait();
+    double part = 0.0;
+    if (warp >= 30) {
+        const double h = scalar_mean(p.states, p.K, slen, warp - 30, lane);
+        if (lane == 0) head_s[warp - 30] = h;
+    } else if (warp < stripes * p.l) {
+        const int i = warp % p.l;
+        for (int c = (warp / p.l) * 32 + lane; c < p.m; c += stripes * 32) {
+            const double t = column_sum(p.states + 2 + (size_t)i * p.m + c, 0, 1, p.K, slen) / (double)p.K;
+            part += t * t;
+        }
+        part = warp_sum(part);
+    }
+    if (lane == 0) part_s[warp] = part;
+    __syncthreads();
+    if (warp != 0) return;
+    double row = 0.0;
+    if (lane < p.l)
+        for (int q = 0; q < stripes; ++q) row += part_s[q * p.l + lane];
+    finish(p, row, head_s[0], head_s[1], lane);
+}
+
+// Block b: the 64 columns b % chunks of row b / chunks; two warps of block 0 also take the scalars.
+__global__ void __launch_bounds__(kUnitThreads) k_combine(const CombineParams p)
+{
+    __shared__ double slice_s[kUnitThreads], part_s[kUnitColumns / 32];
+    __shared__ bool last_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const size_t slen = 2 + (size_t)p.l * (size_t)p.m;
+    fda_grid_wait();
+    const int i = (int)blockIdx.x / p.chunks, sl = tid / kUnitColumns;
+    const int c = ((int)blockIdx.x % p.chunks) * kUnitColumns + tid % kUnitColumns;
+    slice_s[tid] = c < p.m ? column_sum(p.states + 2 + (size_t)i * p.m + c, sl, kUnitSlices, p.K, slen) : 0.0;
+    if (blockIdx.x == 0 && warp < 2) {
+        const double h = scalar_mean(p.states, p.K, slen, warp, lane);
+        if (lane == 0) { p.scratch[warp] = h; __threadfence(); }
+    }
+    __syncthreads();
+    if (tid < kUnitColumns) {
+        double t = 0.0;
+#pragma unroll
+        for (int q = 0; q < kUnitSlices; ++q) t += slice_s[q * kUnitColumns + tid];
+        t /= (double)p.K;
+        t = warp_sum(t * t);
+        if (lane == 0) part_s[warp] = t;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double t = 0.0;
+#pragma unroll
+        for (int q = 0; q < kUnitColumns / 32; ++q) t += part_s[q];
+        p.scratch[2 + blockIdx.x] = t;
+        __threadfence();
+        last_s = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last_s || warp != 0) return;
+    __threadfence();
+    double row = 0.0;
+    if (lane < p.l)
+        for (int q = 0; q < p.chunks; ++q) row += __ldcg(p.scratch + 2 + lane * p.chunks + q);
+    finish(p, row, __ldcg(p.scratch), __ldcg(p.scratch + 1), lane);
+    if (lane == 0) *p.ticket = 0u;                         // ready for the next launch on this context
 }
 
 }  // namespace
 
 cudaError_t fda_launch_combine(const fda_ctx *ctx, const float *states, int K, int variant,
-                               float epsilon, float theta, fda_estimate *est_dev, cudaStream_t s)
+                               float epsilon, float theta, fda_estimate *est_dev, fda_estimate *est_host,
+                               cudaStream_t s)
 {
-    // columns per pass: the power of two that covers m (at most the block); the other threads
-    // of the block split the workers
-    int cw = 32;
-    while (cw < ctx->m && cw < kCombineThreads) cw <<= 1;
-    int threads = cw;
-    while (threads < kCombineThreads && threads / cw < (K + 7) / 8) threads <<= 1;
-    k_combine<<<ctx->l + 1, threads, 0, s>>>(states, K, ctx->l, ctx->m, cw, variant, epsilon, theta,
-                                            ctx->combine_scratch, ctx->combine_ticket, est_dev);
-    return cudaGetLastError();
+    CombineParams p{};
+    p.states = states; p.K = K; p.l = ctx->l; p.m = ctx->m;
+    p.variant = variant; p.epsilon = epsilon; p.theta = theta;
+    p.scratch = ctx->combine_scratch; p.ticket = ctx->combine_ticket;
+    p.est = est_dev; p.est_host = est_host;
+    if (ctx->l == 0 || (int64_t)K * ctx->lm <= kOneBlock)
+        return fda_launch_dependent(k_combine_small, 1, kThreads, 0, s, p);
+    p.chunks = (ctx->m + kUnitColumns - 1) / kUnitColumns;
+    return fda_launch_dependent(k_combine, ctx->l * p.chunks, kUnitThreads, 0, s, p);
 }
+
+// doubles of the context's combine scratch: the two scalars and one partial per block
+size_t fda_combine_scratch_doubles(int l, int m) { return 2 + (size_t)l * ((size_t)(m + kUnitColumns - 1) / kUnitColumns); }

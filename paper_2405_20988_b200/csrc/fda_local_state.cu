@@ -42,7 +42,7 @@ __device__ __forceinline__ float flip(float v, uint32_t signbit)   // signbit: 0
     return __uint_as_float(__float_as_uint(v) ^ signbit);
 }
 
-template <int LWK, bool SKETCH, bool LINEAR, bool VEC>
+template <int LWK, bool LINEAR, bool VEC>
 __global__ void __launch_bounds__(1024, 1) k_local_state(const LsParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -58,10 +58,8 @@ __global__ void __launch_bounds__(1024, 1) k_local_state(const LsParams p)
     const bool active = kl < kg_here;
     const int columns = 1 << p.cshift;
 
-    if (SKETCH) {
-        for (int i = tid; i < p.lm * columns; i += blockDim.x) bins[i] = 0.f;
-        __syncthreads();
-    }
+    for (int i = tid; i < p.lm * columns; i += blockDim.x) bins[i] = 0.f;
+    __syncthreads();
 
     double acc_n = 0.0, acc_p = 0.0;
     if (active) {
@@ -107,32 +105,30 @@ __global__ void __launch_bounds__(1024, 1) k_local_state(const LsParams p)
             acc_n += (double)pn;
             if (LINEAR) acc_p += (double)pp;
 
-            if (SKETCH) {
 #pragma unroll
-                for (int v = 0; v < kQuadsPerLane; ++v) {
-                    if (jq[v] >= p.d) continue;      // whole quad past the end: u is all zero
-                    for (int i = 0; i < p.l; ++i) {
-                        // 4 consecutive 16-bit entries; the table is padded past d_max
-                        const uint2 h = __ldg(reinterpret_cast<const uint2 *>(
-                            p.tab + (size_t)i * (size_t)p.tab_stride + jq[v]));
-                        const int rowbase = i * p.m;
-                        const uint32_t e0 = h.x & 0xffffu, e1 = h.x >> 16, e2 = h.y & 0xffffu, e3 = h.y >> 16;
-                        atomicAdd(&bins[((rowbase + (int)(e0 & 0x7fffu)) << p.cshift) + col],
-                                  flip(u[v][0], (e0 & FDA_TAB_SIGN_BIT) << 16));
-                        atomicAdd(&bins[((rowbase + (int)(e1 & 0x7fffu)) << p.cshift) + col],
-                                  flip(u[v][1], (e1 & FDA_TAB_SIGN_BIT) << 16));
-                        atomicAdd(&bins[((rowbase + (int)(e2 & 0x7fffu)) << p.cshift) + col],
-                                  flip(u[v][2], (e2 & FDA_TAB_SIGN_BIT) << 16));
-                        atomicAdd(&bins[((rowbase + (int)(e3 & 0x7fffu)) << p.cshift) + col],
-                                  flip(u[v][3], (e3 & FDA_TAB_SIGN_BIT) << 16));
-                    }
+            for (int v = 0; v < kQuadsPerLane; ++v) {
+                if (jq[v] >= p.d) continue;      // whole quad past the end: u is all zero
+                for (int i = 0; i < p.l; ++i) {
+                    // 4 consecutive 16-bit entries; the table is padded past d_max
+                    const uint2 h = __ldg(reinterpret_cast<const uint2 *>(
+                        p.tab + (size_t)i * (size_t)p.tab_stride + jq[v]));
+                    const int rowbase = i * p.m;
+                    const uint32_t e0 = h.x & 0xffffu, e1 = h.x >> 16, e2 = h.y & 0xffffu, e3 = h.y >> 16;
+                    atomicAdd(&bins[((rowbase + (int)(e0 & 0x7fffu)) << p.cshift) + col],
+                              flip(u[v][0], (e0 & FDA_TAB_SIGN_BIT) << 16));
+                    atomicAdd(&bins[((rowbase + (int)(e1 & 0x7fffu)) << p.cshift) + col],
+                              flip(u[v][1], (e1 & FDA_TAB_SIGN_BIT) << 16));
+                    atomicAdd(&bins[((rowbase + (int)(e2 & 0x7fffu)) << p.cshift) + col],
+                              flip(u[v][2], (e2 & FDA_TAB_SIGN_BIT) << 16));
+                    atomicAdd(&bins[((rowbase + (int)(e3 & 0x7fffu)) << p.cshift) + col],
+                              flip(u[v][3], (e3 & FDA_TAB_SIGN_BIT) << 16));
                 }
             }
         }
     }
 
     // ---- flush the block's sketch partial: sum the columns of each worker ----------------
-    if (SKETCH) {
+    {
         __syncthreads();
         float *out = p.part_sk + (size_t)blockIdx.x * (size_t)p.lm * LWK;
         const int reps = columns / LWK;
@@ -358,6 +354,7 @@ __global__ void k_finalize_states(const float *__restrict__ part_sk, const doubl
                                   int K, int Kg, int groups, int cpg, int lm, uint32_t flags,
                                   bool have_xi, float *__restrict__ states)
 {
+    fda_grid_wait();
     const int slen = 2 + lm;
     const bool sketch = (flags & FDA_STATE_SKETCH) != 0;
     const int64_t per_group = (int64_t)(lm + 2) * LWK;
@@ -409,7 +406,6 @@ template <int LWK>
 cudaError_t launch_for_lwk(fda_ctx *ctx, LsParams &p, uint32_t flags, bool vec, bool fast, int groups,
                            int blocks, int threads, size_t smem, float *states, cudaStream_t s)
 {
-    const bool sketch = (flags & FDA_STATE_SKETCH) != 0;
     const bool linear = (flags & FDA_STATE_LINEAR) != 0 && p.xi != nullptr;
     if (fast) {
         if constexpr (LWK >= 8) {
@@ -420,31 +416,19 @@ cudaError_t launch_for_lwk(fda_ctx *ctx, LsParams &p, uint32_t flags, bool vec, 
             return cudaErrorInvalidValue;     // the fast path is never selected for fewer than 8 worker lanes
         }
     } else {
-#define FDA_LS_LAUNCH(SK, LI, VE)                                                              \
-    do {                                                                                       \
-        auto kern = k_local_state<LWK, SK, LI, VE>;                                            \
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                             ctx->smem_optin);                                 \
-        if (e != cudaSuccess) return e;                                                        \
-        kern<<<blocks, threads, smem, s>>>(p);                                                 \
-    } while (0)
-    if (sketch) {
-        if (linear) { if (vec) FDA_LS_LAUNCH(true, true, true); else FDA_LS_LAUNCH(true, true, false); }
-        else        { if (vec) FDA_LS_LAUNCH(true, false, true); else FDA_LS_LAUNCH(true, false, false); }
-    } else {
-        if (linear) { if (vec) FDA_LS_LAUNCH(false, true, true); else FDA_LS_LAUNCH(false, true, false); }
-        else        { if (vec) FDA_LS_LAUNCH(false, false, true); else FDA_LS_LAUNCH(false, false, false); }
+        auto kern = linear ? (vec ? k_local_state<LWK, true, true> : k_local_state<LWK, true, false>)
+                           : (vec ? k_local_state<LWK, false, true> : k_local_state<LWK, false, false>);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
+        if (e != cudaSuccess) return e;
+        kern<<<blocks, threads, smem, s>>>(p);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
     }
-#undef FDA_LS_LAUNCH
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     const int64_t total = (int64_t)groups * (2 + p.lm) * LWK;
     int fb = (int)((total + 255) / 256);
     if (fb > ctx->n_sm * 8) fb = ctx->n_sm * 8;
-    k_finalize_states<LWK><<<fb, 256, 0, s>>>(p.part_sk, p.part_np, p.K, p.Kg, groups, p.cpg, p.lm, flags,
-                                             p.xi != nullptr, states);
-    return cudaGetLastError();
+    return fda_launch_dependent(k_finalize_states<LWK>, fb, 256, 0, s, p.part_sk, p.part_np, p.K, p.Kg, groups, p.cpg,
+                                p.lm, flags, p.xi != nullptr, states);
 }
 
 }  // namespace
@@ -470,15 +454,12 @@ cudaError_t fda_launch_local_state(fda_ctx *ctx, const float *w, int64_t row_str
         cudaError_t e = fda_launch_local_state_gather(ctx, w, row_stride, K, d, w_t0, xi, flags, states, s);
         if (e != cudaErrorNotSupported) { ctx->last_ls_kernel = "k_local_state_gather"; return e; }   // (counts its launches itself)
         e = fda_launch_local_state_linear(ctx, w, row_stride, K, d, w_t0, xi, flags, states, s);
-        if (e != cudaErrorNotSupported) { ctx->last_ls_kernel = "k_local_state_linear"; ctx->last_ls_launches = 2; return e; }
+        if (e != cudaErrorNotSupported) { ctx->last_ls_kernel = "k_local_state_linear"; ctx->last_ls_launches = 1; return e; }
     }
-    if (flags & FDA_STATE_SKETCH) {
-        const cudaError_t e = fda_ensure_table(ctx, s);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = fda_ensure_table(ctx, s);
+    if (e != cudaSuccess) return e;
     ctx->last_ls_kernel = "k_local_state";
     ctx->last_ls_launches = 2;
-    const bool sketch = (flags & FDA_STATE_SKETCH) != 0;
     LsParams p{};
     p.w = w; p.row_stride = row_stride; p.K = K; p.d = d; p.w_t0 = w_t0;
     p.xi = (flags & FDA_STATE_LINEAR) ? xi : nullptr;
@@ -487,24 +468,23 @@ cudaError_t fda_launch_local_state(fda_ctx *ctx, const float *w, int64_t row_str
     p.part_sk = ctx->part_sk; p.part_np = ctx->part_np;
 
     // workers per group: a power of two lane count LWK, limited by the bin columns
-    const int lane_cap = sketch ? ctx->columns : 32;
+    const int lane_cap = ctx->columns;
     int lwk = pow2_ceil(K < 32 ? K : 32);
     if (lwk > lane_cap) lwk = lane_cap;
     if (lwk < 8) lwk = 8 <= lane_cap ? 8 : lane_cap;
     const int groups = (K + lwk - 1) / lwk;
     p.Kg = (K + groups - 1) / groups;
-    const int columns = sketch ? ctx->columns : lwk;
+    const int columns = ctx->columns;
     p.cshift = ilog2(columns);
 
     const bool vec = ((((uintptr_t)w | (uintptr_t)w_t0 | (uintptr_t)(p.xi ? p.xi : w)) & 15u) == 0) &&
                      (row_stride % 4 == 0);
-    const bool fast = sketch && vec && lwk >= 8 && (ctx->l == 5 || ctx->l == 7);
-    const int threads = fast ? kFastThreads : (sketch ? 1024 : 512);
-    const int blocks_per_sm = sketch ? 1 : 2;
+    const bool fast = vec && lwk >= 8 && (ctx->l == 5 || ctx->l == 7);
+    const int threads = fast ? kFastThreads : 1024;
     const int js = 32 / lwk;
     const int64_t tile_j = (int64_t)(threads / 32) * js * (fast ? kFastQuads : kQuadsPerLane) * 4;
     p.tiles = (d + tile_j - 1) / tile_j;
-    int64_t cpg = (int64_t)ctx->n_sm * blocks_per_sm / groups;
+    int64_t cpg = (int64_t)ctx->n_sm / groups;
     if (cpg < 1) cpg = 1;
     if (cpg > p.tiles) cpg = p.tiles;
     if ((int64_t)groups * cpg > ctx->max_blocks) cpg = ctx->max_blocks / groups;
@@ -512,16 +492,14 @@ cudaError_t fda_launch_local_state(fda_ctx *ctx, const float *w, int64_t row_str
     const int blocks = groups * p.cpg;
     // the partial sums of a launch must fit the context's scratch (sized for n_sm blocks of 32
     // worker lanes and 4 * n_sm blocks of K_max workers): more worker groups than that is refused
-    if (blocks < 1 || (sketch && (size_t)blocks * p.lm * lwk > ctx->part_sk_floats) ||
+    if (blocks < 1 || (size_t)blocks * p.lm * lwk > ctx->part_sk_floats ||
         (size_t)blocks * lwk * 2 > ctx->part_np_doubles)
         return cudaErrorNotSupported;
     ctx->last_ls_kernel = fast ? "k_local_state_fast" : "k_local_state";
 
     size_t smem = (size_t)(threads / 32) * lwk * 2 * sizeof(double);
-    if (sketch) {
-        const size_t b = (size_t)p.lm * columns * sizeof(float);
-        if (b > smem) smem = b;
-    }
+    const size_t b = (size_t)p.lm * columns * sizeof(float);
+    if (b > smem) smem = b;
     switch (lwk) {
         case 1:  return launch_for_lwk<1>(ctx, p, flags, vec, fast, groups, blocks, threads, smem, states, s);
         case 2:  return launch_for_lwk<2>(ctx, p, flags, vec, fast, groups, blocks, threads, smem, states, s);

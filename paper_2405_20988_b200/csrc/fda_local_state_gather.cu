@@ -85,6 +85,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     if (tid < 2) ctr[tid] = 0;
     if (tid < kProducerWarps * GW * 2) sums[tid] = 0.0;
     __syncthreads();
+    fda_grid_wait();
 
     const int64_t n_tiles = p.tiles > c ? (p.tiles - c + p.cpg - 1) / p.cpg : 0;
 
@@ -315,6 +316,7 @@ __global__ void k_finalize_gather(const ListParams p, const ListParts parts, uin
     const bool sketch = (flags & FDA_STATE_SKETCH) != 0;
     const int64_t total = (int64_t)p.groups * slen * GW * 4;
     const int64_t padded = (total + 31) & ~(int64_t)31;                 // whole warps take part in the shuffles
+    fda_grid_wait();
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < padded;
          t += (int64_t)gridDim.x * blockDim.x) {
         const bool valid = t < total;
@@ -357,18 +359,30 @@ __global__ void k_finalize_gather(const ListParams p, const ListParts parts, uin
 }
 
 template <int PW, int WW>
-cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, int smem_optin, cudaStream_t s)
+cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent, cudaStream_t s)
 {
     if (p.T % (PW * 128) != 0 || PW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
     p.nb = p.T / (PW * 128);
     auto kern = p.have_xi ? k_local_state_gather<true, PW, WW> : k_local_state_gather<false, PW, WW>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin);
-    if (e != cudaSuccess) return e;
+    if (dependent) return fda_launch_dependent(kern, blocks, (PW + WW) * 32, smem, s, p);
     kern<<<blocks, (PW + WW) * 32, smem, s>>>(p);
     return cudaGetLastError();
 }
 
 }  // namespace
+
+// The kernels' dynamic shared memory limit, set once per context (on the context's device).
+cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx)
+{
+    auto set = [&](void (*kern)(ListParams)) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
+    };
+    cudaError_t e = set(k_local_state_gather<true, 8, 20>);
+    if (e == cudaSuccess) e = set(k_local_state_gather<false, 8, 20>);
+    if (e == cudaSuccess) e = set(k_local_state_gather<true, 4, 24>);
+    if (e == cudaSuccess) e = set(k_local_state_gather<false, 4, 24>);
+    return e;
+}
 
 // Returns cudaErrorNotSupported when the request does not fit this path (the caller then uses
 // the other kernels); any other value is the result of the launches.
@@ -406,9 +420,9 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     // 8 producer + 20 walker warps, or 4 + 24 when a loaded index pays for more walking.  Measured:
     // 7 x 500, K = 60, d = 20M: 3.34 ms with 4 + 24 against 3.71 ms with 8 + 20; 5 x 250, K = 8,
     // d = 198M: 3.49 against 2.49 ms; 5 x 250, K = 30, d = 7M: 0.535 against 0.387 ms.
-    auto launch = [&](ListParams &q, int grid, cudaStream_t st) {
-        return ctx->l >= 7 ? launch_lists<4, 24>(q, grid, smem, ctx->smem_optin, st)
-                           : launch_lists<8, 20>(q, grid, smem, ctx->smem_optin, st);
+    auto launch = [&](ListParams &q, int grid, cudaStream_t st, bool dependent) {
+        return ctx->l >= 7 ? launch_lists<4, 24>(q, grid, smem, dependent, st)
+                           : launch_lists<8, 20>(q, grid, smem, dependent, st);
     };
     ListParts parts{};
     parts.n = 1;
@@ -452,21 +466,22 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         parts.slot_base[2] = blocks + extra; parts.g_first[2] = extra; parts.groups[2] = rest; parts.cpg[2] = cpg_b;
         ListParams main = p;
         main.tiles = t1; main.d = shift;
-        e = cudaEventRecord(ctx->ev_fork, s);
+        e = cudaEventRecord(ctx->ev_fork, s);                  // (launches that events order are ordinary ones)
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0);
-        if (e == cudaSuccess) e = launch(ta, extra, ctx->side_stream);
-        if (e == cudaSuccess) e = launch(tb, rest * cpg_b, ctx->side_stream);
+        if (e == cudaSuccess) e = launch(ta, extra, ctx->side_stream, false);
+        if (e == cudaSuccess) e = launch(tb, rest * cpg_b, ctx->side_stream, false);
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_join, ctx->side_stream);
-        if (e == cudaSuccess) e = launch(main, blocks, s);
+        if (e == cudaSuccess) e = launch(main, blocks, s, false);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->ev_join, 0);
     } else {
-        e = launch(p, blocks, s);
+        e = launch(p, blocks, s, true);
     }
     if (e != cudaSuccess) return e;
     const int64_t total = (int64_t)p.groups * (2 + ctx->lm) * GW * 4;
     int fb = (int)((total + 255) / 256);
     if (fb > ctx->n_sm * 8) fb = ctx->n_sm * 8;
-    k_finalize_gather<<<fb, 256, 0, s>>>(p, parts, flags, states);
     ctx->last_ls_launches = parts.n + 1;
+    if (parts.n == 1) return fda_launch_dependent(k_finalize_gather, fb, 256, 0, s, p, parts, flags, states);
+    k_finalize_gather<<<fb, 256, 0, s>>>(p, parts, flags, states);       // waits for an event too: an ordinary launch
     return cudaGetLastError();
 }
