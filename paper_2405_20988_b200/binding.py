@@ -46,6 +46,7 @@ class Estimate(ctypes.Structure):
 
 
 _lib = None
+_native = None      # the calls of a monitoring step, marshalled in C (csrc/fda_py.c)
 
 
 def library_path() -> str:
@@ -54,7 +55,7 @@ def library_path() -> str:
 
 def load_library():
     """Load libfda.so from the package directory (never from anywhere else)."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     path = library_path()
@@ -94,7 +95,12 @@ def load_library():
     for name in ("fda_create", "fda_destroy", "fda_local_state", "fda_combine_estimate",
                  "fda_average_models", "fda_round_host", "fda_debug_hash"):
         getattr(lib, name).restype = c_int
-    _lib = lib
+    if not os.path.exists(os.path.join(os.path.dirname(path), "_native.so")):
+        raise FdaError(3, "load_library", "_native.so not found - run `python -m paper_2405_20988_b200.build`")
+    import torch
+    from . import _native as native
+    native.init(torch.float32, torch.uint8, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+    _native, _lib = native, lib
     return lib
 
 
@@ -133,15 +139,9 @@ def fda_local_state_linear_noalloc(w, w_t0, xi, flags: int, states, stream=None)
     this wrapper creates no tensor either - ``states`` is supplied by the caller.  K may not
     exceed FDA_NOALLOC_MAX_WORKERS.  Calls that overlap on the device race on that scratch.
     """
-    import torch
-    lib = load_library()
-    stride, K, d = _rows(w)
-    if states.dim() != 2 or states.shape[0] != K or states.shape[1] != 2 or not states.is_contiguous():
-        raise ValueError("states must be a contiguous K x 2 tensor")
-    st = lib.fda_local_state_linear_noalloc(w.device.index or 0, _dev_ptr(w, torch.float32, "w"), stride, K, d,
-                                            _dev_ptr(w_t0, torch.float32, "w_t0"),
-                                            _dev_ptr(xi, torch.float32, "xi"), flags,
-                                            _dev_ptr(states, torch.float32, "states"), _stream_ptr(stream))
+    if _native is None:
+        load_library()
+    st = _native.local_state_linear_noalloc(w, w_t0, xi, flags, states, stream)
     if st != 0:
         raise FdaError(st, "fda_local_state_linear_noalloc",
                        "K exceeds FDA_NOALLOC_MAX_WORKERS" if st == 2 else "")
@@ -212,56 +212,37 @@ class FdaContext:
     # -- the C entry points ----------------------------------------------------------------
     def fda_local_state(self, w, w_t0, xi, flags: int, states, stream=None):
         """states[K, state_len] <- local states of the K rows of w (device tensors)."""
-        import torch
-        stride, K, d = _rows(w)
-        st = self._lib.fda_local_state(self._h, _dev_ptr(w, torch.float32, "w"), stride, K, d,
-                                       _dev_ptr(w_t0, torch.float32, "w_t0"),
-                                       _dev_ptr(xi, torch.float32, "xi"), flags,
-                                       _dev_ptr(states, torch.float32, "states"), _stream_ptr(stream))
-        self._check(st, "fda_local_state")
+        st = _native.local_state(self._h.value, w, w_t0, xi, flags, states, stream)
+        if st:
+            self._check(st, "fda_local_state")
 
     def fda_mean_state(self, w, w_t0, xi, flags: int, mean_state, stream=None):
         """mean_state[state_len] <- averaged state S-bar of the K rows of w (device tensors)."""
-        import torch
-        stride, K, d = _rows(w)
-        st = self._lib.fda_mean_state(self._h, _dev_ptr(w, torch.float32, "w"), stride, K, d,
-                                      _dev_ptr(w_t0, torch.float32, "w_t0"),
-                                      _dev_ptr(xi, torch.float32, "xi"), flags,
-                                      _dev_ptr(mean_state, torch.float32, "mean_state"), _stream_ptr(stream))
-        self._check(st, "fda_mean_state")
+        st = _native.mean_state(self._h.value, w, w_t0, xi, flags, mean_state, stream)
+        if st:
+            self._check(st, "fda_mean_state")
 
     def fda_combine_estimate(self, states, K: int, variant: int, epsilon: float, theta: float,
                              est_dev, want_host: bool = True, stream=None):
         """est_dev: uint8 CUDA tensor of sizeof(fda_estimate) bytes.  Returns an Estimate
         (host copy, synchronises the stream) when ``want_host``, else None."""
-        import torch
         host = Estimate() if want_host else None
-        st = self._lib.fda_combine_estimate(self._h, _dev_ptr(states, torch.float32, "states"), K,
-                                            variant, epsilon, theta, _dev_ptr(est_dev, torch.uint8, "est_dev"),
-                                            ctypes.byref(host) if host is not None else None,
-                                            _stream_ptr(stream))
-        self._check(st, "fda_combine_estimate")
+        st = _native.combine_estimate(self._h.value, states, K, variant, epsilon, theta, est_dev,
+                                      ctypes.addressof(host) if want_host else 0, stream)
+        if st:
+            self._check(st, "fda_combine_estimate")
         return host
 
     def fda_average_models(self, w, w_t0, est_dev, flags: int, stream=None):
-        import torch
-        stride, K, d = _rows(w)
-        st = self._lib.fda_average_models(self._h, _dev_ptr(w, torch.float32, "w"), stride, K, d,
-                                          _dev_ptr(w_t0, torch.float32, "w_t0"),
-                                          _dev_ptr(est_dev, torch.uint8, "est_dev"), flags,
-                                          _stream_ptr(stream))
-        self._check(st, "fda_average_models")
+        st = _native.average_models(self._h.value, w, w_t0, est_dev, flags, stream)
+        if st:
+            self._check(st, "fda_average_models")
 
     def fda_average_models_xi(self, w, w_t0, xi_out, est_dev, flags: int, stream=None):
         """fda_average_models that also writes the refreshed unit direction xi_out (d floats)."""
-        import torch
-        stride, K, d = _rows(w)
-        st = self._lib.fda_average_models_xi(self._h, _dev_ptr(w, torch.float32, "w"), stride, K, d,
-                                             _dev_ptr(w_t0, torch.float32, "w_t0"),
-                                             _dev_ptr(xi_out, torch.float32, "xi_out"),
-                                             _dev_ptr(est_dev, torch.uint8, "est_dev"), flags,
-                                             _stream_ptr(stream))
-        self._check(st, "fda_average_models_xi")
+        st = _native.average_models_xi(self._h.value, w, w_t0, xi_out, est_dev, flags, stream)
+        if st:
+            self._check(st, "fda_average_models_xi")
 
     def fda_round_host(self, w_host, w_t0_host, xi_host, state_flags: int, variant: int,
                        epsilon: float, theta: float, avg_flags: int, states_host=None, stream=None):

@@ -1,4 +1,4 @@
-"""Build libfda.so (sm_100a only) next to this file with nvcc.
+"""Build libfda.so (sm_100a only) with nvcc and _native.so (its CPython module) next to this file.
 
 Usage: ``python -m paper_2405_20988_b200.build [--force] [--verbose]``
 """
@@ -7,11 +7,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libfda.so")
+OUT_PY = os.path.join(HERE, "_native.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 SOURCES = ["fda_api.cu", "fda_hash.cu", "fda_local_state.cu", "fda_local_state_gather.cu", "fda_mean_state_gather.cu", "fda_sched.cu", "fda_local_state_linear.cu", "fda_mean_state.cu", "fda_combine.cu", "fda_average.cu", "fda_noalloc.cu", "fda_probe.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
@@ -30,7 +32,7 @@ def _deps_mtime() -> float:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and os.path.exists(OUT) and os.path.getmtime(OUT) >= _deps_mtime():
+    if not force and all(os.path.exists(o) and os.path.getmtime(o) >= _deps_mtime() for o in (OUT, OUT_PY)):
         return OUT
     os.makedirs(OBJ_DIR, exist_ok=True)
     extra = ["-Xptxas", "-v"] if verbose else []
@@ -50,6 +52,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = OUT + ".tmp%d" % os.getpid()
     subprocess.check_call([_nvcc(), *ARCH, "-shared", "-o", tmp, *objs])
     os.replace(tmp, OUT)
+    tmp = OUT_PY + ".tmp%d" % os.getpid()
+    subprocess.check_call(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
+                           os.path.join(CSRC, "fda_py.c"), "-o", tmp, "-L" + HERE, "-l:libfda.so",
+                           "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, OUT_PY)
     return OUT
 
 
