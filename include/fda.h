@@ -86,7 +86,7 @@ typedef struct {
  * Device memory the context takes (fda_context_info reports the figures):
  *   - per-block partial sums: (SM count) * l*m * 128 bytes plus 64 * (SM count) * max(K_max, 32) bytes;
  *   - the list schedule of the sketch kernel, when the sketch allows one (tiles of at least 6*m
- *     indices fit the shared memory): about 2.4 * l bytes per index of d_max (2.4 GB for
+ *     indices fit the shared memory, or of 5*m with the rows in two or four equal parts): about 2.4 * l bytes per index of d_max (2.4 GB for
  *     d_max = 2 * 10^8 and l = 5), built here in about 4 ms per million indices; it is dropped,
  *     and sketch requests are then served by the slower plain-load kernels, when it would take
  *     more than a third of the free device memory (see fda_create_limited for another cap);
@@ -266,6 +266,8 @@ fda_status fda_debug_read_probe(fda_ctx *ctx, const float *src, int64_t n, float
  *       chunk[lane][4] u16 entries for steps 4c .. 4c+3 of an item; entry = row of the drift
  *       tile (bits 0..12) | sign << 15, where index r of the tile is stored in row
  *       r ^ ((r >> 3) & 3) and rows tile_indices + r, r < 8, are padding (zeros).
+ * A sketch whose rows are in several parts (see fda_create) has the records of the first part, tile
+ * after tile, then those of the next one; l and the rows of a record are then those of the part.
  * In every step the eight lanes 8q .. 8q+7 of an item address rows in eight different 16-byte
  * bank groups (row mod 8), so that the shared-memory load of the step is conflict free.
  * record_host: host buffer of `capacity` bytes, receives min(capacity, record_bytes) bytes.

@@ -406,7 +406,7 @@ fda_status fda_debug_schedule(const fda_ctx *ctx, int64_t tile, void *record_hos
 {
     if (!ctx || !record_host || !info) return FDA_ERR_INVALID_ARG;
     if (!ctx->sched) return FDA_ERR_UNSUPPORTED;
-    if (tile < 0 || tile >= ctx->sched_tiles) return FDA_ERR_INVALID_ARG;
+    if (tile < 0 || tile >= ctx->sched_tiles * ctx->sched_parts) return FDA_ERR_INVALID_ARG;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return FDA_ERR_CUDA;
     uint64_t off[2] = {0, 0};
@@ -417,7 +417,7 @@ fda_status fda_debug_schedule(const fda_ctx *ctx, int64_t tile, void *record_hos
     info[1] = kListSlots;
     info[2] = kListMaxLen;
     info[3] = (int64_t)(off[1] - off[0]);
-    info[4] = ctx->sched_tiles;
+    info[4] = ctx->sched_tiles * ctx->sched_parts;
     info[5] = kListPadRows;
     info[6] = kListOct;
     info[7] = (int64_t)ctx->sched_bytes;
@@ -431,7 +431,7 @@ fda_status fda_context_info(const fda_ctx *ctx, int64_t *info)
 {
     if (!ctx || !info) return FDA_ERR_INVALID_ARG;
     const int64_t table = ctx->tab ? (int64_t)(sizeof(uint16_t) * (size_t)ctx->l * ctx->tab_stride) : 0;
-    const int64_t sched = ctx->sched ? (int64_t)(ctx->sched_bytes + sizeof(uint64_t) * (size_t)(ctx->sched_tiles + 1)) : 0;
+    const int64_t sched = ctx->sched ? (int64_t)(ctx->sched_bytes + sizeof(uint64_t) * (size_t)(ctx->sched_tiles * ctx->sched_parts + 1)) : 0;
     const int64_t partial = (int64_t)(sizeof(float) * ctx->part_sk_floats + sizeof(double) * ctx->part_np_doubles +
                                       sizeof(double) * fda_combine_scratch_doubles(ctx->l, ctx->m) + sizeof(unsigned int) * (1 + ctx->n_row_tickets)) +
                             (ctx->coeffs_dev ? (int64_t)sizeof(uint64_t) * 6 * ctx->l : 0);

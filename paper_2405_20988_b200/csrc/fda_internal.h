@@ -59,13 +59,14 @@ struct fda_ctx {
     int max_blocks = 0;
     // list schedule of the sorted-list sketch kernel (null when not built)
     unsigned char *sched = nullptr;   // records of the tiles, 256-byte aligned
-    uint64_t *sched_off = nullptr;    // [tiles + 1] byte offsets of the records
+    uint64_t *sched_off = nullptr;    // [parts * tiles + 1] byte offsets of the records
     uint64_t sched_bytes = 0;         // size of the schedule
     uint64_t sched_skipped_bytes = 0; // size of a schedule that was not kept (memory limit)
     int64_t sched_limit_bytes = 0;    // caller's cap on the schedule (0: a third of the free memory)
     int sched_T = 0;                  // indices per tile
     int sched_ni_max = 0;             // items a record can have
     int64_t sched_tiles = 0;
+    int sched_parts = 1;              // equal parts of the sketch rows that have records of their own
     double sched_build_ms = 0.0;      // host time spent building it
     float *mean_model = nullptr;      // d_max floats (average drift), allocated by the first fda_mean_state
     // a second stream for the launches that fill the SMs the main launch of the list kernel leaves idle

@@ -18,8 +18,11 @@ struct ListParams {
     int64_t d;
     int have_xi;
     int vec;                         // 16-byte aligned inputs: the producers load 128 bits at a time
-    int l, m;
+    int l, m;                        // sketch rows of a part, columns
     int groups, cpg;                 // block = c * groups + g
+    int wgroups;                     // worker groups: g = part * wgroups + worker group
+    int part_tiles;                  // several parts: records of a part of the sketch rows;
+                                     // one part: blocks that share the items of a tile
     int T, nb;                       // indices and batches per tile
     int64_t tiles;                   // tiles that hold indices below d
     int tab_bytes;                   // bytes of one item-table buffer in shared memory
@@ -103,6 +106,39 @@ __device__ __forceinline__ void gather_lo(uint32_t w, uint32_t base, unsigned lo
 __device__ __forceinline__ void gather_hi(uint32_t w, uint32_t base, unsigned long long &a01, unsigned long long &a23)
 {
     gather_row((w >> 12) & 0x1fff0u, (w & 0x80000000u) ^ 0x3f800000u, base, a01, a23);
+}
+
+// one chunk of an item: the steps that are left of it, at most four
+__device__ __forceinline__ void walk_chunk(const uint2 &ch, int left, uint32_t base, unsigned long long &a01, unsigned long long &a23)
+{
+    if (left >= 4) {
+        gather_lo(ch.x, base, a01, a23);
+        gather_hi(ch.x, base, a01, a23);
+        gather_lo(ch.y, base, a01, a23);
+        gather_hi(ch.y, base, a01, a23);
+    } else if (left > 0) {
+        gather_lo(ch.x, base, a01, a23);
+        if (left > 1) gather_hi(ch.x, base, a01, a23);
+        if (left > 2) gather_lo(ch.y, base, a01, a23);
+    }
+}
+// the sums of an item's 32 lists into the bins
+__device__ __forceinline__ void flush_item(float *bins, int lm, uint32_t cell, unsigned long long a01, unsigned long long a23)
+{
+    float4 acc;
+    asm("mov.b64 {%0,%1}, %2;" : "=f"(acc.x), "=f"(acc.y) : "l"(a01));
+    asm("mov.b64 {%0,%1}, %2;" : "=f"(acc.z), "=f"(acc.w) : "l"(a23));
+    if ((cell & 0x7fffu) < (uint32_t)lm) {
+        float *b = bins + (cell & 0x7fffu) * GW;
+        if (cell & 0x8000u) {                           // a cell with several lists
+            atomicAdd(b + 0, acc.x); atomicAdd(b + 1, acc.y);
+            atomicAdd(b + 2, acc.z); atomicAdd(b + 3, acc.w);
+        } else {
+            float4 o = *reinterpret_cast<float4 *>(b);
+            o.x += acc.x; o.y += acc.y; o.z += acc.z; o.w += acc.w;
+            *reinterpret_cast<float4 *>(b) = o;
+        }
+    }
 }
 
 }  // namespace fda_list

@@ -30,6 +30,17 @@
 // buffer with tile n + 1, and one block-wide barrier per tile hands the buffers over.  Nothing
 // in this kernel waits on another block or spins on memory.
 //
+// What bounds it: the load/store unit's data pipe (about 72 % busy; 6.3 wavefronts per 128 updates
+// are the floor of this design, 8.3 are spent).  Between two items a walker has nothing to gather,
+// so the way from item to item is kept short: the record's offset comes from shared memory (read
+// from L2 after the barrier it stood in front of the first entries of every tile), the first item of
+// a tile goes to a warp by its number, and the next item's number and descriptor are fetched before
+// the walk of the current one.  5 x 250, K = 8, d = 198M: 2.44 -> 2.38 ms; K = 30, d = 7M: 372 -> 356 us;
+// 7 x 500, K = 60, d = 20M: 2.98 -> 2.89 ms.  Tried and slower: hand-over through mbarriers instead of
+// the barrier (2.52 ms: the bins still need the walkers to meet between tiles, or two of them would
+// add to one cell at a time), entries of the next item asked for before the flush (2.61 ms), 24
+// walkers at 64 registers (2.40 ms).
+//
 // fda_mean_state_gather.cu holds the sibling of this kernel that computes the averaged state of
 // fda_mean_state from the same schedule.
 
@@ -44,13 +55,20 @@ using namespace fda_list;
 
 // Shared-memory plan (bytes from the start of dynamic shared memory):
 //   [0, 8)    item counters of the two tile buffers
+//   [16, 48)  offsets of the schedule records of the tiles n, n + 1 (slot n mod 4)
 //   [64, 1088) sums[producer warp][worker][2] (fp64): ||u||^2 and <xi,u> over the tiles so far
 //   [1088, ..) two item tables (tab_bytes each): the head of a tile's schedule record
 //   then      bins[l*m][4]
 //   then      ut[2][T + 8][4]   (drift tiles, index-major; eight zero rows behind each)
 // PW producer warps and WW walker warps: the split that is fastest depends on how much walking a
-// loaded index pays for (l updates per worker).
-template <bool LINEAR, int PW, int WW>
+// loaded index pays for (l updates per worker).  PARTS: the sketch rows are in several parts with
+// records of their own, and a block serves one part of one worker group.  SPLIT: a vector of few
+// tiles leaves most SMs without a block, so p.part_tiles blocks share the tile of each: all of them form
+// the drifts, each walks every p.part_tiles-th item, and their bins, which differ in the cells they touch,
+// are partial sums like those of any other blocks (so the cells come out the same bit for bit).
+// Measured: 8 x 1000 as two parts, K = 20, d = 2.6M: 224 us, against 510 us on the compare-and-swap
+// kernel that served it before; shared tiles, 5 x 250, K = 5, d = 61,706: 12.5 -> 10 us.
+template <bool LINEAR, int PW, int WW, bool PARTS, bool SPLIT>
 __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const ListParams p)
 {
     constexpr int kProducerWarps = PW;
@@ -61,15 +79,20 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     // average 28 steps), or five with the 4 + 24 split, whose items average eleven steps.  Measured:
     // 7 x 500, K = 60, d = 20M: 2.94 ms with 5, 2.98 with 4, 2.96 with 6, 3.01 with 7, 3.06 with 8;
     // 5 x 250, K = 8, d = 198M with 8 + 20 warps: 2.474 ms with 7, 2.481 with 8, 2.51 with 6, 2.52 with 10
-    constexpr int kAhead = (WW == 24) ? 5 : 7;
+    constexpr int kAhead = PARTS ? 2 : (WW == 24) ? 5 : 7;
     static_assert(PW <= kMaxProducerWarps, "the fp64 sums have room for kMaxProducerWarps warps");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = (int)blockIdx.x % p.groups, c = (int)blockIdx.x / p.groups;
+    const int sub = SPLIT ? (int)blockIdx.x / (p.groups * p.cpg) : 0, split = SPLIT ? p.part_tiles : 1;
+    const int blk = SPLIT ? (int)blockIdx.x % (p.groups * p.cpg) : (int)blockIdx.x;
+    const int vg = blk % p.groups, c = blk / p.groups;
+    const int g = PARTS ? vg % p.wgroups : vg;
+    const uint64_t *sched_off = PARTS ? p.sched_off + (size_t)(vg / p.wgroups) * p.part_tiles : p.sched_off;
     const int T = p.T, lm = p.l * p.m;
 
     const uint32_t smem_base = (uint32_t)__cvta_generic_to_shared(smem_raw);
     int *ctr = reinterpret_cast<int *>(smem_raw);
+    unsigned long long *rec_off = reinterpret_cast<unsigned long long *>(smem_raw + 16);
     double *sums = reinterpret_cast<double *>(smem_raw + 64);
     const uint32_t tab_off = kListSmemHead;
     const uint32_t bins_off = tab_off + 2u * (uint32_t)p.tab_bytes;
@@ -127,9 +150,10 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
         // head of the schedule record of the tile being stored (the walkers' item table) and the
         // record offsets of the next tile, loaded one and two tiles ahead of their use
         uint4 tabv = make_uint4(0u, 0u, 0u, 0u);
-        unsigned long long off0 = load_u64(p.sched_off + c), off1 = load_u64(p.sched_off + c + 1);
+        unsigned long long off0 = load_u64(sched_off + c), off1 = load_u64(sched_off + c + 1);
         if (pt * 16 < p.tab_bytes) tabv = load_u4(p.sched + off0 + pt * 16);
-        if (n_tiles > 1) { off0 = load_u64(p.sched_off + c + p.cpg); off1 = load_u64(p.sched_off + c + p.cpg + 1); }
+        if (pt == 0) rec_off[0] = off0;
+        if (n_tiles > 1) { off0 = load_u64(sched_off + c + p.cpg); off1 = load_u64(sched_off + c + p.cpg + 1); }
         auto issue = [&](int slot) {
             if (n_i < n_tiles) {
                 const float *q = wbase + j_i;
@@ -196,7 +220,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                 // of the one after: nothing here waits for memory
                 if (pt * 16 < p.tab_bytes)
                     *reinterpret_cast<uint4 *>(smem_raw + tab_off + (size_t)buf * p.tab_bytes + pt * 16) = tabv;
-                if (pt == 0) ctr[buf] = 0;
+                if (pt == 0) { ctr[buf] = WW; rec_off[(n_c + 1) & 3] = off0; }
                 if (n_c + 1 < n_tiles) {
                     const unsigned char *nrec = p.sched + off0;
                     if (pt * 16 < p.tab_bytes) tabv = load_u4(nrec + pt * 16);
@@ -205,8 +229,8 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                 }
                 if (n_c + 2 < n_tiles) {
                     const int64_t t2 = c + (n_c + 2) * p.cpg;
-                    off0 = load_u64(p.sched_off + t2);
-                    off1 = load_u64(p.sched_off + t2 + 1);
+                    off0 = load_u64(sched_off + t2);
+                    off1 = load_u64(sched_off + t2 + 1);
                 }
                 prefetch_tile(n_c + 2);
                 block_barrier<kThreads>();
@@ -227,22 +251,60 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
         for (int64_t n = 0; n < n_tiles; ++n) {
             block_barrier<kThreads>();                                   // tile n is stored, tile n - 1 is walked
             const int buf = (int)(n & 1);
-            const unsigned char *rec = p.sched + p.sched_off[c + n * p.cpg];
+            // (the record's offset comes from shared memory: a load from L2 here would stand in front of
+            // the first entries of every tile)
+            const unsigned char *rec = p.sched + rec_off[n & 3];
             const uint32_t *tab = reinterpret_cast<const uint32_t *>(smem_raw + tab_off + (size_t)buf * p.tab_bytes);
             const int n_items = (int)tab[0];
             const uint16_t *cells = reinterpret_cast<const uint16_t *>(rec + fda_sched_cells_off(n_items));
             const unsigned char *ent0 = rec + fda_sched_entries_off(n_items);
             const uint32_t base = smem_base + ut_off + (uint32_t)buf * ut_bytes;
-            for (;;) {
-                int it = 0;
-                if (lane == 0) it = atomicAdd(&ctr[buf], 1);
-                it = __shfl_sync(0xffffffffu, it, 0);
-                if (it >= n_items) break;
-                const uint32_t d0 = tab[4 + 2 * it], chunk0 = tab[5 + 2 * it];
+            if constexpr (PARTS) {
+                // Short lists (a few steps an item): what an item costs is the way to its entries.  The
+                // next item's cell and entries are asked for before this one is walked.
+                struct Item { int steps; uint32_t cell; const uint2 *ent; uint2 ch[kAhead]; };
+                int it = warp - kProducerWarps;
+                auto fetch = [&](Item &x) {
+                    const uint32_t d0 = tab[4 + 2 * it], chunk0 = tab[5 + 2 * it];
+                    x.steps = (int)(d0 & 0xffffu);
+                    x.cell = cells[(size_t)(d0 >> 16) * kListSlots + lane];
+                    x.ent = reinterpret_cast<const uint2 *>(ent0 + (size_t)chunk0 * 256) + lane;
+#pragma unroll
+                    for (int q = 0; q < kAhead; ++q)
+                        if (4 * q < x.steps) x.ch[q] = __ldg(x.ent + (size_t)q * kListSlots);
+                };
+                auto take = [&]() {
+                    if (lane == 0) it = atomicAdd(&ctr[buf], 1);
+                    it = __shfl_sync(0xffffffffu, it, 0);
+                };
+                auto walk = [&](Item &x) {
+                    unsigned long long a01 = 0ull, a23 = 0ull;
+#pragma unroll
+                    for (int q = 0; q < kAhead; ++q) walk_chunk(x.ch[q], x.steps - 4 * q, base, a01, a23);
+                    for (int c0 = kAhead; 4 * c0 < x.steps; ++c0)
+                        walk_chunk(__ldg(x.ent + (size_t)c0 * kListSlots), x.steps - 4 * c0, base, a01, a23);
+                    flush_item(bins, lm, x.cell, a01, a23);
+                };
+                Item a;
+                if (it < n_items) fetch(a);
+                while (it < n_items) {
+                    Item b = a;
+                    take();
+                    if (it < n_items) fetch(a);
+                    walk(b);
+                }
+            } else {
+            int it = (warp - kProducerWarps) * split + sub;
+            uint32_t d0 = 0, chunk0 = 0;
+            if (it < n_items) { d0 = tab[4 + 2 * it]; chunk0 = tab[5 + 2 * it]; }
+            while (it < n_items) {
                 const int steps = (int)(d0 & 0xffffu);
                 const uint32_t cell = cells[(size_t)(d0 >> 16) * kListSlots + lane];
                 const uint2 *ent = reinterpret_cast<const uint2 *>(ent0 + (size_t)chunk0 * 256) + lane;
                 const int nch = (steps + 3) >> 2;
+                if (lane == 0) it = atomicAdd(&ctr[buf], 1) * split + sub;
+                it = __shfl_sync(0xffffffffu, it, 0);
+                if (it < n_items) { d0 = tab[4 + 2 * it]; chunk0 = tab[5 + 2 * it]; }
                 unsigned long long a01 = 0ull, a23 = 0ull;
                 // all entry loads of (up to) kAhead chunks first, then the walk: the entries come
                 // from global memory (L2), one round trip per kAhead chunks instead of one per chunk
@@ -252,34 +314,10 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                     for (int q = 0; q < kAhead; ++q)
                         if (c0 + q < nch) ch[q] = __ldg(ent + (size_t)(c0 + q) * kListSlots);
 #pragma unroll
-                    for (int q = 0; q < kAhead; ++q) {
-                        const int left = steps - 4 * (c0 + q);
-                        if (left >= 4) {
-                            gather_lo(ch[q].x, base, a01, a23);
-                            gather_hi(ch[q].x, base, a01, a23);
-                            gather_lo(ch[q].y, base, a01, a23);
-                            gather_hi(ch[q].y, base, a01, a23);
-                        } else if (left > 0) {
-                            gather_lo(ch[q].x, base, a01, a23);
-                            if (left > 1) gather_hi(ch[q].x, base, a01, a23);
-                            if (left > 2) gather_lo(ch[q].y, base, a01, a23);
-                        }
-                    }
+                    for (int q = 0; q < kAhead; ++q) walk_chunk(ch[q], steps - 4 * (c0 + q), base, a01, a23);
                 }
-                float4 acc;
-                asm("mov.b64 {%0,%1}, %2;" : "=f"(acc.x), "=f"(acc.y) : "l"(a01));
-                asm("mov.b64 {%0,%1}, %2;" : "=f"(acc.z), "=f"(acc.w) : "l"(a23));
-                if ((cell & 0x7fffu) < (uint32_t)lm) {
-                    float *b = bins + (cell & 0x7fffu) * GW;
-                    if (cell & 0x8000u) {                           // a cell with several lists
-                        atomicAdd(b + 0, acc.x); atomicAdd(b + 1, acc.y);
-                        atomicAdd(b + 2, acc.z); atomicAdd(b + 3, acc.w);
-                    } else {
-                        float4 o = *reinterpret_cast<float4 *>(b);
-                        o.x += acc.x; o.y += acc.y; o.z += acc.z; o.w += acc.w;
-                        *reinterpret_cast<float4 *>(b) = o;
-                    }
-                }
+                flush_item(bins, lm, cell, a01, a23);
+            }
             }
         }
     }
@@ -294,7 +332,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     if (tid < GW * 2) {
         double t = 0.0;
         for (int q = 0; q < kProducerWarps; ++q) t += sums[q * GW * 2 + tid];
-        p.part_np[(size_t)blockIdx.x * GW * 2 + tid] = t;
+        p.part_np[(size_t)blockIdx.x * GW * 2 + tid] = sub == 0 ? t : 0.0;
     }
 }
 
@@ -312,9 +350,9 @@ struct ListParts {
 // each launch in order (eight loads in flight), and the four sums are added as (s0 + s1) + (s2 + s3).
 __global__ void k_finalize_gather(const ListParams p, const ListParts parts, uint32_t flags, float *__restrict__ states)
 {
-    const int lm = p.l * p.m, slen = 2 + lm;
+    const int lm = p.l * p.m, slen = 2 + lm * (p.groups / p.wgroups);       // lm: cells of a part
     const bool sketch = (flags & FDA_STATE_SKETCH) != 0;
-    const int64_t total = (int64_t)p.groups * slen * GW * 4;
+    const int64_t total = (int64_t)p.wgroups * slen * GW * 4;
     const int64_t padded = (total + 31) & ~(int64_t)31;                 // whole warps take part in the shuffles
     fda_grid_wait();
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < padded;
@@ -328,7 +366,8 @@ __global__ void k_finalize_gather(const ListParams p, const ListParts parts, uin
         const int k = g * GW + kl;
         double acc = 0.0;
         for (int q = 0; q < parts.n; ++q) {
-            const int gl = g - parts.g_first[q];
+            const int part = e < 2 ? 0 : (e - 2) / lm;                  // part 0 also has the norm and the projection
+            const int gl = part * p.wgroups + g - parts.g_first[q];
             if (!valid || gl < 0 || gl >= parts.groups[q]) continue;
             const int nb = parts.cpg[q];                                // blocks of this group: gl, gl + groups, ...
             const size_t first = (size_t)(parts.slot_base[q] + gl);
@@ -340,7 +379,7 @@ __global__ void k_finalize_gather(const ListParams p, const ListParts parts, uin
                         acc += p.part_np[((first + (size_t)j * parts.groups[q]) * GW + kl) * 2 + e];
             } else if (sketch) {
                 const size_t step = (size_t)lm * GW * parts.groups[q];  // from one block of the group to the next
-                const float *src = p.part_sk + first * lm * GW + (size_t)(e - 2) * GW + kl + (size_t)sub * step;
+                const float *src = p.part_sk + first * lm * GW + (size_t)(e - 2 - part * lm) * GW + kl + (size_t)sub * step;
                 int j = sub;
                 for (; j + 28 < nb; j += 32, src += 32 * step) {
                     float v[8];
@@ -358,12 +397,12 @@ __global__ void k_finalize_gather(const ListParams p, const ListParts parts, uin
     }
 }
 
-template <int PW, int WW>
+template <int PW, int WW, bool PARTS, bool SPLIT>
 cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent, cudaStream_t s)
 {
     if (p.T % (PW * 128) != 0 || PW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
     p.nb = p.T / (PW * 128);
-    auto kern = p.have_xi ? k_local_state_gather<true, PW, WW> : k_local_state_gather<false, PW, WW>;
+    auto kern = p.have_xi ? k_local_state_gather<true, PW, WW, PARTS, SPLIT> : k_local_state_gather<false, PW, WW, PARTS, SPLIT>;
     if (dependent) return fda_launch_dependent(kern, blocks, (PW + WW) * 32, smem, s, p);
     kern<<<blocks, (PW + WW) * 32, smem, s>>>(p);
     return cudaGetLastError();
@@ -374,14 +413,15 @@ cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent,
 // The kernels' dynamic shared memory limit, set once per context (on the context's device).
 cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx)
 {
-    auto set = [&](void (*kern)(ListParams)) {
-        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
-    };
-    cudaError_t e = set(k_local_state_gather<true, 8, 20>);
-    if (e == cudaSuccess) e = set(k_local_state_gather<false, 8, 20>);
-    if (e == cudaSuccess) e = set(k_local_state_gather<true, 4, 24>);
-    if (e == cudaSuccess) e = set(k_local_state_gather<false, 4, 24>);
-    return e;
+    for (auto kern : {k_local_state_gather<true, 8, 20, false, false>, k_local_state_gather<false, 8, 20, false, false>,
+                      k_local_state_gather<true, 4, 24, false, false>, k_local_state_gather<false, 4, 24, false, false>,
+                      k_local_state_gather<true, 8, 24, true, false>, k_local_state_gather<false, 8, 24, true, false>,
+                      k_local_state_gather<true, 16, 12, false, true>, k_local_state_gather<false, 16, 12, false, true>,
+                      k_local_state_gather<true, 8, 20, false, true>, k_local_state_gather<false, 8, 20, false, true>}) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Returns cudaErrorNotSupported when the request does not fit this path (the caller then uses
@@ -397,36 +437,49 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     p.w = w; p.w_t0 = w_t0; p.xi = xi_used; p.row_stride = row_stride;
     p.K = K; p.d = d; p.have_xi = xi_used != nullptr;
     p.vec = ((((uintptr_t)w | (uintptr_t)w_t0 | (uintptr_t)(xi_used ? xi_used : w)) & 15u) == 0) && (row_stride % 4 == 0);
-    p.l = ctx->l; p.m = ctx->m;
+    p.l = ctx->l / ctx->sched_parts; p.m = ctx->m;
+    p.part_tiles = (int)ctx->sched_tiles;
     p.T = ctx->sched_T;
     p.sched = ctx->sched; p.sched_off = ctx->sched_off;
     p.part_sk = ctx->part_sk; p.part_np = ctx->part_np;
     p.tiles = (d + p.T - 1) / p.T;
     p.tab_bytes = fda_list_table_bytes(ctx->sched_ni_max);
-    p.groups = (K + GW - 1) / GW;
+    p.wgroups = (K + GW - 1) / GW;
+    p.groups = p.wgroups * ctx->sched_parts;
     if (p.groups > ctx->n_sm) return cudaErrorNotSupported;
     int64_t cpg = ctx->n_sm / p.groups;
     if (cpg > p.tiles) cpg = p.tiles;
     // short jobs stay with the other kernels
     if (p.tiles < (int64_t)kListMinTilesPerBlock * cpg) return cudaErrorNotSupported;
     p.cpg = (int)cpg;
-    const int blocks = p.groups * p.cpg;
-    if ((size_t)blocks * ctx->lm * GW > ctx->part_sk_floats || blocks > ctx->max_blocks ||
+    const int blocks = p.groups * p.cpg, lm = p.l * p.m;
+    if ((size_t)blocks * lm * GW > ctx->part_sk_floats || blocks > ctx->max_blocks ||
         (size_t)blocks * GW * 2 > ctx->part_np_doubles)
         return cudaErrorNotSupported;
     const size_t smem = fda_list_smem_bytes(p.l, p.m, p.T, ctx->sched_ni_max);
     if (smem > (size_t)ctx->smem_optin) return cudaErrorNotSupported;
 
+    // A vector with at most one tile per block and SMs left for as many blocks again: the items of a
+    // tile are split, and with less walking per block more of its warps load (the drifts of a tile are
+    // a chain of round trips, one per batch: three with 16 producer warps, six with 8).
+    int split = 1;
+    if (ctx->sched_parts == 1) {
+        if (p.tiles == p.cpg && 2 * blocks <= ctx->n_sm) split = std::min(8, ctx->n_sm / blocks);
+        p.part_tiles = split;
+    }
     // 8 producer + 20 walker warps, or 4 + 24 when a loaded index pays for more walking.  Measured:
     // 7 x 500, K = 60, d = 20M: 3.34 ms with 4 + 24 against 3.71 ms with 8 + 20; 5 x 250, K = 8,
     // d = 198M: 3.49 against 2.49 ms; 5 x 250, K = 30, d = 7M: 0.535 against 0.387 ms.
     auto launch = [&](ListParams &q, int grid, cudaStream_t st, bool dependent) {
-        return ctx->l >= 7 ? launch_lists<4, 24>(q, grid, smem, dependent, st)
-                           : launch_lists<8, 20>(q, grid, smem, dependent, st);
+        if (ctx->sched_parts > 1) return launch_lists<8, 24, true, false>(q, grid, smem, dependent, st);
+        if (split > 1) return q.T % 2048 == 0 ? launch_lists<16, 12, false, true>(q, grid, smem, dependent, st)
+                                                : launch_lists<8, 20, false, true>(q, grid, smem, dependent, st);
+        return p.l >= 7 ? launch_lists<4, 24, false, false>(q, grid, smem, dependent, st)
+                        : launch_lists<8, 20, false, false>(q, grid, smem, dependent, st);
     };
     ListParts parts{};
     parts.n = 1;
-    parts.slot_base[0] = 0; parts.g_first[0] = 0; parts.groups[0] = p.groups; parts.cpg[0] = p.cpg;
+    parts.slot_base[0] = 0; parts.g_first[0] = 0; parts.groups[0] = p.groups; parts.cpg[0] = p.cpg * split;
 
     // When the groups do not divide the SMs (K = 60: 15 groups x 9 blocks on 148 SMs) the SMs left
     // over get the last tiles of every group, from the same kernel launched on a second stream with
@@ -438,7 +491,7 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     const int rest = p.groups - extra;                         // groups of the second tail launch (extra < groups)
     int64_t t1 = p.tiles;
     int cpg_b = 0;
-    if (extra > 0 && rest > 0 && extra / rest >= 1 && ctx->side_stream && p.tiles >= 64 * (int64_t)p.cpg) {
+    if (ctx->sched_parts == 1 && extra > 0 && rest > 0 && extra / rest >= 1 && ctx->side_stream && p.tiles >= 64 * (int64_t)p.cpg) {
         cpg_b = extra / rest;
         // tail walks per block: n_tail + n_tail / cpg_b; main walks per block: (tiles - n_tail) / cpg
         const double per_tail = 1.0 + 1.0 / (double)cpg_b;
@@ -447,7 +500,7 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         const int64_t main_walks = (p.tiles - n_tail + p.cpg - 1) / p.cpg;
         const size_t slots = (size_t)blocks + extra + (size_t)rest * cpg_b;
         if (n_tail >= 4 * cpg_b && main_walks + 2 < (p.tiles + p.cpg - 1) / p.cpg &&
-            slots * ctx->lm * GW <= ctx->part_sk_floats && slots * GW * 2 <= ctx->part_np_doubles)
+            slots * lm * GW <= ctx->part_sk_floats && slots * GW * 2 <= ctx->part_np_doubles)
             t1 = p.tiles - n_tail;
     }
     cudaError_t e;
@@ -457,10 +510,10 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         ta.w = p.w + shift; ta.w_t0 = p.w_t0 + shift; ta.xi = p.xi ? p.xi + shift : nullptr;
         ta.d = p.d - shift; ta.tiles = p.tiles - t1; ta.sched_off = p.sched_off + t1;
         ListParams tb = ta;
-        ta.K = extra * GW; ta.groups = extra; ta.cpg = 1;
-        ta.part_sk = p.part_sk + (size_t)blocks * ctx->lm * GW; ta.part_np = p.part_np + (size_t)blocks * GW * 2;
-        tb.w = ta.w + (size_t)extra * GW * (size_t)row_stride; tb.K = K - extra * GW; tb.groups = rest; tb.cpg = cpg_b;
-        tb.part_sk = ta.part_sk + (size_t)extra * ctx->lm * GW; tb.part_np = ta.part_np + (size_t)extra * GW * 2;
+        ta.K = extra * GW; ta.groups = ta.wgroups = extra; ta.cpg = 1;
+        ta.part_sk = p.part_sk + (size_t)blocks * lm * GW; ta.part_np = p.part_np + (size_t)blocks * GW * 2;
+        tb.w = ta.w + (size_t)extra * GW * (size_t)row_stride; tb.K = K - extra * GW; tb.groups = tb.wgroups = rest; tb.cpg = cpg_b;
+        tb.part_sk = ta.part_sk + (size_t)extra * lm * GW; tb.part_np = ta.part_np + (size_t)extra * GW * 2;
         parts.n = 3;
         parts.slot_base[1] = blocks; parts.g_first[1] = 0; parts.groups[1] = extra; parts.cpg[1] = 1;
         parts.slot_base[2] = blocks + extra; parts.g_first[2] = extra; parts.groups[2] = rest; parts.cpg[2] = cpg_b;
@@ -474,10 +527,10 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         if (e == cudaSuccess) e = launch(main, blocks, s, false);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->ev_join, 0);
     } else {
-        e = launch(p, blocks, s, true);
+        e = launch(p, blocks * split, s, true);
     }
     if (e != cudaSuccess) return e;
-    const int64_t total = (int64_t)p.groups * (2 + ctx->lm) * GW * 4;
+    const int64_t total = (int64_t)p.wgroups * (2 + ctx->lm) * GW * 4;
     int fb = (int)((total + 255) / 256);
     if (fb > ctx->n_sm * 8) fb = ctx->n_sm * 8;
     ctx->last_ls_launches = parts.n + 1;

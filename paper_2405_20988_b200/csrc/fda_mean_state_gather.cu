@@ -138,6 +138,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
     if (tid < 2) ctr[tid] = 0;
     if (tid < kPW * 2) sums[tid] = 0.0;
     __syncthreads();
+    fda_grid_wait();
 
     const int64_t n_tiles = p.tiles > c ? (p.tiles - c + p.cpg - 1) / p.cpg : 0;
 
@@ -325,10 +326,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
 // part_np[b * 2 + e], b < np_blocks - this kernel's own partials, or those of the pass that
 // averaged the drifts - and divided by K.
 __global__ void k_finalize_mean_gather(const float *__restrict__ part_sk, const double *__restrict__ part_np,
-                                       int blocks, int np_blocks, int lm, int K, uint32_t flags, bool have_xi,
-                                       double cell_div, float *__restrict__ mean_state)
+                                       int blocks, int np_blocks, int cells, int lm /* of a part */, int K, uint32_t flags,
+                                       bool have_xi, double cell_div, float *__restrict__ mean_state)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    fda_grid_wait();
     if (blockIdx.x == 0 && warp < 2) {          // the scalars: lanes stride the partials, fixed shuffle tree
         const int e = warp;
         const bool on = (e == 0) ? (flags & FDA_STATE_NORM) != 0 : ((flags & FDA_STATE_LINEAR) != 0 && have_xi);
@@ -340,10 +342,10 @@ __global__ void k_finalize_mean_gather(const float *__restrict__ part_sk, const 
         if (lane == 0) mean_state[e] = (float)(acc / (double)K);
     }
     const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= lm) return;
+    if (cell >= cells) return;
     double acc = 0.0;
     if (flags & FDA_STATE_SKETCH) {
-        const float *src = part_sk + cell;
+        const float *src = part_sk + (size_t)(cell / lm) * blocks * lm + cell % lm;
         int b = 0;
         for (; b + 8 <= blocks; b += 8) {
             float v[8];
@@ -375,7 +377,10 @@ cudaError_t launch_mean(fda_ctx *ctx, const float *w, int64_t row_stride, int ro
     mp.sketch_only = base_zero;
     p.vec = ((((uintptr_t)w | (uintptr_t)(base_zero ? w : w_t0) | (uintptr_t)(xi_used ? xi_used : w)) & 15u) == 0) &&
             (row_stride % 4 == 0);
-    p.l = ctx->l; p.m = ctx->m;
+    const int parts = ctx->sched_parts;
+    if (parts > 1 && !base_zero) return cudaErrorNotSupported;      // every part would read the K rows again
+    p.l = ctx->l / parts; p.m = ctx->m;
+    const int lm = p.l * p.m;
     p.T = ctx->sched_T;
     p.sched = ctx->sched; p.sched_off = ctx->sched_off;
     p.part_sk = ctx->part_sk; p.part_np = ctx->part_np;
@@ -386,7 +391,7 @@ cudaError_t launch_mean(fda_ctx *ctx, const float *w, int64_t row_stride, int ro
     if (cpg > p.tiles) cpg = p.tiles;
     p.cpg = (int)cpg;
     const int blocks = p.cpg;
-    if ((size_t)blocks * ctx->lm > ctx->part_sk_floats || blocks > ctx->max_blocks ||
+    if ((size_t)blocks * lm * parts > ctx->part_sk_floats || blocks > ctx->max_blocks ||
         (size_t)blocks * 2 > ctx->part_np_doubles)
         return cudaErrorNotSupported;
     if (p.T % kBatch != 0 || kPW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
@@ -400,17 +405,20 @@ cudaError_t launch_mean(fda_ctx *ctx, const float *w, int64_t row_stride, int ro
     mp.depth = (int)(depth < (size_t)kMaxDepth ? depth : (size_t)kMaxDepth);
     const size_t smem = fixed + (size_t)mp.depth * per_quad;
 
-    auto kern = ctx->l >= 7 ? (xi_used ? k_mean_state_gather<true, 5> : k_mean_state_gather<false, 5>)
+    auto kern = p.l >= 7 || parts > 1 ? (xi_used ? k_mean_state_gather<true, 5> : k_mean_state_gather<false, 5>)
                             : (xi_used ? k_mean_state_gather<true, kChunksAhead> : k_mean_state_gather<false, kChunksAhead>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, kThreads, smem, s>>>(mp);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    for (int part = 0; part < parts; ++part) {                       // (the row of averaged drifts is in L2)
+        p.sched_off = ctx->sched_off + (size_t)part * ctx->sched_tiles;
+        p.part_sk = ctx->part_sk + (size_t)part * blocks * lm;
+        e = fda_launch_dependent(kern, blocks, kThreads, smem, s, mp);
+        if (e != cudaSuccess) return e;
+    }
     const int fblocks = ((ctx->lm > 64 ? ctx->lm : 64) + 127) / 128;      // at least two warps for the scalars
-    k_finalize_mean_gather<<<fblocks, 128, 0, s>>>(ctx->part_sk, ctx->part_np, blocks, base_zero ? np_blocks : blocks,
-                                                    ctx->lm, K, flags, have_xi, base_zero ? 1.0 : (double)K, mean_state);
-    return cudaGetLastError();
+    return fda_launch_dependent(k_finalize_mean_gather, fblocks, 128, 0, s, ctx->part_sk, ctx->part_np, blocks,
+                                base_zero ? np_blocks : blocks, ctx->lm, lm, K, flags, have_xi,
+                                base_zero ? 1.0 : (double)K, mean_state);
 }
 
 }  // namespace

@@ -50,9 +50,10 @@ constexpr int kSpread = FDA_SPREAD;       // every kSpread-th thread of the bloc
 
 struct SchedParams {
     const uint64_t *coeffs;
-    int l, m;
+    int l, m;              // rows of a part, columns
     uint64_t magic;
     int T;
+    uint32_t tiles;        // block = part * tiles + tile
     int nl_max;            // lists of a (tile, row)
     int no_max;            // octets of a (tile, row)
     int ni_row_max;        // items of a (tile, row)
@@ -73,13 +74,20 @@ struct Carve {
     }
 };
 
+// 32-bit words of the two arrays of hash words, which the matching tables of a row's octets reuse
+__host__ __device__ inline size_t hash_words(int T, int ni_row_max)
+{
+    const size_t tables = (size_t)4 * ni_row_max * kMatchBytes / sizeof(uint32_t);
+    return tables > 2 * (size_t)T ? tables : 2 * (size_t)T;
+}
+
 // shared memory of a builder block (must match the carve-up in the kernel)
 size_t build_smem(int l, int m, int T, int nl_max, int no_max, int ni_row_max)
 {
     auto a16 = [](size_t b) { return (b + 15) / 16 * 16; };
     size_t s = 0;
     s += a16(sizeof(int) * m) * 3 + a16(sizeof(int) * (m + 1)) * 2;      // cnt, fill, npiece | start, lfirst
-    s += a16(sizeof(uint32_t) * T) * 2;                                   // key, bycell
+    s += a16(sizeof(uint32_t) * hash_words(T, ni_row_max));               // key, bycell
     s += a16(sizeof(uint16_t) * T);                                       // sorted
     s += a16(sizeof(uint16_t) * nl_max) * 4;                              // ls_start, ls_len, ls_cell, order
     s += a16(8 * (size_t)nl_max);                                         // ls_res
@@ -90,14 +98,16 @@ size_t build_smem(int l, int m, int T, int nl_max, int no_max, int ni_row_max)
     return s + 64;
 }
 
-// One block per tile.  WRITE = false: count the items and entry chunks of the record;
+// One block per tile (and part of the sketch rows).  WRITE = false: count the items and entry chunks of the record;
 // WRITE = true: write the record at its offset.
 template <bool WRITE>
 __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     const int tid = threadIdx.x, lane = tid & 31;
-    const int64_t tile = blockIdx.x;
+    const int64_t rec_no = blockIdx.x;             // records are in order of (part, tile)
+    const int64_t tile = blockIdx.x % p.tiles;
+    const uint64_t *coeffs = p.coeffs + (size_t)6 * p.l * (blockIdx.x / p.tiles);
     const int T = p.T, m = p.m, NL = p.nl_max, NO = p.no_max;
 
     Carve cv{sm};
@@ -106,8 +116,8 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
     int *npiece = cv.take<int>(m);
     int *start = cv.take<int>(m + 1);
     int *lfirst = cv.take<int>(m + 1);
-    uint32_t *key = cv.take<uint32_t>(T);          // by index: cell << 16 | sign << 15 | index
-    uint32_t *bycell = cv.take<uint32_t>(T);       // the same words grouped by cell
+    uint32_t *key = cv.take<uint32_t>(hash_words(T, p.ni_row_max));   // by index: cell << 16 | sign << 15 | index
+    uint32_t *bycell = key + T;                    // the same words grouped by cell
     uint16_t *sorted = cv.take<uint16_t>(T);       // entries (sign << 15 | index), list after list
     uint16_t *ls_start = cv.take<uint16_t>(NL);
     uint16_t *ls_len = cv.take<uint16_t>(NL);
@@ -128,8 +138,8 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
     uint32_t rec_ni = 0;
     size_t cells_off = 0, ent_off = 0;
     if (WRITE) {
-        rec = p.sched + p.rec_off[tile];
-        rec_ni = p.rec_items[tile];
+        rec = p.sched + p.rec_off[rec_no];
+        rec_ni = p.rec_items[rec_no];
         cells_off = fda_sched_cells_off(rec_ni);
         ent_off = fda_sched_entries_off(rec_ni);
     }
@@ -137,8 +147,8 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
     __syncthreads();
 
     for (int i = 0; i < p.l; ++i) {
-        const uint64_t c[6] = {p.coeffs[6 * i + 0], p.coeffs[6 * i + 1], p.coeffs[6 * i + 2],
-                               p.coeffs[6 * i + 3], p.coeffs[6 * i + 4], p.coeffs[6 * i + 5]};
+        const uint64_t c[6] = {coeffs[6 * i + 0], coeffs[6 * i + 1], coeffs[6 * i + 2],
+                               coeffs[6 * i + 3], coeffs[6 * i + 4], coeffs[6 * i + 5]};
         for (int t = tid; t < m; t += kBT) { cnt[t] = 0; fill[t] = 0; }
         if (tid < ML + 2) cls[tid] = 0;
         __syncthreads();
@@ -478,14 +488,14 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
     }
     __syncthreads();
     if (!WRITE) {
-        if (tid == 0) { p.rec_items[tile] = (uint32_t)ni; p.rec_chunks[tile] = (uint32_t)nch; }
+        if (tid == 0) { p.rec_items[rec_no] = (uint32_t)ni; p.rec_chunks[rec_no] = (uint32_t)nch; }
     } else {
         uint32_t *hdr = reinterpret_cast<uint32_t *>(rec);
         if (tid == 0) {
             hdr[0] = (uint32_t)ni;
             hdr[1] = (uint32_t)(ent_off + (size_t)nch * 256);
             hdr[2] = (uint32_t)nch;
-            hdr[3] = (ni == (int)rec_ni && nch == (int)p.rec_chunks[tile]) ? 0u : 1u;   // 1: the two passes disagree
+            hdr[3] = (ni == (int)rec_ni && nch == (int)p.rec_chunks[rec_no]) ? 0u : 1u;   // 1: the two passes disagree
         }
         for (int q = tid; q < ni; q += kBT) {
             uint32_t *dsc = hdr + 4 + 2 * it_rank[q];
@@ -497,42 +507,55 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
 
 }  // namespace
 
-// Geometry of the schedule for a sketch of l x m: the largest tile (a multiple of kListBatch
-// indices) whose two drift buffers fit beside the bins, or 0 when the lists would be too short.
-static int list_tile_indices(const fda_ctx *ctx, int *ni_max_out)
+// The largest tile (a multiple of kListBatch indices) whose two drift buffers fit beside the bins of
+// `rows` sketch rows, or 0 when its lists would be shorter than min_len entries on average: short lists
+// do not pay for their flushes.
+static int list_tile_indices(const fda_ctx *ctx, int rows, int min_len, int *ni_max_out)
 {
-    const int l = ctx->l, m = ctx->m;
-    if (l == 0 || ctx->lm + 1 >= 0x8000) return 0;
+    const int m = ctx->m;
+    if (rows * m + 1 >= 0x8000) return 0;
     for (int T = kListMaxTile; T >= 2 * kListBatch; T -= kListBatch) {
         const int nl = (m < T ? m : T) + T / kListMaxLen;
-        const int ni_max = l * ((nl + kListSlots - 1) / kListSlots);
-        if (fda_list_smem_bytes(l, m, T, ni_max) > (size_t)ctx->smem_optin) continue;
-        // Lists shorter than six entries on average do not pay for their flushes.
-        if (T < 6 * m) return 0;
+        const int ni_max = rows * ((nl + kListSlots - 1) / kListSlots);
+        if (fda_list_smem_bytes(rows, m, T, ni_max) > (size_t)ctx->smem_optin) continue;
+        if (T < min_len * m) return 0;
         *ni_max_out = ni_max;
         return T;
     }
     return 0;
 }
 
+// Geometry of the schedule: all rows in one part where lists of six entries fit, else two or four
+// equal parts of the rows, each with bins, records and blocks of its own, from five entries on: a part
+// forms the drifts again (its loads hit L2), but the bins it does not hold make room for lists twice as
+// long.  8 x 1000 as two parts of 4 x 1000: tiles of 5120 indices instead of 3072.
+static int list_geometry(const fda_ctx *ctx, int *parts_out, int *ni_max_out)
+{
+    if (ctx->l == 0) return 0;
+    for (int parts = 1; parts <= 4; parts *= 2) {
+        if (ctx->l % parts) break;
+        const int T = list_tile_indices(ctx, ctx->l / parts, parts == 1 ? 6 : 5, ni_max_out);
+        if (T) { *parts_out = parts; return T; }
+    }
+    return 0;
+}
+
 cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s)
 {
-    int ni_max = 0;
-    const int T = list_tile_indices(ctx, &ni_max);
+    int ni_max = 0, parts = 1;
+    const int T = list_geometry(ctx, &parts, &ni_max);
     if (T == 0) return cudaSuccess;
-    const int64_t tiles = (ctx->d_max + T - 1) / T;
+    const int64_t part_tiles = (ctx->d_max + T - 1) / T, tiles = part_tiles * parts;      // records
     if (tiles > 0x7fffffffLL) return cudaSuccess;
 
     SchedParams p{};
-    p.coeffs = ctx->coeffs_dev; p.l = ctx->l; p.m = ctx->m; p.magic = ~0ull / (uint64_t)ctx->m;
+    p.coeffs = ctx->coeffs_dev; p.l = ctx->l / parts; p.tiles = (uint32_t)part_tiles; p.m = ctx->m; p.magic = ~0ull / (uint64_t)ctx->m;
     p.T = T;
     p.nl_max = (ctx->m < T ? ctx->m : T) + T / kListMaxLen;
     p.no_max = (p.nl_max + kListOct - 1) / kListOct;
     p.ni_row_max = (p.nl_max + kListSlots - 1) / kListSlots;
     const size_t bsmem = build_smem(p.l, p.m, T, p.nl_max, p.no_max, p.ni_row_max);
     if (bsmem > (size_t)ctx->smem_optin) return cudaSuccess;
-    // the matching tables of a row's octets reuse the two arrays of hash words (8 bytes per index)
-    if ((size_t)4 * p.ni_row_max * kMatchBytes > 2 * sizeof(uint32_t) * (size_t)T) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k_build_schedule<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_build_schedule<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem);
@@ -583,6 +606,6 @@ cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s)
     cudaFree(items); cudaFree(chunks);
     if (e != cudaSuccess) { cudaFree(off); cudaFree(buf); return e; }
     ctx->sched = buf; ctx->sched_off = off; ctx->sched_bytes = total; ctx->sched_T = T;
-    ctx->sched_ni_max = ni_max; ctx->sched_tiles = tiles;
+    ctx->sched_ni_max = ni_max; ctx->sched_tiles = part_tiles; ctx->sched_parts = parts;
     return cudaSuccess;
 }
