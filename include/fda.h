@@ -91,8 +91,8 @@ typedef struct {
  *     and sketch requests are then served by the slower plain-load kernels, when it would take
  *     more than a third of the free device memory (see fda_create_limited for another cap);
  *   - lazily, by the first call that needs them: a 16-bit hash table of 2*l bytes per index
- *     (sketch requests on a context without a schedule), d_max floats (fda_mean_state with
- *     more than 2*l workers, or without a schedule), K_max*d_max floats of staging
+ *     (sketch requests on a context without a schedule), d_max floats (fda_mean_state on
+ *     short vectors, many unaligned rows, or without a schedule), K_max*d_max floats of staging
  *     (fda_round_host).
  * Blocking: allocates, builds the schedule, synchronises the device.
  * Errors: INVALID_ARG (out == NULL, l < 0 or > FDA_MAX_ROWS, m < 1 or > 32768 with l > 0,
@@ -162,7 +162,7 @@ fda_status fda_local_state(fda_ctx *ctx, const float *w, int64_t row_stride, int
  * yields the same H and trigger as the per-worker route, with l instead of K*l bin updates
  * per index.  Arguments and errors as fda_local_state; mean_state is state_len floats.  On a
  * context with a list schedule the cells come from the list kernel: in one pass over the K rows
- * for K <= 2*l, else from the vector of averaged drifts that a first pass leaves in device
+ * of a long vector, else from the vector of averaged drifts that a first pass leaves in device
  * memory; that vector (d_max floats) is allocated by the first call that needs it (NOMEM if that
  * fails), and so is the 16-bit hash table on a context without a schedule.
  */

@@ -23,6 +23,7 @@
 #include <algorithm>
 
 #include "fda_internal.h"
+#include "fda_quads.cuh"
 
 namespace {
 
@@ -53,54 +54,78 @@ __device__ __forceinline__ void red_shared_add(uint32_t addr, float v)
 constexpr int kModelThreads = 256;
 
 // ubar[j] = (1/K) sum_k (w_k[j] - w_t0[j]);  partial sums of sum_k ||u_k||^2 and sum_k <xi,u_k>
-template <bool LINEAR, bool VEC>
-__global__ void __launch_bounds__(kModelThreads)
-k_mean_model(const float *__restrict__ w, int64_t row_stride, int K, int64_t d, const float *__restrict__ w_t0,
-             const float *__restrict__ xi, float *__restrict__ ubar, double *__restrict__ part_np)
+// Bound: HBM.  A thread takes a quad of indices and asks for eight rows of it (four when some rows are
+// not 16-byte aligned: SHIFT, each then two loads, fda_quads.cuh) before it uses any.  Measured, K = 30,
+// d = 6,964,106: 150 us aligned, 165 us at a pitch of d (222 us with 32-bit loads, as before).
+template <bool LINEAR, bool SHIFT>
+__global__ void __launch_bounds__(kModelThreads, SHIFT ? 4 : 3)
+k_mean_model(const float *w, int64_t row_stride, int K, int64_t d, const float *w_t0,
+             const float *xi, float *__restrict__ ubar, double *__restrict__ part_np)
 {
+    using namespace fda_quads;
+    constexpr int kRows = SHIFT ? 4 : kBatch;
+    fda_grid_wait();
     const float inv_k = 1.0f / (float)K;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double acc_n = 0.0, acc_p = 0.0;
-    if (VEC) {
-        const int64_t nq = d / 4;
-        for (int64_t q = t0; q < nq; q += nthreads) {
-            const float4 b = __ldg(reinterpret_cast<const float4 *>(w_t0 + q * 4));
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (LINEAR) x = __ldg(reinterpret_cast<const float4 *>(xi + q * 4));
-            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-            float pn = 0.f;
-            for (int k0 = 0; k0 < K; k0 += kBatch) {
-                float4 a[kBatch];
-#pragma unroll
-                for (int t = 0; t < kBatch; ++t)
-                    if (k0 + t < K)
-                        a[t] = __ldcs(reinterpret_cast<const float4 *>(w + (size_t)(k0 + t) * row_stride + q * 4));
-#pragma unroll
-                for (int t = 0; t < kBatch; ++t)
-                    if (k0 + t < K) {
-                        const float ux = a[t].x - b.x, uy = a[t].y - b.y, uz = a[t].z - b.z, uw = a[t].w - b.w;
-                        pn = fmaf(ux, ux, pn); pn = fmaf(uy, uy, pn); pn = fmaf(uz, uz, pn); pn = fmaf(uw, uw, pn);
-                        sum.x += ux; sum.y += uy; sum.z += uz; sum.w += uw;
-                    }
-            }
-            acc_n += (double)pn;
-            if (LINEAR)   // sum_k <xi,u_k> = <xi, sum_k u_k>
-                acc_p += (double)(x.x * sum.x + x.y * sum.y + x.z * sum.z + x.w * sum.w);
-            *reinterpret_cast<float4 *>(ubar + q * 4) = make_float4(sum.x * inv_k, sum.y * inv_k, sum.z * inv_k, sum.w * inv_k);
+    // whole quads q0 .. nq - 1; with SHIFT the windows around them lie inside [0, d)
+    const int64_t q0 = SHIFT ? 1 : 0, nq = SHIFT ? (d >= 12 ? (d - 8) / 4 + 1 : 1) : d / 4;
+    for (int64_t q = q0 + t0; q < nq; q += nthreads) {
+        const int64_t j = 4 * q;
+        float4 b, x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (SHIFT) {
+            b = value(load_window(w_t0 + j), w_t0 + j);
+            if (LINEAR) x = value(load_window(xi + j), xi + j);
+        } else {
+            b = *reinterpret_cast<const float4 *>(w_t0 + j);
+            if (LINEAR) x = *reinterpret_cast<const float4 *>(xi + j);
         }
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        float pn = 0.f;
+        auto add = [&](const float4 &a) {
+            const float ux = a.x - b.x, uy = a.y - b.y, uz = a.z - b.z, uw = a.w - b.w;
+            pn = fmaf(ux, ux, pn); pn = fmaf(uy, uy, pn); pn = fmaf(uz, uz, pn); pn = fmaf(uw, uw, pn);
+            sum.x += ux; sum.y += uy; sum.z += uz; sum.w += uw;
+        };
+        for (int k0 = 0; k0 < K; k0 += kRows) {
+            const float *row = w + (size_t)k0 * row_stride + j;
+            if (SHIFT) {
+                Window v[kRows];
+#pragma unroll
+                for (int t = 0; t < kRows; ++t)
+                    if (k0 + t < K) v[t] = load_window(row + (size_t)t * row_stride);
+#pragma unroll
+                for (int t = 0; t < kRows; ++t)
+                    if (k0 + t < K) add(value(v[t], row + (size_t)t * row_stride));
+            } else {
+                float4 a[kRows];
+#pragma unroll
+                for (int t = 0; t < kRows; ++t)
+                    if (k0 + t < K) a[t] = __ldcs(reinterpret_cast<const float4 *>(row + (size_t)t * row_stride));
+#pragma unroll
+                for (int t = 0; t < kRows; ++t)
+                    if (k0 + t < K) add(a[t]);
+            }
+        }
+        acc_n += (double)pn;
+        if (LINEAR)   // sum_k <xi,u_k> = <xi, sum_k u_k>
+            acc_p += (double)(x.x * sum.x + x.y * sum.y + x.z * sum.z + x.w * sum.w);
+        *reinterpret_cast<float4 *>(ubar + j) = make_float4(sum.x * inv_k, sum.y * inv_k, sum.z * inv_k, sum.w * inv_k);
     }
-    const int64_t begin = VEC ? (d / 4) * 4 : 0;
-    for (int64_t j = begin + t0; j < d; j += nthreads) {
-        const float b = __ldg(w_t0 + j);
+    // what the quads leave out at the ends
+    const int64_t head = min(d, 4 * q0), tail = 4 * nq, n_ends = head + (tail < d ? d - tail : 0);
+    for (int64_t t = t0; t < n_ends; t += nthreads) {
+        const int64_t j = t < head ? t : tail + (t - head);
+        const float b = w_t0[j];
         float sum = 0.f, pn = 0.f;
         for (int k = 0; k < K; ++k) {
-            const float a = __ldg(w + (size_t)k * row_stride + j);
+            const float a = w[(size_t)k * row_stride + j];
             pn = fmaf(a - b, a - b, pn);
             sum += a - b;
         }
         acc_n += (double)pn;
-        if (LINEAR) acc_p += (double)(__ldg(xi + j) * sum);
+        if (LINEAR) acc_p += (double)(xi[j] * sum);
         ubar[j] = sum * inv_k;
     }
     // block partial (fixed order)
@@ -141,6 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sketch_vector(const SketchVecPa
     const int columns = 1 << p.cshift;
     for (int i = tid; i < p.lm * columns; i += blockDim.x) bins[i] = 0.f;
     __syncthreads();
+    fda_grid_wait();
     const uint32_t col_addr = (uint32_t)__cvta_generic_to_shared(bins) + (uint32_t)(lane & (columns - 1)) * 4u;
     const int bshift = p.cshift + 2;
     const uint32_t row_bytes = (uint32_t)p.m << bshift;
@@ -157,7 +183,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sketch_vector(const SketchVecPa
             u[0] = a.x; u[1] = a.y; u[2] = a.z; u[3] = a.w; u[4] = b.x; u[5] = b.y; u[6] = b.z; u[7] = b.w;
         } else {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) u[e] = j8 + e < p.d ? __ldg(p.v + j8 + e) : 0.f;
+            for (int e = 0; e < 8; ++e) u[e] = j8 + e < p.d ? p.v[j8 + e] : 0.f;
         }
         // the table planes are padded to a multiple of 64 entries past d_max: whole 16-byte reads stay inside
         const bool any = j8 < p.d;
@@ -227,6 +253,7 @@ __global__ void __launch_bounds__(32 * FDA_MAX_ROWS, 1) k_sketch_vector_rows(con
     const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;      // blockDim = 32 * l
     for (int i = tid; i < p.lm * 32; i += blockDim.x) bins[i] = 0.f;
     __syncthreads();
+    fda_grid_wait();
     const uint32_t rowaddr = (uint32_t)__cvta_generic_to_shared(bins) + (uint32_t)row * ((uint32_t)p.m << 7) +
                              (uint32_t)lane * 4u;
     const uint16_t *__restrict__ plane = p.tab + (size_t)row * (size_t)p.tab_stride;
@@ -237,11 +264,11 @@ __global__ void __launch_bounds__(32 * FDA_MAX_ROWS, 1) k_sketch_vector_rows(con
         const int64_t j = st * kStep + lane * 4;
         a = make_float4(0.f, 0.f, 0.f, 0.f);
         h = make_uint2(0u, 0u);                      // past d: u = 0 goes to cell 0
-        if (j + 3 < p.d) a = __ldg(reinterpret_cast<const float4 *>(p.v + j));
+        if (j + 3 < p.d) a = *reinterpret_cast<const float4 *>(p.v + j);
         else {
-            if (j + 0 < p.d) a.x = __ldg(p.v + j + 0);
-            if (j + 1 < p.d) a.y = __ldg(p.v + j + 1);
-            if (j + 2 < p.d) a.z = __ldg(p.v + j + 2);
+            if (j + 0 < p.d) a.x = p.v[j + 0];
+            if (j + 1 < p.d) a.y = p.v[j + 1];
+            if (j + 2 < p.d) a.z = p.v[j + 2];
         }
         if (j < p.d) h = __ldg(reinterpret_cast<const uint2 *>(plane + j));      // plane padded past d_max
     };
@@ -304,6 +331,7 @@ __global__ void k_finalize_mean(const float *__restrict__ part_sk, const double 
                                 float *__restrict__ mean_state)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    fda_grid_wait();
     if (blockIdx.x == 0 && warp < 2) {
         const int e = warp;
         const bool on = e == 0 ? (flags & FDA_STATE_NORM) != 0 : ((flags & FDA_STATE_LINEAR) != 0 && have_xi);
@@ -330,8 +358,7 @@ cudaError_t launch_sketch_vector(fda_ctx *ctx, const SketchVecParams &p, int blo
     auto kern = k_sketch_vector<L>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, kThreads, smem, s>>>(p);
-    return cudaGetLastError();
+    return fda_launch_dependent(kern, blocks, kThreads, smem, s, p);
 }
 
 }  // namespace
@@ -342,16 +369,19 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
 {
     const bool sketch = (flags & FDA_STATE_SKETCH) != 0;
     const float *xi_used = (flags & FDA_STATE_LINEAR) ? xi : nullptr;
+    const bool vec = ((((uintptr_t)w | (uintptr_t)w_t0 | (uintptr_t)(xi_used ? xi_used : w)) & 15u) == 0) &&
+                     (row_stride % 4 == 0);
     // With a list schedule in the context the cells can come from the list kernel.  In one pass over
-    // the K rows when there are few of them and the vector is long: 1.50 against 2.58 ms at 5 x 250,
-    // K = 8, d = 198M, but no gain at d = 7M, where the averaged drifts and the 16-bit table of the
-    // two-kernel route stay in L2.  From the averaged drifts that phase 1 below leaves in memory when
-    // the sketch is too large for the lane-private bins of k_sketch_vector_rows: 0.93 against 1.42 ms
-    // at 7 x 500, K = 60, d = 20M (at 5 x 250 that kernel is the faster one: 0.22 against 0.25 ms at
-    // K = 30, d = 7M).
+    // the K rows when the vector has at least two tiles per SM (5 x 250, K = 30, d = 7M: 182 against
+    // 214 us; K = 20, d = 2.6M: 77 against 85 us; below that the first tile's loads and the rounding of
+    // the tiles per block cost more than the second kernel).  Rows that are not 16-byte aligned arrive
+    // there by 32-bit copies, which pays for few workers on long vectors only (K = 8, d = 20M: 243 against
+    // about 290 us; K = 30, d = 7M: 350 against 210 us).  From the averaged drifts that phase 1 below leaves in memory when
+    // the sketch is too large for the lane-private bins of k_sketch_vector_rows.
     const bool lists = sketch && ctx->sched != nullptr;
     const int64_t tiles = lists ? (d + ctx->sched_T - 1) / ctx->sched_T : 0;
-    if (lists && K <= 2 * ctx->l && tiles >= 8 * (int64_t)ctx->n_sm) {
+    const bool one_pass = vec ? tiles >= 2 * (int64_t)ctx->n_sm : K <= 2 * ctx->l && tiles >= 8 * (int64_t)ctx->n_sm;
+    if (lists && one_pass) {
         const cudaError_t e = fda_launch_mean_state_gather(ctx, w, row_stride, K, d, w_t0, xi, flags, mean_state, s);
         if (e != cudaErrorNotSupported) {
             if (e == cudaSuccess) ctx->last_ls_kernel = "k_mean_state_gather";
@@ -363,21 +393,14 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
         if (e != cudaSuccess) return e;
     }
     // phase 1: one pass over the K rows
-    const bool vec = ((((uintptr_t)w | (uintptr_t)w_t0 | (uintptr_t)(xi_used ? xi_used : w)) & 15u) == 0) &&
-                     (row_stride % 4 == 0);
     const bool linear = xi_used != nullptr;
-    int64_t work = vec ? (d + 3) / 4 : d;
-    int64_t nblk = (work + kModelThreads - 1) / kModelThreads;
+    int64_t nblk = ((d + 3) / 4 + kModelThreads - 1) / kModelThreads;
     if (nblk > (int64_t)ctx->n_sm * 8) nblk = (int64_t)ctx->n_sm * 8;
     if (nblk > ctx->max_blocks * 2) nblk = ctx->max_blocks * 2;      // part_np holds >= max_blocks*64 doubles
-    if (linear) {
-        if (vec) k_mean_model<true, true><<<(unsigned)nblk, kModelThreads, 0, s>>>(w, row_stride, K, d, w_t0, xi_used, ctx->mean_model, ctx->part_np);
-        else     k_mean_model<true, false><<<(unsigned)nblk, kModelThreads, 0, s>>>(w, row_stride, K, d, w_t0, xi_used, ctx->mean_model, ctx->part_np);
-    } else {
-        if (vec) k_mean_model<false, true><<<(unsigned)nblk, kModelThreads, 0, s>>>(w, row_stride, K, d, w_t0, xi_used, ctx->mean_model, ctx->part_np);
-        else     k_mean_model<false, false><<<(unsigned)nblk, kModelThreads, 0, s>>>(w, row_stride, K, d, w_t0, xi_used, ctx->mean_model, ctx->part_np);
-    }
-    cudaError_t e = cudaGetLastError();
+    auto model = linear ? (vec ? k_mean_model<true, false> : k_mean_model<true, true>)
+                        : (vec ? k_mean_model<false, false> : k_mean_model<false, true>);
+    cudaError_t e = fda_launch_dependent(model, (int)nblk, kModelThreads, 0, s, w, row_stride, K, d, w_t0, xi_used,
+                                         ctx->mean_model, ctx->part_np);
     if (e != cudaSuccess) return e;
 
     // phase 2: sketch of u-bar
@@ -409,8 +432,7 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
             sk_blocks = (int)rb;
             e = cudaFuncSetAttribute(k_sketch_vector_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
             if (e != cudaSuccess) return e;
-            k_sketch_vector_rows<<<sk_blocks, 32 * ctx->l, smem, s>>>(p);
-            e = cudaGetLastError();
+            e = fda_launch_dependent(k_sketch_vector_rows, sk_blocks, 32 * ctx->l, smem, s, p);
         } else
         switch (ctx->l) {
             case 1: e = launch_sketch_vector<1>(ctx, p, sk_blocks, smem, s); break;
@@ -425,7 +447,6 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
         if (e != cudaSuccess) return e;
     }
     const int n = ctx->lm > 64 ? ctx->lm : 64;        // at least two warps for the scalars
-    k_finalize_mean<<<(n + 255) / 256, 256, 0, s>>>(ctx->part_sk, ctx->part_np, (int)nblk, sk_blocks, ctx->lm, K,
-                                                   flags, linear, mean_state);
-    return cudaGetLastError();
+    return fda_launch_dependent(k_finalize_mean, (n + 255) / 256, 256, 0, s, ctx->part_sk, ctx->part_np, (int)nblk,
+                                sk_blocks, ctx->lm, K, flags, linear, mean_state);
 }

@@ -13,11 +13,12 @@
 //     octets may still share a bank) and keeps one sum; everything is divided by K at the end;
 //   * the single-column tile leaves most of the shared memory free, and the loads land there
 //     instead of in registers: the rows of a quad of indices (the K workers, w_t0, xi) are copied
-//     asynchronously, `depth` quads ahead per thread, and the thread that asked for them reads
-//     them back when their group has landed (cp.async.wait_group: nothing here can wait for
-//     ever).  The bytes in flight then depend neither on registers nor on the number of producer
-//     warps.  Elements past d and the rows of a model that is not 16-byte aligned are copied
-//     four bytes at a time, with zeros for what lies past the end;
+//     asynchronously, `depth` slots ahead per thread, and read back when their group has landed
+//     (cp.async.wait_group: nothing here can wait for ever).  A slot holds the quad of up to ten
+//     rows; more workers arrive in several slots, so that the bytes in flight depend on neither
+//     registers, the number of producer warps nor K.  Rows that are not 16-byte aligned, and the end
+//     of the model, are copied four bytes at a time, 32 consecutive indices per warp instruction,
+//     with zeros for what lies past the end;
 //   * 8 producer and 24 walker warps at 64 registers.
 //
 // Two callers: the K rows of w (one pass, for few workers), or the single row of averaged drifts
@@ -27,7 +28,8 @@
 // a four-column tile and 12 + 16 warps 2.15 ms; single-column tile 2.07; landing zone with 8 + 20
 // warps 1.73, with 8 + 24 warps 1.67 (6 + 26: 1.86; 12 + 16: 2.01; 4 + 24: 2.12; depth capped at
 // 3 / 2: 1.76 / 1.95); without the L2 prefetch of the next tiles' rows that the per-worker kernel
-// issues, 1.56; with every shared-memory region on a 128-byte boundary, 1.50.
+// issues, 1.56; with every shared-memory region on a 128-byte boundary, 1.50.  7 x 500, K = 60,
+// d = 20M, where the drifts used to be averaged in a pass of their own first: 0.93 -> 0.82 ms.
 
 #include "fda_internal.h"
 #include "fda_list_kernel.cuh"
@@ -37,17 +39,19 @@ namespace {
 using namespace fda_list;
 
 constexpr int kPW = 8;                         // producer warps
+constexpr int kBatch = kPW * 32 * 4;           // a batch is four consecutive indices per producer thread
 constexpr int kWW = 24;                        // walker warps
 constexpr int kThreads = (kPW + kWW) * 32;
-constexpr int kBatch = kPW * 32 * 4;           // a batch is four consecutive indices per producer thread
 constexpr uint32_t kRowPitch = kPW * 32u * 16u;   // one row of a landing-zone slot: 16 bytes per producer thread
 constexpr int kMaxDepth = 8;
+constexpr int kMaxPiece = 10;                  // rows of a landing-zone slot
 
 struct MeanParams {
     ListParams q;                    // rows, schedule, partial-sum buffers; q.K = rows that are read
     int base_zero;                   // the rows are drifts already (no w_t0 to subtract)
     int sketch_only;                 // leave part_np alone
-    int depth;                       // quads a producer thread keeps in flight (1 .. kMaxDepth)
+    int piece;                       // rows of a landing-zone slot: a quad of K rows arrives in K / piece slots
+    int depth;                       // slots a producer thread keeps in flight (1 .. kMaxDepth)
 };
 
 // 16 bytes from global memory straight into shared memory (no register in between), in groups
@@ -105,6 +109,7 @@ inline size_t mean_smem_fixed(int l, int m, int T, int tab_bytes)
 
 // Shared-memory plan (bytes from the start of dynamic shared memory):
 //   [0, 8)      item counters of the two tile buffers
+//   [16, 48)    offsets of the schedule records of the tiles n, n + 1 (slot n mod 4)
 //   [64, 192)   sums[producer warp][2] (fp64): sum_k ||u_k||^2 and <xi, sum_k u_k> over the tiles so far
 //   [1088, ..)  two item tables (tab_bytes each): the head of a tile's schedule record
 //   then        bins[l*m]
@@ -113,7 +118,9 @@ inline size_t mean_smem_fixed(int l, int m, int T, int tab_bytes)
 // (each region on a 128-byte boundary)
 // AHEAD: entry chunks (four steps each) a walker loads before it walks them (five for sketches of
 // seven or more rows, whose items are short; else eight - as in k_local_state_gather).
-template <bool LINEAR, int AHEAD>
+// MULTI: the rows of a quad arrive in several slots (more than kMaxPiece rows).
+// VEC: w, w_t0 and xi are 16-byte aligned.
+template <bool LINEAR, int AHEAD, bool MULTI, bool VEC>
 __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanParams mp)
 {
     const ListParams &p = mp.q;
@@ -124,6 +131,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
 
     const uint32_t smem_base = (uint32_t)__cvta_generic_to_shared(smem_raw);
     int *ctr = reinterpret_cast<int *>(smem_raw);
+    unsigned long long *rec_off = reinterpret_cast<unsigned long long *>(smem_raw + 16);
     double *sums = reinterpret_cast<double *>(smem_raw + 64);
     const uint32_t tab_off = kListSmemHead;
     const uint32_t bins_off = mean_bins_off(p.tab_bytes);
@@ -145,48 +153,67 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
     if (warp < kPW) {
         // =============================== producers ===============================
         const int pt = tid;                                   // quad of indices inside a batch
-        const bool vec_in = p.vec != 0;
         float nf = 0.f, pf = 0.f;
         // head of the schedule record of the tile being stored (the walkers' item table) and the
         // record offsets of the next tile, loaded one and two tiles ahead of their use
         uint4 tabv = make_uint4(0u, 0u, 0u, 0u);
         unsigned long long off0 = load_u64(p.sched_off + c), off1 = load_u64(p.sched_off + c + 1);
         if (pt * 16 < p.tab_bytes) tabv = load_u4(p.sched + off0 + pt * 16);
+        if (pt == 0) rec_off[0] = off0;
         if (n_tiles > 1) { off0 = load_u64(p.sched_off + c + p.cpg); off1 = load_u64(p.sched_off + c + p.cpg + 1); }
 
-        // Slot s, row r of thread pt: lz + (s * R + r) * kRowPitch.
-        const int D = mp.depth;
-        const int R = p.K + (mp.base_zero ? 0 : 1) + (LINEAR ? 1 : 0);
+        // Slot s, row r: lz + (s * R + r) * kRowPitch, a thread's 16 bytes of it.  A slot
+        // holds up to rp rows of w; the slot of a quad's first rows also w_t0 and xi, behind them.
+        const int D = mp.depth, rp = MULTI ? mp.piece : p.K;
+        const int R = rp + (mp.base_zero ? 0 : 1) + (LINEAR ? 1 : 0);
         const uint32_t lz = smem_base + lz_off + (uint32_t)pt * 16u;
-        const int64_t quads = n_tiles * p.nb;                 // this thread's quads
-        int64_t s_i = 0;                                      // next quad to ask for
-        int b_i = 0;
-        int64_t j_i = (int64_t)c * T + 4 * pt;
-        const int64_t wrap = (int64_t)(p.cpg - 1) * T;        // from the end of a tile to this block's next one
-        // the slow copy: what lies past d becomes zero
-        auto copy_ragged = [&](uint32_t dst, const float *row, int64_t j) {
-            const int64_t left = p.d - j;
+        int left_i = (int)n_tiles * p.nb;                     // quads of this thread that are still to be asked for,
+        int b_i = 0, k_i = 0;                                 // the next one's batch in the tile and first row
+        uint32_t j_i = (uint32_t)c * (uint32_t)T + 4u * pt;
+        const uint32_t wrap = (uint32_t)(p.cpg - 1) * (uint32_t)T;   // from the end of a tile to this block's next one
+        // n rows from `row` on into a slot
+        auto copy = [&](uint32_t dst, const float *row, int n) {
+            const float *q = row + j_i;
+            if (VEC) {
+                if (j_i + 4u <= (uint32_t)p.d) {
+#pragma unroll 4
+                    for (int k = 0; k < n; ++k) cp_async16(dst + (uint32_t)k * kRowPitch, q + (int64_t)k * p.row_stride);
+                } else {                                       // the end of the model
+#pragma unroll 1
+                    for (int k = 0; k < n; ++k, q += p.row_stride, dst += kRowPitch)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) cp_async4(dst + 4u * e, e < left ? row + j + e : row, e < left);
+                        for (uint32_t e = 0; e < 4; ++e) cp_async4(dst + 4u * e, j_i + e < (uint32_t)p.d ? q + e : row, j_i + e < (uint32_t)p.d);
+                }
+            } else {
+                // the warp's 128 indices, 32 consecutive ones at a time (a lane's quad is copied by other lanes)
+                q -= 3 * lane;
+                dst -= 12u * lane;
+                const uint32_t j0 = j_i - 3u * lane;
+#pragma unroll 1
+                for (int k = 0; k < n; ++k, q += p.row_stride, dst += kRowPitch)
+#pragma unroll
+                    for (uint32_t e = 0; e < 128; e += 32) {
+                        const bool on = j0 + e < (uint32_t)p.d;
+                        cp_async4(dst + 4u * e, on ? q + e : row, on);
+                    }
+            }
         };
         auto issue = [&](int slot) {
-            if (s_i < quads) {
-                const uint32_t dst = lz + (uint32_t)(slot * R) * kRowPitch;
-                if (vec_in && j_i + 4 <= p.d) {
-                    const float *q = p.w + j_i;
-                    for (int k = 0; k < p.K; ++k) cp_async16(dst + (uint32_t)k * kRowPitch, q + (int64_t)k * p.row_stride);
-                    int r = p.K;
-                    if (!mp.base_zero) { cp_async16(dst + (uint32_t)r * kRowPitch, p.w_t0 + j_i); ++r; }
-                    if (LINEAR) cp_async16(dst + (uint32_t)r * kRowPitch, p.xi + j_i);
-                } else {
-                    for (int k = 0; k < p.K; ++k) copy_ragged(dst + (uint32_t)k * kRowPitch, p.w + (int64_t)k * p.row_stride, j_i);
-                    int r = p.K;
-                    if (!mp.base_zero) { copy_ragged(dst + (uint32_t)r * kRowPitch, p.w_t0, j_i); ++r; }
-                    if (LINEAR) copy_ragged(dst + (uint32_t)r * kRowPitch, p.xi, j_i);
+            if (left_i > 0) {
+                uint32_t dst = lz + (uint32_t)(slot * R) * kRowPitch;
+                copy(dst, p.w + (int64_t)k_i * p.row_stride, MULTI ? min(rp, p.K - k_i) : rp);
+                if (k_i == 0) {
+                    dst += (uint32_t)rp * kRowPitch;
+                    if (!mp.base_zero) { copy(dst, p.w_t0, 1); dst += kRowPitch; }
+                    if (LINEAR) copy(dst, p.xi, 1);
                 }
-                ++s_i;
-                j_i += kBatch;
-                if (++b_i == p.nb) { b_i = 0; j_i += wrap; }
+                if (MULTI) k_i += rp;
+                if (!MULTI || k_i >= p.K) {
+                    k_i = 0;
+                    --left_i;
+                    j_i += kBatch;
+                    if (++b_i == p.nb) { b_i = 0; j_i += wrap; }
+                }
             }
             cp_async_commit();                                 // (an empty group past the end keeps the count)
         };
@@ -195,21 +222,33 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
         for (int64_t n = 0; n < n_tiles; ++n) {
             const int buf = (int)(n & 1);
             for (int b = 0; b < p.nb; ++b) {
-                cp_async_wait_upto(D - 1);                     // the oldest group has landed
-                const uint32_t src = lz + (uint32_t)(slot * R) * kRowPitch;
-                int r = p.K;
-                float4 w0 = make_float4(0.f, 0.f, 0.f, 0.f), a = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (!mp.base_zero) { w0 = lds128(src + (uint32_t)r * kRowPitch); ++r; }
+                float4 w0 = make_float4(0.f, 0.f, 0.f, 0.f), x = w0, a = w0;
+                float qn = 0.f;
+                for (int k0 = 0; k0 < p.K; k0 += rp) {
+                    cp_async_wait_upto(D - 1);                 // the oldest group has landed
+                    if (!VEC) __syncwarp();                    // (all lanes' parts of it)
+                    const uint32_t src = lz + (uint32_t)(slot * R) * kRowPitch;
+                    if (k0 == 0) {
+                        uint32_t q = src + (uint32_t)rp * kRowPitch;
+                        if (!mp.base_zero) { w0 = lds128(q); q += kRowPitch; }
+                        if (LINEAR) x = lds128(q);
+                    }
+                    const int m = MULTI ? min(rp, p.K - k0) : rp;
 #pragma unroll 4
-                for (int k = 0; k < p.K; ++k) {
-                    const float4 v = lds128(src + (uint32_t)k * kRowPitch);
-                    const float ux = v.x - w0.x, uy = v.y - w0.y, uz = v.z - w0.z, uw = v.w - w0.w;
-                    nf = fmaf(ux, ux, nf); nf = fmaf(uy, uy, nf);
-                    nf = fmaf(uz, uz, nf); nf = fmaf(uw, uw, nf);
-                    a.x += ux; a.y += uy; a.z += uz; a.w += uw;
+                    for (int k = 0; k < m; ++k) {
+                        const float4 v = lds128(src + (uint32_t)k * kRowPitch);
+                        const float ux = v.x - w0.x, uy = v.y - w0.y, uz = v.z - w0.z, uw = v.w - w0.w;
+                        qn = fmaf(ux, ux, qn); qn = fmaf(uy, uy, qn);
+                        qn = fmaf(uz, uz, qn); qn = fmaf(uw, uw, qn);
+                        a.x += ux; a.y += uy; a.z += uz; a.w += uw;
+                    }
+                    if (!VEC) __syncwarp();                    // (read by all lanes)
+                    issue(slot);                               // the slot is free again
+                    slot = slot + 1 == D ? 0 : slot + 1;
+                    if (!MULTI) break;
                 }
+                nf += qn;
                 if (LINEAR) {
-                    const float4 x = lds128(src + (uint32_t)r * kRowPitch);
                     pf = fmaf(x.x, a.x, pf); pf = fmaf(x.y, a.y, pf);
                     pf = fmaf(x.z, a.z, pf); pf = fmaf(x.w, a.w, pf);
                 }
@@ -219,8 +258,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
                 const int sw = (int)((r0 >> 3) & 3u);
                 store_row(smem_base + ut_off + (uint32_t)buf * ut_bytes + r0 * 4u,
                           comp(a, 0 ^ sw), comp(a, 1 ^ sw), comp(a, 2 ^ sw), comp(a, 3 ^ sw));
-                issue(slot);                                   // the slot is free again
-                slot = slot + 1 == D ? 0 : slot + 1;
             }
             // ---- the tile is stored: its sums, its item table, its counter, then the hand-over ----
             // (fp32 within the tile: a thread's few indices, then the warp's tree; fp64 across tiles)
@@ -241,7 +278,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
             // the one after: nothing here waits for memory
             if (pt * 16 < p.tab_bytes)
                 *reinterpret_cast<uint4 *>(smem_raw + tab_off + (size_t)buf * p.tab_bytes + pt * 16) = tabv;
-            if (pt == 0) ctr[buf] = 0;
+            if (pt == 0) { ctr[buf] = kWW; rec_off[(n + 1) & 3] = off0; }
             if (n + 1 < n_tiles) {
                 const unsigned char *nrec = p.sched + off0;
                 if (pt * 16 < p.tab_bytes) tabv = load_u4(nrec + pt * 16);
@@ -261,22 +298,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
         for (int64_t n = 0; n < n_tiles; ++n) {
             block_barrier<kThreads>();                                   // tile n is stored, tile n - 1 is walked
             const int buf = (int)(n & 1);
-            const unsigned char *rec = p.sched + p.sched_off[c + n * p.cpg];
+            const unsigned char *rec = p.sched + rec_off[n & 3];
             const uint32_t *tab = reinterpret_cast<const uint32_t *>(smem_raw + tab_off + (size_t)buf * p.tab_bytes);
             const int n_items = (int)tab[0];
             const uint16_t *cells = reinterpret_cast<const uint16_t *>(rec + fda_sched_cells_off(n_items));
             const unsigned char *ent0 = rec + fda_sched_entries_off(n_items);
             const uint32_t base = smem_base + ut_off + (uint32_t)buf * ut_bytes;
-            for (;;) {
-                int it = 0;
-                if (lane == 0) it = atomicAdd(&ctr[buf], 1);
-                it = __shfl_sync(0xffffffffu, it, 0);
-                if (it >= n_items) break;
-                const uint32_t d0 = tab[4 + 2 * it], chunk0 = tab[5 + 2 * it];
+            // the first kWW items go to the warps in order, the others to whoever asks next
+            int it = warp - kPW;
+            uint32_t d0 = 0, chunk0 = 0;
+            if (it < n_items) { d0 = tab[4 + 2 * it]; chunk0 = tab[5 + 2 * it]; }
+            while (it < n_items) {
                 const int steps = (int)(d0 & 0xffffu);
                 const uint32_t cell = cells[(size_t)(d0 >> 16) * kListSlots + lane];
                 const uint2 *ent = reinterpret_cast<const uint2 *>(ent0 + (size_t)chunk0 * 256) + lane;
                 const int nch = (steps + 3) >> 2;
+                if (lane == 0) it = atomicAdd(&ctr[buf], 1);
+                it = __shfl_sync(0xffffffffu, it, 0);
+                if (it < n_items) { d0 = tab[4 + 2 * it]; chunk0 = tab[5 + 2 * it]; }
                 float a = 0.f;
                 // all entry loads of (up to) AHEAD chunks first, then the walk
                 for (int c0 = 0; c0 < nch; c0 += AHEAD) {
@@ -359,6 +398,14 @@ __global__ void k_finalize_mean_gather(const float *__restrict__ part_sk, const 
     mean_state[2 + cell] = (float)(acc / cell_div);
 }
 
+template <int AHEAD>
+void (*pick_kernel(bool linear, bool multi, bool vec))(MeanParams)
+{
+    if (!vec) return linear ? k_mean_state_gather<true, AHEAD, true, false> : k_mean_state_gather<false, AHEAD, true, false>;
+    if (multi) return linear ? k_mean_state_gather<true, AHEAD, true, true> : k_mean_state_gather<false, AHEAD, true, true>;
+    return linear ? k_mean_state_gather<true, AHEAD, false, true> : k_mean_state_gather<false, AHEAD, false, true>;
+}
+
 // rows == K: the averaged state of the K rows of w in one pass.  rows == 1 and base_zero: w is the
 // row of averaged drifts; the cells come from it, the two scalars from np_blocks partial pairs that
 // the averaging pass left at the start of ctx->part_np.
@@ -398,15 +445,18 @@ cudaError_t launch_mean(fda_ctx *ctx, const float *w, int64_t row_stride, int ro
     p.nb = p.T / kBatch;
     // what the single-column tile leaves free becomes the producers' landing zone
     const size_t fixed = mean_smem_fixed(p.l, p.m, p.T, p.tab_bytes);
-    const size_t per_quad = (size_t)kRowPitch * (size_t)(rows + (base_zero ? 0 : 1) + (xi_used ? 1 : 0));
-    const size_t depth = (size_t)ctx->smem_optin > fixed ? ((size_t)ctx->smem_optin - fixed) / per_quad : 0;
-    // too many rows to keep three quads per thread in flight: the pass would wait for its loads
+    // (up to kMaxPiece rows arrive in one slot, more of them in several of nearly equal size)
+    const int slots = (rows + kMaxPiece - 1) / kMaxPiece;
+    mp.piece = (rows + slots - 1) / slots;
+    const size_t per_slot = (size_t)kRowPitch * (size_t)(mp.piece + (base_zero ? 0 : 1) + (xi_used ? 1 : 0));
+    const size_t depth = (size_t)ctx->smem_optin > fixed ? ((size_t)ctx->smem_optin - fixed) / per_slot : 0;
+    // too little room to keep three slots per thread in flight: the pass would wait for its loads
     if (depth < (size_t)(base_zero ? 1 : 3)) return cudaErrorNotSupported;
     mp.depth = (int)(depth < (size_t)kMaxDepth ? depth : (size_t)kMaxDepth);
-    const size_t smem = fixed + (size_t)mp.depth * per_quad;
+    const size_t smem = fixed + (size_t)mp.depth * per_slot;
 
-    auto kern = p.l >= 7 || parts > 1 ? (xi_used ? k_mean_state_gather<true, 5> : k_mean_state_gather<false, 5>)
-                            : (xi_used ? k_mean_state_gather<true, kChunksAhead> : k_mean_state_gather<false, kChunksAhead>);
+    auto kern = p.l >= 7 || parts > 1 ? pick_kernel<5>(xi_used != nullptr, slots > 1, p.vec != 0)
+                                      : pick_kernel<kChunksAhead>(xi_used != nullptr, slots > 1, p.vec != 0);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
     if (e != cudaSuccess) return e;
     for (int part = 0; part < parts; ++part) {                       // (the row of averaged drifts is in L2)
