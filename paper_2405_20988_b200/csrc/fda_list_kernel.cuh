@@ -69,6 +69,13 @@ __device__ __forceinline__ float4 load_quad(const float *ptr, bool vec, int n)
     v.x = load1(ptr, n > 0); v.y = load1(ptr + 1, n > 1); v.z = load1(ptr + 2, n > 2); v.w = load1(ptr + 3, n > 3);
     return v;
 }
+// the first n of the four floats ptr, ptr + 32, ptr + 64, ptr + 96, zeros for the others
+__device__ __forceinline__ float4 load_strided(const float *ptr, int n)
+{
+    float4 v;
+    v.x = load1(ptr, n > 0); v.y = load1(ptr + 32, n > 1); v.z = load1(ptr + 64, n > 2); v.w = load1(ptr + 96, n > 3);
+    return v;
+}
 __device__ __forceinline__ uint4 load_u4(const void *ptr)
 {
     uint4 v;
@@ -121,6 +128,20 @@ __device__ __forceinline__ void walk_chunk(const uint2 &ch, int left, uint32_t b
         if (left > 1) gather_hi(ch.x, base, a01, a23);
         if (left > 2) gather_lo(ch.y, base, a01, a23);
     }
+}
+// two chunks: one block of code while eight steps are left
+__device__ __forceinline__ void walk_chunks2(const uint2 &c0, const uint2 &c1, int left, uint32_t base, unsigned long long &a01, unsigned long long &a23)
+{
+    if (left >= 8) {
+        gather_lo(c0.x, base, a01, a23);
+        gather_hi(c0.x, base, a01, a23);
+        gather_lo(c0.y, base, a01, a23);
+        gather_hi(c0.y, base, a01, a23);
+        gather_lo(c1.x, base, a01, a23);
+        gather_hi(c1.x, base, a01, a23);
+        gather_lo(c1.y, base, a01, a23);
+        gather_hi(c1.y, base, a01, a23);
+    } else { walk_chunk(c0, left, base, a01, a23); walk_chunk(c1, left - 4, base, a01, a23); }
 }
 // the sums of an item's 32 lists into the bins
 __device__ __forceinline__ void flush_item(float *bins, int lm, uint32_t cell, unsigned long long a01, unsigned long long a23)

@@ -11,8 +11,8 @@
 // to be cut into pieces are added atomically).  One update costs one 4-byte shared-memory read.
 //
 // A block serves a group of 4 workers and a strided set of tiles, with two kinds of warps:
-//   producers  8 warps (4 for sketches of 7 or more rows).  A thread owns four consecutive indices
-//              of a batch (1024 indices with 8 warps): it loads the four workers' values and w_t0
+//   producers  8 warps (5 for sketches of 7 or more rows).  A thread owns four consecutive indices
+//              of a batch (1024 indices with 8 warps; the last batch of a tile may be a part): it loads the four workers' values and w_t0
 //              (xi) with 128-bit loads into registers (the landing zone: nothing else is staged),
 //              subtracts, adds up ||u||^2 and <xi,u> (fp32 within a tile, fp64 across tiles) and
 //              stores the four drifts of an index as one 16-byte row of the tile: ut[index][4].
@@ -21,7 +21,7 @@
 //              in flight (4.6 TB/s with 8 warps per SM, 6.5 with 16, 7.0 with 24), not with the
 //              loads a warp has in flight; deeper software pipelines here changed nothing, and
 //              32-bit loads ran at a quarter of the speed;
-//   walkers    20 warps (24).  They take the tile's items (32 lists, one per lane) from a counter,
+//   walkers    20 warps (23).  They take the tile's items (32 lists, one per lane) from a counter,
 //              longest first; per step a lane loads one 16-bit entry's row with a 128-bit load
 //              (the schedule orders the entries so that the eight lanes of a pass through
 //              shared memory hit eight different bank groups) and adds it with the entry's
@@ -36,7 +36,8 @@
 // from L2 after the barrier it stood in front of the first entries of every tile), the first item of
 // a tile goes to a warp by its number, and the next item's number and descriptor are fetched before
 // the walk of the current one.  5 x 250, K = 8, d = 198M: 2.44 -> 2.38 ms; K = 30, d = 7M: 372 -> 356 us;
-// 7 x 500, K = 60, d = 20M: 2.98 -> 2.89 ms.  Tried and slower: hand-over through mbarriers instead of
+// 7 x 500, K = 60, d = 20M: 2.98 -> 2.89 ms.  Fewer live registers (tile counts and indices in 32 bits,
+// eight steps in one block of code) took them to 2.33 ms, 347 us and, with 5 + 23 warps, 2.57 ms.  Tried and slower: hand-over through mbarriers instead of
 // the barrier (2.52 ms: the bins still need the walkers to meet between tiles, or two of them would
 // add to one cell at a time), entries of the next item asked for before the flush (2.61 ms), 24
 // walkers at 64 registers (2.40 ms).
@@ -66,9 +67,12 @@ using namespace fda_list;
 // tiles leaves most SMs without a block, so p.part_tiles blocks share the tile of each: all of them form
 // the drifts, each walks every p.part_tiles-th item, and their bins, which differ in the cells they touch,
 // are partial sums like those of any other blocks (so the cells come out the same bit for bit).
-// Measured: 8 x 1000 as two parts, K = 20, d = 2.6M: 224 us, against 510 us on the compare-and-swap
+// Measured: 8 x 1000 as two parts, K = 20, d = 2.6M: 212 us, against 510 us on the compare-and-swap
 // kernel that served it before; shared tiles, 5 x 250, K = 5, d = 61,706: 12.5 -> 10 us.
-template <bool LINEAR, int PW, int WW, bool PARTS, bool SPLIT>
+// VEC: w, w_t0 and xi are 16-byte aligned.  If not, a producer thread owns the four indices lane, lane + 32,
+// ... of its warp's 128 instead of four consecutive ones, so that its 32-bit loads are coalesced (K = 30,
+// d = 6,964,106 at a pitch of d: 529 -> 370 us; 7 x 500, K = 60, d = 20M: 4.38 -> 2.75 ms).
+template <bool LINEAR, int PW, int WW, bool PARTS, bool SPLIT, bool VEC>
 __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const ListParams p)
 {
     constexpr int kProducerWarps = PW;
@@ -76,10 +80,10 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     constexpr int kBatch = PW * 32 * 4;                       // a batch is four consecutive indices per producer thread
     constexpr int kDepth = 1;                                 // batches a producer thread keeps in flight
     // entry chunks (four steps each) a walker loads before it walks them: seven (items of 5 x 250
-    // average 28 steps), or five with the 4 + 24 split, whose items average eleven steps.  Measured:
-    // 7 x 500, K = 60, d = 20M: 2.94 ms with 5, 2.98 with 4, 2.96 with 6, 3.01 with 7, 3.06 with 8;
-    // 5 x 250, K = 8, d = 198M with 8 + 20 warps: 2.474 ms with 7, 2.481 with 8, 2.51 with 6, 2.52 with 10
-    constexpr int kAhead = PARTS ? 2 : (WW == 24) ? 5 : 7;
+    // average 28 steps), four with the 5 + 23 split, whose items average eleven, two for the short
+    // items of parts.  Measured: 7 x 500, K = 60, d = 20M: 2.76 ms with 4 or 3, 2.79 with 5;
+    // 5 x 250, K = 8, d = 198M: 2.33 ms with 7 or 8, 2.43 with 6, 2.38 with 5
+    constexpr int kAhead = PARTS ? 2 : (PW == 5 && WW == 23) ? 4 : 7;
     static_assert(PW <= kMaxProducerWarps, "the fp64 sums have room for kMaxProducerWarps warps");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -110,7 +114,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     __syncthreads();
     fda_grid_wait();
 
-    const int64_t n_tiles = p.tiles > c ? (p.tiles - c + p.cpg - 1) / p.cpg : 0;
+    const int n_tiles = p.tiles > c ? (int)((p.tiles - c + p.cpg - 1) / p.cpg) : 0;
 
     if (warp < kProducerWarps) {
         // =============================== producers ===============================
@@ -125,23 +129,29 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
         float nf[GW], pf[GW];
 #pragma unroll
         for (int k = 0; k < GW; ++k) { nf[k] = 0.f; pf[k] = 0.f; }
-        int64_t n_i = 0, n_c = 0;                             // tile being loaded / stored
+        int n_i = 0, n_c = 0;                             // tile being loaded / stored
         int b_i = 0, b_c = 0;                                 // batch inside it
-        int64_t j_i = (int64_t)c * T + 4 * pt;                // first index of this thread's next loads
-        int64_t end_i = (int64_t)(c + 1) * T;                 // end of the tile they belong to
-        const int64_t wrap = (int64_t)(p.cpg - 1) * T;        // from the end of a tile to this block's next one
-        const bool vec_in = p.vec != 0;
-
+        uint32_t j_i = (uint32_t)c * (uint32_t)T + (VEC ? 4 * pt : 128 * warp + lane);   // first index of this thread's next loads
+        uint32_t end_i = (uint32_t)(c + 1) * (uint32_t)T;                 // end of the tile they belong to
+        // 128-index chunks warp, warp + PW, ... of a tile, and the way from behind the last one to the
+        // first of this block's next tile
+        const int nb = (T / 128 - warp + PW - 1) / PW;
+        const uint32_t wrap = (uint32_t)p.cpg * (uint32_t)T - (uint32_t)(nb * kBatch);
         // The rows of a tile two tiles ahead of the one being stored, into L2 (one bulk prefetch per
         // worker row, w_t0 and xi): the producers' loads then find their data in L2.
-        auto prefetch_tile = [&](int64_t n) {
-            if (n >= n_tiles || !vec_in || pt >= GW + 2) return;
+        auto prefetch_tile = [&](int n) {
+            if (n >= n_tiles || pt >= GW + 2) return;
             const int64_t j = (c + n * p.cpg) * (int64_t)T;
             int64_t cnt = p.d - j;
             if (cnt > T) cnt = T;
-            const uint32_t bytes = (uint32_t)(cnt * 4) & ~15u;
+            uint32_t bytes = (uint32_t)(cnt * 4) & ~15u;
             const float *src = pt < GW ? (g * GW + pt < p.K ? wbase + (int64_t)pt * p.row_stride + j : nullptr)
                                        : (pt == GW ? p.w_t0 + j : (LINEAR ? p.xi + j : nullptr));
+            if (!VEC && src) {                                // the 16-byte pieces inside the row
+                const uint32_t off = (16u - ((uint32_t)(uintptr_t)src & 15u)) & 15u;
+                bytes = (uint32_t)(cnt * 4) > off ? ((uint32_t)(cnt * 4) - off) & ~15u : 0u;
+                src += off / 4;
+            }
             if (src && bytes)
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
         };
@@ -157,22 +167,28 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
         auto issue = [&](int slot) {
             if (n_i < n_tiles) {
                 const float *q = wbase + j_i;
-                if (vec_in && end_i <= p.d) {                 // a whole tile of aligned rows: 128-bit loads
+                if (!VEC) {
+                    const int64_t left = p.d - (int64_t)j_i;
+                    const int n = left > 96 ? 4 : (left > 0 ? (int)(left + 31) / 32 : 0);
+#pragma unroll
+                    for (int k = 0; k < GW; ++k) wv[slot][k] = load_strided(q + roff[k], n);
+                    w0v[slot] = load_strided(p.w_t0 + j_i, n);
+                    if (LINEAR) xv[slot] = load_strided(p.xi + j_i, n);
+                } else if (end_i <= (uint32_t)p.d) {                    // a whole tile: 128-bit loads
 #pragma unroll
                     for (int k = 0; k < GW; ++k) wv[slot][k] = load4_stream(q + roff[k]);
                     w0v[slot] = load4_keep(p.w_t0 + j_i);
                     if (LINEAR) xv[slot] = load4_keep(p.xi + j_i);
-                } else {                                      // the last tile of the model, or unaligned rows
-                    const int64_t left = p.d - j_i;
+                } else {                                      // the last tile of the model
+                    const int64_t left = p.d - (int64_t)j_i;
                     const int n = left >= 4 ? 4 : (left > 0 ? (int)left : 0);
-                    const bool vec = vec_in && n == 4;
 #pragma unroll
-                    for (int k = 0; k < GW; ++k) wv[slot][k] = load_quad<true>(q + roff[k], vec, n);
-                    w0v[slot] = load_quad<false>(p.w_t0 + j_i, vec, n);
-                    if (LINEAR) xv[slot] = load_quad<false>(p.xi + j_i, vec, n);
+                    for (int k = 0; k < GW; ++k) wv[slot][k] = load_quad<true>(q + roff[k], n == 4, n);
+                    w0v[slot] = load_quad<false>(p.w_t0 + j_i, n == 4, n);
+                    if (LINEAR) xv[slot] = load_quad<false>(p.xi + j_i, n == 4, n);
                 }
                 j_i += kBatch;
-                if (++b_i == p.nb) { b_i = 0; ++n_i; j_i += wrap; end_i += wrap + T; }
+                if (++b_i == nb) { b_i = 0; ++n_i; j_i += wrap; end_i += (uint32_t)p.cpg * (uint32_t)T; }
             }
         };
         auto consume = [&](int slot) {
@@ -180,7 +196,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
             // rows 4*pt .. 4*pt+3 of the batch; row r is stored at r ^ ((r >> 3) & 3), so that the
             // eight lanes of a store pass hit eight different bank groups (the schedule's entries
             // hold the swizzled row)
-            const uint32_t r0 = (uint32_t)(b_c * kBatch + 4 * pt);
+            const uint32_t r0 = (uint32_t)(b_c * kBatch) + (VEC ? 4u * pt : fda_list_row(128u * warp + lane));
             const uint32_t dst0 = smem_base + ut_off + (uint32_t)buf * ut_bytes + r0 * 16u;
             const uint32_t sw = (r0 >> 3) & 3u;
 #pragma unroll
@@ -197,9 +213,9 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                     pf[0] = fmaf(xq, u0, pf[0]); pf[1] = fmaf(xq, u1, pf[1]);
                     pf[2] = fmaf(xq, u2, pf[2]); pf[3] = fmaf(xq, u3, pf[3]);
                 }
-                store_row(dst0 + (((uint32_t)q ^ sw) << 4), u0, u1, u2, u3);
+                store_row(dst0 + (VEC ? ((uint32_t)q ^ sw) << 4 : 512u * q), u0, u1, u2, u3);
             }
-            if (++b_c == p.nb) {
+            if (++b_c == nb) {
                 // ---- the tile is stored: its item table, its counter, then the hand-over ----
                 // (fp32 within the tile: a thread's few indices, then the warp's tree; fp64 across tiles)
 #pragma unroll
@@ -228,7 +244,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(nrec + o));
                 }
                 if (n_c + 2 < n_tiles) {
-                    const int64_t t2 = c + (n_c + 2) * p.cpg;
+                    const int64_t t2 = c + (int64_t)(n_c + 2) * p.cpg;
                     off0 = load_u64(sched_off + t2);
                     off1 = load_u64(sched_off + t2 + 1);
                 }
@@ -248,7 +264,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
         }
     } else {
         // =============================== walkers ===============================
-        for (int64_t n = 0; n < n_tiles; ++n) {
+        for (int n = 0; n < n_tiles; ++n) {
             block_barrier<kThreads>();                                   // tile n is stored, tile n - 1 is walked
             const int buf = (int)(n & 1);
             // (the record's offset comes from shared memory: a load from L2 here would stand in front of
@@ -314,7 +330,8 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                     for (int q = 0; q < kAhead; ++q)
                         if (c0 + q < nch) ch[q] = __ldg(ent + (size_t)(c0 + q) * kListSlots);
 #pragma unroll
-                    for (int q = 0; q < kAhead; ++q) walk_chunk(ch[q], steps - 4 * (c0 + q), base, a01, a23);
+                    for (int q = 0; q + 1 < kAhead; q += 2) walk_chunks2(ch[q], ch[q + 1], steps - 4 * (c0 + q), base, a01, a23);
+                    if (kAhead & 1) walk_chunk(ch[kAhead - 1], steps - 4 * (c0 + kAhead - 1), base, a01, a23);
                 }
                 flush_item(bins, lm, cell, a01, a23);
             }
@@ -398,11 +415,17 @@ __global__ void k_finalize_gather(const ListParams p, const ListParts parts, uin
 }
 
 template <int PW, int WW, bool PARTS, bool SPLIT>
+void (*pick_kernel(bool linear, bool vec))(ListParams)
+{
+    if (linear) return vec ? k_local_state_gather<true, PW, WW, PARTS, SPLIT, true> : k_local_state_gather<true, PW, WW, PARTS, SPLIT, false>;
+    return vec ? k_local_state_gather<false, PW, WW, PARTS, SPLIT, true> : k_local_state_gather<false, PW, WW, PARTS, SPLIT, false>;
+}
+
+template <int PW, int WW, bool PARTS, bool SPLIT>
 cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent, cudaStream_t s)
 {
-    if (p.T % (PW * 128) != 0 || PW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
-    p.nb = p.T / (PW * 128);
-    auto kern = p.have_xi ? k_local_state_gather<true, PW, WW, PARTS, SPLIT> : k_local_state_gather<false, PW, WW, PARTS, SPLIT>;
+    if (p.T % 128 != 0 || p.T < PW * 128 || PW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
+    auto kern = pick_kernel<PW, WW, PARTS, SPLIT>(p.have_xi != 0, p.vec != 0);
     if (dependent) return fda_launch_dependent(kern, blocks, (PW + WW) * 32, smem, s, p);
     kern<<<blocks, (PW + WW) * 32, smem, s>>>(p);
     return cudaGetLastError();
@@ -413,13 +436,14 @@ cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent,
 // The kernels' dynamic shared memory limit, set once per context (on the context's device).
 cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx)
 {
-    for (auto kern : {k_local_state_gather<true, 8, 20, false, false>, k_local_state_gather<false, 8, 20, false, false>,
-                      k_local_state_gather<true, 4, 24, false, false>, k_local_state_gather<false, 4, 24, false, false>,
-                      k_local_state_gather<true, 8, 24, true, false>, k_local_state_gather<false, 8, 24, true, false>,
-                      k_local_state_gather<true, 16, 12, false, true>, k_local_state_gather<false, 16, 12, false, true>,
-                      k_local_state_gather<true, 8, 20, false, true>, k_local_state_gather<false, 8, 20, false, true>}) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
-        if (e != cudaSuccess) return e;
+    for (int i = 0; i < 4; ++i) {
+        const bool linear = i & 1, vec = i & 2;
+        for (auto kern : {pick_kernel<8, 20, false, false>(linear, vec), pick_kernel<5, 23, false, false>(linear, vec),
+                          pick_kernel<8, 20, true, false>(linear, vec), pick_kernel<16, 12, false, true>(linear, vec),
+                          pick_kernel<8, 20, false, true>(linear, vec)}) {
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
+            if (e != cudaSuccess) return e;
+        }
     }
     return cudaSuccess;
 }
@@ -467,14 +491,16 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         if (p.tiles == p.cpg && 2 * blocks <= ctx->n_sm) split = std::min(8, ctx->n_sm / blocks);
         p.part_tiles = split;
     }
-    // 8 producer + 20 walker warps, or 4 + 24 when a loaded index pays for more walking.  Measured:
-    // 7 x 500, K = 60, d = 20M: 3.34 ms with 4 + 24 against 3.71 ms with 8 + 20; 5 x 250, K = 8,
-    // d = 198M: 3.49 against 2.49 ms; 5 x 250, K = 30, d = 7M: 0.535 against 0.387 ms.
+    // 8 producer + 20 walker warps, or 5 + 23 when a loaded index pays for more walking.  Measured,
+    // 7 x 500, K = 60, d = 20M: 2.76 ms with 5 + 23, 2.90 with 4 + 24, 2.95 with 8 + 20, 2.68 against
+    // 2.64 with 6 + 22; 5 x 250, K = 8, d = 198M: 2.35 ms with 8 + 20, 2.46 with 7 + 21, 2.48 with 9 + 19,
+    // 2.61 with 12 + 16; 8 x 1000 in parts, K = 20, d = 2.6M: 214 us with 8 + 20, 216 with 10 + 18,
+    // 231 with 6 + 22, 226 with 8 + 24 (64 registers).
     auto launch = [&](ListParams &q, int grid, cudaStream_t st, bool dependent) {
-        if (ctx->sched_parts > 1) return launch_lists<8, 24, true, false>(q, grid, smem, dependent, st);
+        if (ctx->sched_parts > 1) return launch_lists<8, 20, true, false>(q, grid, smem, dependent, st);
         if (split > 1) return q.T % 2048 == 0 ? launch_lists<16, 12, false, true>(q, grid, smem, dependent, st)
                                                 : launch_lists<8, 20, false, true>(q, grid, smem, dependent, st);
-        return p.l >= 7 ? launch_lists<4, 24, false, false>(q, grid, smem, dependent, st)
+        return p.l >= 7 ? launch_lists<5, 23, false, false>(q, grid, smem, dependent, st)
                         : launch_lists<8, 20, false, false>(q, grid, smem, dependent, st);
     };
     ListParts parts{};
