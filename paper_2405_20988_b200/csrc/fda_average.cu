@@ -158,6 +158,45 @@ k_average_shifted(float *w, int64_t row_stride, int K, int64_t d, float *w_t0,
     if (XI) block_partial(dsq, part);
 }
 
+// Short vectors: one index per thread, whatever the alignment.  A quad per thread would leave most of
+// the SMs' warps without work, and what a thread waits for is a chain of round trips, one per
+// batch of rows, so a batch is sixteen rows deep.
+template <bool XI>
+__global__ void __launch_bounds__(256)
+k_average_short(float *w, int64_t row_stride, int K, int64_t d, float *w_t0,
+                const fda_estimate *est, int broadcast, float *__restrict__ xi_out, double *__restrict__ part)
+{
+    constexpr int kDeep = 16;
+    fda_grid_wait();
+    if (est != nullptr && est->trigger == 0) return;
+    double dsq = 0.0;
+    const float inv_k = 1.0f / (float)K;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < d; j += (int64_t)gridDim.x * blockDim.x) {
+        float acc = 0.f;
+        for (int k0 = 0; k0 < K; k0 += kDeep) {
+            float v[kDeep];
+#pragma unroll
+            for (int b = 0; b < kDeep; ++b)
+                if (k0 + b < K) v[b] = __ldcs(w + (size_t)(k0 + b) * row_stride + j);
+#pragma unroll
+            for (int b = 0; b < kDeep; ++b)
+                if (k0 + b < K) acc += v[b];
+        }
+        acc *= inv_k;
+        if (XI) {
+            const float dl = acc - w_t0[j];
+            xi_out[j] = dl;
+            dsq += (double)(dl * dl);
+        }
+        w_t0[j] = acc;
+        if (broadcast) {
+#pragma unroll 8
+            for (int k = 0; k < K; ++k) __stcs(w + (size_t)k * row_stride + j, acc);
+        }
+    }
+    if (XI) block_partial(dsq, part);
+}
+
 // xi_out *= 1 / ||delta||  (0 when the step is zero); gated like the average itself
 __global__ void __launch_bounds__(256)
 k_scale_xi(float *__restrict__ xi_out, int64_t d, const double *__restrict__ part, int nparts,
@@ -195,16 +234,20 @@ cudaError_t fda_launch_average(const fda_ctx *ctx, float *w, int64_t row_stride,
     const fda_estimate *gate = (flags & FDA_AVG_UNCONDITIONAL) ? nullptr : est_dev;
     const int broadcast = (flags & FDA_AVG_BROADCAST) ? 1 : 0;
     const int threads = 256;
-    int64_t blocks = ((d + 3) / 4 + threads - 1) / threads;
+    // One index per thread up to 512 indices per SM, and up to 4096 when the chain of batches is long.
+    // Measured with broadcast, calls back to back: K = 44, d = 84K, pitch d 6.7 us against 16.8 us with quads
+    // (aligned 5.7 against 7.9); K = 40, d = 500K 30 against 34 us; K = 20, d = 250K 6.6 against 5.6 us.
+    const bool shrt = d <= (int64_t)ctx->n_sm * (K > 32 ? 4096 : 512);
+    int64_t blocks = ((shrt ? d : (d + 3) / 4) + threads - 1) / threads;
     const int64_t cap = (int64_t)ctx->n_sm * 8;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     if (xi_out) {
-        cudaError_t e = fda_launch_dependent(vec ? k_average<true> : k_average_shifted<true>, (int)blocks, threads, 0, s,
+        cudaError_t e = fda_launch_dependent(shrt ? k_average_short<true> : vec ? k_average<true> : k_average_shifted<true>, (int)blocks, threads, 0, s,
                                              w, row_stride, K, d, w_t0, gate, broadcast, xi_out, ctx->part_np);
         if (e != cudaSuccess) return e;
         return fda_launch_dependent(k_scale_xi, (int)blocks, threads, 0, s, xi_out, d, ctx->part_np, (int)blocks, gate);
     }
-    return fda_launch_dependent(vec ? k_average<false> : k_average_shifted<false>, (int)blocks, threads, 0, s,
+    return fda_launch_dependent(shrt ? k_average_short<false> : vec ? k_average<false> : k_average_shifted<false>, (int)blocks, threads, 0, s,
                                 w, row_stride, K, d, w_t0, gate, broadcast, (float *)nullptr, (double *)nullptr);
 }
