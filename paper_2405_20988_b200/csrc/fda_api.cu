@@ -46,37 +46,72 @@ fda_status fail_cuda(fda_ctx *ctx, cudaError_t e, const char *where)
 // and freeing it with every context would add milliseconds to fda_create and fda_destroy), a slot
 // per context, given back when the context goes.  Contexts beyond the page's slots copy instead.
 struct EstimateSlots {
-    static constexpr int kSlots = 64, kBytes = 128;
+    static constexpr int kSlots = 32, kWords = 4 + FDA_MAX_ROWS;
     std::mutex mutex;
-    unsigned char *page = nullptr;
-    uint64_t used = 0;
-    fda_estimate *take()
+    unsigned long long *page = nullptr;
+    uint32_t used = 0;
+    unsigned long long *take()
     {
-        static_assert(sizeof(fda_estimate) <= kBytes, "a slot holds an estimate");
         std::lock_guard<std::mutex> lock(mutex);
         if (!page) {
             void *ptr = nullptr;
-            if (cudaHostAlloc(&ptr, kSlots * kBytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+            if (cudaHostAlloc(&ptr, sizeof(unsigned long long) * kSlots * kWords, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
                 cudaGetLastError();
                 return nullptr;
             }
-            page = static_cast<unsigned char *>(ptr);
+            page = static_cast<unsigned long long *>(ptr);
         }
         for (int i = 0; i < kSlots; ++i)
             if (!((used >> i) & 1u)) {
-                used |= (uint64_t)1 << i;
-                return reinterpret_cast<fda_estimate *>(page + i * kBytes);
+                used |= (uint32_t)1 << i;
+                // the number of no estimate: the slot may have served another context
+                std::memset(page + i * kWords, 0, sizeof(unsigned long long) * kWords);
+                return page + i * kWords;
             }
         return nullptr;
     }
-    void give_back(fda_estimate *slot)
+    void give_back(unsigned long long *slot)
     {
         if (!slot) return;
         std::lock_guard<std::mutex> lock(mutex);
-        used &= ~((uint64_t)1 << ((reinterpret_cast<unsigned char *>(slot) - page) / kBytes));
+        used &= ~((uint32_t)1 << ((slot - page) / kWords));
     }
 };
 EstimateSlots g_estimates;
+
+// Waits until all words of the estimate numbered `seq` are in the slot.  They are the last thing that
+// the call's kernel writes, so everything enqueued on the stream before it is complete then.  The slot
+// is polled for a while - a stream synchronisation would add some 4 us to a step of a small model -
+// and the stream is waited for after that, which also reports an error.
+cudaError_t wait_for_estimate(const volatile unsigned long long *slot, int words, unsigned int seq, cudaStream_t s)
+{
+    const auto t0 = std::chrono::steady_clock::now();
+    int have = 0;
+    do {
+        for (int i = 0; i < 64; ++i) {
+            while (have < words && (unsigned int)(slot[have] >> 32) == seq) ++have;
+            if (have == words) return cudaSuccess;
+        }
+    } while (std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(200));
+    return cudaStreamSynchronize(s);
+}
+
+void read_estimate(const volatile unsigned long long *slot, int l, float theta, fda_estimate *est)
+{
+    auto value = [&](int i) {
+        const uint32_t bits = (uint32_t)slot[i];
+        float f;
+        std::memcpy(&f, &bits, sizeof(f));
+        return f;
+    };
+    est->mean_sq_norm = value(0);
+    est->est_sq_norm_of_mean = value(1);
+    est->H = value(2);
+    est->theta = theta;
+    est->trigger = (int32_t)(uint32_t)slot[3];
+    est->l = l;
+    for (int r = 0; r < FDA_MAX_ROWS; ++r) est->row_sq_norm[r] = r < l ? value(4 + r) : 0.f;
+}
 
 void free_device(fda_ctx *ctx)
 {
@@ -271,12 +306,15 @@ fda_status fda_combine_estimate(fda_ctx *ctx, const float *states, int K, int va
     if (!guard.ok) return fail(ctx, FDA_ERR_CUDA, "fda_combine_estimate: cannot select device");
     cudaStream_t s = (cudaStream_t)stream;
     // the kernel writes the estimate to mapped host memory as well: no copy stands between it and the host
-    cudaError_t e = fda_launch_combine(ctx, states, K, variant, epsilon, theta, est_dev,
-                                       est_host ? ctx->est_pinned : nullptr, s);
-    if (e == cudaSuccess && est_host) {
-        if (!ctx->est_pinned) e = cudaMemcpyAsync(est_host, est_dev, sizeof(fda_estimate), cudaMemcpyDeviceToHost, s);
+    unsigned long long *slot = est_host ? ctx->est_pinned : nullptr;
+    if (slot && ++ctx->est_seq == 0) ctx->est_seq = 1;
+    cudaError_t e = fda_launch_combine(ctx, states, K, variant, epsilon, theta, est_dev, slot, ctx->est_seq, s);
+    if (e == cudaSuccess && slot) {
+        e = wait_for_estimate(slot, 4 + ctx->l, ctx->est_seq, s);
+        if (e == cudaSuccess) read_estimate(slot, ctx->l, theta, est_host);
+    } else if (e == cudaSuccess && est_host) {
+        e = cudaMemcpyAsync(est_host, est_dev, sizeof(fda_estimate), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess && ctx->est_pinned) std::memcpy(est_host, ctx->est_pinned, sizeof(fda_estimate));
     }
     if (e != cudaSuccess) return fail_cuda(ctx, e, "fda_combine_estimate");
     return FDA_OK;

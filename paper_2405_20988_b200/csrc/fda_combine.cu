@@ -3,7 +3,7 @@
 //
 // Bound: latency.  The K x (2 + l*m) floats are a few kilobytes to a megabyte; what takes time is
 // the chain launch - loads - reductions - (meeting of the blocks) - median - result.  So a thread
-// asks for sixteen workers' values of a column before it adds any, and a warp meets the others once.
+// asks for eight workers' values of a column before it adds any, and a warp meets the others once.
 // Tables of up to kOneBlock floats are taken by one block (a ticket and a second trip to L2 cost more
 // than reading them on one SM); larger ones by one block per 64 columns of a row, its threads
 // splitting the workers four ways, and the block that finishes last (a ticket counter, no waiting)
@@ -23,10 +23,13 @@ struct CombineParams {
     const float *states;
     int K, l, m, chunks;                   // chunks: blocks per sketch row (several blocks only)
     int variant;
-    float epsilon, theta;
+    float theta;
     double *scratch;                       // [0..1] S-bar[0..1], then one partial per block
     unsigned int *ticket;                  // 0 between launches
-    fda_estimate *est, *est_host;          // est_host: mapped host memory or null
+    double inv_k, inv_eps;                 // 1 / K, 1 / (1 + epsilon)
+    fda_estimate *est;
+    unsigned long long *host;              // mapped host memory (fda_host_estimate) or null,
+    unsigned int seq;                      // and the number of this estimate
 };
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -36,27 +39,28 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// sum over the workers first, first + step, ... of one column, in order, sixteen loads in flight
+// sum over the workers first, first + step, ... of one column: eight loads in flight, the eight added
+// as a tree (a chain of fp64 additions as long as the loads themselves would follow them), the trees in order
 __device__ __forceinline__ double column_sum(const float *col, int first, int step, int K, size_t slen)
 {
-    constexpr int kBatch = 16;
+    constexpr int kBatch = 8;
     double acc = 0.0;
     for (int k = first; k < K; k += kBatch * step) {
         float v[kBatch];
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) v[u] = k + u * step < K ? __ldcg(col + (size_t)(k + u * step) * slen) : 0.f;
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) acc += (double)v[u];
+        acc += (((double)v[0] + (double)v[1]) + ((double)v[2] + (double)v[3])) +
+               (((double)v[4] + (double)v[5]) + ((double)v[6] + (double)v[7]));
     }
     return acc;
 }
 
-// S-bar[e] (e = 0, 1): lanes stride the workers, fixed shuffle tree
-__device__ __forceinline__ double scalar_mean(const float *states, int K, size_t slen, int e, int lane)
+// sum over the workers of entry e (0, 1): lanes stride the workers, fixed shuffle tree
+__device__ __forceinline__ double scalar_sum(const float *states, int K, size_t slen, int e, int lane)
 {
     double acc = 0.0;
     for (int k = lane; k < K; k += 32) acc += (double)__ldcg(states + (size_t)k * slen + e);
-    return warp_sum(acc) / (double)K;
+    return warp_sum(acc);
 }
 
 // One warp: lane r < l holds ||row r of the averaged sketch||^2; writes the estimate.
@@ -73,22 +77,27 @@ __device__ __forceinline__ void finish(const CombineParams &p, double row, doubl
         const unsigned hi = __ballot_sync(0xffffffffu, lane < p.l && rank == p.l / 2);
         const double a = __shfl_sync(0xffffffffu, row, lo ? __ffs(lo) - 1 : 0);
         const double b = __shfl_sync(0xffffffffu, row, hi ? __ffs(hi) - 1 : 0);
-        est_sq = ((p.l & 1) ? a : 0.5 * (a + b)) / (1.0 + (double)p.epsilon);
+        est_sq = ((p.l & 1) ? a : 0.5 * (a + b)) * p.inv_eps;
     }
     const double H = head0 - est_sq;
     const int trigger = (H > (double)p.theta) ? 1 : 0;    // decided in fp64, strict '>'
-    for (int t = 0; t < 2; ++t) {
-        fda_estimate *est = t == 0 ? p.est : p.est_host;
-        if (!est) continue;
-        if (lane == 0) {
-            est->mean_sq_norm = (float)head0;
-            est->est_sq_norm_of_mean = (float)est_sq;
-            est->H = (float)H;
-            est->theta = p.theta;
-            est->trigger = trigger;
-            est->l = p.l;
-        }
-        if (lane < FDA_MAX_ROWS) est->row_sq_norm[lane] = lane < p.l ? (float)row : 0.f;
+    fda_estimate *est = p.est;
+    if (lane == 0) {
+        est->mean_sq_norm = (float)head0;
+        est->est_sq_norm_of_mean = (float)est_sq;
+        est->H = (float)H;
+        est->theta = p.theta;
+        est->trigger = trigger;
+        est->l = p.l;
+    }
+    const float norm = lane < p.l ? (float)row : 0.f;
+    if (lane < FDA_MAX_ROWS) est->row_sq_norm[lane] = norm;
+    if (p.host) {      // lane 4 + r: row r; every word carries the estimate's number, so no fence orders them
+        const float shifted = __shfl_up_sync(0xffffffffu, norm, 4);
+        const uint32_t word = lane == 0 ? __float_as_uint((float)head0) : lane == 1 ? __float_as_uint((float)est_sq)
+                            : lane == 2 ? __float_as_uint((float)H) : lane == 3 ? (uint32_t)trigger : __float_as_uint(shifted);
+        if (lane < 4 + p.l)
+            *reinterpret_cast<volatile unsigned long long *>(p.host + lane) = ((unsigned long long)p.seq << 32) | word;
     }
 }
 
@@ -102,12 +111,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_combine_small(const CombinePara
     fda_grid_wait();
     double part = 0.0;
     if (warp >= 30) {
-        const double h = scalar_mean(p.states, p.K, slen, warp - 30, lane);
+        const double h = scalar_sum(p.states, p.K, slen, warp - 30, lane) * p.inv_k;
         if (lane == 0) head_s[warp - 30] = h;
     } else if (warp < stripes * p.l) {
         const int i = warp % p.l;
         for (int c = (warp / p.l) * 32 + lane; c < p.m; c += stripes * 32) {
-            const double t = column_sum(p.states + 2 + (size_t)i * p.m + c, 0, 1, p.K, slen) / (double)p.K;
+            const double t = column_sum(p.states + 2 + (size_t)i * p.m + c, 0, 1, p.K, slen) * p.inv_k;
             part += t * t;
         }
         part = warp_sum(part);
@@ -133,7 +142,7 @@ __global__ void __launch_bounds__(kUnitThreads) k_combine(const CombineParams p)
     const int c = ((int)blockIdx.x % p.chunks) * kUnitColumns + tid % kUnitColumns;
     slice_s[tid] = c < p.m ? column_sum(p.states + 2 + (size_t)i * p.m + c, sl, kUnitSlices, p.K, slen) : 0.0;
     if (blockIdx.x == 0 && warp < 2) {
-        const double h = scalar_mean(p.states, p.K, slen, warp, lane);
+        const double h = scalar_sum(p.states, p.K, slen, warp, lane) * p.inv_k;
         if (lane == 0) { p.scratch[warp] = h; __threadfence(); }
     }
     __syncthreads();
@@ -141,7 +150,7 @@ __global__ void __launch_bounds__(kUnitThreads) k_combine(const CombineParams p)
         double t = 0.0;
 #pragma unroll
         for (int q = 0; q < kUnitSlices; ++q) t += slice_s[q * kUnitColumns + tid];
-        t /= (double)p.K;
+        t *= p.inv_k;
         t = warp_sum(t * t);
         if (lane == 0) part_s[warp] = t;
     }
@@ -167,14 +176,15 @@ __global__ void __launch_bounds__(kUnitThreads) k_combine(const CombineParams p)
 }  // namespace
 
 cudaError_t fda_launch_combine(const fda_ctx *ctx, const float *states, int K, int variant,
-                               float epsilon, float theta, fda_estimate *est_dev, fda_estimate *est_host,
-                               cudaStream_t s)
+                               float epsilon, float theta, fda_estimate *est_dev, unsigned long long *host,
+                               unsigned int seq, cudaStream_t s)
 {
     CombineParams p{};
     p.states = states; p.K = K; p.l = ctx->l; p.m = ctx->m;
-    p.variant = variant; p.epsilon = epsilon; p.theta = theta;
+    p.variant = variant; p.theta = theta;
+    p.inv_k = 1.0 / (double)K; p.inv_eps = 1.0 / (1.0 + (double)epsilon);
     p.scratch = ctx->combine_scratch; p.ticket = ctx->combine_ticket;
-    p.est = est_dev; p.est_host = est_host;
+    p.est = est_dev; p.host = host; p.seq = seq;
     if (ctx->l == 0 || (int64_t)K * ctx->lm <= kOneBlock)
         return fda_launch_dependent(k_combine_small, 1, kThreads, 0, s, p);
     p.chunks = (ctx->m + kUnitColumns - 1) / kUnitColumns;

@@ -74,7 +74,11 @@ struct fda_ctx {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     double *combine_scratch = nullptr;        // fda_combine_scratch_doubles: S-bar[0..1] and the partial row norms
     unsigned int *combine_ticket = nullptr;   // blocks of the combine kernel that have finished (0 between launches)
-    fda_estimate *est_pinned = nullptr;       // slot of mapped host memory for callers that read the estimate at once (may be null)
+    // Slot of mapped host memory for callers that read the estimate at once (may be null): 64-bit words, the
+    // estimate's number in the upper halves, in the lower ones mean_sq_norm, est_sq_norm_of_mean, H,
+    // trigger and the l row norms.
+    unsigned long long *est_pinned = nullptr;
+    unsigned int est_seq = 0;                 // number of the last estimate asked for through est_pinned
     unsigned int *row_tickets = nullptr;      // the same per row group of the pass without a sketch
     int n_row_tickets = 0;
     // staging for fda_round_host (lazy)
@@ -97,13 +101,13 @@ struct fda_ctx {
 #ifdef __CUDACC__
 __device__ __forceinline__ void fda_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... Params, typename... Args>
-cudaError_t fda_launch_dependent(void (*kern)(Params...), int blocks, int threads, size_t smem, cudaStream_t s, Args... args)
+cudaError_t fda_launch_dependent(void (*kern)(Params...), dim3 blocks, int threads, size_t smem, cudaStream_t s, Args... args)
 {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3((unsigned)threads);
+    cfg.gridDim = blocks; cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem; cfg.stream = s; cfg.attrs = &attr; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
 }
@@ -136,8 +140,8 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
                                   cudaStream_t s);
 cudaError_t fda_setup_local_state(fda_ctx *ctx);   // opt-in shared memory, pick geometry
 cudaError_t fda_launch_combine(const fda_ctx *ctx, const float *states, int K, int variant,
-                               float epsilon, float theta, fda_estimate *est_dev, fda_estimate *est_host,
-                               cudaStream_t s);
+                               float epsilon, float theta, fda_estimate *est_dev, unsigned long long *host,
+                               unsigned int seq, cudaStream_t s);
 size_t fda_combine_scratch_doubles(int l, int m);
 cudaError_t fda_launch_average(const fda_ctx *ctx, float *w, int64_t row_stride, int K, int64_t d,
                                float *w_t0, float *xi_out, const fda_estimate *est_dev, uint32_t flags,

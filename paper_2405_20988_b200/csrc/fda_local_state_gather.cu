@@ -63,16 +63,13 @@ using namespace fda_list;
 //   then      ut[2][T + 8][4]   (drift tiles, index-major; eight zero rows behind each)
 // PW producer warps and WW walker warps: the split that is fastest depends on how much walking a
 // loaded index pays for (l updates per worker).  PARTS: the sketch rows are in several parts with
-// records of their own, and a block serves one part of one worker group.  SPLIT: a vector of few
-// tiles leaves most SMs without a block, so p.part_tiles blocks share the tile of each: all of them form
-// the drifts, each walks every p.part_tiles-th item, and their bins, which differ in the cells they touch,
-// are partial sums like those of any other blocks (so the cells come out the same bit for bit).
+// records of their own, and a block serves one part of one worker group.
 // Measured: 8 x 1000 as two parts, K = 20, d = 2.6M: 212 us, against 510 us on the compare-and-swap
-// kernel that served it before; shared tiles, 5 x 250, K = 5, d = 61,706: 12.5 -> 10 us.
+// kernel that served it before.
 // VEC: w, w_t0 and xi are 16-byte aligned.  If not, a producer thread owns the four indices lane, lane + 32,
 // ... of its warp's 128 instead of four consecutive ones, so that its 32-bit loads are coalesced (K = 30,
 // d = 6,964,106 at a pitch of d: 529 -> 370 us; 7 x 500, K = 60, d = 20M: 4.38 -> 2.75 ms).
-template <bool LINEAR, int PW, int WW, bool PARTS, bool SPLIT, bool VEC>
+template <bool LINEAR, int PW, int WW, bool PARTS, bool VEC>
 __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const ListParams p)
 {
     constexpr int kProducerWarps = PW;
@@ -87,9 +84,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     static_assert(PW <= kMaxProducerWarps, "the fp64 sums have room for kMaxProducerWarps warps");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int sub = SPLIT ? (int)blockIdx.x / (p.groups * p.cpg) : 0, split = SPLIT ? p.part_tiles : 1;
-    const int blk = SPLIT ? (int)blockIdx.x % (p.groups * p.cpg) : (int)blockIdx.x;
-    const int vg = blk % p.groups, c = blk / p.groups;
+    const int vg = (int)blockIdx.x % p.groups, c = (int)blockIdx.x / p.groups;
     const int g = PARTS ? vg % p.wgroups : vg;
     const uint64_t *sched_off = PARTS ? p.sched_off + (size_t)(vg / p.wgroups) * p.part_tiles : p.sched_off;
     const int T = p.T, lm = p.l * p.m;
@@ -310,7 +305,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                     walk(b);
                 }
             } else {
-            int it = (warp - kProducerWarps) * split + sub;
+            int it = warp - kProducerWarps;
             uint32_t d0 = 0, chunk0 = 0;
             if (it < n_items) { d0 = tab[4 + 2 * it]; chunk0 = tab[5 + 2 * it]; }
             while (it < n_items) {
@@ -318,7 +313,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                 const uint32_t cell = cells[(size_t)(d0 >> 16) * kListSlots + lane];
                 const uint2 *ent = reinterpret_cast<const uint2 *>(ent0 + (size_t)chunk0 * 256) + lane;
                 const int nch = (steps + 3) >> 2;
-                if (lane == 0) it = atomicAdd(&ctr[buf], 1) * split + sub;
+                if (lane == 0) it = atomicAdd(&ctr[buf], 1);
                 it = __shfl_sync(0xffffffffu, it, 0);
                 if (it < n_items) { d0 = tab[4 + 2 * it]; chunk0 = tab[5 + 2 * it]; }
                 unsigned long long a01 = 0ull, a23 = 0ull;
@@ -349,7 +344,135 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     if (tid < GW * 2) {
         double t = 0.0;
         for (int q = 0; q < kProducerWarps; ++q) t += sums[q * GW * 2 + tid];
-        p.part_np[(size_t)blockIdx.x * GW * 2 + tid] = sub == 0 ? t : 0.0;
+        p.part_np[(size_t)blockIdx.x * GW * 2 + tid] = t;
+    }
+}
+
+constexpr int kShortWarps = 24;
+constexpr int kShortChunks = 2;                // chunks of 128 indices a warp forms: tiles of up to 6144 indices
+constexpr uint32_t kShortBins = kShortWarps * GW * 2 * 8;      // offset of the bins, behind the warps' sums
+inline size_t short_smem_bytes(int lm, int T) { return kShortBins + (size_t)lm * GW * 4 + (size_t)(T + kListPadRows) * GW * 4; }
+
+// The sketch pass of vectors with so few tiles that every SM can have a block of its own and more:
+// a block serves one tile, p.part_tiles blocks share it - all of them form its drifts, each walks every
+// p.part_tiles-th item - and their bins, which differ in the cells they touch, are partial sums like
+// those of any other blocks, so the cells come out the same bit for bit.
+// Bound: latency, so there are no roles and no second buffer: every warp has its first item's entries
+// on their way (the schedule is older than the kernel before this one, so even in front of
+// fda_grid_wait), then all the loads of its two chunks of indices, stores the drifts, and after one barrier walks.
+// Measured, 5 x 250, K = 5, d = 61,706, with its finalize kernel, back to back: 8.7 us with up to three blocks
+// to a tile (8.9 with two or four), against 10.3 with 16 producer and 12 walker warps on shared tiles and
+// 14.4 with 8 + 20 warps on a tile of its own.
+template <bool LINEAR, bool VEC>
+__global__ void __launch_bounds__(kShortWarps * 32, 1) k_local_state_short(const ListParams p)
+{
+    constexpr int kThreads = kShortWarps * 32;
+    constexpr int kAhead = 7;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int split = p.part_tiles, sub = (int)blockIdx.x / (p.groups * p.cpg), blk = (int)blockIdx.x % (p.groups * p.cpg);
+    const int g = blk % p.groups, c = blk / p.groups;         // the block's tile is tile c
+    const int T = p.T, lm = p.l * p.m;
+    const uint32_t smem_base = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    const uint32_t base = smem_base + kShortBins + (uint32_t)lm * 16u;
+    double *sums = reinterpret_cast<double *>(smem_raw);
+    float *bins = reinterpret_cast<float *>(smem_raw + kShortBins);
+
+    const unsigned char *rec = p.sched + load_u64(p.sched_off + c);
+    const uint32_t *tab = reinterpret_cast<const uint32_t *>(rec);
+    int it = warp * split + sub;
+    const int n_items = (int)__ldg(tab);
+    const uint16_t *cells = reinterpret_cast<const uint16_t *>(rec + fda_sched_cells_off(n_items));
+    const unsigned char *ent0 = rec + fda_sched_entries_off(n_items);
+    int steps = 0;
+    uint32_t cell = 0;
+    const uint2 *ent = nullptr;
+    uint2 ch[kAhead];
+    auto fetch = [&]() {
+        const uint32_t d0 = __ldg(tab + 4 + 2 * it), chunk0 = __ldg(tab + 5 + 2 * it);
+        steps = (int)(d0 & 0xffffu);
+        cell = __ldg(cells + (size_t)(d0 >> 16) * kListSlots + lane);
+        ent = reinterpret_cast<const uint2 *>(ent0 + (size_t)chunk0 * 256) + lane;
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q)
+            if (4 * q < steps) ch[q] = __ldg(ent + (size_t)q * kListSlots);
+    };
+    if (it < n_items) fetch();
+    for (int t = tid; t < lm * GW; t += kThreads) bins[t] = 0.f;
+    if (tid < kListPadRows) store_row(base + (uint32_t)(T + tid) * 16u, 0.f, 0.f, 0.f, 0.f);
+    fda_grid_wait();
+
+    // ---- the drifts of chunks warp, warp + kShortWarps, ... of 128 indices ----
+    // (workers past K alias the group's first row: their sums are never written out)
+    const float *wbase = p.w + (size_t)(g * GW) * (size_t)p.row_stride;
+    float4 wv[kShortChunks][GW], w0v[kShortChunks], xv[kShortChunks];
+#pragma unroll
+    for (int b = 0; b < kShortChunks; ++b) {
+        const int first = 128 * (warp + kShortWarps * b);
+        const int64_t j = (int64_t)c * T + first + (VEC ? 4 * lane : lane), left = first < T ? p.d - j : 0;
+        const int n = VEC ? (left >= 4 ? 4 : left > 0 ? (int)left : 0) : (left > 96 ? 4 : left > 0 ? (int)(left + 31) / 32 : 0);
+        auto load = [&](const float *ptr) { return VEC ? load_quad<false>(ptr, n == 4, n) : load_strided(ptr, n); };
+#pragma unroll
+        for (int k = 0; k < GW; ++k) wv[b][k] = load(wbase + (g * GW + k < p.K ? (int64_t)k * p.row_stride : 0) + j);
+        w0v[b] = load(p.w_t0 + j);
+        if (LINEAR) xv[b] = load(p.xi + j);
+    }
+    float nf[GW], pf[GW];
+#pragma unroll
+    for (int k = 0; k < GW; ++k) { nf[k] = 0.f; pf[k] = 0.f; }
+#pragma unroll
+    for (int b = 0; b < kShortChunks; ++b) {
+        const uint32_t first = 128u * (uint32_t)(warp + kShortWarps * b);
+        if (first >= (uint32_t)T) break;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float w0 = comp(w0v[b], q);
+            float u[GW];
+#pragma unroll
+            for (int k = 0; k < GW; ++k) {
+                u[k] = comp(wv[b][k], q) - w0;
+                nf[k] = fmaf(u[k], u[k], nf[k]);
+                if (LINEAR) pf[k] = fmaf(comp(xv[b], q), u[k], pf[k]);
+            }
+            const uint32_t r = first + (VEC ? 4u * lane + q : (uint32_t)lane + 32u * q);
+            store_row(base + fda_list_row(r) * 16u, u[0], u[1], u[2], u[3]);
+        }
+    }
+    if (sub == 0) {                                           // fp32 within a warp's indices of the tile, then fp64
+#pragma unroll
+        for (int k = 0; k < GW; ++k) {
+            float a = nf[k], bq = LINEAR ? pf[k] : 0.f;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, off);
+                if (LINEAR) bq += __shfl_xor_sync(0xffffffffu, bq, off);
+            }
+            if (lane == 0) { sums[(warp * GW + k) * 2] = (double)a; sums[(warp * GW + k) * 2 + 1] = (double)bq; }
+        }
+    }
+    __syncthreads();
+
+    // ---- items warp * split + sub, then every (kShortWarps * split)-th ----
+    while (it < n_items) {
+        unsigned long long a01 = 0ull, a23 = 0ull;
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) walk_chunk(ch[q], steps - 4 * q, base, a01, a23);
+        for (int c0 = kAhead; 4 * c0 < steps; ++c0)
+            walk_chunk(__ldg(ent + (size_t)c0 * kListSlots), steps - 4 * c0, base, a01, a23);
+        const uint32_t done = cell;
+        it += kShortWarps * split;
+        if (it < n_items) fetch();
+        flush_item(bins, lm, done, a01, a23);
+    }
+    __syncthreads();
+
+    float *out = p.part_sk + (size_t)blockIdx.x * (size_t)lm * GW;
+    for (int t = tid; t < lm; t += kThreads) reinterpret_cast<float4 *>(out)[t] = reinterpret_cast<const float4 *>(bins)[t];
+    if (tid < GW * 2) {
+        double t = 0.0;
+        if (sub == 0)
+            for (int q = 0; q < kShortWarps; ++q) t += sums[q * GW * 2 + tid];
+        p.part_np[(size_t)blockIdx.x * GW * 2 + tid] = t;
     }
 }
 
@@ -364,68 +487,71 @@ struct ListParts {
 
 // states[k][.] = sum of the partials of worker k's blocks in fp64, in a fixed order: four
 // adjacent lanes share one output, lane s adds the blocks s, s + 4, ... of the worker's group in
-// each launch in order (eight loads in flight), and the four sums are added as (s0 + s1) + (s2 + s3).
-__global__ void k_finalize_gather(const ListParams p, const ListParts parts, uint32_t flags, float *__restrict__ states)
+// each launch in order, and the four sums are added as (s0 + s1) + (s2 + s3).
+// Bound: latency (a few megabytes at most, from L2): twelve values are asked for at a time,
+// whatever the number of blocks, and blockIdx.y is the worker group, so that no index is divided.
+// Measured with the kernel before it, 5 x 250, K = 10, d = 150K (25 blocks a group): 12.1 us with eight or sixteen
+// values at a time and 64-bit divisions, 11.7 now; four at a time cost 3 us.
+__global__ void __launch_bounds__(256) k_finalize_gather(const ListParams p, const ListParts parts, uint32_t flags, float *__restrict__ states)
 {
+    constexpr int kLoads = 12;
     const int lm = p.l * p.m, slen = 2 + lm * (p.groups / p.wgroups);       // lm: cells of a part
-    const bool sketch = (flags & FDA_STATE_SKETCH) != 0;
-    const int64_t total = (int64_t)p.wgroups * slen * GW * 4;
-    const int64_t padded = (total + 31) & ~(int64_t)31;                 // whole warps take part in the shuffles
+    const int t = blockIdx.x * 256 + threadIdx.x, sub = t & 3, kl = (t >> 2) % GW, e = t / (4 * GW), g = blockIdx.y;
+    const bool on = e >= slen ? false
+                  : e == 0    ? (flags & FDA_STATE_NORM) != 0
+                  : e == 1    ? (flags & FDA_STATE_LINEAR) != 0 && p.have_xi != 0
+                              : (flags & FDA_STATE_SKETCH) != 0;
+    const int part = e < 2 ? 0 : (e - 2) / lm;                  // part 0 also has the norm and the projection
     fda_grid_wait();
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < padded;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const bool valid = t < total;
-        const int sub = (int)(t & 3);
-        const int64_t o = t >> 2;
-        const int kl = (int)(o % GW);
-        const int e = (int)((o / GW) % slen);
-        const int g = (int)(o / ((int64_t)GW * slen));
-        const int k = g * GW + kl;
-        double acc = 0.0;
-        for (int q = 0; q < parts.n; ++q) {
-            const int part = e < 2 ? 0 : (e - 2) / lm;                  // part 0 also has the norm and the projection
-            const int gl = part * p.wgroups + g - parts.g_first[q];
-            if (!valid || gl < 0 || gl >= parts.groups[q]) continue;
-            const int nb = parts.cpg[q];                                // blocks of this group: gl, gl + groups, ...
-            const size_t first = (size_t)(parts.slot_base[q] + gl);
-            if (e < 2) {
-                const bool on = (e == 0) ? (flags & FDA_STATE_NORM) != 0
-                                         : ((flags & FDA_STATE_LINEAR) != 0 && p.have_xi);
-                if (on)
-                    for (int j = sub; j < nb; j += 4)
-                        acc += p.part_np[((first + (size_t)j * parts.groups[q]) * GW + kl) * 2 + e];
-            } else if (sketch) {
-                const size_t step = (size_t)lm * GW * parts.groups[q];  // from one block of the group to the next
-                const float *src = p.part_sk + first * lm * GW + (size_t)(e - 2 - part * lm) * GW + kl + (size_t)sub * step;
-                int j = sub;
-                for (; j + 28 < nb; j += 32, src += 32 * step) {
-                    float v[8];
+    double acc = 0.0;
+    for (int q = 0; q < parts.n; ++q) {
+        const int gl = part * p.wgroups + g - parts.g_first[q];
+        if (!on || gl < 0 || gl >= parts.groups[q]) continue;
+        const int nb = parts.cpg[q];                            // blocks of this group: gl, gl + groups, ...
+        const size_t first = (size_t)(parts.slot_base[q] + gl), step = (size_t)parts.groups[q];
+        const double *np = p.part_np + (first * GW + kl) * 2 + e;
+        const float *sk = p.part_sk + first * lm * GW + (size_t)(e - 2 - part * lm) * GW + kl;
+        if (e < 2) {
+            for (int j = sub; j < nb; j += 4 * kLoads) {
+                double v[kLoads];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) v[u] = src[(size_t)(4 * u) * step];
+                for (int u = 0; u < kLoads; ++u) v[u] = np[(size_t)(j + 4 * u < nb ? j + 4 * u : j) * step * GW * 2];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) acc += (double)v[u];
-                }
-                for (; j < nb; j += 4, src += 4 * step) acc += (double)src[0];
+                for (int u = 0; u < kLoads; ++u) acc += j + 4 * u < nb ? v[u] : 0.0;
+            }
+        } else {
+            for (int j = sub; j < nb; j += 4 * kLoads) {
+                float v[kLoads];
+#pragma unroll
+                for (int u = 0; u < kLoads; ++u) v[u] = sk[(size_t)(j + 4 * u < nb ? j + 4 * u : j) * step * lm * GW];
+#pragma unroll
+                for (int u = 0; u < kLoads; ++u) acc += j + 4 * u < nb ? (double)v[u] : 0.0;
             }
         }
-        const double pair = acc + __shfl_xor_sync(0xffffffffu, acc, 1);      // lanes 0,1: s0 + s1; lanes 2,3: s2 + s3
-        const double other = __shfl_xor_sync(0xffffffffu, pair, 2);
-        if (valid && sub == 0 && k < p.K) states[(size_t)k * slen + e] = (float)(pair + other);
     }
+    const double pair = acc + __shfl_xor_sync(0xffffffffu, acc, 1);      // lanes 0,1: s0 + s1; lanes 2,3: s2 + s3
+    const double other = __shfl_xor_sync(0xffffffffu, pair, 2);
+    const int k = g * GW + kl;
+    if (e < slen && sub == 0 && k < p.K) states[(size_t)k * slen + e] = (float)(pair + other);
 }
 
-template <int PW, int WW, bool PARTS, bool SPLIT>
+template <int PW, int WW, bool PARTS>
 void (*pick_kernel(bool linear, bool vec))(ListParams)
 {
-    if (linear) return vec ? k_local_state_gather<true, PW, WW, PARTS, SPLIT, true> : k_local_state_gather<true, PW, WW, PARTS, SPLIT, false>;
-    return vec ? k_local_state_gather<false, PW, WW, PARTS, SPLIT, true> : k_local_state_gather<false, PW, WW, PARTS, SPLIT, false>;
+    if (linear) return vec ? k_local_state_gather<true, PW, WW, PARTS, true> : k_local_state_gather<true, PW, WW, PARTS, false>;
+    return vec ? k_local_state_gather<false, PW, WW, PARTS, true> : k_local_state_gather<false, PW, WW, PARTS, false>;
+}
+void (*pick_short(bool linear, bool vec))(ListParams)
+{
+    if (linear) return vec ? k_local_state_short<true, true> : k_local_state_short<true, false>;
+    return vec ? k_local_state_short<false, true> : k_local_state_short<false, false>;
 }
 
-template <int PW, int WW, bool PARTS, bool SPLIT>
+template <int PW, int WW, bool PARTS>
 cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent, cudaStream_t s)
 {
     if (p.T % 128 != 0 || p.T < PW * 128 || PW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
-    auto kern = pick_kernel<PW, WW, PARTS, SPLIT>(p.have_xi != 0, p.vec != 0);
+    auto kern = pick_kernel<PW, WW, PARTS>(p.have_xi != 0, p.vec != 0);
     if (dependent) return fda_launch_dependent(kern, blocks, (PW + WW) * 32, smem, s, p);
     kern<<<blocks, (PW + WW) * 32, smem, s>>>(p);
     return cudaGetLastError();
@@ -438,9 +564,8 @@ cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx)
 {
     for (int i = 0; i < 4; ++i) {
         const bool linear = i & 1, vec = i & 2;
-        for (auto kern : {pick_kernel<8, 20, false, false>(linear, vec), pick_kernel<5, 23, false, false>(linear, vec),
-                          pick_kernel<8, 20, true, false>(linear, vec), pick_kernel<16, 12, false, true>(linear, vec),
-                          pick_kernel<8, 20, false, true>(linear, vec)}) {
+        for (auto kern : {pick_kernel<8, 20, false>(linear, vec), pick_kernel<5, 23, false>(linear, vec),
+                          pick_kernel<8, 20, true>(linear, vec), pick_short(linear, vec)}) {
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
             if (e != cudaSuccess) return e;
         }
@@ -483,12 +608,11 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     const size_t smem = fda_list_smem_bytes(p.l, p.m, p.T, ctx->sched_ni_max);
     if (smem > (size_t)ctx->smem_optin) return cudaErrorNotSupported;
 
-    // A vector with at most one tile per block and SMs left for as many blocks again: the items of a
-    // tile are split, and with less walking per block more of its warps load (the drifts of a tile are
-    // a chain of round trips, one per batch: three with 16 producer warps, six with 8).
+    // A vector with at most one tile per block and SMs left for as many blocks again: several blocks
+    // share a tile (k_local_state_short).
     int split = 1;
     if (ctx->sched_parts == 1) {
-        if (p.tiles == p.cpg && 2 * blocks <= ctx->n_sm) split = std::min(8, ctx->n_sm / blocks);
+        if (p.tiles == p.cpg && 2 * blocks <= ctx->n_sm && p.T <= kShortWarps * 128 * kShortChunks) split = std::min(3, ctx->n_sm / blocks);
         p.part_tiles = split;
     }
     // 8 producer + 20 walker warps, or 5 + 23 when a loaded index pays for more walking.  Measured,
@@ -497,11 +621,12 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     // 2.61 with 12 + 16; 8 x 1000 in parts, K = 20, d = 2.6M: 214 us with 8 + 20, 216 with 10 + 18,
     // 231 with 6 + 22, 226 with 8 + 24 (64 registers).
     auto launch = [&](ListParams &q, int grid, cudaStream_t st, bool dependent) {
-        if (ctx->sched_parts > 1) return launch_lists<8, 20, true, false>(q, grid, smem, dependent, st);
-        if (split > 1) return q.T % 2048 == 0 ? launch_lists<16, 12, false, true>(q, grid, smem, dependent, st)
-                                                : launch_lists<8, 20, false, true>(q, grid, smem, dependent, st);
-        return p.l >= 7 ? launch_lists<5, 23, false, false>(q, grid, smem, dependent, st)
-                        : launch_lists<8, 20, false, false>(q, grid, smem, dependent, st);
+        if (ctx->sched_parts > 1) return launch_lists<8, 20, true>(q, grid, smem, dependent, st);
+        if (split > 1)
+            return fda_launch_dependent(pick_short(q.have_xi != 0, q.vec != 0), grid, kShortWarps * 32,
+                                        short_smem_bytes(q.l * q.m, q.T), st, q);
+        return p.l >= 7 ? launch_lists<5, 23, false>(q, grid, smem, dependent, st)
+                        : launch_lists<8, 20, false>(q, grid, smem, dependent, st);
     };
     ListParts parts{};
     parts.n = 1;
@@ -556,9 +681,7 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         e = launch(p, blocks * split, s, true);
     }
     if (e != cudaSuccess) return e;
-    const int64_t total = (int64_t)p.wgroups * (2 + ctx->lm) * GW * 4;
-    int fb = (int)((total + 255) / 256);
-    if (fb > ctx->n_sm * 8) fb = ctx->n_sm * 8;
+    const dim3 fb((unsigned)(((2 + ctx->lm) * GW * 4 + 255) / 256), (unsigned)p.wgroups);
     ctx->last_ls_launches = parts.n + 1;
     if (parts.n == 1) return fda_launch_dependent(k_finalize_gather, fb, 256, 0, s, p, parts, flags, states);
     k_finalize_gather<<<fb, 256, 0, s>>>(p, parts, flags, states);       // waits for an event too: an ordinary launch
