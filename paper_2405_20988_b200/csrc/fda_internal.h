@@ -132,6 +132,8 @@ cudaError_t fda_launch_mean_state_gather(fda_ctx *ctx, const float *w, int64_t r
                                          uint32_t flags, float *mean_state, cudaStream_t s);
 cudaError_t fda_launch_mean_sketch_gather(fda_ctx *ctx, const float *mean_drift, int K, int64_t d, bool have_xi,
                                           uint32_t flags, int np_blocks, float *mean_state, cudaStream_t s);
+cudaError_t fda_launch_finalize_mean(const fda_ctx *ctx, int blocks, int np_blocks, int lm, int K, uint32_t flags,
+                                     bool have_xi, double cell_div, float *mean_state, cudaStream_t s);
 cudaError_t fda_launch_local_state_linear(fda_ctx *ctx, const float *w, int64_t row_stride, int K,
                                           int64_t d, const float *w_t0, const float *xi,
                                           uint32_t flags, float *states, cudaStream_t s);

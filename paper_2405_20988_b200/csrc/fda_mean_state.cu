@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(32 * FDA_MAX_ROWS, 1) k_sketch_vector_rows(con
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *bins = reinterpret_cast<float *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;      // blockDim = 32 * l
-    for (int i = tid; i < p.lm * 32; i += blockDim.x) bins[i] = 0.f;
+    for (int i = tid; i < p.lm * 8; i += blockDim.x) reinterpret_cast<float4 *>(bins)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
     fda_grid_wait();
     const uint32_t rowaddr = (uint32_t)__cvta_generic_to_shared(bins) + (uint32_t)row * ((uint32_t)p.m << 7) +
@@ -321,33 +321,6 @@ __global__ void __launch_bounds__(32 * FDA_MAX_ROWS, 1) k_sketch_vector_rows(con
         for (int c = 0; c < 32; ++c) v += bins[cell * 32 + ((c + tid) & 31)];
         out[cell] = v;
     }
-}
-
-// mean_state[e] = sum over blocks in fp64 [/ K for the two scalars].  Warp 0 and 1 of block 0
-// reduce the scalar partials (lanes stride the blocks, fixed shuffle tree); the cells are summed
-// in block order by one thread each.
-__global__ void k_finalize_mean(const float *__restrict__ part_sk, const double *__restrict__ part_np,
-                                int np_blocks, int sk_blocks, int lm, int K, uint32_t flags, bool have_xi,
-                                float *__restrict__ mean_state)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    fda_grid_wait();
-    if (blockIdx.x == 0 && warp < 2) {
-        const int e = warp;
-        const bool on = e == 0 ? (flags & FDA_STATE_NORM) != 0 : ((flags & FDA_STATE_LINEAR) != 0 && have_xi);
-        double acc = 0.0;
-        if (on)
-            for (int b = lane; b < np_blocks; b += 32) acc += part_np[(size_t)b * 2 + e];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) mean_state[e] = (float)(acc / (double)K);
-    }
-    const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= lm) return;
-    double acc = 0.0;
-    if (flags & FDA_STATE_SKETCH)
-        for (int b = 0; b < sk_blocks; ++b) acc += (double)part_sk[(size_t)b * lm + cell];
-    mean_state[2 + cell] = (float)acc;
 }
 
 int ilog2(int v) { int r = 0; while ((1 << (r + 1)) <= v) ++r; return r; }
@@ -446,7 +419,5 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
         }
         if (e != cudaSuccess) return e;
     }
-    const int n = ctx->lm > 64 ? ctx->lm : 64;        // at least two warps for the scalars
-    return fda_launch_dependent(k_finalize_mean, (n + 255) / 256, 256, 0, s, ctx->part_sk, ctx->part_np, (int)nblk,
-                                sk_blocks, ctx->lm, K, flags, linear, mean_state);
+    return fda_launch_finalize_mean(ctx, sk_blocks, (int)nblk, ctx->lm, K, flags, linear, 1.0, mean_state, s);
 }

@@ -361,41 +361,61 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
 }
 
 // Averaged state: mean_state[e] = (sum over the blocks of the partials) / divisor, in fp64 and in a
-// fixed order (block after block, eight loads in flight).  The two scalars are summed from
-// part_np[b * 2 + e], b < np_blocks - this kernel's own partials, or those of the pass that
-// averaged the drifts - and divided by K.
-__global__ void k_finalize_mean_gather(const float *__restrict__ part_sk, const double *__restrict__ part_np,
-                                       int blocks, int np_blocks, int cells, int lm /* of a part */, int K, uint32_t flags,
-                                       bool have_xi, double cell_div, float *__restrict__ mean_state)
+// fixed order.  Block 0 takes the two scalars, from part_np[b * 2 + e], b < np_blocks - the partials of
+// the list kernel or of the pass that averaged the drifts - and divides them by K; every other block 32
+// cells, eight threads to a cell.  Bound: latency, so twelve loads are in flight per thread.  Averaged
+// state with K = 10, d = 1.2M (148 blocks, 1172 pairs), back to back: 36.4 -> 28.9 us, d = 61,706, K = 5
+// 15.3 -> 12.5 us, against one thread per cell and one warp per scalar.
+constexpr int kFinalThreads = 256, kFinalCells = 32, kFinalLoads = 12;
+
+template <typename T>
+__device__ __forceinline__ double sum_strided(const T *src, int first, int step, int n, size_t pitch)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    fda_grid_wait();
-    if (blockIdx.x == 0 && warp < 2) {          // the scalars: lanes stride the partials, fixed shuffle tree
-        const int e = warp;
-        const bool on = (e == 0) ? (flags & FDA_STATE_NORM) != 0 : ((flags & FDA_STATE_LINEAR) != 0 && have_xi);
-        double acc = 0.0;
-        if (on)
-            for (int b = lane; b < np_blocks; b += 32) acc += part_np[(size_t)b * 2 + e];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) mean_state[e] = (float)(acc / (double)K);
-    }
-    const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= cells) return;
     double acc = 0.0;
-    if (flags & FDA_STATE_SKETCH) {
-        const float *src = part_sk + (size_t)(cell / lm) * blocks * lm + cell % lm;
-        int b = 0;
-        for (; b + 8 <= blocks; b += 8) {
-            float v[8];
+    for (int b = first; b < n; b += kFinalLoads * step) {
+        T v[kFinalLoads];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = src[(size_t)(b + u) * lm];
+        for (int u = 0; u < kFinalLoads; ++u) v[u] = src[(size_t)(b + u * step < n ? b + u * step : b) * pitch];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) acc += (double)v[u];
-        }
-        for (; b < blocks; ++b) acc += (double)src[(size_t)b * lm];
+        for (int u = 0; u < kFinalLoads; ++u) acc += b + u * step < n ? (double)v[u] : 0.0;
     }
-    mean_state[2 + cell] = (float)(acc / cell_div);
+    return acc;
+}
+
+__global__ void __launch_bounds__(kFinalThreads)
+k_finalize_mean(const float *part_sk, const double *part_np, int blocks, int np_blocks, int cells, int lm /* of a part */,
+                int K, uint32_t flags, bool have_xi, double cell_div, float *mean_state)
+{
+    __shared__ double red[kFinalThreads];
+    const int tid = threadIdx.x;
+    fda_grid_wait();
+    if (blockIdx.x == 0) {
+        const int e = tid & 1;
+        const bool on = e == 0 ? (flags & FDA_STATE_NORM) != 0 : ((flags & FDA_STATE_LINEAR) != 0 && have_xi);
+        red[tid] = on ? sum_strided(part_np + e, tid >> 1, kFinalThreads / 2, np_blocks, 2) : 0.0;
+        __syncthreads();
+        if (tid < 64) {                         // warp e adds the values of scalar e
+            double acc = 0.0;
+            for (int q = tid & 31; q < kFinalThreads / 2; q += 32) acc += red[2 * q + (tid >> 5)];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            if ((tid & 31) == 0) mean_state[tid >> 5] = (float)(acc / (double)K);
+        }
+        return;
+    }
+    const int cell = ((int)blockIdx.x - 1) * kFinalCells + tid % kFinalCells, slice = tid / kFinalCells;
+    constexpr int kSlices = kFinalThreads / kFinalCells;
+    double acc = 0.0;
+    if (cell < cells && (flags & FDA_STATE_SKETCH))
+        acc = sum_strided(part_sk + (size_t)(cell / lm) * blocks * lm + cell % lm, slice, kSlices, blocks, (size_t)lm);
+    red[tid] = acc;
+    __syncthreads();
+    if (slice == 0 && cell < cells) {
+        double t = 0.0;
+#pragma unroll
+        for (int q = 0; q < kSlices; ++q) t += red[q * kFinalCells + tid];
+        mean_state[2 + cell] = (float)(t / cell_div);
+    }
 }
 
 template <int AHEAD>
@@ -465,13 +485,20 @@ cudaError_t launch_mean(fda_ctx *ctx, const float *w, int64_t row_stride, int ro
         e = fda_launch_dependent(kern, blocks, kThreads, smem, s, mp);
         if (e != cudaSuccess) return e;
     }
-    const int fblocks = ((ctx->lm > 64 ? ctx->lm : 64) + 127) / 128;      // at least two warps for the scalars
-    return fda_launch_dependent(k_finalize_mean_gather, fblocks, 128, 0, s, ctx->part_sk, ctx->part_np, blocks,
-                                base_zero ? np_blocks : blocks, ctx->lm, lm, K, flags, have_xi,
-                                base_zero ? 1.0 : (double)K, mean_state);
+    return fda_launch_finalize_mean(ctx, blocks, base_zero ? np_blocks : blocks, lm, K, flags, have_xi,
+                                    base_zero ? 1.0 : (double)K, mean_state, s);
 }
 
 }  // namespace
+
+// mean_state from the partial sums: `blocks` partial sketches per part of lm cells, np_blocks partial pairs.
+cudaError_t fda_launch_finalize_mean(const fda_ctx *ctx, int blocks, int np_blocks, int lm, int K, uint32_t flags,
+                                     bool have_xi, double cell_div, float *mean_state, cudaStream_t s)
+{
+    return fda_launch_dependent(k_finalize_mean, 1 + (ctx->lm + kFinalCells - 1) / kFinalCells, kFinalThreads, 0, s,
+                                ctx->part_sk, ctx->part_np, blocks, np_blocks, ctx->lm, lm, K, flags, have_xi, cell_div,
+                                mean_state);
+}
 
 // The averaged state S-bar of fda_mean_state in one pass over the K rows.  Returns
 // cudaErrorNotSupported when the request does not fit this path (the caller then uses the other
