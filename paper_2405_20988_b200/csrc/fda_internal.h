@@ -22,7 +22,7 @@ constexpr int kListPadRows = 8;        // zero rows behind the tile, one per ban
 constexpr int kListBatch = 1024;       // indices a producer step covers; tiles are multiples of it
 constexpr int kListMaxTile = 7168;     // rows + pad rows must fit 13 bits
 constexpr int kListMinTilesPerBlock = 1;
-constexpr int kListSmemHead = 1088;    // counters and the producer warps' fp64 sums in front of the item tables
+constexpr int kListSmemHead = 2112;    // counters and the warps' fp64 sums in front of the item tables
 
 // byte offsets inside the schedule record of a tile with `items` items
 inline __host__ __device__ size_t fda_sched_cells_off(uint32_t items) { return ((size_t)16 + 8 * (size_t)items + 63) / 64 * 64; }

@@ -54,11 +54,72 @@ namespace {
 
 using namespace fda_list;
 
+// The drifts of the chunks first, first + step, ... (CHUNKS of them at a time) of 128 indices of the tile
+// that starts at index j0: all loads before any use, rows into the buffer at `base`, the warp's sums
+// of squares and products with xi (fp32) into sums[8] (fp64, lane 0).  VEC: a lane owns four consecutive
+// indices of a chunk, else the four indices lane, lane + 32, ...  Workers past K alias the group's
+// first row: their sums are never written out.
+template <bool LINEAR, bool VEC, int CHUNKS>
+__device__ __forceinline__ void form_drifts(const ListParams &p, int g, int64_t j0, int first, int step, uint32_t base,
+                                            double *sums)
+{
+    const int lane = threadIdx.x & 31, T = p.T;
+    const float *wbase = p.w + (size_t)(g * GW) * (size_t)p.row_stride;
+    float nf[GW], pf[GW];
+#pragma unroll
+    for (int k = 0; k < GW; ++k) { nf[k] = 0.f; pf[k] = 0.f; }
+#pragma unroll 1
+    for (int c0 = first; c0 < T / 128; c0 += step * CHUNKS) {
+        float4 wv[CHUNKS][GW], w0v[CHUNKS], xv[CHUNKS];
+#pragma unroll
+        for (int b = 0; b < CHUNKS; ++b) {
+            const int r = 128 * (c0 + step * b);
+            const int64_t j = j0 + r + (VEC ? 4 * lane : lane), left = r < T ? p.d - j : 0;
+            const int n = VEC ? (left >= 4 ? 4 : left > 0 ? (int)left : 0) : (left > 96 ? 4 : left > 0 ? (int)(left + 31) / 32 : 0);
+            auto load = [&](const float *ptr) { return VEC ? load_quad<false>(ptr, n == 4, n) : load_strided(ptr, n); };
+#pragma unroll
+            for (int k = 0; k < GW; ++k) wv[b][k] = load(wbase + (g * GW + k < p.K ? (int64_t)k * p.row_stride : 0) + j);
+            w0v[b] = load(p.w_t0 + j);
+            if (LINEAR) xv[b] = load(p.xi + j);
+        }
+#pragma unroll
+        for (int b = 0; b < CHUNKS; ++b) {
+            const uint32_t r0 = 128u * (uint32_t)(c0 + step * b);
+            if (r0 >= (uint32_t)T) break;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float w0 = comp(w0v[b], q);
+                float u[GW];
+#pragma unroll
+                for (int k = 0; k < GW; ++k) {
+                    u[k] = comp(wv[b][k], q) - w0;
+                    nf[k] = fmaf(u[k], u[k], nf[k]);
+                    if (LINEAR) pf[k] = fmaf(comp(xv[b], q), u[k], pf[k]);
+                }
+                const uint32_t r = r0 + (VEC ? 4u * lane + q : (uint32_t)lane + 32u * q);
+                store_row(base + fda_list_row(r) * 16u, u[0], u[1], u[2], u[3]);
+            }
+        }
+        if (CHUNKS > 1) break;                                 // (the caller has checked that one round covers the tile)
+    }
+#pragma unroll
+    for (int k = 0; k < GW; ++k) {
+        float a = nf[k], bq = LINEAR ? pf[k] : 0.f;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, off);
+            if (LINEAR) bq += __shfl_xor_sync(0xffffffffu, bq, off);
+        }
+        if (lane == 0) { sums[2 * k] = (double)a; sums[2 * k + 1] = (double)bq; }
+    }
+}
+
 // Shared-memory plan (bytes from the start of dynamic shared memory):
 //   [0, 8)    item counters of the two tile buffers
 //   [16, 48)  offsets of the schedule records of the tiles n, n + 1 (slot n mod 4)
-//   [64, 1088) sums[producer warp][worker][2] (fp64): ||u||^2 and <xi,u> over the tiles so far
-//   [1088, ..) two item tables (tab_bytes each): the head of a tile's schedule record
+//   [64, 2112) sums[warp][worker][2] (fp64): ||u||^2 and <xi,u>, of the producers over the tiles so far, of
+//             the walkers (FIRST) over their part of the first tile
+//   [2112, ..) two item tables (tab_bytes each): the head of a tile's schedule record
 //   then      bins[l*m][4]
 //   then      ut[2][T + 8][4]   (drift tiles, index-major; eight zero rows behind each)
 // PW producer warps and WW walker warps: the split that is fastest depends on how much walking a
@@ -69,7 +130,9 @@ using namespace fda_list;
 // VEC: w, w_t0 and xi are 16-byte aligned.  If not, a producer thread owns the four indices lane, lane + 32,
 // ... of its warp's 128 instead of four consecutive ones, so that its 32-bit loads are coalesced (K = 30,
 // d = 6,964,106 at a pitch of d: 529 -> 370 us; 7 x 500, K = 60, d = 20M: 4.38 -> 2.75 ms).
-template <bool LINEAR, int PW, int WW, bool PARTS, bool VEC>
+// FIRST: all warps form the first tile.  As the producers' own job it is a chain of round trips with nothing to
+// walk meanwhile, which counts when a block has few tiles; the code for it costs long runs 1 %.
+template <bool LINEAR, int PW, int WW, bool PARTS, bool VEC, bool FIRST>
 __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const ListParams p)
 {
     constexpr int kProducerWarps = PW;
@@ -81,7 +144,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     // items of parts.  Measured: 7 x 500, K = 60, d = 20M: 2.76 ms with 4 or 3, 2.79 with 5;
     // 5 x 250, K = 8, d = 198M: 2.33 ms with 7 or 8, 2.43 with 6, 2.38 with 5
     constexpr int kAhead = PARTS ? 2 : (PW == 5 && WW == 23) ? 4 : 7;
-    static_assert(PW <= kMaxProducerWarps, "the fp64 sums have room for kMaxProducerWarps warps");
+    static_assert(PW + WW <= 32, "the fp64 sums have room for 32 warps");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int vg = (int)blockIdx.x % p.groups, c = (int)blockIdx.x / p.groups;
@@ -105,9 +168,21 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
         reinterpret_cast<float *>(smem_raw + ut_off + (size_t)b * ut_bytes)[T * GW + r] = 0.f;
     }
     if (tid < 2) ctr[tid] = 0;
-    if (tid < kProducerWarps * GW * 2) sums[tid] = 0.0;
-    __syncthreads();
-    fda_grid_wait();
+    uint4 tab0 = make_uint4(0u, 0u, 0u, 0u);
+    if (FIRST) {
+        if (warp < kProducerWarps) {
+            const unsigned long long off = load_u64(sched_off + c);
+            if (tid * 16 < p.tab_bytes) tab0 = load_u4(p.sched + off + tid * 16);
+            if (tid == 0) rec_off[0] = off;
+        }
+        fda_grid_wait();
+        form_drifts<LINEAR, VEC, 1>(p, g, (int64_t)c * T, warp, PW + WW, smem_base + ut_off, sums + warp * GW * 2);
+        __syncthreads();
+    } else {
+        if (tid < kProducerWarps * GW * 2) sums[tid] = 0.0;
+        __syncthreads();
+        fda_grid_wait();
+    }
 
     const int n_tiles = p.tiles > c ? (int)((p.tiles - c + p.cpg - 1) / p.cpg) : 0;
 
@@ -124,10 +199,10 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
         float nf[GW], pf[GW];
 #pragma unroll
         for (int k = 0; k < GW; ++k) { nf[k] = 0.f; pf[k] = 0.f; }
-        int n_i = 0, n_c = 0;                             // tile being loaded / stored
+        int n_i = FIRST ? 1 : 0, n_c = 0;                 // tile being loaded / stored
         int b_i = 0, b_c = 0;                                 // batch inside it
-        uint32_t j_i = (uint32_t)c * (uint32_t)T + (VEC ? 4 * pt : 128 * warp + lane);   // first index of this thread's next loads
-        uint32_t end_i = (uint32_t)(c + 1) * (uint32_t)T;                 // end of the tile they belong to
+        uint32_t j_i = (uint32_t)(FIRST ? c + p.cpg : c) * (uint32_t)T + (VEC ? 4 * pt : 128 * warp + lane);   // first index of this thread's next loads
+        uint32_t end_i = (uint32_t)((FIRST ? c + p.cpg : c) + 1) * (uint32_t)T;   // end of the tile they belong to
         // 128-index chunks warp, warp + PW, ... of a tile, and the way from behind the last one to the
         // first of this block's next tile
         const int nb = (T / 128 - warp + PW - 1) / PW;
@@ -150,15 +225,42 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
             if (src && bytes)
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
         };
-        prefetch_tile(0);
+        if (!FIRST) prefetch_tile(0);
         prefetch_tile(1);
         // head of the schedule record of the tile being stored (the walkers' item table) and the
         // record offsets of the next tile, loaded one and two tiles ahead of their use
-        uint4 tabv = make_uint4(0u, 0u, 0u, 0u);
-        unsigned long long off0 = load_u64(sched_off + c), off1 = load_u64(sched_off + c + 1);
-        if (pt * 16 < p.tab_bytes) tabv = load_u4(p.sched + off0 + pt * 16);
-        if (pt == 0) rec_off[0] = off0;
+        uint4 tabv = tab0;
+        unsigned long long off0 = 0ull, off1 = 0ull;
+        if (!FIRST) {
+            off0 = load_u64(sched_off + c);
+            off1 = load_u64(sched_off + c + 1);
+            if (pt * 16 < p.tab_bytes) tabv = load_u4(p.sched + off0 + pt * 16);
+            if (pt == 0) rec_off[0] = off0;
+        }
         if (n_tiles > 1) { off0 = load_u64(sched_off + c + p.cpg); off1 = load_u64(sched_off + c + p.cpg + 1); }
+        // the walkers get tile n_c, which is in buffer `buf`
+        auto hand_over = [&](int buf) {
+            // the table of this tile (loaded a tile ago), the loads of the next one, the offsets
+            // of the one after: nothing here waits for memory
+            if (pt * 16 < p.tab_bytes)
+                *reinterpret_cast<uint4 *>(smem_raw + tab_off + (size_t)buf * p.tab_bytes + pt * 16) = tabv;
+            if (pt == 0) { ctr[buf] = WW; rec_off[(n_c + 1) & 3] = off0; }
+            if (n_c + 1 < n_tiles) {
+                const unsigned char *nrec = p.sched + off0;
+                if (pt * 16 < p.tab_bytes) tabv = load_u4(nrec + pt * 16);
+                for (uint64_t o = (uint64_t)pt * 128u; o < off1 - off0; o += (uint64_t)kProducerWarps * 32u * 128u)   // the record into L2 ahead of its walk
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(nrec + o));
+            }
+            if (n_c + 2 < n_tiles) {
+                const int64_t t2 = c + (int64_t)(n_c + 2) * p.cpg;
+                off0 = load_u64(sched_off + t2);
+                off1 = load_u64(sched_off + t2 + 1);
+            }
+            prefetch_tile(n_c + 2);
+            block_barrier<kThreads>();
+            b_c = 0;
+            ++n_c;
+        };
         auto issue = [&](int slot) {
             if (n_i < n_tiles) {
                 const float *q = wbase + j_i;
@@ -227,30 +329,12 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                     }
                     nf[k] = 0.f; pf[k] = 0.f;
                 }
-                // the table of this tile (loaded a tile ago), the loads of the next one, the offsets
-                // of the one after: nothing here waits for memory
-                if (pt * 16 < p.tab_bytes)
-                    *reinterpret_cast<uint4 *>(smem_raw + tab_off + (size_t)buf * p.tab_bytes + pt * 16) = tabv;
-                if (pt == 0) { ctr[buf] = WW; rec_off[(n_c + 1) & 3] = off0; }
-                if (n_c + 1 < n_tiles) {
-                    const unsigned char *nrec = p.sched + off0;
-                    if (pt * 16 < p.tab_bytes) tabv = load_u4(nrec + pt * 16);
-                    for (uint64_t o = (uint64_t)pt * 128u; o < off1 - off0; o += (uint64_t)kProducerWarps * 32u * 128u)   // the record into L2 ahead of its walk
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(nrec + o));
-                }
-                if (n_c + 2 < n_tiles) {
-                    const int64_t t2 = c + (int64_t)(n_c + 2) * p.cpg;
-                    off0 = load_u64(sched_off + t2);
-                    off1 = load_u64(sched_off + t2 + 1);
-                }
-                prefetch_tile(n_c + 2);
-                block_barrier<kThreads>();
-                b_c = 0;
-                ++n_c;
+                hand_over(buf);
             }
         };
 #pragma unroll
         for (int s = 0; s < kDepth; ++s) issue(s);
+        if (FIRST && n_tiles > 0) hand_over(0);
         while (n_c < n_tiles) {
 #pragma unroll
             for (int s = 0; s < kDepth; ++s) {
@@ -343,7 +427,7 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
     // ---- block partial of (||u||^2, <xi,u>) per worker: the producer warps' sums, in warp order ----
     if (tid < GW * 2) {
         double t = 0.0;
-        for (int q = 0; q < kProducerWarps; ++q) t += sums[q * GW * 2 + tid];
+        for (int q = 0; q < (FIRST ? PW + WW : kProducerWarps); ++q) t += sums[q * GW * 2 + tid];
         p.part_np[(size_t)blockIdx.x * GW * 2 + tid] = t;
     }
 }
@@ -402,54 +486,7 @@ __global__ void __launch_bounds__(kShortWarps * 32, 1) k_local_state_short(const
     if (tid < kListPadRows) store_row(base + (uint32_t)(T + tid) * 16u, 0.f, 0.f, 0.f, 0.f);
     fda_grid_wait();
 
-    // ---- the drifts of chunks warp, warp + kShortWarps, ... of 128 indices ----
-    // (workers past K alias the group's first row: their sums are never written out)
-    const float *wbase = p.w + (size_t)(g * GW) * (size_t)p.row_stride;
-    float4 wv[kShortChunks][GW], w0v[kShortChunks], xv[kShortChunks];
-#pragma unroll
-    for (int b = 0; b < kShortChunks; ++b) {
-        const int first = 128 * (warp + kShortWarps * b);
-        const int64_t j = (int64_t)c * T + first + (VEC ? 4 * lane : lane), left = first < T ? p.d - j : 0;
-        const int n = VEC ? (left >= 4 ? 4 : left > 0 ? (int)left : 0) : (left > 96 ? 4 : left > 0 ? (int)(left + 31) / 32 : 0);
-        auto load = [&](const float *ptr) { return VEC ? load_quad<false>(ptr, n == 4, n) : load_strided(ptr, n); };
-#pragma unroll
-        for (int k = 0; k < GW; ++k) wv[b][k] = load(wbase + (g * GW + k < p.K ? (int64_t)k * p.row_stride : 0) + j);
-        w0v[b] = load(p.w_t0 + j);
-        if (LINEAR) xv[b] = load(p.xi + j);
-    }
-    float nf[GW], pf[GW];
-#pragma unroll
-    for (int k = 0; k < GW; ++k) { nf[k] = 0.f; pf[k] = 0.f; }
-#pragma unroll
-    for (int b = 0; b < kShortChunks; ++b) {
-        const uint32_t first = 128u * (uint32_t)(warp + kShortWarps * b);
-        if (first >= (uint32_t)T) break;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float w0 = comp(w0v[b], q);
-            float u[GW];
-#pragma unroll
-            for (int k = 0; k < GW; ++k) {
-                u[k] = comp(wv[b][k], q) - w0;
-                nf[k] = fmaf(u[k], u[k], nf[k]);
-                if (LINEAR) pf[k] = fmaf(comp(xv[b], q), u[k], pf[k]);
-            }
-            const uint32_t r = first + (VEC ? 4u * lane + q : (uint32_t)lane + 32u * q);
-            store_row(base + fda_list_row(r) * 16u, u[0], u[1], u[2], u[3]);
-        }
-    }
-    if (sub == 0) {                                           // fp32 within a warp's indices of the tile, then fp64
-#pragma unroll
-        for (int k = 0; k < GW; ++k) {
-            float a = nf[k], bq = LINEAR ? pf[k] : 0.f;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                a += __shfl_xor_sync(0xffffffffu, a, off);
-                if (LINEAR) bq += __shfl_xor_sync(0xffffffffu, bq, off);
-            }
-            if (lane == 0) { sums[(warp * GW + k) * 2] = (double)a; sums[(warp * GW + k) * 2 + 1] = (double)bq; }
-        }
-    }
+    form_drifts<LINEAR, VEC, kShortChunks>(p, g, (int64_t)c * T, warp, kShortWarps, base, sums + warp * GW * 2);
     __syncthreads();
 
     // ---- items warp * split + sub, then every (kShortWarps * split)-th ----
@@ -535,11 +572,11 @@ __global__ void __launch_bounds__(256) k_finalize_gather(const ListParams p, con
     if (e < slen && sub == 0 && k < p.K) states[(size_t)k * slen + e] = (float)(pair + other);
 }
 
-template <int PW, int WW, bool PARTS>
+template <int PW, int WW, bool PARTS, bool FIRST>
 void (*pick_kernel(bool linear, bool vec))(ListParams)
 {
-    if (linear) return vec ? k_local_state_gather<true, PW, WW, PARTS, true> : k_local_state_gather<true, PW, WW, PARTS, false>;
-    return vec ? k_local_state_gather<false, PW, WW, PARTS, true> : k_local_state_gather<false, PW, WW, PARTS, false>;
+    if (linear) return vec ? k_local_state_gather<true, PW, WW, PARTS, true, FIRST> : k_local_state_gather<true, PW, WW, PARTS, false, FIRST>;
+    return vec ? k_local_state_gather<false, PW, WW, PARTS, true, FIRST> : k_local_state_gather<false, PW, WW, PARTS, false, FIRST>;
 }
 void (*pick_short(bool linear, bool vec))(ListParams)
 {
@@ -551,7 +588,12 @@ template <int PW, int WW, bool PARTS>
 cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent, cudaStream_t s)
 {
     if (p.T % 128 != 0 || p.T < PW * 128 || PW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
-    auto kern = pick_kernel<PW, WW, PARTS>(p.have_xi != 0, p.vec != 0);
+    // all warps form the first tile when a block has at most twelve.  Measured, kernel and finalize back to back:
+    // 5 x 250, K = 20, d = 300,000 (two tiles) 18.3 -> 17.4 us, K = 10, d = 1.2M (four) 34.1 -> 32.4 us; 7 x 500, K = 10,
+    // d = 1.2M (five) 46.0 -> 44.5 us; K = 20, d = 2M (twelve) 75.7 -> 75.3 us.
+    const bool first = !PARTS && p.tiles <= 12 * (int64_t)p.cpg;
+    auto kern = first ? pick_kernel<PW, WW, PARTS, !PARTS>(p.have_xi != 0, p.vec != 0)
+                      : pick_kernel<PW, WW, PARTS, false>(p.have_xi != 0, p.vec != 0);
     if (dependent) return fda_launch_dependent(kern, blocks, (PW + WW) * 32, smem, s, p);
     kern<<<blocks, (PW + WW) * 32, smem, s>>>(p);
     return cudaGetLastError();
@@ -564,8 +606,9 @@ cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx)
 {
     for (int i = 0; i < 4; ++i) {
         const bool linear = i & 1, vec = i & 2;
-        for (auto kern : {pick_kernel<8, 20, false>(linear, vec), pick_kernel<5, 23, false>(linear, vec),
-                          pick_kernel<8, 20, true>(linear, vec), pick_short(linear, vec)}) {
+        for (auto kern : {pick_kernel<8, 20, false, false>(linear, vec), pick_kernel<5, 23, false, false>(linear, vec),
+                          pick_kernel<8, 20, false, true>(linear, vec), pick_kernel<5, 23, false, true>(linear, vec),
+                          pick_kernel<8, 20, true, false>(linear, vec), pick_short(linear, vec)}) {
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
             if (e != cudaSuccess) return e;
         }

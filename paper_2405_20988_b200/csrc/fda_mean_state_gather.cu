@@ -111,7 +111,7 @@ inline size_t mean_smem_fixed(int l, int m, int T, int tab_bytes)
 //   [0, 8)      item counters of the two tile buffers
 //   [16, 48)    offsets of the schedule records of the tiles n, n + 1 (slot n mod 4)
 //   [64, 192)   sums[producer warp][2] (fp64): sum_k ||u_k||^2 and <xi, sum_k u_k> over the tiles so far
-//   [1088, ..)  two item tables (tab_bytes each): the head of a tile's schedule record
+//   [2112, ..)  two item tables (tab_bytes each): the head of a tile's schedule record
 //   then        bins[l*m]
 //   then        ut[2][T + 8]   (summed drifts; eight zero rows behind each)
 //   then        the landing zone: depth slots of R rows of kRowPitch bytes
