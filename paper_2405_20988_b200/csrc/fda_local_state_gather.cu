@@ -525,13 +525,15 @@ struct ListParts {
 // states[k][.] = sum of the partials of worker k's blocks in fp64, in a fixed order: four
 // adjacent lanes share one output, lane s adds the blocks s, s + 4, ... of the worker's group in
 // each launch in order, and the four sums are added as (s0 + s1) + (s2 + s3).
-// Bound: latency (a few megabytes at most, from L2): twelve values are asked for at a time,
-// whatever the number of blocks, and blockIdx.y is the worker group, so that no index is divided.
+// Bound: latency (a few megabytes at most, from L2): a lane asks for kLoads values at a time - four, eight
+// or twelve, as few as cover the blocks of a group in one or two rounds - and blockIdx.y is the worker
+// group, so that no index is divided.
 // Measured with the kernel before it, 5 x 250, K = 10, d = 150K (25 blocks a group): 12.1 us with eight or sixteen
-// values at a time and 64-bit divisions, 11.7 now; four at a time cost 3 us.
+// values at a time and 64-bit divisions, 11.7 now; four at a time cost 3 us there, and twelve cost 7 us at
+// 7 x 500, K = 60 (9 blocks a group).
+template <int kLoads>
 __global__ void __launch_bounds__(256) k_finalize_gather(const ListParams p, const ListParts parts, uint32_t flags, float *__restrict__ states)
 {
-    constexpr int kLoads = 12;
     const int lm = p.l * p.m, slen = 2 + lm * (p.groups / p.wgroups);       // lm: cells of a part
     const int t = blockIdx.x * 256 + threadIdx.x, sub = t & 3, kl = (t >> 2) % GW, e = t / (4 * GW), g = blockIdx.y;
     const bool on = e >= slen ? false
@@ -726,7 +728,9 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     if (e != cudaSuccess) return e;
     const dim3 fb((unsigned)(((2 + ctx->lm) * GW * 4 + 255) / 256), (unsigned)p.wgroups);
     ctx->last_ls_launches = parts.n + 1;
-    if (parts.n == 1) return fda_launch_dependent(k_finalize_gather, fb, 256, 0, s, p, parts, flags, states);
-    k_finalize_gather<<<fb, 256, 0, s>>>(p, parts, flags, states);       // waits for an event too: an ordinary launch
+    const int nb = parts.cpg[0];
+    auto fin = nb <= 16 ? k_finalize_gather<4> : nb <= 32 ? k_finalize_gather<8> : k_finalize_gather<12>;
+    if (parts.n == 1) return fda_launch_dependent(fin, fb, 256, 0, s, p, parts, flags, states);
+    fin<<<fb, 256, 0, s>>>(p, parts, flags, states);       // waits for an event too: an ordinary launch
     return cudaGetLastError();
 }
