@@ -574,6 +574,58 @@ __global__ void __launch_bounds__(256) k_finalize_gather(const ListParams p, con
     if (e < slen && sub == 0 && k < p.K) states[(size_t)k * slen + e] = (float)(pair + other);
 }
 
+// The same sums with the four workers of the group in each lane, 128-bit loads of the partials: a quarter of
+// the threads, for launches whose threads would not all be resident at once.  Lane s stores worker s.
+template <int kLoads>
+__global__ void __launch_bounds__(256) k_finalize_gather_wide(const ListParams p, const ListParts parts, uint32_t flags, float *__restrict__ states)
+{
+    const int lm = p.l * p.m, slen = 2 + lm * (p.groups / p.wgroups);
+    const int t = blockIdx.x * 256 + threadIdx.x, sub = t & 3, e = t / 4, g = blockIdx.y;
+    const bool on = e >= slen ? false
+                  : e == 0    ? (flags & FDA_STATE_NORM) != 0
+                  : e == 1    ? (flags & FDA_STATE_LINEAR) != 0 && p.have_xi != 0
+                              : (flags & FDA_STATE_SKETCH) != 0;
+    const int part = e < 2 ? 0 : (e - 2) / lm;
+    fda_grid_wait();
+    double acc[GW] = {};
+    for (int q = 0; q < parts.n; ++q) {
+        const int gl = part * p.wgroups + g - parts.g_first[q];
+        if (!on || gl < 0 || gl >= parts.groups[q]) continue;
+        const int nb = parts.cpg[q];
+        const size_t first = (size_t)(parts.slot_base[q] + gl), step = (size_t)parts.groups[q];
+        if (e < 2) {
+            const double *np = p.part_np + first * GW * 2 + e;
+            for (int j = sub; j < nb; j += 4)
+#pragma unroll
+                for (int k = 0; k < GW; ++k) acc[k] += np[(size_t)j * step * GW * 2 + 2 * k];
+        } else {
+            const float4 *sk = reinterpret_cast<const float4 *>(p.part_sk) + first * lm + (e - 2 - part * lm);
+            for (int j = sub; j < nb; j += 4 * kLoads) {
+                float4 v[kLoads];
+#pragma unroll
+                for (int u = 0; u < kLoads; ++u) v[u] = sk[(size_t)(j + 4 * u < nb ? j + 4 * u : j) * step * lm];
+#pragma unroll
+                for (int u = 0; u < kLoads; ++u) {
+                    const bool in = j + 4 * u < nb;
+                    acc[0] += in ? (double)v[u].x : 0.0;
+                    acc[1] += in ? (double)v[u].y : 0.0;
+                    acc[2] += in ? (double)v[u].z : 0.0;
+                    acc[3] += in ? (double)v[u].w : 0.0;
+                }
+            }
+        }
+    }
+    double mine = 0.0;
+#pragma unroll
+    for (int k = 0; k < GW; ++k) {
+        const double pair = acc[k] + __shfl_xor_sync(0xffffffffu, acc[k], 1);
+        const double other = __shfl_xor_sync(0xffffffffu, pair, 2);
+        if (sub == k) mine = pair + other;
+    }
+    const int k = g * GW + sub;
+    if (e < slen && k < p.K) states[(size_t)k * slen + e] = (float)mine;
+}
+
 template <int PW, int WW, bool PARTS, bool FIRST>
 void (*pick_kernel(bool linear, bool vec))(ListParams)
 {
@@ -726,10 +778,17 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         e = launch(p, blocks * split, s, true);
     }
     if (e != cudaSuccess) return e;
-    const dim3 fb((unsigned)(((2 + ctx->lm) * GW * 4 + 255) / 256), (unsigned)p.wgroups);
     ctx->last_ls_launches = parts.n + 1;
     const int nb = parts.cpg[0];
-    auto fin = nb <= 16 ? k_finalize_gather<4> : nb <= 32 ? k_finalize_gather<8> : k_finalize_gather<12>;
+    // one worker per lane while all those threads are resident at once (2048 to an SM), four beyond that.  Measured,
+    // kernel and finalize back to back, one and four per lane: 5 x 250, K = 10, d = 1.2M (60K threads) 30.0 and 34.3 us;
+    // 5 x 250, K = 30, d = 2M (160K) 110.6 both; 7 x 500, K = 60, d = 1.2M (841K) 191.0 and 184.7 us; 8 x 1000,
+    // K = 30, d = 300,000 (1.02M) 55.7 and 48.0 us.
+    const int64_t lanes = (int64_t)(2 + ctx->lm) * 4;
+    const bool wide = lanes * GW * p.wgroups > (int64_t)ctx->n_sm * 2048;
+    auto fin = wide ? (nb <= 16 ? k_finalize_gather_wide<4> : nb <= 32 ? k_finalize_gather_wide<8> : k_finalize_gather_wide<12>)
+                    : (nb <= 16 ? k_finalize_gather<4> : nb <= 32 ? k_finalize_gather<8> : k_finalize_gather<12>);
+    const dim3 fb((unsigned)((lanes * (wide ? 1 : GW) + 255) / 256), (unsigned)p.wgroups);
     if (parts.n == 1) return fda_launch_dependent(fin, fb, 256, 0, s, p, parts, flags, states);
     fin<<<fb, 256, 0, s>>>(p, parts, flags, states);       // waits for an event too: an ordinary launch
     return cudaGetLastError();

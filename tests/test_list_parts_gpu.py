@@ -16,7 +16,8 @@ P = (1 << 61) - 1
     (8, 1000, 5, 1, True), (8, 1000, 20, 5 * 5120 - 1, True), (8, 1000, 21, 150_001, False),       # two parts
     (16, 600, 9, 40_961, True), (4, 1200, 3, 30_720, False),
     (5, 250, 5, 6144, True), (5, 250, 4, 6145, False), (5, 250, 37, 12_289, True),                 # shared tiles
-    (7, 500, 10, 10_241, True), (3, 100, 6, 61_706, False)])
+    (7, 500, 10, 10_241, True), (3, 100, 6, 61_706, False),
+    (7, 500, 21, 150_001, True), (8, 1000, 9, 120_003, False), (16, 600, 8, 200_002, True)])       # finalize, four workers to a lane
 def test_parts_and_shared_tiles(l, m, K, d, aligned):
     import torch
     import oracle
