@@ -295,7 +295,8 @@ const char *fda_debug_last_kernel(const fda_ctx *ctx);
 
 /*
  * Number of kernels the context's last fda_local_state call launched (the paper has no
- * counterpart): 2 (the pass and the kernel that adds up its per-block partial sums), or 4 when the
+ * counterpart): 1 for the pass without a sketch (its last block per worker group writes the states),
+ * 2 for a sketch (the pass and the kernel that adds up its per-block partial sums), or 4 when the
  * sketch pass over index lists also ran its two tail launches on the context's second stream (worker
  * groups that do not divide the SMs, long vectors).  0 before the first call or for ctx == NULL.
  * The benchmark uses it to count the launches of a step.
