@@ -180,8 +180,8 @@ fda_status fda_mean_state(fda_ctx *ctx, const float *w, int64_t row_stride, int 
  *   trigger = (H > theta).  Accumulation is in fp64, results are rounded to fp32.
  *   states      K x state_len floats (as written by fda_local_state)
  *   est_dev     out, DEVICE fda_estimate
- *   est_host    out, HOST fda_estimate or NULL.  If not NULL the call copies the result
- *               and synchronises `stream` before returning.
+ *   est_host    out, HOST fda_estimate or NULL.  If not NULL the call returns when the result has
+ *               reached the host; all earlier work on `stream` and *est_dev are then complete.
  * Errors: INVALID_ARG (NULL, K < 1 or > K_max, bad variant, SKETCH variant with l == 0,
  * epsilon <= -1 or not finite, theta not finite), CUDA.
  */

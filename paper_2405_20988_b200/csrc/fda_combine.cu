@@ -92,7 +92,11 @@ __device__ __forceinline__ void finish(const CombineParams &p, double row, doubl
     }
     const float norm = lane < p.l ? (float)row : 0.f;
     if (lane < FDA_MAX_ROWS) est->row_sq_norm[lane] = norm;
-    if (p.host) {      // lane 4 + r: row r; every word carries the estimate's number, so no fence orders them
+    if (p.host) {      // lane 4 + r: row r; every word carries the estimate's number, so nothing orders the words
+        // among each other.  The fence puts *est (and the ticket) in front of them: the host that has read
+        // the words may launch a reader of *est on any stream.  It costs 0.4 us.
+        __threadfence();
+        __syncwarp();
         const float shifted = __shfl_up_sync(0xffffffffu, norm, 4);
         const uint32_t word = lane == 0 ? __float_as_uint((float)head0) : lane == 1 ? __float_as_uint((float)est_sq)
                             : lane == 2 ? __float_as_uint((float)H) : lane == 3 ? (uint32_t)trigger : __float_as_uint(shifted);
@@ -169,8 +173,8 @@ __global__ void __launch_bounds__(kUnitThreads) k_combine(const CombineParams p)
     double row = 0.0;
     if (lane < p.l)
         for (int q = 0; q < p.chunks; ++q) row += __ldcg(p.scratch + 2 + lane * p.chunks + q);
-    finish(p, row, __ldcg(p.scratch), __ldcg(p.scratch + 1), lane);
     if (lane == 0) *p.ticket = 0u;                         // ready for the next launch on this context
+    finish(p, row, __ldcg(p.scratch), __ldcg(p.scratch + 1), lane);
 }
 
 }  // namespace
