@@ -211,8 +211,9 @@ fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uin
     ctx->part_np_doubles = (size_t)ctx->max_blocks * (size_t)(K_max > 32 ? K_max : 32) * 2;
     if (e == cudaSuccess) e = cudaMalloc(&ctx->part_np, sizeof(double) * ctx->part_np_doubles);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->combine_scratch, sizeof(double) * fda_combine_scratch_doubles(ctx->l, ctx->m));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->combine_ticket, sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMemset(ctx->combine_ticket, 0, sizeof(unsigned int));
+    // one word for the combine kernel, two for the chunks of the model average
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->combine_ticket, 3 * sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemset(ctx->combine_ticket, 0, 3 * sizeof(unsigned int));
     ctx->est_pinned = g_estimates.take();
     ctx->n_row_tickets = (K_max + fda_rows::kRows - 1) / fda_rows::kRows;
     if (e == cudaSuccess) e = cudaMalloc(&ctx->row_tickets, sizeof(unsigned int) * ctx->n_row_tickets);
@@ -471,7 +472,7 @@ fda_status fda_context_info(const fda_ctx *ctx, int64_t *info)
     const int64_t table = ctx->tab ? (int64_t)(sizeof(uint16_t) * (size_t)ctx->l * ctx->tab_stride) : 0;
     const int64_t sched = ctx->sched ? (int64_t)(ctx->sched_bytes + sizeof(uint64_t) * (size_t)(ctx->sched_tiles * ctx->sched_parts + 1)) : 0;
     const int64_t partial = (int64_t)(sizeof(float) * ctx->part_sk_floats + sizeof(double) * ctx->part_np_doubles +
-                                      sizeof(double) * fda_combine_scratch_doubles(ctx->l, ctx->m) + sizeof(unsigned int) * (1 + ctx->n_row_tickets)) +
+                                      sizeof(double) * fda_combine_scratch_doubles(ctx->l, ctx->m) + sizeof(unsigned int) * (3 + ctx->n_row_tickets)) +
                             (ctx->coeffs_dev ? (int64_t)sizeof(uint64_t) * 6 * ctx->l : 0);
     const int64_t mean = ctx->mean_model ? (int64_t)sizeof(float) * ((ctx->d_max + 3) / 4 * 4) : 0;
     int64_t stage = 0;

@@ -25,14 +25,45 @@ __device__ __forceinline__ void block_partial(double dsq, double *part)
     }
 }
 
+// Chunks of a vector in the order in which blocks come free.  With a fixed stride some SMs run ahead of others,
+// so that the launch reads and writes rows all over a wide window and ends with few SMs at work; with tickets
+// the blocks stay side by side.  A block asks for its next chunk before it works on the one it has.
+// ticket[0]: chunks handed out beyond the first of every block, ticket[1]: blocks that are done; both 0 between launches.
+template <bool TICKETS>
+struct ChunkOrder {
+    unsigned int *ticket;
+    unsigned int *taken;        // two words of shared memory
+    unsigned int c = blockIdx.x;
+    int phase = 0;
+    __device__ __forceinline__ void ask()
+    {
+        if (TICKETS && threadIdx.x == 0) taken[phase] = gridDim.x + atomicAdd(ticket, 1u);
+    }
+    __device__ __forceinline__ void next()
+    {
+        if (!TICKETS) { c += gridDim.x; return; }
+        __syncthreads();
+        c = taken[phase];
+        phase ^= 1;
+    }
+    __device__ __forceinline__ void done()
+    {
+        if (!TICKETS || threadIdx.x != 0) return;
+        __threadfence();
+        if (atomicAdd(ticket + 1, 1u) == gridDim.x - 1) { ticket[0] = 0u; ticket[1] = 0u; }
+    }
+};
+
 // XI: also write the unnormalised direction of the global step, delta = w-bar_new - w_t0_old, to
 // xi_out and the block's partial of ||delta||^2 to part (Section 3.2: xi is the normalised
 // difference of the models of the last two synchronisations).
-template <bool XI>
+// TICKETS: chunks by ticket (not with XI: the partials of ||delta||^2 keep a fixed order).
+template <bool XI, bool TICKETS>
 __global__ void __launch_bounds__(256)
 k_average(float *w, int64_t row_stride, int K, int64_t d, float *__restrict__ w_t0,
-          const fda_estimate *est, int broadcast, float *__restrict__ xi_out, double *__restrict__ part)
+          const fda_estimate *est, int broadcast, float *__restrict__ xi_out, double *__restrict__ part, unsigned int *ticket)
 {
+    __shared__ unsigned int taken[2];
     fda_grid_wait();
     if (est != nullptr && est->trigger == 0) return;
     double dsq = 0.0;
@@ -40,30 +71,38 @@ k_average(float *w, int64_t row_stride, int K, int64_t d, float *__restrict__ w_
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nq = d / 4;
-    for (int64_t q = t0; q < nq; q += nthreads) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int k0 = 0; k0 < K; k0 += kBatch) {
-            float4 v[kBatch];
+    const unsigned int chunks = (unsigned int)((nq + 255) / 256);
+    ChunkOrder<TICKETS> order{ticket, taken};
+    while (order.c < chunks) {
+        order.ask();
+        const int64_t q = (int64_t)order.c * 256 + threadIdx.x;
+        if (q < nq) {
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k0 = 0; k0 < K; k0 += kBatch) {
+                float4 v[kBatch];
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b)
-                if (k0 + b < K)
-                    v[b] = __ldcs(reinterpret_cast<const float4 *>(w + (size_t)(k0 + b) * row_stride + q * 4));
+                for (int b = 0; b < kBatch; ++b)
+                    if (k0 + b < K)
+                        v[b] = __ldcs(reinterpret_cast<const float4 *>(w + (size_t)(k0 + b) * row_stride + q * 4));
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b)
-                if (k0 + b < K) { acc.x += v[b].x; acc.y += v[b].y; acc.z += v[b].z; acc.w += v[b].w; }
+                for (int b = 0; b < kBatch; ++b)
+                    if (k0 + b < K) { acc.x += v[b].x; acc.y += v[b].y; acc.z += v[b].z; acc.w += v[b].w; }
+            }
+            acc.x *= inv_k; acc.y *= inv_k; acc.z *= inv_k; acc.w *= inv_k;
+            if (XI) {
+                const float4 old = *reinterpret_cast<const float4 *>(w_t0 + q * 4);
+                const float4 dl = make_float4(acc.x - old.x, acc.y - old.y, acc.z - old.z, acc.w - old.w);
+                *reinterpret_cast<float4 *>(xi_out + q * 4) = dl;
+                dsq += (double)(dl.x * dl.x + dl.y * dl.y + dl.z * dl.z + dl.w * dl.w);
+            }
+            __stcs(reinterpret_cast<float4 *>(w_t0 + q * 4), acc);
+            if (broadcast)
+                for (int k = 0; k < K; ++k)
+                    __stcs(reinterpret_cast<float4 *>(w + (size_t)k * row_stride + q * 4), acc);
         }
-        acc.x *= inv_k; acc.y *= inv_k; acc.z *= inv_k; acc.w *= inv_k;
-        if (XI) {
-            const float4 old = *reinterpret_cast<const float4 *>(w_t0 + q * 4);
-            const float4 dl = make_float4(acc.x - old.x, acc.y - old.y, acc.z - old.z, acc.w - old.w);
-            *reinterpret_cast<float4 *>(xi_out + q * 4) = dl;
-            dsq += (double)(dl.x * dl.x + dl.y * dl.y + dl.z * dl.z + dl.w * dl.w);
-        }
-        __stcs(reinterpret_cast<float4 *>(w_t0 + q * 4), acc);
-        if (broadcast)
-            for (int k = 0; k < K; ++k)
-                __stcs(reinterpret_cast<float4 *>(w + (size_t)k * row_stride + q * 4), acc);
+        order.next();
     }
+    order.done();
     // the d % 4 tail
     for (int64_t j = nq * 4 + t0; j < d; j += nthreads) {
         float acc = 0.f;
@@ -86,12 +125,13 @@ k_average(float *w, int64_t row_stride, int K, int64_t d, float *__restrict__ w_
 // last but one is left to single floats, one thread each.
 // Measured on B200 with broadcast, K = 30, d = 6,964,106 at a pitch of d: 293 us (297 with aligned rows); with
 // 32-bit accesses throughout, as before, 346 us; eight rows a batch 310 us.
-template <bool XI>
+template <bool XI, bool TICKETS>
 __global__ void __launch_bounds__(256)
 k_average_shifted(float *w, int64_t row_stride, int K, int64_t d, float *w_t0,
-                  const fda_estimate *est, int broadcast, float *__restrict__ xi_out, double *__restrict__ part)
+                  const fda_estimate *est, int broadcast, float *__restrict__ xi_out, double *__restrict__ part, unsigned int *ticket)
 {
     using namespace fda_quads;
+    __shared__ unsigned int taken[2];
     fda_grid_wait();
     if (est != nullptr && est->trigger == 0) return;
     double dsq = 0.0;
@@ -100,45 +140,52 @@ k_average_shifted(float *w, int64_t row_stride, int K, int64_t d, float *w_t0,
     const int c0 = first_aligned(w_t0);
     // whole quads 1 .. Q - 1: the windows of all rows around them lie inside [0, d)
     const int64_t Q = d >= c0 + 12 ? (d - c0 - 8) / 4 + 1 : 1;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const unsigned int chunks = (unsigned int)((Q - 1 + 255) / 256);
     const bool xi_al = XI && misaligned(xi_out + c0) == 0;
-    for (int64_t q0 = 1 + 32 * ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); q0 < Q; q0 += 32 * nwarps) {
-        const int64_t q = q0 + lane;
-        const bool on = q < Q;
-        const int64_t j = c0 + 4 * (on ? q : q0);          // lanes past the end repeat the first quad
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int k0 = 0; k0 < K; k0 += kShiftedBatch) {
-            Window v[kShiftedBatch];
+    ChunkOrder<TICKETS> order{ticket, taken};
+    while (order.c < chunks) {
+        order.ask();
+        const int64_t q0 = 1 + 32 * ((int64_t)order.c * 8 + (threadIdx.x >> 5));
+        if (q0 < Q) {
+            const int64_t q = q0 + lane;
+            const bool on = q < Q;
+            const int64_t j = c0 + 4 * (on ? q : q0);          // lanes past the end repeat the first quad
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k0 = 0; k0 < K; k0 += kShiftedBatch) {
+                Window v[kShiftedBatch];
 #pragma unroll
-            for (int b = 0; b < kShiftedBatch; ++b)
-                if (k0 + b < K) v[b] = load_window(w + (size_t)(k0 + b) * row_stride + j);
+                for (int b = 0; b < kShiftedBatch; ++b)
+                    if (k0 + b < K) v[b] = load_window(w + (size_t)(k0 + b) * row_stride + j);
 #pragma unroll
-            for (int b = 0; b < kShiftedBatch; ++b)
-                if (k0 + b < K) {
-                    const float4 x = value(v[b], w + (size_t)(k0 + b) * row_stride + j);
-                    acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
-                }
+                for (int b = 0; b < kShiftedBatch; ++b)
+                    if (k0 + b < K) {
+                        const float4 x = value(v[b], w + (size_t)(k0 + b) * row_stride + j);
+                        acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
+                    }
+            }
+            acc.x *= inv_k; acc.y *= inv_k; acc.z *= inv_k; acc.w *= inv_k;
+            if (XI && on) {
+                const float4 old = *reinterpret_cast<const float4 *>(w_t0 + j);
+                const float4 dl = make_float4(acc.x - old.x, acc.y - old.y, acc.z - old.z, acc.w - old.w);
+                if (xi_al) *reinterpret_cast<float4 *>(xi_out + j) = dl;
+                else { xi_out[j] = dl.x; xi_out[j + 1] = dl.y; xi_out[j + 2] = dl.z; xi_out[j + 3] = dl.w; }
+                dsq += (double)(dl.x * dl.x + dl.y * dl.y + dl.z * dl.z + dl.w * dl.w);
+            }
+            if (on) __stcs(reinterpret_cast<float4 *>(w_t0 + j), acc);
+            if (broadcast) {
+                float4 nx;
+                nx.x = __shfl_down_sync(0xffffffffu, acc.x, 1);
+                nx.y = __shfl_down_sync(0xffffffffu, acc.y, 1);
+                nx.z = __shfl_down_sync(0xffffffffu, acc.z, 1);
+                nx.w = 0.f;
+                if (on)
+                    for (int k = 0; k < K; ++k)
+                        store_shifted(w + (size_t)k * row_stride + j, acc, nx, lane == 0, lane == 31 || q + 1 == Q);
+            }
         }
-        acc.x *= inv_k; acc.y *= inv_k; acc.z *= inv_k; acc.w *= inv_k;
-        if (XI && on) {
-            const float4 old = *reinterpret_cast<const float4 *>(w_t0 + j);
-            const float4 dl = make_float4(acc.x - old.x, acc.y - old.y, acc.z - old.z, acc.w - old.w);
-            if (xi_al) *reinterpret_cast<float4 *>(xi_out + j) = dl;
-            else { xi_out[j] = dl.x; xi_out[j + 1] = dl.y; xi_out[j + 2] = dl.z; xi_out[j + 3] = dl.w; }
-            dsq += (double)(dl.x * dl.x + dl.y * dl.y + dl.z * dl.z + dl.w * dl.w);
-        }
-        if (on) __stcs(reinterpret_cast<float4 *>(w_t0 + j), acc);
-        if (broadcast) {
-            float4 nx;
-            nx.x = __shfl_down_sync(0xffffffffu, acc.x, 1);
-            nx.y = __shfl_down_sync(0xffffffffu, acc.y, 1);
-            nx.z = __shfl_down_sync(0xffffffffu, acc.z, 1);
-            nx.w = 0.f;
-            if (on)
-                for (int k = 0; k < K; ++k)
-                    store_shifted(w + (size_t)k * row_stride + j, acc, nx, lane == 0, lane == 31 || q + 1 == Q);
-        }
+        order.next();
     }
+    order.done();
     // the ends
     const int64_t head = d < c0 + 4 ? d : c0 + 4, tail = c0 + 4 * Q, n_ends = head + (tail < d ? d - tail : 0);
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_ends; t += (int64_t)gridDim.x * blockDim.x) {
@@ -238,16 +285,28 @@ cudaError_t fda_launch_average(const fda_ctx *ctx, float *w, int64_t row_stride,
     // Measured with broadcast, calls back to back: K = 44, d = 84K, pitch d 6.7 us against 16.8 us with quads
     // (aligned 5.7 against 7.9); K = 40, d = 500K 30 against 34 us; K = 20, d = 250K 6.6 against 5.6 us.
     const bool shrt = d <= (int64_t)ctx->n_sm * (K > 32 ? 4096 : 512);
+    // By ticket when a fixed stride takes every block round many times; four blocks of either kernel fit an SM.
+    // Measured, fixed stride and tickets, with broadcast: K = 20, d = 2.6M 71.6 and 72.7 us (two rounds); K = 30,
+    // d = 7M 287 and 280 us (six); K = 60, d = 20M 1555 and 1524 us; K = 8, d = 198M 2179 and 2035 us (without broadcast
+    // 1100 and 1019 us).  Rows at any alignment: K = 30, d = 7M 288 and 287 us (without broadcast 132 and 135 us), K = 60,
+    // d = 20M 1804 and 1644 us.  Two quads per thread spilled at three blocks per SM: 2052 us at d = 198M.
+    const bool tickets = !shrt && !xi_out && (d + 3) / 4 > (int64_t)ctx->n_sm * 8 * threads * (vec ? 4 : 8);
     int64_t blocks = ((shrt ? d : (d + 3) / 4) + threads - 1) / threads;
-    const int64_t cap = (int64_t)ctx->n_sm * 8;
+    const int64_t cap = (int64_t)ctx->n_sm * (!tickets ? 8 : 4);
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    if (xi_out) {
-        cudaError_t e = fda_launch_dependent(shrt ? k_average_short<true> : vec ? k_average<true> : k_average_shifted<true>, (int)blocks, threads, 0, s,
-                                             w, row_stride, K, d, w_t0, gate, broadcast, xi_out, ctx->part_np);
-        if (e != cudaSuccess) return e;
-        return fda_launch_dependent(k_scale_xi, (int)blocks, threads, 0, s, xi_out, d, ctx->part_np, (int)blocks, gate);
+    unsigned int *ticket = ctx->combine_ticket + 1;
+    if (shrt) {
+        const cudaError_t e = fda_launch_dependent(xi_out ? k_average_short<true> : k_average_short<false>, (int)blocks, threads, 0, s,
+                                                   w, row_stride, K, d, w_t0, gate, broadcast, xi_out, ctx->part_np);
+        if (e != cudaSuccess || !xi_out) return e;
+    } else {
+        auto kern = xi_out    ? (vec ? k_average<true, false> : k_average_shifted<true, false>)
+                    : tickets ? (vec ? k_average<false, true> : k_average_shifted<false, true>)
+                              : (vec ? k_average<false, false> : k_average_shifted<false, false>);
+        const cudaError_t e = fda_launch_dependent(kern, (int)blocks, threads, 0, s,
+                                                   w, row_stride, K, d, w_t0, gate, broadcast, xi_out, ctx->part_np, ticket);
+        if (e != cudaSuccess || !xi_out) return e;
     }
-    return fda_launch_dependent(shrt ? k_average_short<false> : vec ? k_average<false> : k_average_shifted<false>, (int)blocks, threads, 0, s,
-                                w, row_stride, K, d, w_t0, gate, broadcast, (float *)nullptr, (double *)nullptr);
+    return fda_launch_dependent(k_scale_xi, (int)blocks, threads, 0, s, xi_out, d, ctx->part_np, (int)blocks, gate);
 }

@@ -54,6 +54,26 @@ def test_average_at_any_alignment(d, K, extra, mis):
         assert np.max(np.abs(xi.cpu().numpy() - xi_ref)) <= 1e-5
 
 
+@pytest.mark.parametrize("rounds,extra,pitch_extra", [(4, 0, 0), (4, 1, 0), (5, 1023, 0), (8, 3, 1), (8, 12, 1), (9, 501, 2)])
+def test_average_of_long_vectors(rounds, extra, pitch_extra):
+    # around the size from which blocks take chunks by ticket (4 rounds of the grid, 8 when rows are not aligned), called again and again
+    import torch
+    import paper_2405_20988_b200 as F
+    K, d = 3, rounds * torch.cuda.get_device_properties(0).multi_processor_count * 8 * 1024 + extra
+    pitch = (d + 3) // 4 * 4 + pitch_extra
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    with F.FdaContext(0, 0, None, d_max=d, K_max=K) as ctx:
+        for bc in (0, F.FDA_AVG_BROADCAST, 0):
+            wbuf = torch.randn((K, pitch), device="cuda", generator=gen)
+            before, w0 = wbuf.clone(), torch.zeros(d, device="cuda")
+            rows = before.cpu().numpy()[:, :d]
+            mean = (rows[0] + rows[1] + rows[2]) * (np.float32(1.0) / np.float32(K))
+            ctx.fda_average_models(wbuf[:, :d], w0, None, bc)
+            assert np.array_equal(w0.cpu().numpy(), mean)
+            assert torch.equal(wbuf[:, d:], before[:, d:])
+            assert torch.equal(wbuf[:, :d], w0.expand(K, d) if bc else before[:, :d])
+
+
 @pytest.mark.parametrize("K,tiles,extra,pitch_extra", [(11, 2, 13, 0), (21, 2, 0, 0), (3, 8, 2, 1)])
 def test_averaged_state_in_one_pass(K, tiles, extra, pitch_extra):
     import torch
