@@ -1,0 +1,44 @@
+"""The estimate of fda_combine_estimate as its host caller gets it: what is promised when the call
+returns, and contexts beyond those that the library keeps mapped host memory for."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import fda_synth as S
+
+pytestmark = pytest.mark.gpu
+
+
+def _fields(raw):
+    import paper_2405_20988_b200 as F
+    e = F.Estimate.from_buffer_copy(bytes(raw))
+    return (e.mean_sq_norm, e.est_sq_norm_of_mean, e.H, e.theta, e.trigger, e.l, tuple(e.row_sq_norm))
+
+
+# states of 24 x (2 + 5 x 250) floats are taken by several blocks, of 3 x (2 + 16 x 64) and of a context without sketch by one
+@pytest.mark.parametrize("l,m,K", [(5, 250, 24), (16, 64, 3), (0, 1, 5)])
+def test_device_estimate_is_complete_when_the_call_returns(l, m, K):
+    """est_dev is read on another stream, with nothing but the call's return in front of it."""
+    import torch
+    import paper_2405_20988_b200 as F
+    rng = np.random.default_rng(l + K)
+    size, calls = ctypes.sizeof(F.Estimate), 300
+    with F.FdaContext(l, m, S.hash_coefficients(3, l), d_max=64, K_max=K) as ctx:
+        variant = F.FDA_VARIANT_SKETCH if l else F.FDA_VARIANT_LINEAR
+        states = torch.from_numpy(rng.normal(0, 1, size=(calls, K, ctx.state_len)).astype(np.float32)).cuda()
+        states[:, :, 0].abs_()
+        est = ctx.new_estimate_buffer()
+        read = torch.zeros((calls, size), dtype=torch.uint8, device="cuda")
+        writer, reader = torch.cuda.Stream(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        host = []
+        for t in range(calls):
+            host.append(_fields(ctx.fda_combine_estimate(states[t], K, variant, 0.06, 0.5, est, stream=writer)))
+            with torch.cuda.stream(reader):
+                read[t].copy_(est)
+            reader.synchronize()                 # (the next call writes est again)
+        got = read.cpu().numpy()
+    assert len(set(host)) == calls               # every call's estimate is another one
+    for t in range(calls):
+        assert _fields(got[t]) == host[t]
