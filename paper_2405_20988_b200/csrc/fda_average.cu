@@ -246,7 +246,7 @@ k_average_short(float *w, int64_t row_stride, int K, int64_t d, float *w_t0,
 
 // xi_out *= 1 / ||delta||  (0 when the step is zero); gated like the average itself
 __global__ void __launch_bounds__(256)
-k_scale_xi(float *__restrict__ xi_out, int64_t d, const double *__restrict__ part, int nparts,
+k_scale_xi(float *xi_out, int64_t d, const double *part, int nparts,
            const fda_estimate *est)
 {
     fda_grid_wait();

@@ -38,7 +38,8 @@ __device__ __forceinline__ void block_barrier()
 }
 
 // Loads and stores of the producers as volatile statements: the compiler keeps them in program
-// order, so a batch's loads are issued kDepth batches before its values are used.
+// order, so a batch's loads are issued kDepth batches before its values are used.  What the kernel before
+// this one may have written (w, w_t0, xi) is not read through ld.global.nc: see fda_launch_dependent.
 __device__ __forceinline__ float4 load4_stream(const float *ptr)
 {
     float4 v;
@@ -48,7 +49,7 @@ __device__ __forceinline__ float4 load4_stream(const float *ptr)
 __device__ __forceinline__ float4 load4_keep(const float *ptr)
 {
     float4 v;
-    asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(ptr));
+    asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(ptr));
     return v;
 }
 __device__ __forceinline__ float load1(const float *ptr, bool on)

@@ -350,9 +350,9 @@ __global__ void __launch_bounds__(kFastThreads, 1) k_local_state_fast(const LsPa
 // Threads run over (group, cell, worker-in-group) with the worker fastest, which is the order
 // of the partial buffers, so the reads of every block's partial are contiguous.
 template <int LWK>
-__global__ void k_finalize_states(const float *__restrict__ part_sk, const double *__restrict__ part_np,
+__global__ void k_finalize_states(const float *part_sk, const double *part_np,
                                   int K, int Kg, int groups, int cpg, int lm, uint32_t flags,
-                                  bool have_xi, float *__restrict__ states)
+                                  bool have_xi, float *states)
 {
     fda_grid_wait();
     const int slen = 2 + lm;

@@ -84,8 +84,7 @@ __device__ __forceinline__ float4 pick(const float4 &a, const float4 &b, int r)
     }
 }
 
-// Ordinary loads (not ld.global.nc, which the compiler may move in front of fda_grid_wait: the kernel
-// before this one may have written what they read).
+// Ordinary loads, not ld.global.nc: the kernel before this one may have written what they read (fda_launch_dependent).
 __device__ __forceinline__ float4 load4(const float *ptr) { return *reinterpret_cast<const float4 *>(ptr); }
 __device__ __forceinline__ float4 load4_any(const float *ptr)
 {
