@@ -104,15 +104,20 @@ struct fda_ctx {
 #ifdef __CUDACC__
 __device__ __forceinline__ void fda_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... Params, typename... Args>
-cudaError_t fda_launch_dependent(void (*kern)(Params...), dim3 blocks, int threads, size_t smem, cudaStream_t s, Args... args)
+cudaError_t fda_launch_dependent_if(bool dependent, void (*kern)(Params...), dim3 blocks, int threads, size_t smem, cudaStream_t s, Args... args)
 {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    attr.val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
     cfg.gridDim = blocks; cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem; cfg.stream = s; cfg.attrs = &attr; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
+template <typename... Params, typename... Args>
+cudaError_t fda_launch_dependent(void (*kern)(Params...), dim3 blocks, int threads, size_t smem, cudaStream_t s, Args... args)
+{
+    return fda_launch_dependent_if(true, kern, blocks, threads, smem, s, args...);
 }
 #endif
 

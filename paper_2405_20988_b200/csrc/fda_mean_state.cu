@@ -326,12 +326,12 @@ __global__ void __launch_bounds__(32 * FDA_MAX_ROWS, 1) k_sketch_vector_rows(con
 int ilog2(int v) { int r = 0; while ((1 << (r + 1)) <= v) ++r; return r; }
 
 template <int L>
-cudaError_t launch_sketch_vector(fda_ctx *ctx, const SketchVecParams &p, int blocks, size_t smem, cudaStream_t s)
+cudaError_t launch_sketch_vector(fda_ctx *ctx, const SketchVecParams &p, int blocks, size_t smem, bool dependent, cudaStream_t s)
 {
     auto kern = k_sketch_vector<L>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
     if (e != cudaSuccess) return e;
-    return fda_launch_dependent(kern, blocks, kThreads, smem, s, p);
+    return fda_launch_dependent_if(dependent, kern, blocks, kThreads, smem, s, p);
 }
 
 }  // namespace
@@ -387,7 +387,10 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
     ctx->last_ls_kernel = sketch ? "k_mean_model + k_sketch_vector" : "k_mean_model";
     int sk_blocks = 0;
     if (sketch) {
-        e = fda_ensure_table(ctx, s);        // first use: the 16-bit hash table
+        // first use: the 16-bit hash table.  The kernels below read it with __ldg, which nothing keeps behind
+        // fda_grid_wait, so behind the kernel that builds it they are ordinary launches.
+        const bool dependent = ctx->tab != nullptr;
+        e = fda_ensure_table(ctx, s);
         if (e != cudaSuccess) return e;
         SketchVecParams p{};
         p.v = ctx->mean_model; p.d = d; p.tab = ctx->tab; p.tab_stride = ctx->tab_stride;
@@ -405,17 +408,17 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
             sk_blocks = (int)rb;
             e = cudaFuncSetAttribute(k_sketch_vector_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
             if (e != cudaSuccess) return e;
-            e = fda_launch_dependent(k_sketch_vector_rows, sk_blocks, 32 * ctx->l, smem, s, p);
+            e = fda_launch_dependent_if(dependent, k_sketch_vector_rows, sk_blocks, 32 * ctx->l, smem, s, p);
         } else
         switch (ctx->l) {
-            case 1: e = launch_sketch_vector<1>(ctx, p, sk_blocks, smem, s); break;
-            case 2: e = launch_sketch_vector<2>(ctx, p, sk_blocks, smem, s); break;
-            case 3: e = launch_sketch_vector<3>(ctx, p, sk_blocks, smem, s); break;
-            case 4: e = launch_sketch_vector<4>(ctx, p, sk_blocks, smem, s); break;
-            case 5: e = launch_sketch_vector<5>(ctx, p, sk_blocks, smem, s); break;
-            case 6: e = launch_sketch_vector<6>(ctx, p, sk_blocks, smem, s); break;
-            case 7: e = launch_sketch_vector<7>(ctx, p, sk_blocks, smem, s); break;
-            default: e = launch_sketch_vector<0>(ctx, p, sk_blocks, smem, s); break;
+            case 1: e = launch_sketch_vector<1>(ctx, p, sk_blocks, smem, dependent, s); break;
+            case 2: e = launch_sketch_vector<2>(ctx, p, sk_blocks, smem, dependent, s); break;
+            case 3: e = launch_sketch_vector<3>(ctx, p, sk_blocks, smem, dependent, s); break;
+            case 4: e = launch_sketch_vector<4>(ctx, p, sk_blocks, smem, dependent, s); break;
+            case 5: e = launch_sketch_vector<5>(ctx, p, sk_blocks, smem, dependent, s); break;
+            case 6: e = launch_sketch_vector<6>(ctx, p, sk_blocks, smem, dependent, s); break;
+            case 7: e = launch_sketch_vector<7>(ctx, p, sk_blocks, smem, dependent, s); break;
+            default: e = launch_sketch_vector<0>(ctx, p, sk_blocks, smem, dependent, s); break;
         }
         if (e != cudaSuccess) return e;
     }

@@ -38,3 +38,22 @@ def test_states_behind_an_average_are_zero(l, m, K, d, limit, packed):
             ctx.fda_average_models_xi(w, w_t0, xi, None, F.FDA_AVG_BROADCAST)
             ctx.fda_mean_state(w, w_t0, xi, flags, means[t])
         assert not states.any() and not means.any()
+
+
+# lane-private bins (5 x 250) and compare-and-swap bins (7 x 500, 9 x 700); the first call builds the hash table
+@pytest.mark.parametrize("l,m", [(5, 250), (7, 500), (9, 700)])
+def test_first_averaged_state_of_a_context_equals_the_second(l, m):
+    import torch
+    import paper_2405_20988_b200 as F
+    K, d = 4, 40_003
+    gen = torch.Generator(device="cuda").manual_seed(l)
+    w_t0 = torch.zeros(d, device="cuda")
+    # quarters of whole numbers: every sum is exact, so the order of the additions does not show
+    w = torch.randint(-8, 9, (K, d), device="cuda", generator=gen).float()
+    for seed in range(8):
+        with F.FdaContext(l, m, S.hash_coefficients(seed, l), d_max=d, K_max=K, schedule_limit_bytes=-1) as ctx:
+            first, second = (torch.full((ctx.state_len,), float("nan"), device="cuda") for _ in range(2))
+            ctx.fda_mean_state(w, w_t0, None, 5, first)
+            assert ctx.fda_debug_last_kernel() == "k_mean_model + k_sketch_vector"
+            ctx.fda_mean_state(w, w_t0, None, 5, second)
+            assert torch.equal(first, second)
