@@ -68,10 +68,12 @@ __device__ __forceinline__ void finish(const CombineParams &p, double row, doubl
 {
     double est_sq = head1 * head1;
     if (p.variant == FDA_VARIANT_SKETCH) {
-        int rank = 0;                      // of this lane's row, ties by row number
+        int rank = 0;                      // of this lane's row, ties by row number; NaN behind all numbers, so that
+        const bool nan = row != row;       // the ranks are 0 .. l - 1 whatever the rows hold
         for (int q = 0; q < p.l; ++q) {
             const double o = __shfl_sync(0xffffffffu, row, q);
-            rank += (o < row || (o == row && q < lane)) ? 1 : 0;
+            const bool tie = o == row || (nan && o != o);
+            rank += (tie ? q < lane : (o < row || nan)) ? 1 : 0;
         }
         const unsigned lo = __ballot_sync(0xffffffffu, lane < p.l && rank == (p.l - 1) / 2);
         const unsigned hi = __ballot_sync(0xffffffffu, lane < p.l && rank == p.l / 2);

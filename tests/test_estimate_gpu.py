@@ -42,3 +42,23 @@ def test_device_estimate_is_complete_when_the_call_returns(l, m, K):
     assert len(set(host)) == calls               # every call's estimate is another one
     for t in range(calls):
         assert _fields(got[t]) == host[t]
+
+
+@pytest.mark.parametrize("m", [4, 5000])              # one block, several blocks
+@pytest.mark.parametrize("cells", [[1, np.nan, np.nan, np.nan, 2], [3, np.nan, 1, 2, 5], [np.nan] * 5, [np.inf, 1, np.inf, np.inf, 2],
+                                   [1, np.nan, 2, 3], [np.nan, 1, np.nan, 2], [2, np.inf, np.nan, 1], [4, 4, 1, 4, np.nan, 1]])
+def test_median_of_rows_that_are_not_all_numbers(cells, m):
+    """NaN counts as the largest: the median is a number while fewer than half of the rows are NaN."""
+    import torch
+    import paper_2405_20988_b200 as F
+    l = len(cells)
+    state = np.zeros((1, 2 + l * m), dtype=np.float32)
+    state[0, 0] = 7.0
+    state[0, 3::m] = cells
+    rows = np.sort(np.square(np.array(cells, dtype=np.float64)))
+    want = rows[l // 2] if l % 2 else 0.5 * (rows[l // 2 - 1] + rows[l // 2])
+    with F.FdaContext(l, m, S.hash_coefficients(3, l), d_max=64, K_max=1) as ctx:
+        est = ctx.fda_combine_estimate(torch.from_numpy(state).cuda(), 1, F.FDA_VARIANT_SKETCH, 0.0, 1.0, ctx.new_estimate_buffer())
+    assert np.array_equal(np.float32(est.est_sq_norm_of_mean), np.float32(want), equal_nan=True)
+    assert np.array_equal(np.float32(est.H), np.float32(7.0 - want), equal_nan=True)
+    assert est.trigger == int(7.0 - want > 1.0)
