@@ -62,3 +62,35 @@ def test_median_of_rows_that_are_not_all_numbers(cells, m):
     assert np.array_equal(np.float32(est.est_sq_norm_of_mean), np.float32(want), equal_nan=True)
     assert np.array_equal(np.float32(est.H), np.float32(7.0 - want), equal_nan=True)
     assert est.trigger == int(7.0 - want > 1.0)
+
+
+def test_contexts_beyond_the_mapped_page():
+    """The page of mapped host memory has 32 slots: the contexts beyond them copy the estimate, and
+    a slot that a context has given back serves another one, whose first estimate is not the old one."""
+    import torch
+    import paper_2405_20988_b200 as F
+    K, l, m = 3, 2, 16
+    rng = np.random.default_rng(1)
+
+    def estimate(ctx):
+        states = torch.from_numpy(np.abs(rng.normal(0, 1, size=(K, ctx.state_len))).astype(np.float32)).cuda()
+        est = ctx.new_estimate_buffer()
+        host = ctx.fda_combine_estimate(states, K, F.FDA_VARIANT_SKETCH, 0.06, 0.5, est)
+        mean = states.double().mean(dim=0).cpu().numpy()
+        rows = np.square(mean[2:].reshape(l, m)).sum(axis=1)
+        assert host.mean_sq_norm == pytest.approx(mean[0], rel=1e-6)
+        assert host.est_sq_norm_of_mean == pytest.approx(rows.mean() / 1.06, rel=1e-6)
+        assert list(host.row_sq_norm[:l]) == pytest.approx(rows, rel=1e-6)
+        assert _fields(est.cpu().numpy()) == _fields(bytes(host))
+
+    held = [F.FdaContext(l, m, S.hash_coefficients(k, l), d_max=64, K_max=K) for k in range(36)]
+    try:
+        for _ in range(2):
+            for ctx in held:
+                estimate(ctx)
+            for k in range(0, 36, 5):            # slots go round, to contexts that had none among others
+                held[k].close()
+                held[k] = F.FdaContext(l, m, S.hash_coefficients(k, l), d_max=64, K_max=K)
+    finally:
+        for ctx in held:
+            ctx.close()
