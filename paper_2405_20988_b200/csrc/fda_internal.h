@@ -21,7 +21,6 @@ constexpr int kListMaxLen = 64;        // longest list (longer cells are cut int
 constexpr int kListPadRows = 8;        // zero rows behind the tile, one per bank group
 constexpr int kListBatch = 1024;       // indices a producer step covers; tiles are multiples of it
 constexpr int kListMaxTile = 7168;     // rows + pad rows must fit 13 bits
-constexpr int kListMinTilesPerBlock = 1;
 constexpr int kListSmemHead = 2112;    // counters and the warps' fp64 sums in front of the item tables
 
 // byte offsets inside the schedule record of a tile with `items` items

@@ -695,8 +695,6 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     if (p.groups > ctx->n_sm) return cudaErrorNotSupported;
     int64_t cpg = ctx->n_sm / p.groups;
     if (cpg > p.tiles) cpg = p.tiles;
-    // short jobs stay with the other kernels
-    if (p.tiles < (int64_t)kListMinTilesPerBlock * cpg) return cudaErrorNotSupported;
     p.cpg = (int)cpg;
     const int blocks = p.groups * p.cpg, lm = p.l * p.m;
     if ((size_t)blocks * lm * GW > ctx->part_sk_floats || blocks > ctx->max_blocks ||

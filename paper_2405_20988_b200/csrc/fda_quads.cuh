@@ -1,5 +1,6 @@
 // Quads of four consecutive floats at any alignment, for the passes that combine the K rows of w index
-// by index (fda_average.cu, fda_mean_state.cu).  The pass runs in the frame of one vector (w_t0, or the
+// by index (fda_average.cu, fda_mean_state.cu; fda_rows.cuh, which cuts every row at its own
+// boundaries, takes the helpers).  The pass runs in the frame of one vector (w_t0, or the
 // averaged drifts): quad q covers indices c0 + 4q .. + 3, where that vector is 16-byte aligned.  A row
 // aligned otherwise is read as the two aligned quads around those indices, with 128-bit loads of which
 // the second hits L1, and written as quads at its own boundaries, put together from two neighbouring lanes.

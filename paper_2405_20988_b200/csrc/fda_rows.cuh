@@ -21,8 +21,12 @@
 #define FDA_ROWS_CUH_
 
 #include "fda_internal.h"
+#include "fda_quads.cuh"
 
 namespace fda_rows {
+
+using fda_quads::first_aligned;
+using fda_quads::pick;
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
@@ -51,8 +55,6 @@ __device__ __forceinline__ int group_first(const Params &p, int g)
 }
 __device__ __forceinline__ int group_rows(const Params &p, int g) { return p.K / p.groups + (g < p.K % p.groups ? 1 : 0); }
 
-__device__ __forceinline__ int misaligned(const float *ptr) { return (int)(((uintptr_t)ptr >> 2) & 3u); }
-
 // Adds the pairs of all blocks of group g in a fixed order (16 threads per value, then their sums in
 // order) and writes the rows' states.  Called by one block; red: kThreads doubles of shared memory.
 __device__ __forceinline__ void finish_group(const Params &p, int g, double *red)
@@ -70,17 +72,6 @@ __device__ __forceinline__ void finish_group(const Params &p, int g, double *red
         const int k = tid >> 1;
         const bool on = (tid & 1) == 0 ? (p.flags & FDA_STATE_NORM) != 0 : p.xi != nullptr;
         if (k < group_rows(p, g)) p.states[(size_t)(group_first(p, g) + k) * p.slen + (tid & 1)] = on ? (float)s : 0.f;
-    }
-}
-
-// four values of the window v[0..7] from position r (r is the same for the whole block)
-__device__ __forceinline__ float4 pick(const float4 &a, const float4 &b, int r)
-{
-    switch (r) {
-        case 0: return a;
-        case 1: return make_float4(a.y, a.z, a.w, b.x);
-        case 2: return make_float4(a.z, a.w, b.x, b.y);
-        default: return make_float4(a.w, b.x, b.y, b.z);
     }
 }
 
@@ -104,11 +95,11 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) k_rows_state(const Par
     const int first = group_first(p, g), n = group_rows(p, g);
     const float *wg = p.w + (size_t)first * (size_t)p.row_stride;
 
-    const int c0 = (4 - misaligned(p.w_t0)) & 3;              // first index at which w_t0 is aligned
+    const int c0 = first_aligned(p.w_t0);                     // first index at which w_t0 is aligned
     unsigned rs = 0;                                          // r_k of the rows, two bits each
 #pragma unroll
     for (int k = 0; k < kRows; ++k)
-        rs |= (unsigned)((4 - misaligned(wg + c0 + (int64_t)(k < n ? k : 0) * p.row_stride)) & 3) << (2 * k);
+        rs |= (unsigned)first_aligned(wg + c0 + (int64_t)(k < n ? k : 0) * p.row_stride) << (2 * k);
     fda_grid_wait();
     // quads whose two-quad window lies inside the vectors
     const int64_t Q = p.d >= c0 + 8 ? (p.d - 8 - c0) / 4 + 1 : 0;

@@ -42,11 +42,8 @@ constexpr int kBT = 256;                  // threads of a builder block
 constexpr int ML = kListMaxLen;
 constexpr int NRES = kListOct;            // residue classes = lanes per shared-memory pass
 constexpr int kWindow = 64;               // candidates looked at for every place in an octet
-#ifndef FDA_SPREAD
-#define FDA_SPREAD 8
-#endif
 constexpr int kMatchBytes = 288;          // shared memory of the thread that orders an octet's entries
-constexpr int kSpread = FDA_SPREAD;       // every kSpread-th thread of the block orders the entries of an octet
+constexpr int kSpread = 8;                // every kSpread-th thread of the block orders the entries of an octet
 
 struct SchedParams {
     const uint64_t *coeffs;
