@@ -437,10 +437,10 @@ constexpr int kShortChunks = 2;                // chunks of 128 indices a warp f
 constexpr uint32_t kShortBins = kShortWarps * GW * 2 * 8;      // offset of the bins, behind the warps' sums
 inline size_t short_smem_bytes(int lm, int T) { return kShortBins + (size_t)lm * GW * 4 + (size_t)(T + kListPadRows) * GW * 4; }
 
-// The sketch pass of vectors with so few tiles that every SM can have a block of its own and more:
-// a block serves one tile, p.part_tiles blocks share it - all of them form its drifts, each walks every
-// p.part_tiles-th item - and their bins, which differ in the cells they touch, are partial sums like
-// those of any other blocks, so the cells come out the same bit for bit.
+// The sketch pass of vectors with so few tiles that no block has more than one: p.part_tiles blocks (one
+// to three) share a tile - all of them form its drifts, each walks every p.part_tiles-th item - and their
+// bins, which differ in the cells they touch, are partial sums like those of any other blocks, so the
+// cells come out the same bit for bit.
 // Bound: latency, so there are no roles and no second buffer: every warp has its first item's entries
 // on their way (the schedule is older than the kernel before this one, so even in front of
 // fda_grid_wait), then all the loads of its two chunks of indices, stores the drifts, and after one barrier walks.
@@ -703,11 +703,20 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     const size_t smem = fda_list_smem_bytes(p.l, p.m, p.T, ctx->sched_ni_max);
     if (smem > (size_t)ctx->smem_optin) return cudaErrorNotSupported;
 
-    // A vector with at most one tile per block and SMs left for as many blocks again: several blocks
-    // share a tile (k_local_state_short).
+    // A vector with at most one tile per block runs on k_local_state_short, whose tiles hold up to 6144 indices:
+    // several blocks share a tile while the SMs last, and sketches of up to six rows stay with it when they do not.
+    // Measured with the finalize kernel, back to back, d at 75 to 148 blocks of one tile, the short kernel against the
+    // one with roles: 5 x 250, K = 10, d = 154K 10.5 and 11.4 us, K = 5, d = 455K 11.5 and 12.3; 3 x 200, K = 10,
+    // d = 154K 9.5 and 11.0; 6 x 400, K = 10, d = 128K 13.0 and 13.7; but 7 x 500, K = 10, d = 128K 15.0 and 14.8,
+    // 8 x 250 15.0 and 14.3, 16 x 100 21.6 and 20.8, where the walk is most of the work and 28 warps are better than 24.  With
+    // blocks to share the tiles: 7 x 500, K = 10, d = 123K 13.4 and 14.8, 16 x 100, d = 147K 17.5 and 20.7.
     int split = 1;
+    bool one_tile = false;
     if (ctx->sched_parts == 1) {
-        if (p.tiles == p.cpg && 2 * blocks <= ctx->n_sm && p.T <= kShortWarps * 128 * kShortChunks) split = std::min(3, ctx->n_sm / blocks);
+        if (p.tiles == p.cpg && p.T <= kShortWarps * 128 * kShortChunks) {
+            split = std::min(3, ctx->n_sm / blocks);
+            one_tile = split > 1 || p.l <= 6;
+        }
         p.part_tiles = split;
     }
     // 8 producer + 20 walker warps, or 5 + 23 when a loaded index pays for more walking.  Measured,
@@ -717,7 +726,7 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     // 231 with 6 + 22, 226 with 8 + 24 (64 registers).
     auto launch = [&](ListParams &q, int grid, cudaStream_t st, bool dependent) {
         if (ctx->sched_parts > 1) return launch_lists<8, 20, true>(q, grid, smem, dependent, st);
-        if (split > 1)
+        if (one_tile)
             return fda_launch_dependent(pick_short(q.have_xi != 0, q.vec != 0), grid, kShortWarps * 32,
                                         short_smem_bytes(q.l * q.m, q.T), st, q);
         return p.l >= 7 ? launch_lists<5, 23, false>(q, grid, smem, dependent, st)

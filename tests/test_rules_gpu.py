@@ -1,0 +1,42 @@
+"""Both sides of the lines at which a call goes to another kernel, against the oracle."""
+import numpy as np
+import pytest
+
+import fda_synth as S
+from fda_testlib import check_states
+
+pytestmark = pytest.mark.gpu
+
+SMS = 148
+
+
+def _inputs(l, K, d, pitch_extra, seed):
+    rng = np.random.default_rng(seed)
+    pitch = (d + 3) // 4 * 4 + pitch_extra
+    w_t0 = rng.normal(0, 0.05, size=d).astype(np.float32)
+    wbuf = np.full((K, pitch), 1e6, dtype=np.float32)
+    wbuf[:, :d] = w_t0 + rng.normal(2e-4, 1e-3, size=(K, d)).astype(np.float32)
+    xi = rng.normal(size=d)
+    return wbuf, w_t0, (xi / np.linalg.norm(xi)).astype(np.float32), S.hash_coefficients(seed, l)
+
+
+# blocks of one tile: the most that still share tiles (74), one more, one for every SM, and the first vector with
+# two tiles to a block; sketches of up to six rows and of more go to different kernels in between
+@pytest.mark.parametrize("pitch_extra", [0, 1])
+@pytest.mark.parametrize("l,m,K,tiles,more", [(5, 250, 10, 24, 0), (5, 250, 10, 24, 1), (5, 250, 9, 49, 0), (5, 250, 10, 49, 1),
+                                              (6, 400, 5, 74, 0), (6, 400, 20, 14, 5), (7, 500, 10, 25, -3), (7, 500, 3, 75, 0),
+                                              (1, 250, 3, 148, -1)])
+def test_vectors_of_one_tile_per_block(l, m, K, tiles, more, pitch_extra):
+    import torch
+    import oracle
+    import paper_2405_20988_b200 as F
+    T = 6144 if m == 250 else 5120
+    d = tiles * T + more
+    wbuf, w_t0, xi, coeffs = _inputs(l, K, d, pitch_extra, l * m + tiles)
+    ora = oracle.local_state(wbuf[:, :d], w_t0, xi, coeffs, l, m, threads=8)
+    with F.FdaContext(l, m, coeffs, d_max=d, K_max=K) as ctx:
+        assert ctx.fda_context_info()["tile_indices"] == T
+        st = torch.full((K, ctx.state_len), float("nan"), device="cuda")
+        ctx.fda_local_state(torch.from_numpy(wbuf).cuda()[:, :d], torch.from_numpy(w_t0).cuda(), torch.from_numpy(xi).cuda(), 7, st)
+        assert ctx.fda_debug_last_kernel() == "k_local_state_gather"
+    check_states(st.cpu().numpy(), ora, l, m, d)
