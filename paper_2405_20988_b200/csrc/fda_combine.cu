@@ -4,8 +4,8 @@
 // Bound: latency.  The K x (2 + l*m) floats are a few kilobytes to a megabyte; what takes time is
 // the chain launch - loads - reductions - (meeting of the blocks) - median - result.  So a thread
 // asks for eight workers' values of a column before it adds any, and a warp meets the others once.
-// Tables of up to kOneBlock floats are taken by one block (a ticket and a second trip to L2 cost more
-// than reading them on one SM); larger ones by one block per 64 columns of a row, its threads
+// Tables that a block reads in up to kOneBlockTrips round trips are taken by one block (a ticket and a second
+// trip to L2 cost more than that); larger ones by one block per 64 columns of a row, its threads
 // splitting the workers four ways, and the block that finishes last (a ticket counter, no waiting)
 // takes the median.  The median comes from the ranks of the row norms, all rows at once.
 // fp64 accumulation in a fixed order, so the result is reproducible.
@@ -17,7 +17,13 @@ constexpr int kThreads = 1024;             // of the block that takes everything
 constexpr int kUnitColumns = 64;           // columns of a block that takes a part of a row,
 constexpr int kUnitSlices = 4;             // and the slices of workers its threads split into
 constexpr int kUnitThreads = kUnitColumns * kUnitSlices;
-constexpr int64_t kOneBlock = 12 * 1024;   // states (floats) one block reads in about the time of a meeting
+// Round trips (batches of eight workers of a warp's 32 columns, one after the other) that cost one block what a
+// meeting of several costs.  Measured, one block and several, back to back: two trips 3.54 and 3.79 us (16 x 64, K = 8),
+// 3.80 and 3.72 (5 x 250, K = 8); three 3.70 and 3.95 (3 x 100, K = 20); four 4.45 and 3.73 (5 x 250, K = 10), 4.46 and
+// 3.73 (7 x 500, K = 1), 4.25 and 4.08 (3 x 100, K = 27); eleven 7.30 and 4.48 us (8 x 1000, K = 1).  Behind a sketch
+// pass the difference at four trips is lost in the chain (a round with 5 x 250, K = 10, d = 1.2M: 49.8 us with either).
+constexpr int kOneBlockTrips = 3;
+constexpr int kBatch = 8;                  // workers whose values of a column are asked for at once
 
 struct CombineParams {
     const float *states;
@@ -43,7 +49,6 @@ __device__ __forceinline__ double warp_sum(double v)
 // as a tree (a chain of fp64 additions as long as the loads themselves would follow them), the trees in order
 __device__ __forceinline__ double column_sum(const float *col, int first, int step, int K, size_t slen)
 {
-    constexpr int kBatch = 8;
     double acc = 0.0;
     for (int k = first; k < K; k += kBatch * step) {
         float v[kBatch];
@@ -194,7 +199,9 @@ cudaError_t fda_launch_combine(const fda_ctx *ctx, const float *states, int K, i
     p.inv_k = 1.0 / (double)K; p.inv_eps = 1.0 / (1.0 + (double)epsilon);
     p.scratch = ctx->combine_scratch; p.ticket = ctx->combine_ticket;
     p.est = est_dev; p.host = host; p.seq = seq;
-    if (ctx->l == 0 || (int64_t)K * ctx->lm <= kOneBlock)
+    // k_combine_small: 30 / l warps to a row, 32 columns a warp
+    const int64_t columns = ctx->l > 0 ? 30 / ctx->l * 32 : 1, trips = (ctx->m + columns - 1) / columns * ((K + kBatch - 1) / kBatch);
+    if (ctx->l == 0 || trips <= kOneBlockTrips)
         return fda_launch_dependent(k_combine_small, 1, kThreads, 0, s, p);
     p.chunks = (ctx->m + kUnitColumns - 1) / kUnitColumns;
     return fda_launch_dependent(k_combine, ctx->l * p.chunks, kUnitThreads, 0, s, p);

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 import fda_synth as S
-from fda_testlib import check_states
+from fda_testlib import check_estimate, check_states
 
 pytestmark = pytest.mark.gpu
 
@@ -40,3 +40,20 @@ def test_vectors_of_one_tile_per_block(l, m, K, tiles, more, pitch_extra):
         ctx.fda_local_state(torch.from_numpy(wbuf).cuda()[:, :d], torch.from_numpy(w_t0).cuda(), torch.from_numpy(xi).cuda(), 7, st)
         assert ctx.fda_debug_last_kernel() == "k_local_state_gather"
     check_states(st.cpu().numpy(), ora, l, m, d)
+
+
+# round trips of a warp: 3 | 4 of one batch of columns, 2 | 4 of two, 4 of four, 3 | 4 of batches of columns
+@pytest.mark.parametrize("l,m,K", [(3, 100, 24), (3, 100, 25), (5, 250, 8), (5, 250, 9), (7, 500, 1), (16, 96, 8), (16, 97, 8), (1, 960, 24), (1, 960, 25)])
+def test_combine_by_one_block_and_by_several(l, m, K):
+    import torch
+    import oracle
+    import paper_2405_20988_b200 as F
+    rng = np.random.default_rng(l * m + K)
+    st = rng.normal(0, 0.1, size=(K, 2 + l * m)).astype(np.float32)
+    st[:, 0] = np.abs(st[:, 0]) + 1.0
+    with F.FdaContext(l, m, S.hash_coefficients(2, l), d_max=1000, K_max=K) as ctx:
+        g, buf = torch.from_numpy(st).cuda(), ctx.new_estimate_buffer()
+        for variant in (0, 1, 1):
+            est = ctx.fda_combine_estimate(g, K, variant, float(np.float32(0.06)), 0.5, buf)
+            check_estimate(est.as_dict(), oracle.combine(st, l, m, variant, 0.06, 0.5), l)
+            assert bytes(buf.cpu().numpy()) == bytes(est)
