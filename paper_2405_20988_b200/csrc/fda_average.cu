@@ -281,10 +281,16 @@ cudaError_t fda_launch_average(const fda_ctx *ctx, float *w, int64_t row_stride,
     const fda_estimate *gate = (flags & FDA_AVG_UNCONDITIONAL) ? nullptr : est_dev;
     const int broadcast = (flags & FDA_AVG_BROADCAST) ? 1 : 0;
     const int threads = 256;
-    // One index per thread up to 512 indices per SM, and up to 4096 when the chain of batches is long.
-    // Measured with broadcast, calls back to back: K = 44, d = 84K, pitch d 6.7 us against 16.8 us with quads
-    // (aligned 5.7 against 7.9); K = 40, d = 500K 30 against 34 us; K = 20, d = 250K 6.6 against 5.6 us.
-    const bool shrt = d <= (int64_t)ctx->n_sm * (K > 32 ? 4096 : 512);
+    // One index per thread on short vectors, up to a number of indices per SM that depends on what the quads cost
+    // there: rows at any alignment pay for windows and shifted stores, many rows for the chain of their batches.
+    // Measured with broadcast, calls back to back, one index per thread and quads.
+    // Aligned: K = 32, d = 84K 4.8 and 6.3 us, 150K 5.9 and 5.8; K = 20, 100K 4.0 and 4.0, 250K 6.9 and 5.9; K = 60, 100K 8.1
+    // and 9.2, 200K 12.5 and 14.1, 300K 18.2 and 15.5, 600K 51 and 37.
+    // Any alignment: K = 4, 100K 3.9 and 3.7, 400K 5.4 and 4.0; K = 16, 150K 4.4 and 7.7, 300K 6.7 and 8.1, 600K 11.3 and 12.3
+    // (without broadcast 3.8 and 4.1, 4.2 and 4.5, 6.7 and 6.1); K = 20, 150K 5.4 and 9.4, without broadcast 200K 4.5 and 5.0, 300K 5.7
+    // and 5.1; K = 44, 75,776 6.4 and 17.9, 450K 21.8 and 23.6; K = 60, 600K 54 and 54, 900K 80 and 91.
+    const int64_t per_sm = K > 32 ? (vec ? 1536 : 4096) : (vec || K < 8 ? 768 : 1536);
+    const bool shrt = d <= (int64_t)ctx->n_sm * per_sm;
     // By ticket when a fixed stride takes every block round many times; four blocks of either kernel fit an SM.
     // Measured, fixed stride and tickets, with broadcast: K = 20, d = 2.6M 71.6 and 72.7 us (two rounds); K = 30,
     // d = 7M 287 and 280 us (six); K = 60, d = 20M 1555 and 1524 us; K = 8, d = 198M 2179 and 2035 us (without broadcast

@@ -19,7 +19,7 @@ def at(torch, a, misalign):
     return view
 
 
-@pytest.mark.parametrize("d", [1, 11, 12, 17, 139, 140, 1029, 75_776, 75_777, 75_916, 76_803])   # 512 x 148 = 75,776: short up to there
+@pytest.mark.parametrize("d", [1, 11, 12, 17, 139, 140, 1029, 75_776, 75_777, 75_916, 76_803])   # (both sides of the lines: test_rules_gpu.py)
 @pytest.mark.parametrize("K,extra,mis", [(1, 0, (1, 0, 0)), (3, 1, (0, 0, 0)), (4, 2, (0, 3, 0)), (5, 3, (2, 2, 2)), (9, 1, (3, 1, 2)),
                                          (33, 3, (0, 0, 0)), (4, 0, (0, 0, 0))])
 def test_average_at_any_alignment(d, K, extra, mis):

@@ -57,3 +57,42 @@ def test_combine_by_one_block_and_by_several(l, m, K):
             est = ctx.fda_combine_estimate(g, K, variant, float(np.float32(0.06)), 0.5, buf)
             check_estimate(est.as_dict(), oracle.combine(st, l, m, variant, 0.06, 0.5), l)
             assert bytes(buf.cpu().numpy()) == bytes(est)
+
+
+def _at(torch, a, misalign):
+    buf = torch.zeros(a.size + 8, dtype=torch.float32, device="cuda")
+    view = buf[misalign:misalign + a.size].view(a.shape)
+    view.copy_(torch.from_numpy(a))
+    return view
+
+
+# indices per SM up to which an index has a thread of its own; behind that line the quads, whose edges the offsets meet
+@pytest.mark.parametrize("over", [0, 1, 2, 140, 1027])
+@pytest.mark.parametrize("K,per_sm,extra,mis", [(4, 768, 0, (0, 0, 0)), (7, 768, 1, (1, 3, 2)), (8, 1536, 0, (0, 1, 0)), (11, 1536, 3, (3, 0, 1)),
+                                                (32, 768, 0, (0, 0, 0)), (33, 1536, 0, (0, 0, 0)), (33, 4096, 2, (0, 0, 3))])
+def test_average_by_index_and_by_quads(K, per_sm, extra, mis, over):
+    import torch
+    import paper_2405_20988_b200 as F
+    d = SMS * per_sm + over
+    rng = np.random.default_rng(d + K)
+    wbuf = rng.normal(0, 0.05, size=(K, (d + 3) // 4 * 4 + extra)).astype(np.float32)
+    w_t0 = rng.normal(0, 0.05, size=d).astype(np.float32)
+    acc = np.zeros(d, dtype=np.float32)
+    for k in range(K):
+        acc = acc + wbuf[k, :d]
+    mean = acc * (np.float32(1.0) / np.float32(K))
+    delta = (mean - w_t0).astype(np.float64)
+    delta /= np.linalg.norm(delta)
+    with F.FdaContext(0, 0, None, d_max=d, K_max=K) as ctx:
+        for bc in (0, F.FDA_AVG_BROADCAST):
+            w, w0 = _at(torch, wbuf, mis[0]), _at(torch, w_t0, mis[1])
+            ctx.fda_average_models(w[:, :d], w0, None, bc)
+            got = w.cpu().numpy()
+            assert np.array_equal(w0.cpu().numpy(), mean)
+            assert np.array_equal(got[:, d:], wbuf[:, d:])
+            assert np.array_equal(got[:, :d], np.broadcast_to(mean, (K, d)) if bc else wbuf[:, :d])
+        w, w0, xi = _at(torch, wbuf, mis[0]), _at(torch, w_t0, mis[1]), _at(torch, np.zeros(d, np.float32), mis[2])
+        ctx.fda_average_models_xi(w[:, :d], w0, xi, None, F.FDA_AVG_BROADCAST)
+        assert np.array_equal(w0.cpu().numpy(), mean) and np.array_equal(w.cpu().numpy()[:, :d], np.broadcast_to(mean, (K, d)))
+        # single precision on both sides of a difference of numbers around mean |w|, unit length
+        assert np.max(np.abs(xi.cpu().numpy() - delta)) <= 1e-5
