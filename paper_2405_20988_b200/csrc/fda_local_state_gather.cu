@@ -11,7 +11,7 @@
 // to be cut into pieces are added atomically).  One update costs one 4-byte shared-memory read.
 //
 // A block serves a group of 4 workers and a strided set of tiles, with two kinds of warps:
-//   producers  8 warps (5 for sketches of 7 or more rows).  A thread owns four consecutive indices
+//   producers  8 warps (5 when the walk is most of the work).  A thread owns four consecutive indices
 //              of a batch (1024 indices with 8 warps; the last batch of a tile may be a part): it loads the four workers' values and w_t0
 //              (xi) with 128-bit loads into registers (the landing zone: nothing else is staged),
 //              subtracts, adds up ||u||^2 and <xi,u> (fp32 within a tile, fp64 across tiles) and
@@ -719,17 +719,22 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         }
         p.part_tiles = split;
     }
-    // 8 producer + 20 walker warps, or 5 + 23 when a loaded index pays for more walking.  Measured,
-    // 7 x 500, K = 60, d = 20M: 2.76 ms with 5 + 23, 2.90 with 4 + 24, 2.95 with 8 + 20, 2.68 against
-    // 2.64 with 6 + 22; 5 x 250, K = 8, d = 198M: 2.35 ms with 8 + 20, 2.46 with 7 + 21, 2.48 with 9 + 19,
-    // 2.61 with 12 + 16; 8 x 1000 in parts, K = 20, d = 2.6M: 214 us with 8 + 20, 216 with 10 + 18,
-    // 231 with 6 + 22, 226 with 8 + 24 (64 registers).
+    // 8 producer + 20 walker warps, or 5 + 23 when a loaded index pays for more walking: l steps, and its share of the
+    // starts and flushes of the lists, which cost about ten steps each (T / m indices to a list and row).  Measured, 8 + 20
+    // and 5 + 23, K = 8, d = 20M, by l * (1 + 10 * m / T): 7.4 (5 x 300) 257 and 311 us; 9.9 (5 x 500) 311 and
+    // 313, (7 x 250) 300 and 329; 10.1 (6 x 350) 330 and 322; 10.9 (5 x 600) 348 and 317; 11.9 (6 x 500) 367 and 332; 13.8
+    // (7 x 500) 421 and 355; from eight rows on 5 + 23 whatever the lists (8 x 100, 9.3: 406 and 376; 8 x 250 346 and 340;
+    // 9 x 250 397 both; 12 x 250 495 and 500; 16 x 100 757 and 695).  Other splits: 7 x 500, K = 60, d = 20M: 2.76 ms
+    // with 5 + 23, 2.90 with 4 + 24, 2.95 with 8 + 20, 2.68 against 2.64 with 6 + 22; 5 x 250, K = 8, d = 198M: 2.35 ms
+    // with 8 + 20, 2.46 with 7 + 21, 2.48 with 9 + 19, 2.61 with 12 + 16; 8 x 1000 in parts, K = 20, d = 2.6M: 214 us with
+    // 8 + 20, 216 with 10 + 18, 231 with 6 + 22, 226 with 8 + 24 (64 registers).
+    const bool walking = p.l >= 8 || (int64_t)p.l * (p.T + 10 * p.m) >= 10 * (int64_t)p.T;
     auto launch = [&](ListParams &q, int grid, cudaStream_t st, bool dependent) {
         if (ctx->sched_parts > 1) return launch_lists<8, 20, true>(q, grid, smem, dependent, st);
         if (one_tile)
             return fda_launch_dependent(pick_short(q.have_xi != 0, q.vec != 0), grid, kShortWarps * 32,
                                         short_smem_bytes(q.l * q.m, q.T), st, q);
-        return p.l >= 7 ? launch_lists<5, 23, false>(q, grid, smem, dependent, st)
+        return walking ? launch_lists<5, 23, false>(q, grid, smem, dependent, st)
                         : launch_lists<8, 20, false>(q, grid, smem, dependent, st);
     };
     ListParts parts{};

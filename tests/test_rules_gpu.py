@@ -96,3 +96,19 @@ def test_average_by_index_and_by_quads(K, per_sm, extra, mis, over):
         assert np.array_equal(w0.cpu().numpy(), mean) and np.array_equal(w.cpu().numpy()[:, :d], np.broadcast_to(mean, (K, d)))
         # single precision on both sides of a difference of numbers around mean |w|, unit length
         assert np.max(np.abs(xi.cpu().numpy() - delta)) <= 1e-5
+
+
+# the split of the warps: l * (1 + 10 * m / T) below ten and from ten on, seven rows on either side of it, eight and more
+@pytest.mark.parametrize("l,m", [(5, 500), (5, 600), (6, 250), (6, 400), (7, 250), (7, 300), (8, 100)])
+@pytest.mark.parametrize("K,d,pitch_extra", [(9, 200_003, 0), (4, 2_500_001, 2)])
+def test_both_splits_of_the_warps(l, m, K, d, pitch_extra):
+    import torch
+    import oracle
+    import paper_2405_20988_b200 as F
+    wbuf, w_t0, xi, coeffs = _inputs(l, K, d, pitch_extra, l * m)
+    ora = oracle.local_state(wbuf[:, :d], w_t0, xi, coeffs, l, m, threads=8)
+    with F.FdaContext(l, m, coeffs, d_max=d, K_max=K) as ctx:
+        st = torch.full((K, ctx.state_len), float("nan"), device="cuda")
+        ctx.fda_local_state(torch.from_numpy(wbuf).cuda()[:, :d], torch.from_numpy(w_t0).cuda(), torch.from_numpy(xi).cuda(), 7, st)
+        assert ctx.fda_debug_last_kernel() == "k_local_state_gather"
+    check_states(st.cpu().numpy(), ora, l, m, d)
