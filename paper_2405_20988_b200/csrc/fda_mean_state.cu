@@ -347,13 +347,21 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
     // With a list schedule in the context the cells can come from the list kernel.  In one pass over
     // the K rows when the vector has at least two tiles per SM (5 x 250, K = 30, d = 7M: 182 against
     // 214 us; K = 20, d = 2.6M: 77 against 85 us; below that the first tile's loads and the rounding of
-    // the tiles per block cost more than the second kernel).  Rows that are not 16-byte aligned arrive
-    // there by 32-bit copies, which pays for few workers on long vectors only (K = 8, d = 20M: 243 against
-    // about 290 us; K = 30, d = 7M: 350 against 210 us).  From the averaged drifts that phase 1 below leaves in memory when
-    // the sketch is too large for the lane-private bins of k_sketch_vector_rows.
-    const bool lists = sketch && ctx->sched != nullptr;
+    // the tiles per block cost more than the second kernel).  Rows that are not 16-byte aligned arrive there by
+    // 32-bit copies.  That pays while the rows of a quad fit one slot of the landing zone (ten), and for a few more
+    // the more rows the sketch has.  Measured, rows at a pitch of an odd d, one pass and two:
+    //   second kernel k_sketch_vector_rows, from eight tiles per SM (at three and four the two are within 13 % either way):
+    //   5 x 250, d = 7.3M, K = 8 96 and 104 us, K = 10 103 and 116, K = 12 128 and 123; 3 x 100, d = 8.5M, K = 8 101 and 112,
+    //   K = 10 108 and 125, K = 14 149 and 146;
+    //   second kernel k_mean_state_gather, from two tiles per SM: 7 x 500, d = 1.5M, K = 10 38 and 42 us, d = 6.1M, K = 14 129
+    //   and 132, K = 16 137 both; 10 x 250, K = 20 3 % and 16 x 250, K = 20 10 % faster in one.
+    // Where sketches of many rows lose by it (7 x 250, K = 12 and 16 x 250, K = 32 6 to 8 %, 16 x 100 10 to 15 %) the call
+    // stays in one pass, which allocates nothing.
+    // From the averaged drifts that phase 1 below leaves in memory when the sketch is too large for the lane-private
+    // bins of k_sketch_vector_rows.
+    const bool lists = sketch && ctx->sched != nullptr, rows_kernel = ctx->columns == 32;
     const int64_t tiles = lists ? (d + ctx->sched_T - 1) / ctx->sched_T : 0;
-    const bool one_pass = vec ? tiles >= 2 * (int64_t)ctx->n_sm : K <= 2 * ctx->l && tiles >= 8 * (int64_t)ctx->n_sm;
+    const bool one_pass = (vec || K <= std::max(2 * ctx->l, 10)) && tiles >= (vec || !rows_kernel ? 2 : 8) * (int64_t)ctx->n_sm;
     if (lists && one_pass) {
         const cudaError_t e = fda_launch_mean_state_gather(ctx, w, row_stride, K, d, w_t0, xi, flags, mean_state, s);
         if (e != cudaErrorNotSupported) {
@@ -377,7 +385,7 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
     if (e != cudaSuccess) return e;
 
     // phase 2: sketch of u-bar
-    if (lists && ctx->columns != 32) {
+    if (lists && !rows_kernel) {
         e = fda_launch_mean_sketch_gather(ctx, ctx->mean_model, K, d, linear, flags, (int)nblk, mean_state, s);
         if (e != cudaErrorNotSupported) {
             if (e == cudaSuccess) ctx->last_ls_kernel = "k_mean_model + k_mean_state_gather";
@@ -401,7 +409,7 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
         if (blocks > p.tiles) blocks = p.tiles;
         sk_blocks = (int)blocks;
         const size_t smem = (size_t)ctx->lm * ctx->columns * sizeof(float);
-        if (ctx->columns == 32) {
+        if (rows_kernel) {
             const int64_t ngroups = (d + 1023) / 1024;            // 8 steps of 128 indices
             int64_t rb = (int64_t)ctx->n_sm;
             if (rb > ngroups) rb = ngroups;

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 import fda_synth as S
-from fda_testlib import check_estimate, check_states
+from fda_testlib import REL, check_estimate, check_states
 
 pytestmark = pytest.mark.gpu
 
@@ -112,3 +112,33 @@ def test_both_splits_of_the_warps(l, m, K, d, pitch_extra):
         ctx.fda_local_state(torch.from_numpy(wbuf).cuda()[:, :d], torch.from_numpy(w_t0).cuda(), torch.from_numpy(xi).cuda(), 7, st)
         assert ctx.fda_debug_last_kernel() == "k_local_state_gather"
     check_states(st.cpu().numpy(), ora, l, m, d)
+
+
+# rows that are not 16-byte aligned: one pass up to ten workers or twice the sketch rows, from eight tiles per SM where
+# the second kernel of the other route has lane-private bins, from two where it walks the lists too
+@pytest.mark.parametrize("l,m,K,tiles,one_pass", [(3, 100, 10, 8, True), (3, 100, 11, 8, False), (3, 100, 3, 7, False), (5, 250, 10, 8, True),
+                                                  (7, 500, 14, 2, True), (7, 500, 15, 2, False), (7, 500, 3, 1, False)])
+def test_averaged_state_of_unaligned_rows(l, m, K, tiles, one_pass):
+    import torch
+    import oracle
+    import paper_2405_20988_b200 as F
+    T = 5120 if m == 500 else 6144
+    d = tiles * SMS * T - 7
+    wbuf, w_t0, xi, coeffs = _inputs(l, K, d, 2, l * m + K)
+    # the sketch is linear: the oracle's state of the averaged drift, and the averages of the scalars
+    u = wbuf[:, :d].astype(np.float64) - w_t0
+    ubar = u.mean(axis=0)
+    ora = oracle.local_state(ubar.astype(np.float32)[None], np.zeros(d, np.float32), xi, coeffs, l, m, threads=8)[0]
+    norm, proj = float((u * u).sum(axis=1).mean()), float((u @ xi.astype(np.float64)).mean())
+    ubar_sq = float(ubar @ ubar)
+    with F.FdaContext(l, m, coeffs, d_max=d, K_max=K) as ctx:
+        assert ctx.fda_context_info()["tile_indices"] == T
+        mean = torch.full((ctx.state_len,), float("nan"), device="cuda")
+        ctx.fda_mean_state(torch.from_numpy(wbuf).cuda()[:, :d], torch.from_numpy(w_t0).cuda(), torch.from_numpy(xi).cuda(), 7, mean)
+        assert (ctx.fda_debug_last_kernel() == "k_mean_state_gather") == one_pass
+        assert (ctx.fda_context_info()["other_lazy_bytes"] == 0) == one_pass
+    got = mean.cpu().numpy().astype(np.float64)
+    assert abs(got[0] - norm) <= REL * norm
+    assert abs(got[1] - proj) <= REL * max(abs(proj), np.sqrt(ubar_sq / d))
+    # u-bar reaches the oracle in single precision (2^-24), a cell is held to REL of its scale
+    assert np.max(np.abs(got[2:] - ora[2:]) / np.maximum(np.abs(ora[2:]), np.sqrt(ubar_sq / m))) <= REL
