@@ -86,10 +86,13 @@ typedef struct {
  * Device memory the context takes (fda_context_info reports the figures):
  *   - per-block partial sums: (SM count) * l*m * 128 bytes plus 64 * (SM count) * max(K_max, 32) bytes;
  *   - the list schedule of the sketch kernel, when the sketch allows one (tiles of at least 6*m
- *     indices fit the shared memory, or of 5*m with the rows in two or four equal parts): about 2.4 * l bytes per index of d_max (2.4 GB for
- *     d_max = 2 * 10^8 and l = 5), built here in about 4 ms per million indices; it is dropped,
- *     and sketch requests are then served by the slower plain-load kernels, when it would take
- *     more than a third of the free device memory (see fda_create_limited for another cap);
+ *     indices fit the shared memory, or of 5*m with the rows in two or four equal parts).  Per index of d_max
+ *     it takes 2.4 * l bytes at m = 250 (2.4 GB for d_max = 2 * 10^8 and l = 5), 2.8 * l at m = 500 and 3.1 to
+ *     3.6 * l at m = 1000, and it is built here: per million indices and sketch row in 0.22 ms at m = 250,
+ *     0.4 at m = 500 and 0.65 at m = 1000 (5 x 250: 1.1 ms per million indices, 8 x 1000, whose rows are in two
+ *     parts: 5.1), about twice that for vectors of a million indices and less.  It is dropped, and sketch
+ *     requests are then served by the slower plain-load kernels, when it would take more than a third of the
+ *     free device memory (see fda_create_limited for another cap);
  *   - lazily, by the first call that needs them: a 16-bit hash table of 2*l bytes per index
  *     (sketch requests on a context without a schedule), d_max floats (fda_mean_state on
  *     short vectors, many unaligned rows, or without a schedule), K_max*d_max floats of staging
@@ -141,9 +144,11 @@ const char *fda_last_error(const fda_ctx *ctx);
  *   states      out, K x state_len floats
  * Any alignment of w, w_t0, xi is accepted; 16-byte aligned pointers with row_stride a
  * multiple of 4 take the vector path.  Errors: INVALID_ARG (NULL, K < 1 or > K_max, d < 1
- * or > d_max, row_stride < d, unknown flag, SKETCH without a sketch), UNSUPPORTED (more worker
- * groups than the context's partial-sum scratch holds: K above 4 x the SM count with a list
- * schedule, above 32 x the SM count without; nothing is launched), CUDA.
+ * or > d_max, row_stride < d, unknown flag, SKETCH without a sketch), UNSUPPORTED (a sketch for more
+ * workers than the context's partial-sum scratch holds: K above 32 x the SM count, or above 4 x the SM
+ * count x the copies of the l*m bins that fit the shared memory when fewer than eight do; nothing is
+ * launched), CUDA.  K above 4 x the SM count (2 x or 1 x with the rows in two or four parts) is served by
+ * the plain-load kernels also on a context with a list schedule.
  * Stream order: the call's work starts after what `stream` held before it and is complete before
  * anything enqueued on `stream` after it.  Part of it may run on a second stream that the context
  * owns (forked from and joined to `stream` with events; also legal while `stream` is being
@@ -282,9 +287,9 @@ fda_status fda_debug_schedule(const fda_ctx *ctx, int64_t tile, void *record_hos
 
 /*
  * Name of the kernel that served the context's last fda_local_state or fda_mean_state call (the
- * paper has no counterpart): "k_local_state_gather" (sketch pass over per-cell index lists: every sketch request
- * on a context that holds a list schedule), "k_local_state_linear" (no sketch requested),
- * "k_local_state_fast" / "k_local_state" (sketch requests without a schedule: aligned rows with 5
+ * paper has no counterpart): "k_local_state_gather" (sketch pass over per-cell index lists, in all its
+ * forms: every sketch request that a context's list schedule can serve), "k_local_state_linear" (no
+ * sketch requested), "k_local_state_fast" / "k_local_state" (other sketch requests: aligned rows with 5
  * or 7 sketch rows / everything else); for fda_mean_state "k_mean_state_gather" (one pass on
  * the list kernel), "k_mean_model + k_mean_state_gather" (averaged drifts, then the list
  * kernel on them), "k_mean_model + k_sketch_vector" (no schedule) or "k_mean_model" (no sketch

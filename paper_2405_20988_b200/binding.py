@@ -224,8 +224,9 @@ class FdaContext:
 
     def fda_combine_estimate(self, states, K: int, variant: int, epsilon: float, theta: float,
                              est_dev, want_host: bool = True, stream=None):
-        """est_dev: uint8 CUDA tensor of sizeof(fda_estimate) bytes.  Returns an Estimate
-        (host copy, synchronises the stream) when ``want_host``, else None."""
+        """est_dev: uint8 CUDA tensor of sizeof(fda_estimate) bytes.  When ``want_host``, returns an
+        Estimate as soon as it has reached the host (earlier work on the stream and est_dev are complete
+        then), else None."""
         host = Estimate() if want_host else None
         st = _native.combine_estimate(self._h.value, states, K, variant, epsilon, theta, est_dev,
                                       ctypes.addressof(host) if want_host else 0, stream)

@@ -404,7 +404,7 @@ fda_status fda_round_host(fda_ctx *ctx, float *w_host, int64_t row_stride, int K
                                     ctx->stage_states, stream);
     if (st != FDA_OK) return st;
     st = fda_combine_estimate(ctx, ctx->stage_states, K, variant, epsilon, theta, ctx->stage_est,
-                              est_host, stream);          // synchronises: est_host is valid
+                              est_host, stream);          // returns when est_host is valid
     if (st != FDA_OK) return st;
     if (states_host) {
         e = cudaMemcpyAsync(states_host, ctx->stage_states, sizeof(float) * (size_t)K * slen,

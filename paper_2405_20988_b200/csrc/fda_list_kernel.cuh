@@ -8,7 +8,7 @@
 namespace fda_list {
 
 constexpr int GW = kListWorkers;
-constexpr int kChunksAhead = 8;                // entry chunks (four steps each) the walkers of the averaged state load ahead (sketches below 7 rows)
+constexpr int kChunksAhead = 8;                // entry chunks (four steps each) the walkers of the averaged state load ahead (long items)
 
 struct ListParams {
     const float *w, *w_t0, *xi;

@@ -30,8 +30,8 @@
 // buffer with tile n + 1, and one block-wide barrier per tile hands the buffers over.  Nothing
 // in this kernel waits on another block or spins on memory.
 //
-// What bounds it: the load/store unit's data pipe (about 72 % busy; 6.3 wavefronts per 128 updates
-// are the floor of this design, 8.3 are spent).  Between two items a walker has nothing to gather,
+// What bounds it: the load/store unit's data pipe (74 % busy; 6.3 wavefronts per 128 updates
+// are the floor of this design, 8.2 are spent).  Between two items a walker has nothing to gather,
 // so the way from item to item is kept short: the record's offset comes from shared memory (read
 // from L2 after the barrier it stood in front of the first entries of every tile), the first item of
 // a tile goes to a warp by its number, and the next item's number and descriptor are fetched before

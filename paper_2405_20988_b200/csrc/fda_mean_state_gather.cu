@@ -21,7 +21,7 @@
 //     with zeros for what lies past the end;
 //   * 8 producer and 24 walker warps at 64 registers.
 //
-// Two callers: the K rows of w (one pass, for few workers), or the single row of averaged drifts
+// Two callers: the K rows of w (one pass, any number of workers), or the single row of averaged drifts
 // that k_mean_model has left in device memory (no w_t0; the two scalars then come from that
 // kernel's partial sums).  Measured on B200, 5 x 250, K = 8, d = 198M, one pass: 1.50 ms (0.73 of
 // the measured copy bandwidth).  On the way: loads landing in registers four rows at a time with
@@ -116,8 +116,8 @@ inline size_t mean_smem_fixed(int l, int m, int T, int tab_bytes)
 //   then        ut[2][T + 8]   (summed drifts; eight zero rows behind each)
 //   then        the landing zone: depth slots of R rows of kRowPitch bytes
 // (each region on a 128-byte boundary)
-// AHEAD: entry chunks (four steps each) a walker loads before it walks them (five for sketches of
-// seven or more rows, whose items are short; else eight - as in k_local_state_gather).
+// AHEAD: entry chunks (four steps each) a walker loads before it walks them: eight, or five for the short
+// items of sketches of seven or more rows and of rows in parts (k_local_state_gather has a rule of its own).
 // MULTI: the rows of a quad arrive in several slots (more than kMaxPiece rows).
 // VEC: w, w_t0 and xi are 16-byte aligned.
 template <bool LINEAR, int AHEAD, bool MULTI, bool VEC>

@@ -142,3 +142,20 @@ def test_averaged_state_of_unaligned_rows(l, m, K, tiles, one_pass):
     assert abs(got[1] - proj) <= REL * max(abs(proj), np.sqrt(ubar_sq / d))
     # u-bar reaches the oracle in single precision (2^-24), a cell is held to REL of its scale
     assert np.max(np.abs(got[2:] - ora[2:]) / np.maximum(np.abs(ora[2:]), np.sqrt(ubar_sq / m))) <= REL
+
+
+# more worker groups than SMs: the plain-load kernels, also on a context with a schedule
+@pytest.mark.parametrize("l,m,K", [(2, 16, 4 * SMS), (2, 16, 4 * SMS + 1), (8, 1000, 2 * SMS), (8, 1000, 2 * SMS + 1)])
+def test_more_worker_groups_than_sms(l, m, K):
+    import torch
+    import oracle
+    import paper_2405_20988_b200 as F
+    d = 1027
+    wbuf, w_t0, xi, coeffs = _inputs(l, K, d, 0, K)
+    ora = oracle.local_state(wbuf[:, :d], w_t0, xi, coeffs, l, m, threads=8)
+    with F.FdaContext(l, m, coeffs, d_max=d, K_max=K) as ctx:
+        assert ctx.fda_context_info()["list_kernel"] == 1
+        st = torch.full((K, ctx.state_len), float("nan"), device="cuda")
+        ctx.fda_local_state(torch.from_numpy(wbuf).cuda()[:, :d], torch.from_numpy(w_t0).cuda(), torch.from_numpy(xi).cuda(), 7, st)
+        assert (ctx.fda_debug_last_kernel() == "k_local_state_gather") == (K % SMS == 0)
+    check_states(st.cpu().numpy(), ora, l, m, d)
