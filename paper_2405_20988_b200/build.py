@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libfda.so")
 OUT_PY = os.path.join(HERE, "_native.so")
 OBJ_DIR = os.path.join(HERE, "_build")
-SOURCES = ["fda_api.cu", "fda_hash.cu", "fda_local_state.cu", "fda_local_state_gather.cu", "fda_mean_state_gather.cu", "fda_sched.cu", "fda_local_state_linear.cu", "fda_mean_state.cu", "fda_combine.cu", "fda_average.cu", "fda_noalloc.cu", "fda_probe.cu"]
+SOURCES = ["fda_api.cu", "fda_hash.cu", "fda_local_state.cu", "fda_local_state_gather.cu", "fda_lanes_12.cu", "fda_lanes_16.cu", "fda_lanes_20.cu", "fda_lanes_22.cu", "fda_lanes_23.cu", "fda_lanes_24.cu", "fda_mean_state_gather.cu", "fda_sched.cu", "fda_local_state_linear.cu", "fda_mean_state.cu", "fda_combine.cu", "fda_average.cu", "fda_noalloc.cu", "fda_probe.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]
 

@@ -119,6 +119,10 @@ void free_device(fda_ctx *ctx)
     cudaFree(ctx->tab);
     cudaFree(ctx->sched);
     cudaFree(ctx->sched_off);
+    cudaFree(ctx->lane_sched);
+    cudaFree(ctx->lane_off);
+    cudaFree(ctx->lane_prog);
+    cudaFree(ctx->lane_rows);
     cudaFree(ctx->part_sk);
     cudaFree(ctx->part_np);
     cudaFree(ctx->combine_scratch);
@@ -198,6 +202,7 @@ fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uin
         if (e == cudaSuccess && schedule_limit_bytes >= 0) {
             const auto t0 = std::chrono::steady_clock::now();
             e = fda_build_list_schedule(ctx, nullptr);
+            if (e == cudaSuccess && ctx->sched) e = fda_build_lane_schedule(ctx, nullptr);
             ctx->sched_build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
         if (e == cudaSuccess) e = cudaMalloc(&ctx->part_sk, sizeof(float) * ctx->part_sk_floats);
@@ -470,7 +475,7 @@ fda_status fda_context_info(const fda_ctx *ctx, int64_t *info)
 {
     if (!ctx || !info) return FDA_ERR_INVALID_ARG;
     const int64_t table = ctx->tab ? (int64_t)(sizeof(uint16_t) * (size_t)ctx->l * ctx->tab_stride) : 0;
-    const int64_t sched = ctx->sched ? (int64_t)(ctx->sched_bytes + sizeof(uint64_t) * (size_t)(ctx->sched_tiles * ctx->sched_parts + 1)) : 0;
+    const int64_t sched = ctx->sched ? (int64_t)(ctx->sched_bytes + sizeof(uint64_t) * (size_t)(ctx->sched_tiles * ctx->sched_parts + 1) + ctx->lane_bytes) : 0;
     const int64_t partial = (int64_t)(sizeof(float) * ctx->part_sk_floats + sizeof(double) * ctx->part_np_doubles +
                                       sizeof(double) * fda_combine_scratch_doubles(ctx->l, ctx->m) + sizeof(unsigned int) * (3 + ctx->n_row_tickets)) +
                             (ctx->coeffs_dev ? (int64_t)sizeof(uint64_t) * 6 * ctx->l : 0);

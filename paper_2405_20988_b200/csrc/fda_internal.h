@@ -21,6 +21,8 @@ constexpr int kListMaxLen = 64;        // longest list (longer cells are cut int
 constexpr int kListPadRows = 8;        // zero rows behind the tile, one per bank group
 constexpr int kListBatch = 1024;       // indices a producer step covers; tiles are multiples of it
 constexpr int kListMaxTile = 7168;     // rows + pad rows must fit 13 bits
+constexpr int kLaneStepBits = 12;      // bits of an item's steps in a word of lane_prog
+constexpr int kLaneMaxItems = 154;     // items that the lanes of a block can keep the cells of (seven to each of 22 warps)
 constexpr int kListSmemHead = 2112;    // counters and the warps' fp64 sums in front of the item tables
 
 // byte offsets inside the schedule record of a tile with `items` items
@@ -66,6 +68,19 @@ struct fda_ctx {
     int sched_ni_max = 0;             // items a record can have
     int64_t sched_tiles = 0;
     int sched_parts = 1;              // equal parts of the sketch rows that have records of their own
+    // A second schedule, in which every cell stays with one lane of one warp (null when not built): its records
+    // have the same form.  The program of a record, [record][1 + lane_items], says where its chunks begin, in units
+    // of 256 bytes, and for each item its first chunk << kLaneStepBits | its steps; lane_rows holds the order of
+    // the cells of every sketch row, {cell step, cycle length}.
+    unsigned char *lane_sched = nullptr;
+    uint64_t *lane_off = nullptr;
+    uint32_t *lane_prog = nullptr;
+    int2 *lane_rows = nullptr;
+    uint64_t lane_bytes = 0;          // records, offsets and programs
+    int lane_T = 0, lane_parts = 1;
+    int64_t lane_tiles = 0;
+    int lane_items = 0;               // items of a tile (and part of the sketch rows)
+    int lane_walkers = 0;             // warps that share them
     double sched_build_ms = 0.0;      // host time spent building it
     float *mean_model = nullptr;      // d_max floats (average drift), allocated by the first fda_mean_state
     // a second stream for the launches that fill the SMs the main launch of the list kernel leaves idle
@@ -89,6 +104,16 @@ struct fda_ctx {
     int last_ls_launches = 0;          // kernels the last fda_local_state launched
     std::string err;
 };
+
+// Lanes that keep their cells: worth a schedule of their own, and used, when a block has more than twelve tiles.
+inline bool fda_lanes_pay(int64_t tiles, int groups, int n_sm) { return groups <= n_sm && tiles > 12 * (int64_t)(n_sm / groups); }
+
+// Cell at place `pos` of the order (step, cycle) of a sketch row: the cells 0, step, 2 step, ... (mod m) up to the
+// end of the cycle, then those of the cycle through 1, and so on.
+inline __host__ __device__ int fda_lane_cell(int pos, int step, int cycle, int m)
+{
+    return (int)(((int64_t)(pos % cycle) * step + pos / cycle) % m);
+}
 
 // ---- kernels that overlap their start with the end of the kernel before them -----------
 // A kernel launched with fda_launch_dependent is set up while its predecessor on the stream is still
@@ -130,6 +155,7 @@ cudaError_t fda_launch_local_state(fda_ctx *ctx, const float *w, int64_t row_str
                                    int64_t d, const float *w_t0, const float *xi, uint32_t flags,
                                    float *states, cudaStream_t s);
 cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s);   // allocates and fills ctx->sched when it fits
+cudaError_t fda_build_lane_schedule(fda_ctx *ctx, cudaStream_t s);   // the same for ctx->lane_sched, where it pays
 cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx);
 cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t row_stride, int K,
                                           int64_t d, const float *w_t0, const float *xi,

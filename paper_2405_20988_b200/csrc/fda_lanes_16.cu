@@ -1,0 +1,6 @@
+#include "fda_worker_kernel.cuh"
+
+cudaError_t fda_lanes_16(const fda_list::ListParams &p, int blocks, bool dependent, cudaStream_t s)
+{
+    return launch_lanes<16, 16, false, 1, 2>(p, blocks, dependent, s);
+}

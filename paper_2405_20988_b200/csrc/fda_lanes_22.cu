@@ -1,0 +1,6 @@
+#include "fda_worker_kernel.cuh"
+
+cudaError_t fda_lanes_22(const fda_list::ListParams &p, int blocks, bool dependent, cudaStream_t s)
+{
+    return launch_lanes<10, 22, true, 1, 7>(p, blocks, dependent, s);
+}

@@ -27,6 +27,9 @@ struct ListParams {
     int tab_bytes;                   // bytes of one item-table buffer in shared memory
     const unsigned char *sched;
     const uint64_t *sched_off;
+    const uint32_t *lane_prog;         // cells that stay with their lanes (else null): see fda_ctx
+    const int2 *lane_rows;
+    int lane_items;
     float *part_sk;                  // [block][cell][GW]
     double *part_np;                 // [block][GW][2]
 };
@@ -80,6 +83,12 @@ __device__ __forceinline__ uint4 load_u4(const void *ptr)
 {
     uint4 v;
     asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(ptr));
+    return v;
+}
+__device__ __forceinline__ uint2 load_u2(const void *ptr)
+{
+    uint2 v;
+    asm volatile("ld.global.nc.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(ptr));
     return v;
 }
 __device__ __forceinline__ unsigned long long load_u64(const void *ptr)

@@ -31,7 +31,9 @@
 // in this kernel waits on another block or spins on memory.
 //
 // What bounds it: the load/store unit's data pipe (74 % busy; 6.3 wavefronts per 128 updates
-// are the floor of this design, 8.2 are spent).  Between two items a walker has nothing to gather,
+// are the floor of this design, 8.2 are spent).  The loads of the next tile's first batch are asked for in front of
+// the barrier, and the sums of squares go through six shuffles instead of twenty (they take that pipe, too):
+// with lanes that keep their cells 2065 -> 1876 us at 5 x 250, K = 8, d = 198M, 312 -> 285 at K = 30, d = 7M.  Between two items a walker has nothing to gather,
 // so the way from item to item is kept short: the record's offset comes from shared memory (read
 // from L2 after the barrier it stood in front of the first entries of every tile), the first item of
 // a tile goes to a warp by its number, and the next item's number and descriptor are fetched before
@@ -42,395 +44,51 @@
 // add to one cell at a time), entries of the next item asked for before the flush (2.61 ms), 24
 // walkers at 64 registers (2.40 ms).
 //
+// Lanes that keep their cells.  A bucket is a*j + b mod p mod m, a lattice: in a tile of thousands of consecutive
+// indices nearly every cell has the same number of them (the variance of the counts is a tenth of that of random
+// buckets; one row in twenty or so is an exception).  So lists need not be handed out by length: on long vectors
+// every cell belongs to one lane of one walker warp for the whole launch.  What that saves: the sum of a cell
+// lives in registers (the list of a tile is added up from zero and added to it once per tile, as to a bin before),
+// so there are no bins, no flush with its conflicts, no counters and no item tables; a warp's program is known
+// ahead, so the next eight steps are always asked for, across items and across the hand-over; walkers do not
+// stop between items all at once.  The order of the cells of a row is chosen so that the lists of eight neighbours are
+// copies of one another shifted by an odd number of indices (fda_sched.cu): as long as one another, and spread over
+// the bank groups; steps per entry 1.12 at 5 x 250, 1.19 at 7 x 500 (list kernel 1.16 and 1.23).  Walkers 12 to 24
+// of 28 to 32 warps, so that no lane is without a cell where that can be had; the others produce.  Measured, the
+// list kernel and this one: 5 x 250, K = 8, d = 198M 2322 and 1860 us (2500 and 2218 us after half a second, at the
+// power limit); K = 30, d = 7M 347 and 283; 7 x 500, K = 60, d = 20M 2560 and 2022; 8 x 1000, K = 20, d = 2.6M 203 and
+// 166; K = 8, d = 20M: 1 x 250 191 and 128, 8 x 250 343 and 309, 4 x 1000 412 and 240.
+//
+// Its line: states without a projection, blocks of more than twelve tiles.  Shorter vectors gain little (K = 10,
+// d = 1.2M, four tiles: 33.3 and 31.2 us) for a second schedule in fda_create.  With xi the list kernel stays, although it
+// is slower there too: such a call keeps the order of its additions.  Right after a synchronisation the mean
+// drift is the rounding of the average itself, and the row norms of S-bar then show that order from the fourth digit on.
+//
 // fda_mean_state_gather.cu holds the sibling of this kernel that computes the averaged state of
-// fda_mean_state from the same schedule.
+// fda_mean_state from the list schedule.
 
 #include <algorithm>
 
 #include "fda_internal.h"
-#include "fda_list_kernel.cuh"
+#include "fda_worker_kernel.cuh"
+
+// One launch of the kernel whose lanes keep their cells, with `walkers` warps that walk (blocks == 0: only sets its
+// shared-memory limit).
+static cudaError_t fda_lanes_run(int walkers, bool parts, const fda_list::ListParams &p, int blocks, bool dependent, cudaStream_t s)
+{
+    if (parts) return fda_lanes_22(p, blocks, dependent, s);
+    switch (walkers) {
+        case 12: return fda_lanes_12(p, blocks, dependent, s);
+        case 16: return fda_lanes_16(p, blocks, dependent, s);
+        case 20: return fda_lanes_20(p, blocks, dependent, s);
+        case 23: return fda_lanes_23(p, blocks, dependent, s);
+        default: return fda_lanes_24(p, blocks, dependent, s);
+    }
+}
 
 namespace {
 
 using namespace fda_list;
-
-// The drifts of the chunks first, first + step, ... (CHUNKS of them at a time) of 128 indices of the tile
-// that starts at index j0: all loads before any use, rows into the buffer at `base`, the warp's sums
-// of squares and products with xi (fp32) into sums[8] (fp64, lane 0).  VEC: a lane owns four consecutive
-// indices of a chunk, else the four indices lane, lane + 32, ...  Workers past K alias the group's
-// first row: their sums are never written out.
-template <bool LINEAR, bool VEC, int CHUNKS>
-__device__ __forceinline__ void form_drifts(const ListParams &p, int g, int64_t j0, int first, int step, uint32_t base,
-                                            double *sums)
-{
-    const int lane = threadIdx.x & 31, T = p.T;
-    const float *wbase = p.w + (size_t)(g * GW) * (size_t)p.row_stride;
-    float nf[GW], pf[GW];
-#pragma unroll
-    for (int k = 0; k < GW; ++k) { nf[k] = 0.f; pf[k] = 0.f; }
-#pragma unroll 1
-    for (int c0 = first; c0 < T / 128; c0 += step * CHUNKS) {
-        float4 wv[CHUNKS][GW], w0v[CHUNKS], xv[CHUNKS];
-#pragma unroll
-        for (int b = 0; b < CHUNKS; ++b) {
-            const int r = 128 * (c0 + step * b);
-            const int64_t j = j0 + r + (VEC ? 4 * lane : lane), left = r < T ? p.d - j : 0;
-            const int n = VEC ? (left >= 4 ? 4 : left > 0 ? (int)left : 0) : (left > 96 ? 4 : left > 0 ? (int)(left + 31) / 32 : 0);
-            auto load = [&](const float *ptr) { return VEC ? load_quad<false>(ptr, n == 4, n) : load_strided(ptr, n); };
-#pragma unroll
-            for (int k = 0; k < GW; ++k) wv[b][k] = load(wbase + (g * GW + k < p.K ? (int64_t)k * p.row_stride : 0) + j);
-            w0v[b] = load(p.w_t0 + j);
-            if (LINEAR) xv[b] = load(p.xi + j);
-        }
-#pragma unroll
-        for (int b = 0; b < CHUNKS; ++b) {
-            const uint32_t r0 = 128u * (uint32_t)(c0 + step * b);
-            if (r0 >= (uint32_t)T) break;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float w0 = comp(w0v[b], q);
-                float u[GW];
-#pragma unroll
-                for (int k = 0; k < GW; ++k) {
-                    u[k] = comp(wv[b][k], q) - w0;
-                    nf[k] = fmaf(u[k], u[k], nf[k]);
-                    if (LINEAR) pf[k] = fmaf(comp(xv[b], q), u[k], pf[k]);
-                }
-                const uint32_t r = r0 + (VEC ? 4u * lane + q : (uint32_t)lane + 32u * q);
-                store_row(base + fda_list_row(r) * 16u, u[0], u[1], u[2], u[3]);
-            }
-        }
-        if (CHUNKS > 1) break;                                 // (the caller has checked that one round covers the tile)
-    }
-#pragma unroll
-    for (int k = 0; k < GW; ++k) {
-        float a = nf[k], bq = LINEAR ? pf[k] : 0.f;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, off);
-            if (LINEAR) bq += __shfl_xor_sync(0xffffffffu, bq, off);
-        }
-        if (lane == 0) { sums[2 * k] = (double)a; sums[2 * k + 1] = (double)bq; }
-    }
-}
-
-// Shared-memory plan (bytes from the start of dynamic shared memory):
-//   [0, 8)    item counters of the two tile buffers
-//   [16, 48)  offsets of the schedule records of the tiles n, n + 1 (slot n mod 4)
-//   [64, 2112) sums[warp][worker][2] (fp64): ||u||^2 and <xi,u>, of the producers over the tiles so far, of
-//             the walkers (FIRST) over their part of the first tile
-//   [2112, ..) two item tables (tab_bytes each): the head of a tile's schedule record
-//   then      bins[l*m][4]
-//   then      ut[2][T + 8][4]   (drift tiles, index-major; eight zero rows behind each)
-// PW producer warps and WW walker warps: the split that is fastest depends on how much walking a
-// loaded index pays for (l updates per worker).  PARTS: the sketch rows are in several parts with
-// records of their own, and a block serves one part of one worker group.
-// Measured: 8 x 1000 as two parts, K = 20, d = 2.6M: 212 us, against 510 us on the compare-and-swap
-// kernel that served it before.
-// VEC: w, w_t0 and xi are 16-byte aligned.  If not, a producer thread owns the four indices lane, lane + 32,
-// ... of its warp's 128 instead of four consecutive ones, so that its 32-bit loads are coalesced (K = 30,
-// d = 6,964,106 at a pitch of d: 529 -> 370 us; 7 x 500, K = 60, d = 20M: 4.38 -> 2.75 ms).
-// FIRST: all warps form the first tile.  As the producers' own job it is a chain of round trips with nothing to
-// walk meanwhile, which counts when a block has few tiles; the code for it costs long runs 1 %.
-template <bool LINEAR, int PW, int WW, bool PARTS, bool VEC, bool FIRST>
-__global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const ListParams p)
-{
-    constexpr int kProducerWarps = PW;
-    constexpr int kThreads = (PW + WW) * 32;
-    constexpr int kBatch = PW * 32 * 4;                       // a batch is four consecutive indices per producer thread
-    constexpr int kDepth = 1;                                 // batches a producer thread keeps in flight
-    // entry chunks (four steps each) a walker loads before it walks them: seven (items of 5 x 250
-    // average 28 steps), four with the 5 + 23 split, whose items average eleven, two for the short
-    // items of parts.  Measured: 7 x 500, K = 60, d = 20M: 2.76 ms with 4 or 3, 2.79 with 5;
-    // 5 x 250, K = 8, d = 198M: 2.33 ms with 7 or 8, 2.43 with 6, 2.38 with 5
-    constexpr int kAhead = PARTS ? 2 : (PW == 5 && WW == 23) ? 4 : 7;
-    static_assert(PW + WW <= 32, "the fp64 sums have room for 32 warps");
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int vg = (int)blockIdx.x % p.groups, c = (int)blockIdx.x / p.groups;
-    const int g = PARTS ? vg % p.wgroups : vg;
-    const uint64_t *sched_off = PARTS ? p.sched_off + (size_t)(vg / p.wgroups) * p.part_tiles : p.sched_off;
-    const int T = p.T, lm = p.l * p.m;
-
-    const uint32_t smem_base = (uint32_t)__cvta_generic_to_shared(smem_raw);
-    int *ctr = reinterpret_cast<int *>(smem_raw);
-    unsigned long long *rec_off = reinterpret_cast<unsigned long long *>(smem_raw + 16);
-    double *sums = reinterpret_cast<double *>(smem_raw + 64);
-    const uint32_t tab_off = kListSmemHead;
-    const uint32_t bins_off = tab_off + 2u * (uint32_t)p.tab_bytes;
-    const uint32_t ut_off = bins_off + (uint32_t)lm * 16u;
-    const uint32_t ut_bytes = (uint32_t)(T + kListPadRows) * 16u;
-    float *bins = reinterpret_cast<float *>(smem_raw + bins_off);
-
-    for (int t = tid; t < lm * GW; t += kThreads) bins[t] = 0.f;
-    for (int t = tid; t < 2 * kListPadRows * GW; t += kThreads) {
-        const int b = t / (kListPadRows * GW), r = t % (kListPadRows * GW);
-        reinterpret_cast<float *>(smem_raw + ut_off + (size_t)b * ut_bytes)[T * GW + r] = 0.f;
-    }
-    if (tid < 2) ctr[tid] = 0;
-    uint4 tab0 = make_uint4(0u, 0u, 0u, 0u);
-    if (FIRST) {
-        if (warp < kProducerWarps) {
-            const unsigned long long off = load_u64(sched_off + c);
-            if (tid * 16 < p.tab_bytes) tab0 = load_u4(p.sched + off + tid * 16);
-            if (tid == 0) rec_off[0] = off;
-        }
-        fda_grid_wait();
-        form_drifts<LINEAR, VEC, 1>(p, g, (int64_t)c * T, warp, PW + WW, smem_base + ut_off, sums + warp * GW * 2);
-        __syncthreads();
-    } else {
-        if (tid < kProducerWarps * GW * 2) sums[tid] = 0.0;
-        __syncthreads();
-        fda_grid_wait();
-    }
-
-    const int n_tiles = p.tiles > c ? (int)((p.tiles - c + p.cpg - 1) / p.cpg) : 0;
-
-    if (warp < kProducerWarps) {
-        // =============================== producers ===============================
-        const int pt = tid;                                   // quad of indices inside a batch
-        // rows of the group; workers past K alias the group's first row (their sums are computed
-        // and never written out), so the loop below needs no per-worker predicate
-        const float *wbase = p.w + (size_t)(g * GW) * (size_t)p.row_stride;
-        int64_t roff[GW];
-#pragma unroll
-        for (int k = 0; k < GW; ++k) roff[k] = g * GW + k < p.K ? (int64_t)k * p.row_stride : 0;
-        float4 wv[kDepth][GW], w0v[kDepth], xv[kDepth];       // four consecutive indices each
-        float nf[GW], pf[GW];
-#pragma unroll
-        for (int k = 0; k < GW; ++k) { nf[k] = 0.f; pf[k] = 0.f; }
-        int n_i = FIRST ? 1 : 0, n_c = 0;                 // tile being loaded / stored
-        int b_i = 0, b_c = 0;                                 // batch inside it
-        uint32_t j_i = (uint32_t)(FIRST ? c + p.cpg : c) * (uint32_t)T + (VEC ? 4 * pt : 128 * warp + lane);   // first index of this thread's next loads
-        uint32_t end_i = (uint32_t)((FIRST ? c + p.cpg : c) + 1) * (uint32_t)T;   // end of the tile they belong to
-        // 128-index chunks warp, warp + PW, ... of a tile, and the way from behind the last one to the
-        // first of this block's next tile
-        const int nb = (T / 128 - warp + PW - 1) / PW;
-        const uint32_t wrap = (uint32_t)p.cpg * (uint32_t)T - (uint32_t)(nb * kBatch);
-        // The rows of a tile two tiles ahead of the one being stored, into L2 (one bulk prefetch per
-        // worker row, w_t0 and xi): the producers' loads then find their data in L2.
-        auto prefetch_tile = [&](int n) {
-            if (n >= n_tiles || pt >= GW + 2) return;
-            const int64_t j = (c + n * p.cpg) * (int64_t)T;
-            int64_t cnt = p.d - j;
-            if (cnt > T) cnt = T;
-            uint32_t bytes = (uint32_t)(cnt * 4) & ~15u;
-            const float *src = pt < GW ? (g * GW + pt < p.K ? wbase + (int64_t)pt * p.row_stride + j : nullptr)
-                                       : (pt == GW ? p.w_t0 + j : (LINEAR ? p.xi + j : nullptr));
-            if (!VEC && src) {                                // the 16-byte pieces inside the row
-                const uint32_t off = (16u - ((uint32_t)(uintptr_t)src & 15u)) & 15u;
-                bytes = (uint32_t)(cnt * 4) > off ? ((uint32_t)(cnt * 4) - off) & ~15u : 0u;
-                src += off / 4;
-            }
-            if (src && bytes)
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-        };
-        if (!FIRST) prefetch_tile(0);
-        prefetch_tile(1);
-        // head of the schedule record of the tile being stored (the walkers' item table) and the
-        // record offsets of the next tile, loaded one and two tiles ahead of their use
-        uint4 tabv = tab0;
-        unsigned long long off0 = 0ull, off1 = 0ull;
-        if (!FIRST) {
-            off0 = load_u64(sched_off + c);
-            off1 = load_u64(sched_off + c + 1);
-            if (pt * 16 < p.tab_bytes) tabv = load_u4(p.sched + off0 + pt * 16);
-            if (pt == 0) rec_off[0] = off0;
-        }
-        if (n_tiles > 1) { off0 = load_u64(sched_off + c + p.cpg); off1 = load_u64(sched_off + c + p.cpg + 1); }
-        // the walkers get tile n_c, which is in buffer `buf`
-        auto hand_over = [&](int buf) {
-            // the table of this tile (loaded a tile ago), the loads of the next one, the offsets
-            // of the one after: nothing here waits for memory
-            if (pt * 16 < p.tab_bytes)
-                *reinterpret_cast<uint4 *>(smem_raw + tab_off + (size_t)buf * p.tab_bytes + pt * 16) = tabv;
-            if (pt == 0) { ctr[buf] = WW; rec_off[(n_c + 1) & 3] = off0; }
-            if (n_c + 1 < n_tiles) {
-                const unsigned char *nrec = p.sched + off0;
-                if (pt * 16 < p.tab_bytes) tabv = load_u4(nrec + pt * 16);
-                for (uint64_t o = (uint64_t)pt * 128u; o < off1 - off0; o += (uint64_t)kProducerWarps * 32u * 128u)   // the record into L2 ahead of its walk
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(nrec + o));
-            }
-            if (n_c + 2 < n_tiles) {
-                const int64_t t2 = c + (int64_t)(n_c + 2) * p.cpg;
-                off0 = load_u64(sched_off + t2);
-                off1 = load_u64(sched_off + t2 + 1);
-            }
-            prefetch_tile(n_c + 2);
-            block_barrier<kThreads>();
-            b_c = 0;
-            ++n_c;
-        };
-        auto issue = [&](int slot) {
-            if (n_i < n_tiles) {
-                const float *q = wbase + j_i;
-                if (!VEC) {
-                    const int64_t left = p.d - (int64_t)j_i;
-                    const int n = left > 96 ? 4 : (left > 0 ? (int)(left + 31) / 32 : 0);
-#pragma unroll
-                    for (int k = 0; k < GW; ++k) wv[slot][k] = load_strided(q + roff[k], n);
-                    w0v[slot] = load_strided(p.w_t0 + j_i, n);
-                    if (LINEAR) xv[slot] = load_strided(p.xi + j_i, n);
-                } else if (end_i <= (uint32_t)p.d) {                    // a whole tile: 128-bit loads
-#pragma unroll
-                    for (int k = 0; k < GW; ++k) wv[slot][k] = load4_stream(q + roff[k]);
-                    w0v[slot] = load4_keep(p.w_t0 + j_i);
-                    if (LINEAR) xv[slot] = load4_keep(p.xi + j_i);
-                } else {                                      // the last tile of the model
-                    const int64_t left = p.d - (int64_t)j_i;
-                    const int n = left >= 4 ? 4 : (left > 0 ? (int)left : 0);
-#pragma unroll
-                    for (int k = 0; k < GW; ++k) wv[slot][k] = load_quad<true>(q + roff[k], n == 4, n);
-                    w0v[slot] = load_quad<false>(p.w_t0 + j_i, n == 4, n);
-                    if (LINEAR) xv[slot] = load_quad<false>(p.xi + j_i, n == 4, n);
-                }
-                j_i += kBatch;
-                if (++b_i == nb) { b_i = 0; ++n_i; j_i += wrap; end_i += (uint32_t)p.cpg * (uint32_t)T; }
-            }
-        };
-        auto consume = [&](int slot) {
-            const int buf = (int)(n_c & 1);
-            // rows 4*pt .. 4*pt+3 of the batch; row r is stored at r ^ ((r >> 3) & 3), so that the
-            // eight lanes of a store pass hit eight different bank groups (the schedule's entries
-            // hold the swizzled row)
-            const uint32_t r0 = (uint32_t)(b_c * kBatch) + (VEC ? 4u * pt : fda_list_row(128u * warp + lane));
-            const uint32_t dst0 = smem_base + ut_off + (uint32_t)buf * ut_bytes + r0 * 16u;
-            const uint32_t sw = (r0 >> 3) & 3u;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float w0 = comp(w0v[slot], q);
-                const float u0 = comp(wv[slot][0], q) - w0;
-                const float u1 = comp(wv[slot][1], q) - w0;
-                const float u2 = comp(wv[slot][2], q) - w0;
-                const float u3 = comp(wv[slot][3], q) - w0;
-                nf[0] = fmaf(u0, u0, nf[0]); nf[1] = fmaf(u1, u1, nf[1]);
-                nf[2] = fmaf(u2, u2, nf[2]); nf[3] = fmaf(u3, u3, nf[3]);
-                if (LINEAR) {
-                    const float xq = comp(xv[slot], q);
-                    pf[0] = fmaf(xq, u0, pf[0]); pf[1] = fmaf(xq, u1, pf[1]);
-                    pf[2] = fmaf(xq, u2, pf[2]); pf[3] = fmaf(xq, u3, pf[3]);
-                }
-                store_row(dst0 + (VEC ? ((uint32_t)q ^ sw) << 4 : 512u * q), u0, u1, u2, u3);
-            }
-            if (++b_c == nb) {
-                // ---- the tile is stored: its item table, its counter, then the hand-over ----
-                // (fp32 within the tile: a thread's few indices, then the warp's tree; fp64 across tiles)
-#pragma unroll
-                for (int k = 0; k < GW; ++k) {
-                    float a = nf[k], bq = LINEAR ? pf[k] : 0.f;
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        a += __shfl_xor_sync(0xffffffffu, a, off);
-                        if (LINEAR) bq += __shfl_xor_sync(0xffffffffu, bq, off);
-                    }
-                    if (lane == 0) {
-                        sums[(warp * GW + k) * 2 + 0] += (double)a;
-                        if (LINEAR) sums[(warp * GW + k) * 2 + 1] += (double)bq;
-                    }
-                    nf[k] = 0.f; pf[k] = 0.f;
-                }
-                hand_over(buf);
-            }
-        };
-#pragma unroll
-        for (int s = 0; s < kDepth; ++s) issue(s);
-        if (FIRST && n_tiles > 0) hand_over(0);
-        while (n_c < n_tiles) {
-#pragma unroll
-            for (int s = 0; s < kDepth; ++s) {
-                if (n_c < n_tiles) { consume(s); issue(s); }
-            }
-        }
-    } else {
-        // =============================== walkers ===============================
-        for (int n = 0; n < n_tiles; ++n) {
-            block_barrier<kThreads>();                                   // tile n is stored, tile n - 1 is walked
-            const int buf = (int)(n & 1);
-            // (the record's offset comes from shared memory: a load from L2 here would stand in front of
-            // the first entries of every tile)
-            const unsigned char *rec = p.sched + rec_off[n & 3];
-            const uint32_t *tab = reinterpret_cast<const uint32_t *>(smem_raw + tab_off + (size_t)buf * p.tab_bytes);
-            const int n_items = (int)tab[0];
-            const uint16_t *cells = reinterpret_cast<const uint16_t *>(rec + fda_sched_cells_off(n_items));
-            const unsigned char *ent0 = rec + fda_sched_entries_off(n_items);
-            const uint32_t base = smem_base + ut_off + (uint32_t)buf * ut_bytes;
-            if constexpr (PARTS) {
-                // Short lists (a few steps an item): what an item costs is the way to its entries.  The
-                // next item's cell and entries are asked for before this one is walked.
-                struct Item { int steps; uint32_t cell; const uint2 *ent; uint2 ch[kAhead]; };
-                int it = warp - kProducerWarps;
-                auto fetch = [&](Item &x) {
-                    const uint32_t d0 = tab[4 + 2 * it], chunk0 = tab[5 + 2 * it];
-                    x.steps = (int)(d0 & 0xffffu);
-                    x.cell = cells[(size_t)(d0 >> 16) * kListSlots + lane];
-                    x.ent = reinterpret_cast<const uint2 *>(ent0 + (size_t)chunk0 * 256) + lane;
-#pragma unroll
-                    for (int q = 0; q < kAhead; ++q)
-                        if (4 * q < x.steps) x.ch[q] = __ldg(x.ent + (size_t)q * kListSlots);
-                };
-                auto take = [&]() {
-                    if (lane == 0) it = atomicAdd(&ctr[buf], 1);
-                    it = __shfl_sync(0xffffffffu, it, 0);
-                };
-                auto walk = [&](Item &x) {
-                    unsigned long long a01 = 0ull, a23 = 0ull;
-#pragma unroll
-                    for (int q = 0; q < kAhead; ++q) walk_chunk(x.ch[q], x.steps - 4 * q, base, a01, a23);
-                    for (int c0 = kAhead; 4 * c0 < x.steps; ++c0)
-                        walk_chunk(__ldg(x.ent + (size_t)c0 * kListSlots), x.steps - 4 * c0, base, a01, a23);
-                    flush_item(bins, lm, x.cell, a01, a23);
-                };
-                Item a;
-                if (it < n_items) fetch(a);
-                while (it < n_items) {
-                    Item b = a;
-                    take();
-                    if (it < n_items) fetch(a);
-                    walk(b);
-                }
-            } else {
-            int it = warp - kProducerWarps;
-            uint32_t d0 = 0, chunk0 = 0;
-            if (it < n_items) { d0 = tab[4 + 2 * it]; chunk0 = tab[5 + 2 * it]; }
-            while (it < n_items) {
-                const int steps = (int)(d0 & 0xffffu);
-                const uint32_t cell = cells[(size_t)(d0 >> 16) * kListSlots + lane];
-                const uint2 *ent = reinterpret_cast<const uint2 *>(ent0 + (size_t)chunk0 * 256) + lane;
-                const int nch = (steps + 3) >> 2;
-                if (lane == 0) it = atomicAdd(&ctr[buf], 1);
-                it = __shfl_sync(0xffffffffu, it, 0);
-                if (it < n_items) { d0 = tab[4 + 2 * it]; chunk0 = tab[5 + 2 * it]; }
-                unsigned long long a01 = 0ull, a23 = 0ull;
-                // all entry loads of (up to) kAhead chunks first, then the walk: the entries come
-                // from global memory (L2), one round trip per kAhead chunks instead of one per chunk
-                for (int c0 = 0; c0 < nch; c0 += kAhead) {
-                    uint2 ch[kAhead];
-#pragma unroll
-                    for (int q = 0; q < kAhead; ++q)
-                        if (c0 + q < nch) ch[q] = __ldg(ent + (size_t)(c0 + q) * kListSlots);
-#pragma unroll
-                    for (int q = 0; q + 1 < kAhead; q += 2) walk_chunks2(ch[q], ch[q + 1], steps - 4 * (c0 + q), base, a01, a23);
-                    if (kAhead & 1) walk_chunk(ch[kAhead - 1], steps - 4 * (c0 + kAhead - 1), base, a01, a23);
-                }
-                flush_item(bins, lm, cell, a01, a23);
-            }
-            }
-        }
-    }
-    block_barrier<kThreads>();                                           // the last tile is walked
-
-    // ---- flush: bins -> this block's partial sketch ----
-    {
-        float *out = p.part_sk + (size_t)blockIdx.x * (size_t)lm * GW;
-        for (int t = tid; t < lm * GW; t += kThreads) out[t] = bins[t];
-    }
-    // ---- block partial of (||u||^2, <xi,u>) per worker: the producer warps' sums, in warp order ----
-    if (tid < GW * 2) {
-        double t = 0.0;
-        for (int q = 0; q < (FIRST ? PW + WW : kProducerWarps); ++q) t += sums[q * GW * 2 + tid];
-        p.part_np[(size_t)blockIdx.x * GW * 2 + tid] = t;
-    }
-}
 
 constexpr int kShortWarps = 24;
 constexpr int kShortChunks = 2;                // chunks of 128 indices a warp forms: tiles of up to 6144 indices
@@ -626,12 +284,6 @@ __global__ void __launch_bounds__(256) k_finalize_gather_wide(const ListParams p
     if (e < slen && k < p.K) states[(size_t)k * slen + e] = (float)mine;
 }
 
-template <int PW, int WW, bool PARTS, bool FIRST>
-void (*pick_kernel(bool linear, bool vec))(ListParams)
-{
-    if (linear) return vec ? k_local_state_gather<true, PW, WW, PARTS, true, FIRST> : k_local_state_gather<true, PW, WW, PARTS, false, FIRST>;
-    return vec ? k_local_state_gather<false, PW, WW, PARTS, true, FIRST> : k_local_state_gather<false, PW, WW, PARTS, false, FIRST>;
-}
 void (*pick_short(bool linear, bool vec))(ListParams)
 {
     if (linear) return vec ? k_local_state_short<true, true> : k_local_state_short<true, false>;
@@ -646,8 +298,8 @@ cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent,
     // 5 x 250, K = 20, d = 300,000 (two tiles) 18.3 -> 17.4 us, K = 10, d = 1.2M (four) 34.1 -> 32.4 us; 7 x 500, K = 10,
     // d = 1.2M (five) 46.0 -> 44.5 us; K = 20, d = 2M (twelve) 75.7 -> 75.3 us.
     const bool first = !PARTS && p.tiles <= 12 * (int64_t)p.cpg;
-    auto kern = first ? pick_kernel<PW, WW, PARTS, !PARTS>(p.have_xi != 0, p.vec != 0)
-                      : pick_kernel<PW, WW, PARTS, false>(p.have_xi != 0, p.vec != 0);
+    auto kern = first ? pick_kernel<PW, WW, PARTS, !PARTS, 0>(p.have_xi != 0, p.vec != 0)
+                      : pick_kernel<PW, WW, PARTS, false, 0>(p.have_xi != 0, p.vec != 0);
     if (dependent) return fda_launch_dependent(kern, blocks, (PW + WW) * 32, smem, s, p);
     kern<<<blocks, (PW + WW) * 32, smem, s>>>(p);
     return cudaGetLastError();
@@ -658,11 +310,19 @@ cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent,
 // The kernels' dynamic shared memory limit, set once per context (on the context's device).
 cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx)
 {
+    if (ctx->lane_prog) {
+        ListParams p{};
+        p.lane_items = ctx->lane_items; p.T = ctx->lane_T;
+        for (p.vec = 0; p.vec < 2; ++p.vec) {
+            const cudaError_t e = fda_lanes_run(ctx->lane_walkers, ctx->lane_parts > 1, p, 0, false, nullptr);
+            if (e != cudaSuccess) return e;
+        }
+    }
     for (int i = 0; i < 4; ++i) {
         const bool linear = i & 1, vec = i & 2;
-        for (auto kern : {pick_kernel<8, 20, false, false>(linear, vec), pick_kernel<5, 23, false, false>(linear, vec),
-                          pick_kernel<8, 20, false, true>(linear, vec), pick_kernel<5, 23, false, true>(linear, vec),
-                          pick_kernel<8, 20, true, false>(linear, vec), pick_short(linear, vec)}) {
+        for (auto kern : {pick_kernel<8, 20, false, false, 0>(linear, vec), pick_kernel<5, 23, false, false, 0>(linear, vec),
+                          pick_kernel<8, 20, false, true, 0>(linear, vec), pick_kernel<5, 23, false, true, 0>(linear, vec),
+                          pick_kernel<8, 20, true, false, 0>(linear, vec), pick_short(linear, vec)}) {
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
             if (e != cudaSuccess) return e;
         }
@@ -683,15 +343,19 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     p.w = w; p.w_t0 = w_t0; p.xi = xi_used; p.row_stride = row_stride;
     p.K = K; p.d = d; p.have_xi = xi_used != nullptr;
     p.vec = ((((uintptr_t)w | (uintptr_t)w_t0 | (uintptr_t)(xi_used ? xi_used : w)) & 15u) == 0) && (row_stride % 4 == 0);
-    p.l = ctx->l / ctx->sched_parts; p.m = ctx->m;
-    p.part_tiles = (int)ctx->sched_tiles;
-    p.T = ctx->sched_T;
-    p.sched = ctx->sched; p.sched_off = ctx->sched_off;
+    const int wgroups = (K + GW - 1) / GW;
+    const bool lanes = ctx->lane_prog && !xi_used && fda_lanes_pay((d + ctx->lane_T - 1) / ctx->lane_T, wgroups * ctx->lane_parts, ctx->n_sm);
+    const int sched_parts = lanes ? ctx->lane_parts : ctx->sched_parts;
+    p.l = ctx->l / sched_parts; p.m = ctx->m;
+    p.part_tiles = (int)(lanes ? ctx->lane_tiles : ctx->sched_tiles);
+    p.T = lanes ? ctx->lane_T : ctx->sched_T;
+    p.sched = lanes ? ctx->lane_sched : ctx->sched; p.sched_off = lanes ? ctx->lane_off : ctx->sched_off;
+    if (lanes) { p.lane_prog = ctx->lane_prog; p.lane_rows = ctx->lane_rows; p.lane_items = ctx->lane_items; }
     p.part_sk = ctx->part_sk; p.part_np = ctx->part_np;
     p.tiles = (d + p.T - 1) / p.T;
     p.tab_bytes = fda_list_table_bytes(ctx->sched_ni_max);
-    p.wgroups = (K + GW - 1) / GW;
-    p.groups = p.wgroups * ctx->sched_parts;
+    p.wgroups = wgroups;
+    p.groups = wgroups * sched_parts;
     if (p.groups > ctx->n_sm) return cudaErrorNotSupported;
     int64_t cpg = ctx->n_sm / p.groups;
     if (cpg > p.tiles) cpg = p.tiles;
@@ -701,7 +365,7 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         (size_t)blocks * GW * 2 > ctx->part_np_doubles)
         return cudaErrorNotSupported;
     const size_t smem = fda_list_smem_bytes(p.l, p.m, p.T, ctx->sched_ni_max);
-    if (smem > (size_t)ctx->smem_optin) return cudaErrorNotSupported;
+    if (!lanes && smem > (size_t)ctx->smem_optin) return cudaErrorNotSupported;
 
     // A vector with at most one tile per block runs on k_local_state_short, whose tiles hold up to 6144 indices:
     // several blocks share a tile while the SMs last, and sketches of up to six rows stay with it when they do not.
@@ -712,8 +376,8 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     // blocks to share the tiles: 7 x 500, K = 10, d = 123K 13.4 and 14.8, 16 x 100, d = 147K 17.5 and 20.7.
     int split = 1;
     bool one_tile = false;
-    if (ctx->sched_parts == 1) {
-        if (p.tiles == p.cpg && p.T <= kShortWarps * 128 * kShortChunks) {
+    if (sched_parts == 1) {
+        if (!lanes && p.tiles == p.cpg && p.T <= kShortWarps * 128 * kShortChunks) {
             split = std::min(3, ctx->n_sm / blocks);
             one_tile = split > 1 || p.l <= 6;
         }
@@ -730,7 +394,8 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     // 8 + 20, 216 with 10 + 18, 231 with 6 + 22, 226 with 8 + 24 (64 registers).
     const bool walking = p.l >= 8 || (int64_t)p.l * (p.T + 10 * p.m) >= 10 * (int64_t)p.T;
     auto launch = [&](ListParams &q, int grid, cudaStream_t st, bool dependent) {
-        if (ctx->sched_parts > 1) return launch_lists<8, 20, true>(q, grid, smem, dependent, st);
+        if (lanes) return fda_lanes_run(ctx->lane_walkers, sched_parts > 1, q, grid, dependent, st);
+        if (sched_parts > 1) return launch_lists<8, 20, true>(q, grid, smem, dependent, st);
         if (one_tile)
             return fda_launch_dependent(pick_short(q.have_xi != 0, q.vec != 0), grid, kShortWarps * 32,
                                         short_smem_bytes(q.l * q.m, q.T), st, q);
@@ -751,7 +416,7 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     const int rest = p.groups - extra;                         // groups of the second tail launch (extra < groups)
     int64_t t1 = p.tiles;
     int cpg_b = 0;
-    if (ctx->sched_parts == 1 && extra > 0 && rest > 0 && extra / rest >= 1 && ctx->side_stream && p.tiles >= 64 * (int64_t)p.cpg) {
+    if (sched_parts == 1 && extra > 0 && rest > 0 && extra / rest >= 1 && ctx->side_stream && p.tiles >= (lanes ? 48 : 64) * (int64_t)p.cpg) {
         cpg_b = extra / rest;
         // tail walks per block: n_tail + n_tail / cpg_b; main walks per block: (tiles - n_tail) / cpg
         const double per_tail = 1.0 + 1.0 / (double)cpg_b;
@@ -769,6 +434,7 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
         ListParams ta = p;
         ta.w = p.w + shift; ta.w_t0 = p.w_t0 + shift; ta.xi = p.xi ? p.xi + shift : nullptr;
         ta.d = p.d - shift; ta.tiles = p.tiles - t1; ta.sched_off = p.sched_off + t1;
+        if (p.lane_prog) ta.lane_prog = p.lane_prog + (size_t)t1 * (p.lane_items + 1);
         ListParams tb = ta;
         ta.K = extra * GW; ta.groups = ta.wgroups = extra; ta.cpg = 1;
         ta.part_sk = p.part_sk + (size_t)blocks * lm * GW; ta.part_np = p.part_np + (size_t)blocks * GW * 2;
@@ -796,11 +462,11 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     // kernel and finalize back to back, one and four per lane: 5 x 250, K = 10, d = 1.2M (60K threads) 30.0 and 34.3 us;
     // 5 x 250, K = 30, d = 2M (160K) 110.6 both; 7 x 500, K = 60, d = 1.2M (841K) 191.0 and 184.7 us; 8 x 1000,
     // K = 30, d = 300,000 (1.02M) 55.7 and 48.0 us.
-    const int64_t lanes = (int64_t)(2 + ctx->lm) * 4;
-    const bool wide = lanes * GW * p.wgroups > (int64_t)ctx->n_sm * 2048;
+    const int64_t sums = (int64_t)(2 + ctx->lm) * 4;
+    const bool wide = sums * GW * p.wgroups > (int64_t)ctx->n_sm * 2048;
     auto fin = wide ? (nb <= 16 ? k_finalize_gather_wide<4> : nb <= 32 ? k_finalize_gather_wide<8> : k_finalize_gather_wide<12>)
                     : (nb <= 16 ? k_finalize_gather<4> : nb <= 32 ? k_finalize_gather<8> : k_finalize_gather<12>);
-    const dim3 fb((unsigned)((lanes * (wide ? 1 : GW) + 255) / 256), (unsigned)p.wgroups);
+    const dim3 fb((unsigned)((sums * (wide ? 1 : GW) + 255) / 256), (unsigned)p.wgroups);
     if (parts.n == 1) return fda_launch_dependent(fin, fb, 256, 0, s, p, parts, flags, states);
     fin<<<fb, 256, 0, s>>>(p, parts, flags, states);       // waits for an event too: an ordinary launch
     return cudaGetLastError();

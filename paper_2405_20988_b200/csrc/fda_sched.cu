@@ -56,6 +56,9 @@ struct SchedParams {
     int ni_row_max;        // items of a (tile, row)
     uint32_t *rec_items;   // [tile]  written by the counting pass, read by the writing pass
     uint32_t *rec_chunks;  // [tile]
+    uint32_t *rec_steps;   // [tile] steps of all items; all bits set: a cell has more than one list (counting pass)
+    const int2 *lane_rows; // order of the cells of every sketch row (of all parts), or null
+    uint32_t *lane_prog;   // see fda_ctx (writing pass)
     const uint64_t *rec_off;   // [tile + 1] byte offsets of the records (writing pass)
     unsigned char *sched;
 };
@@ -140,7 +143,7 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
         cells_off = fda_sched_cells_off(rec_ni);
         ent_off = fda_sched_entries_off(rec_ni);
     }
-    if (tid == 0) { tot[0] = 0; tot[1] = 0; }
+    if (tid == 0) { tot[0] = 0; tot[1] = 0; tot[4] = 0; }
     __syncthreads();
 
     for (int i = 0; i < p.l; ++i) {
@@ -250,8 +253,30 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
         // to the longest of the next kWindow lists that keeps all residue classes within the
         // opener's length (ties: a cell whose bank group the octet's flush does not use yet,
         // then the flattest classes); if none fits, to the one that raises the classes least ----
-        const int no = (nl + NRES - 1) / NRES;
-        if (tid < 32) {
+        const int no = p.lane_rows ? (m + NRES - 1) / NRES : (nl + NRES - 1) / NRES;
+        if (p.lane_rows) {
+            // the octets of the cells' fixed order: 32 neighbours of it are an item in every tile
+            const int2 ord = p.lane_rows[(size_t)(blockIdx.x / p.tiles) * p.l + i];
+            for (int o = tid; o < no; o += kBT) {
+                int cols[NRES], cost = 1;
+#pragma unroll
+                for (int r = 0; r < NRES; ++r) cols[r] = 0;
+                for (int q = 0; q < NRES; ++q) {
+                    const int pos = NRES * o + q, cell = pos < m ? fda_lane_cell(pos, ord.x, ord.y, m) : 0;
+                    const bool on = pos < m && cnt[cell] > 0;
+                    const int li = on ? lfirst[cell] : 0xffff;
+                    oc_list[NRES * o + q] = (uint16_t)li;
+                    if (!on) continue;
+                    if (npiece[cell] > 1) tot[4] = 1;
+                    cost = max(cost, (int)ls_len[li]);
+#pragma unroll
+                    for (int r = 0; r < NRES; ++r) cols[r] += ls_res[8 * li + r];
+                }
+#pragma unroll
+                for (int r = 0; r < NRES; ++r) cost = max(cost, cols[r]);
+                oc_cost[o] = (uint16_t)cost;
+            }
+        } else if (tid < 32) {
             // order[head ..) are the lists not yet placed, longest first: a list taken from the
             // window is removed by moving the ones before it up by one, so the order is kept
             int head = 0;
@@ -330,9 +355,9 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
         __syncthreads();
         // ---- octets by steps (most first, ties by number); four of them make an item ----
         for (int o = tid; o < no; o += kBT) {
-            int rank = 0;
+            int rank = p.lane_rows ? o : 0;
             const int co = oc_cost[o];
-            for (int q = 0; q < no; ++q) rank += (oc_cost[q] > co || (oc_cost[q] == co && q < o)) ? 1 : 0;
+            for (int q = 0; q < no && !p.lane_rows; ++q) rank += (oc_cost[q] > co || (oc_cost[q] == co && q < o)) ? 1 : 0;
             oc_order[rank] = (uint16_t)o;
         }
         __syncthreads();
@@ -342,7 +367,8 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
         if (tid == 0) {
             int a = chunk0;
             for (int q = 0; q < ni_row; ++q) {
-                const int steps = oc_cost[oc_order[4 * q]];
+                int steps = oc_cost[oc_order[4 * q]];
+                for (int x = 4 * q + 1; p.lane_rows && x < min(no, 4 * q + 4); ++x) steps = max(steps, (int)oc_cost[x]);
                 it_steps[item0 + q] = (uint32_t)steps;
                 it_chunk[item0 + q] = (uint32_t)a;
                 a += (steps + 3) / 4;
@@ -500,7 +526,13 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
     }
     __syncthreads();
     if (!WRITE) {
-        if (tid == 0) { p.rec_items[rec_no] = (uint32_t)ni; p.rec_chunks[rec_no] = (uint32_t)nch; }
+        if (tid == 0) {
+            uint32_t steps = 0;
+            for (int q = 0; q < ni; ++q) steps += it_steps[q];
+            p.rec_items[rec_no] = (uint32_t)ni;
+            p.rec_chunks[rec_no] = (uint32_t)nch;
+            p.rec_steps[rec_no] = tot[4] ? 0xffffffffu : steps;
+        }
     } else {
         uint32_t *hdr = reinterpret_cast<uint32_t *>(rec);
         if (tid == 0) {
@@ -513,8 +545,93 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
             uint32_t *dsc = hdr + 4 + 2 * it_rank[q];
             dsc[0] = (it_steps[q] & 0xffffu) | ((uint32_t)q << 16);
             dsc[1] = it_chunk[q];
+            // (in the program the items that fill a warp come first)
+            const int per_row = (m + kListSlots - 1) / kListSlots, full = m / kListSlots, of_row = q % per_row;
+            const int at = of_row < full ? q / per_row * full + of_row : p.l * full + q / per_row;
+            if (p.lane_prog) p.lane_prog[(size_t)rec_no * (ni + 1) + 1 + at] = it_chunk[q] << kLaneStepBits | it_steps[q];
         }
+        if (p.lane_prog && tid == 0) p.lane_prog[(size_t)rec_no * (ni + 1)] = (uint32_t)((p.rec_off[rec_no] + ent_off) / 256);
     }
+}
+
+// Score of an order of a sketch row's cells for lanes that keep their cells: steps of its items over
+// kSamples tiles.  Block (shift, row) looks at the order in which index j + e lies in the cell after that of
+// j, for e = 2 * shift + 1, unless the bucket hash wraps around p between the two: bucket(j + e) - bucket(j) is
+// r mod m, r = a * e mod p, except for a share |r| / p of all j.  The lists of eight neighbours of that
+// order are then copies of one another, shifted by e, 2e, ..: as long as one another, and - e being odd - spread
+// over the residue classes.  Scores of cells that need several lists: all bits set.
+constexpr int kShifts = 256, kSamples = 3;
+
+__device__ int2 cell_order(uint64_t a, uint32_t e, int m)
+{
+    uint64_t r = fda::mul_add_mod_p(a, e, 0);
+    int step = (int)(r % (uint64_t)m);
+    if (r > fda::kP61 / 2) {                       // r - p is the nearer one
+        step = (int)((fda::kP61 - r) % (uint64_t)m);
+        step = step ? m - step : 0;
+    }
+    int x = m, y = step;
+    while (y) { const int t = x % y; x = y; y = t; }
+    return make_int2(step, m / x);
+}
+
+__global__ void __launch_bounds__(kBT) k_score_orders(const uint64_t *coeffs, int m, uint64_t magic, int T, uint32_t tiles, uint32_t *score)
+{
+    extern __shared__ int cls8[];                  // [m][8] indices of a cell by residue class
+    __shared__ uint32_t sum[kBT / 32];
+    const uint64_t *c = coeffs + 6 * blockIdx.y;
+    const uint32_t e = 2 * blockIdx.x + 1;
+    const int tid = threadIdx.x;
+    const int2 ord = cell_order(c[0], e, m);
+    const bool same = ord.x == 0 && m > 1;         // j and j + e share a cell: no order
+    uint32_t steps = 0, bad = same;
+    for (int smp = 0; smp < kSamples && !same; ++smp) {
+        const uint32_t tile = (uint32_t)((uint64_t)(tiles - 1) * smp / (kSamples - 1));
+        for (int t = tid; t < 8 * m; t += kBT) cls8[t] = 0;
+        __syncthreads();
+        for (int r = tid; r < T; r += kBT)
+            atomicAdd(&cls8[8 * fda::bucket_of(c, tile * (uint32_t)T + r, (uint32_t)m, magic) + (fda_list_row(r) & 7)], 1);
+        __syncthreads();
+        for (int q = tid; q < (m + 31) / 32; q += kBT) {
+            int most = 1;
+            for (int o = 0; o < 4; ++o) {
+                int cols[8] = {};
+                for (int x = 0; x < 8; ++x) {
+                    const int pos = 32 * q + 8 * o + x;
+                    if (pos >= m) break;
+                    const int *v = cls8 + 8 * fda_lane_cell(pos, ord.x, ord.y, m);
+                    int len = 0;
+                    for (int k = 0; k < 8; ++k) { len += v[k]; cols[k] += v[k]; }
+                    most = max(most, len);
+                    if (len > ML) bad = 1;
+                }
+                for (int k = 0; k < 8; ++k) most = max(most, cols[k]);
+            }
+            steps += most;
+        }
+        __syncthreads();
+    }
+    steps = __reduce_add_sync(0xffffffffu, steps);
+    bad = __any_sync(0xffffffffu, bad);
+    if ((tid & 31) == 0) sum[tid / 32] = bad ? 0xffffffffu : steps;
+    __syncthreads();
+    if (tid == 0) {
+        uint32_t t = 0;
+        for (int w = 0; w < kBT / 32; ++w) t = sum[w] == 0xffffffffu || t == 0xffffffffu ? 0xffffffffu : t + sum[w];
+        score[blockIdx.y * kShifts + blockIdx.x] = t;
+    }
+}
+
+// the best order of every row (a warp each)
+__global__ void k_pick_orders(const uint64_t *coeffs, int m, const uint32_t *score, int2 *rows)
+{
+    const int row = blockIdx.x, lane = threadIdx.x;
+    uint32_t best = 0xffffffffu, at = 0;
+    for (int i = lane; i < kShifts; i += 32)
+        if (score[row * kShifts + i] < best) { best = score[row * kShifts + i]; at = i; }
+    const uint32_t least = __reduce_min_sync(0xffffffffu, best);
+    at = __reduce_min_sync(0xffffffffu, best == least ? at : 0xffffu);
+    if (lane == 0) rows[row] = least == 0xffffffffu ? make_int2(1, m) : cell_order(coeffs[6 * row], 2 * at + 1, m);
 }
 
 }  // namespace
@@ -537,6 +654,48 @@ static int list_tile_indices(const fda_ctx *ctx, int rows, int min_len, int *ni_
     return 0;
 }
 
+// Walker warps for `items` items: as many as leave the fewest lanes without a cell, and of those that leave
+// equally many the fewest (every other warp produces).  Measured, K = 8, d = 20M, us with 12 / 20 / 22 / 23 / 24 walkers:
+// 24 items 184 / 196 / 193 / 205 / 211; 40: 303 / 214 / 215 / 226 / 234; 48: 320 / 283 / 289 / 287 / 252; 56: 385 / 286 / 297 /
+// 298 / 312; 64: 484 / 382 / 314 / 317 / 332; 80: 324 / 253 / 244 / 242 / 256; 112: - / 353 / 355 / 314 / 330.
+static int lane_walkers(int items)
+{
+    if (items <= 24) return 12;
+    if (items <= 32) return 16;
+    int best = 0;
+    for (int w : {20, 23, 24})
+        if ((items + w - 1) / w <= 7 && (best == 0 || (items + w - 1) / w * w < (items + best - 1) / best * best)) best = w;
+    return best;
+}
+
+// Geometry of the schedule when cells stay with their lanes: there are no bins, so the tile depends on the lists only.
+// Six batches of 1024 indices, fewer where lists would come near their limit, seven where they would be
+// shorter than ten entries (5 x 250, K = 8, d = 198M: 1860 us with six, 1907 with seven, 1991 with five; 8 x 1000,
+// K = 20, d = 2.6M: 165 with seven, 189 with six).  The sketch rows go in one part unless their items would
+// be more than a block's lanes can keep.
+static int lane_geometry(const fda_ctx *ctx, int *parts_out, int *ni_max_out)
+{
+    const int m = ctx->m;
+    int T = 6 * kListBatch;
+    if (T < 10 * m) T += kListBatch;
+    while (T > 56 * m && T > 2 * kListBatch) T -= kListBatch;
+    if (T < 5 * m || T > 56 * m) return 0;
+    // where a quarter of the lanes would have no cell and the walk is most of the work, the list kernel is as fast
+    // (8 x 100: 380 us, 390 here; 3 x 100: 216 and 193)
+    if (m < 128 && ctx->l >= 6 && (m + kListSlots - 1) / kListSlots * kListSlots * 5 > 6 * m) return 0;
+    for (int parts = 1; parts <= 4; parts *= 2) {
+        if (ctx->l % parts) break;
+        const int rows = ctx->l / parts, items = rows * ((m + kListSlots - 1) / kListSlots);
+        if (items > kLaneMaxItems || rows * m + 1 >= 0x8000) continue;
+        const int groups = (ctx->K_max + kListWorkers - 1) / kListWorkers * parts;
+        if (!fda_lanes_pay((ctx->d_max + T - 1) / T, groups, ctx->n_sm)) return 0;
+        *parts_out = parts;
+        *ni_max_out = items;
+        return T;
+    }
+    return 0;
+}
+
 // Geometry of the schedule: all rows in one part where lists of six entries fit, else two or four
 // equal parts of the rows, each with bins, records and blocks of its own, from five entries on: a part
 // forms the drifts again (its loads hit L2), but the bins it does not hold make room for lists twice as
@@ -552,10 +711,12 @@ static int list_geometry(const fda_ctx *ctx, int *parts_out, int *ni_max_out)
     return 0;
 }
 
-cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s)
+// Builds one of the two schedules; none is built (and cudaSuccess returned) for a sketch, a hash, a size or a
+// memory limit that it does not suit.
+static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
 {
     int ni_max = 0, parts = 1;
-    const int T = list_geometry(ctx, &parts, &ni_max);
+    const int T = lanes ? lane_geometry(ctx, &parts, &ni_max) : list_geometry(ctx, &parts, &ni_max);
     if (T == 0) return cudaSuccess;
     const int64_t part_tiles = (ctx->d_max + T - 1) / T, tiles = part_tiles * parts;      // records
     if (tiles > 0x7fffffffLL) return cudaSuccess;
@@ -573,25 +734,45 @@ cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s)
         e = cudaFuncSetAttribute(k_build_schedule<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem);
     if (e != cudaSuccess) return e;
 
-    uint32_t *items = nullptr, *chunks = nullptr;
+    uint32_t *items = nullptr, *chunks = nullptr, *steps = nullptr, *score = nullptr;
+    int2 *rows = nullptr;
+    uint32_t *prog = nullptr;
     uint64_t *off = nullptr;
     unsigned char *buf = nullptr;
-    auto cleanup = [&]() { cudaFree(items); cudaFree(chunks); cudaFree(off); cudaFree(buf); };
-    if (cudaMalloc(&items, sizeof(uint32_t) * tiles) != cudaSuccess ||
-        cudaMalloc(&chunks, sizeof(uint32_t) * tiles) != cudaSuccess ||
+    auto cleanup = [&]() { cudaFree(items); cudaFree(rows); cudaFree(prog); cudaFree(off); cudaFree(buf); };
+    if (cudaMalloc(&items, sizeof(uint32_t) * (3 * tiles + (size_t)ctx->l * kShifts)) != cudaSuccess ||
+        cudaMalloc(&rows, sizeof(int2) * ctx->l) != cudaSuccess ||
         cudaMalloc(&off, sizeof(uint64_t) * (tiles + 1)) != cudaSuccess) {
         cudaGetLastError();
         cleanup();
         return cudaSuccess;
     }
-    p.rec_items = items; p.rec_chunks = chunks;
-    k_build_schedule<false><<<(unsigned)tiles, kBT, bsmem, s>>>(p);
-    e = cudaGetLastError();
-    std::vector<uint32_t> h_items((size_t)tiles), h_chunks((size_t)tiles);
+    chunks = items + tiles; steps = chunks + tiles; score = steps + tiles;
+    p.rec_items = items; p.rec_chunks = chunks; p.rec_steps = steps;
+    std::vector<uint32_t> h_count(3 * (size_t)tiles);
+    const uint32_t *h_items = h_count.data(), *h_chunks = h_items + tiles, *h_steps = h_chunks + tiles;
     std::vector<uint64_t> h_off((size_t)tiles + 1);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_items.data(), items, sizeof(uint32_t) * tiles, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h_chunks.data(), chunks, sizeof(uint32_t) * tiles, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    auto count = [&]() {
+        k_build_schedule<false><<<(unsigned)tiles, kBT, bsmem, s>>>(p);
+        cudaError_t r = cudaGetLastError();
+        if (r == cudaSuccess) r = cudaMemcpyAsync(h_count.data(), items, sizeof(uint32_t) * 3 * tiles, cudaMemcpyDeviceToHost, s);
+        return r == cudaSuccess ? cudaStreamSynchronize(s) : r;
+    };
+    if (lanes) {
+        const size_t score_smem = sizeof(int) * 8 * (size_t)ctx->m;
+        if (score_smem > 48 * 1024) { cleanup(); return cudaSuccess; }
+        k_score_orders<<<dim3(kShifts, (unsigned)ctx->l), kBT, score_smem, s>>>(ctx->coeffs_dev, ctx->m, p.magic, T, p.tiles, score);
+        k_pick_orders<<<(unsigned)ctx->l, 32, 0, s>>>(ctx->coeffs_dev, ctx->m, score, rows);
+        p.lane_rows = rows;
+    }
+    e = count();
+    if (e == cudaSuccess && lanes) {
+        uint64_t total_steps = 0;
+        bool fits = true;
+        for (int64_t t = 0; t < tiles; ++t) { fits = fits && h_steps[t] != 0xffffffffu; total_steps += h_steps[t]; }
+        // (even hashes need 1.1 to 1.35 steps per entry, one uneven row of five or seven puts the sum far above 1.6)
+        if (!fits || total_steps * kListSlots * 10 > (uint64_t)16 * tiles * p.l * T) { cleanup(); return cudaSuccess; }
+    }
     if (e != cudaSuccess) { cleanup(); return e; }
     uint64_t total = 0;
     for (int64_t t = 0; t < tiles; ++t) {
@@ -600,24 +781,39 @@ cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s)
         total += fda_sched_entries_off(h_items[t]) + (uint64_t)h_chunks[t] * 256;
     }
     h_off[tiles] = total;
+    const int lane_items = p.l * ((ctx->m + kListSlots - 1) / kListSlots);
+    const uint64_t prog_bytes = lanes ? sizeof(uint32_t) * (uint64_t)(lane_items + 1) * tiles : 0;
+    const uint64_t all_bytes = total + prog_bytes + ctx->sched_bytes;         // (of both schedules, when this is the second)
     size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || total > free_b / 3 ||
-        (ctx->sched_limit_bytes > 0 && total > (uint64_t)ctx->sched_limit_bytes)) {
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || total + prog_bytes > free_b / 3 ||
+        (ctx->sched_limit_bytes > 0 && all_bytes > (uint64_t)ctx->sched_limit_bytes) ||
+        cudaMalloc(&buf, total) != cudaSuccess || (lanes && cudaMalloc(&prog, prog_bytes) != cudaSuccess)) {
         cudaGetLastError();
         cleanup();
-        ctx->sched_skipped_bytes = total;
+        if (!lanes) ctx->sched_skipped_bytes = total;
         return cudaSuccess;                                                   // leave the memory to the models
     }
-    if (cudaMalloc(&buf, total) != cudaSuccess) { cudaGetLastError(); cleanup(); ctx->sched_skipped_bytes = total; return cudaSuccess; }
     e = cudaMemcpyAsync(off, h_off.data(), sizeof(uint64_t) * (tiles + 1), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) { cleanup(); return e; }
     p.rec_off = off; p.sched = buf;
+    p.lane_prog = prog;
     k_build_schedule<true><<<(unsigned)tiles, kBT, bsmem, s>>>(p);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(items); cudaFree(chunks);
-    if (e != cudaSuccess) { cudaFree(off); cudaFree(buf); return e; }
+    if (e != cudaSuccess) { cleanup(); return e; }
+    cudaFree(items);
+    if (lanes) {
+        ctx->lane_sched = buf; ctx->lane_off = off; ctx->lane_prog = prog; ctx->lane_rows = rows;
+        ctx->lane_bytes = total + prog_bytes + sizeof(uint64_t) * (tiles + 1) + sizeof(int2) * ctx->l;
+        ctx->lane_T = T; ctx->lane_parts = parts; ctx->lane_tiles = part_tiles;
+        ctx->lane_items = lane_items; ctx->lane_walkers = lane_walkers(lane_items);
+        return cudaSuccess;
+    }
+    cudaFree(rows);
     ctx->sched = buf; ctx->sched_off = off; ctx->sched_bytes = total; ctx->sched_T = T;
     ctx->sched_ni_max = ni_max; ctx->sched_tiles = part_tiles; ctx->sched_parts = parts;
     return cudaSuccess;
 }
+
+cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s) { return build_schedule(ctx, false, s); }
+cudaError_t fda_build_lane_schedule(fda_ctx *ctx, cudaStream_t s) { return build_schedule(ctx, true, s); }
