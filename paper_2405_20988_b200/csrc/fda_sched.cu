@@ -56,7 +56,7 @@ struct SchedParams {
     int ni_row_max;        // items of a (tile, row)
     uint32_t *rec_items;   // [tile]  written by the counting pass, read by the writing pass
     uint32_t *rec_chunks;  // [tile]
-    uint32_t *rec_steps;   // [tile] steps of all items; all bits set: a cell has more than one list (counting pass)
+    uint32_t *rec_steps;   // [tile] steps of all items; all bits set: a cell has more than one list (k_count_lanes)
     const int2 *lane_rows; // order of the cells of every sketch row (of all parts), or null
     uint32_t *lane_prog;   // see fda_ctx (writing pass)
     const uint64_t *rec_off;   // [tile + 1] byte offsets of the records (writing pass)
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
         cells_off = fda_sched_cells_off(rec_ni);
         ent_off = fda_sched_entries_off(rec_ni);
     }
-    if (tid == 0) { tot[0] = 0; tot[1] = 0; tot[4] = 0; }
+    if (tid == 0) { tot[0] = 0; tot[1] = 0; }
     __syncthreads();
 
     for (int i = 0; i < p.l; ++i) {
@@ -237,12 +237,12 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
         }
         __syncthreads();
         // ---- lists by length, longest first, ties by list number ----
-        if (tid == 0) {
+        if (tid == 0 && !p.lane_rows) {
             int a = 0;
             for (int len = ML; len >= 1; --len) { const int v = cls[len]; cls[len] = a; a += v; }
         }
         __syncthreads();
-        if (tid >= 1 && tid <= ML) {
+        if (tid >= 1 && tid <= ML && !p.lane_rows) {
             int r = cls[tid];
             for (int it = 0; it < nl; ++it)
                 if (ls_len[it] == tid) order[r++] = (uint16_t)it;
@@ -267,7 +267,6 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
                     const int li = on ? lfirst[cell] : 0xffff;
                     oc_list[NRES * o + q] = (uint16_t)li;
                     if (!on) continue;
-                    if (npiece[cell] > 1) tot[4] = 1;
                     cost = max(cost, (int)ls_len[li]);
 #pragma unroll
                     for (int r = 0; r < NRES; ++r) cols[r] += ls_res[8 * li + r];
@@ -527,11 +526,8 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
     __syncthreads();
     if (!WRITE) {
         if (tid == 0) {
-            uint32_t steps = 0;
-            for (int q = 0; q < ni; ++q) steps += it_steps[q];
             p.rec_items[rec_no] = (uint32_t)ni;
             p.rec_chunks[rec_no] = (uint32_t)nch;
-            p.rec_steps[rec_no] = tot[4] ? 0xffffffffu : steps;
         }
     } else {
         uint32_t *hdr = reinterpret_cast<uint32_t *>(rec);
@@ -552,6 +548,39 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
         }
         if (p.lane_prog && tid == 0) p.lane_prog[(size_t)rec_no * (ni + 1)] = (uint32_t)((p.rec_off[rec_no] + ent_off) / 256);
     }
+}
+
+// Steps and entry chunks of the items of one tile and sketch row when the row's cells keep the order `ord`: the sums
+// over the items that this thread looks at.  cls8: m * 8 words of shared memory.  `bad` is set when a cell
+// has more than one list.  (k_build_schedule comes to the same numbers by sorting; only counting is done here.)
+__device__ void count_lane_items(const uint64_t *c, int2 ord, int m, uint64_t magic, int T, uint32_t tile, int *cls8,
+                                 uint32_t &steps, uint32_t &chunks, uint32_t &bad)
+{
+    const int tid = threadIdx.x;
+    for (int t = tid; t < 8 * m; t += kBT) cls8[t] = 0;
+    __syncthreads();
+    for (int r = tid; r < T; r += kBT)
+        atomicAdd(&cls8[8 * fda::bucket_of(c, tile * (uint32_t)T + r, (uint32_t)m, magic) + (fda_list_row(r) & 7)], 1);
+    __syncthreads();
+    for (int q = tid; q < (m + 31) / 32; q += kBT) {
+        int most = 1;
+        for (int o = 0; o < 4; ++o) {
+            int cols[8] = {};
+            for (int x = 0; x < 8; ++x) {
+                const int pos = 32 * q + 8 * o + x;
+                if (pos >= m) break;
+                const int *v = cls8 + 8 * fda_lane_cell(pos, ord.x, ord.y, m);
+                int len = 0;
+                for (int k = 0; k < 8; ++k) { len += v[k]; cols[k] += v[k]; }
+                most = max(most, len);
+                if (len > ML) bad = 1;
+            }
+            for (int k = 0; k < 8; ++k) most = max(most, cols[k]);
+        }
+        steps += most;
+        chunks += (most + 3) / 4;
+    }
+    __syncthreads();
 }
 
 // Score of an order of a sketch row's cells for lanes that keep their cells: steps of its items over
@@ -584,33 +613,9 @@ __global__ void __launch_bounds__(kBT) k_score_orders(const uint64_t *coeffs, in
     const int tid = threadIdx.x;
     const int2 ord = cell_order(c[0], e, m);
     const bool same = ord.x == 0 && m > 1;         // j and j + e share a cell: no order
-    uint32_t steps = 0, bad = same;
-    for (int smp = 0; smp < kSamples && !same; ++smp) {
-        const uint32_t tile = (uint32_t)((uint64_t)(tiles - 1) * smp / (kSamples - 1));
-        for (int t = tid; t < 8 * m; t += kBT) cls8[t] = 0;
-        __syncthreads();
-        for (int r = tid; r < T; r += kBT)
-            atomicAdd(&cls8[8 * fda::bucket_of(c, tile * (uint32_t)T + r, (uint32_t)m, magic) + (fda_list_row(r) & 7)], 1);
-        __syncthreads();
-        for (int q = tid; q < (m + 31) / 32; q += kBT) {
-            int most = 1;
-            for (int o = 0; o < 4; ++o) {
-                int cols[8] = {};
-                for (int x = 0; x < 8; ++x) {
-                    const int pos = 32 * q + 8 * o + x;
-                    if (pos >= m) break;
-                    const int *v = cls8 + 8 * fda_lane_cell(pos, ord.x, ord.y, m);
-                    int len = 0;
-                    for (int k = 0; k < 8; ++k) { len += v[k]; cols[k] += v[k]; }
-                    most = max(most, len);
-                    if (len > ML) bad = 1;
-                }
-                for (int k = 0; k < 8; ++k) most = max(most, cols[k]);
-            }
-            steps += most;
-        }
-        __syncthreads();
-    }
+    uint32_t steps = 0, chunks = 0, bad = same;
+    for (int smp = 0; smp < kSamples && !same; ++smp)
+        count_lane_items(c, ord, m, magic, T, (uint32_t)((uint64_t)(tiles - 1) * smp / (kSamples - 1)), cls8, steps, chunks, bad);
     steps = __reduce_add_sync(0xffffffffu, steps);
     bad = __any_sync(0xffffffffu, bad);
     if ((tid & 31) == 0) sum[tid / 32] = bad ? 0xffffffffu : steps;
@@ -619,6 +624,28 @@ __global__ void __launch_bounds__(kBT) k_score_orders(const uint64_t *coeffs, in
         uint32_t t = 0;
         for (int w = 0; w < kBT / 32; ++w) t = sum[w] == 0xffffffffu || t == 0xffffffffu ? 0xffffffffu : t + sum[w];
         score[blockIdx.y * kShifts + blockIdx.x] = t;
+    }
+}
+
+// Counting pass of the schedule whose cells stay with their lanes: a block per record.
+__global__ void __launch_bounds__(kBT) k_count_lanes(const SchedParams p)
+{
+    extern __shared__ int cls8[];
+    __shared__ uint32_t sum[3];
+    const uint32_t part = blockIdx.x / p.tiles, tile = blockIdx.x % p.tiles;
+    uint32_t steps = 0, chunks = 0, bad = 0;
+    if (threadIdx.x < 3) sum[threadIdx.x] = 0;
+    for (int i = 0; i < p.l; ++i)
+        count_lane_items(p.coeffs + 6 * (part * p.l + i), p.lane_rows[part * p.l + i], p.m, p.magic, p.T, tile, cls8, steps, chunks, bad);
+    steps = __reduce_add_sync(0xffffffffu, steps);
+    chunks = __reduce_add_sync(0xffffffffu, chunks);
+    bad = __reduce_or_sync(0xffffffffu, bad);
+    if ((threadIdx.x & 31) == 0) { atomicAdd(&sum[0], steps); atomicAdd(&sum[1], chunks); atomicOr(&sum[2], bad); }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        p.rec_items[blockIdx.x] = (uint32_t)(p.l * ((p.m + kListSlots - 1) / kListSlots));
+        p.rec_chunks[blockIdx.x] = sum[1];
+        p.rec_steps[blockIdx.x] = sum[2] ? 0xffffffffu : sum[0];
     }
 }
 
@@ -753,7 +780,8 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
     const uint32_t *h_items = h_count.data(), *h_chunks = h_items + tiles, *h_steps = h_chunks + tiles;
     std::vector<uint64_t> h_off((size_t)tiles + 1);
     auto count = [&]() {
-        k_build_schedule<false><<<(unsigned)tiles, kBT, bsmem, s>>>(p);
+        if (lanes) k_count_lanes<<<(unsigned)tiles, kBT, sizeof(int) * 8 * (size_t)ctx->m, s>>>(p);
+        else k_build_schedule<false><<<(unsigned)tiles, kBT, bsmem, s>>>(p);
         cudaError_t r = cudaGetLastError();
         if (r == cudaSuccess) r = cudaMemcpyAsync(h_count.data(), items, sizeof(uint32_t) * 3 * tiles, cudaMemcpyDeviceToHost, s);
         return r == cudaSuccess ? cudaStreamSynchronize(s) : r;
