@@ -93,6 +93,11 @@ typedef struct {
  *     parts: 5.1), about twice that for vectors of a million indices and less.  It is dropped, and sketch
  *     requests are then served by the slower plain-load kernels, when it would take more than a third of the
  *     free device memory (see fda_create_limited for another cap);
+ *   - a second schedule of about the same size for contexts of long vectors (more than twelve tiles of 5120 to 7168
+ *     indices to a block of the sketch kernel at K_max workers: d_max above 11 million for K_max = 8, 1.4
+ *     million for 30) whose hash spreads the indices of a tile evenly over the cells: it makes fda_local_state
+ *     without a projection a fifth faster and takes half as long to build as the first; it is left out
+ *     when it would take more than a third of the memory that is free then;
  *   - lazily, by the first call that needs them: a 16-bit hash table of 2*l bytes per index
  *     (sketch requests on a context without a schedule), d_max floats (fda_mean_state on
  *     short vectors, many unaligned rows, or without a schedule), K_max*d_max floats of staging
@@ -106,8 +111,9 @@ fda_status fda_create(fda_ctx **out, int device, int l, int m, const uint64_t *h
                       int64_t d_max, int K_max);
 
 /*
- * fda_create with a cap on the list schedule (the paper has no counterpart): the schedule is
- * kept only if it takes at most `schedule_limit_bytes` (and a third of the free device memory);
+ * fda_create with a cap on the list schedules (the paper has no counterpart): the schedule is
+ * kept only if it takes at most `schedule_limit_bytes` (and a third of the free device memory), a second one only
+ * if both together do;
  * 0 means no cap of the caller's (fda_create), a negative value builds no schedule at all.
  * Other arguments and errors as fda_create.
  */
@@ -116,11 +122,11 @@ fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uin
 
 /*
  * What the context holds (the paper has no counterpart).  info (host, 8 values):
- *   [0] device bytes the context owns now   [1] of which: the list schedule (0: none)
+ *   [0] device bytes the context owns now   [1] of which: the list schedules (0: none)
  *   [2] 1 when sketch requests run on the list kernel, 0 when on the plain-load kernels
  *   [3] indices per tile of the schedule    [4] bytes of a schedule that was built and dropped
  *       for lack of memory (0: none)        [5] bytes of the lazily built 16-bit hash table
- *   [6] microseconds fda_create spent on the schedule   [7] other lazily allocated bytes.
+ *   [6] microseconds fda_create spent on the schedules  [7] other lazily allocated bytes.
  * Errors: INVALID_ARG (NULL).
  */
 fda_status fda_context_info(const fda_ctx *ctx, int64_t *info);
