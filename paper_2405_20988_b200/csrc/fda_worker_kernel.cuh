@@ -84,6 +84,12 @@ __device__ __forceinline__ void form_drifts(const ListParams &p, int g, int64_t 
     if ((lane & 7) == 0) { sums[lane >> 2] = (double)a; sums[(lane >> 2) + 1] = (double)b; }
 }
 
+// Chunks of entries (four steps each) that a walker whose lanes keep their cells has on their way: four while the block
+// has few walkers, each with one or two items, two beyond that.  Measured, us with two and four, K = 8, d = 20M: 2 x 250 168 and
+// 140, 3 x 250 181 and 159, 3 x 100 194 and 179, 4 x 250 191 and 183, but with 20 and more walkers 5 x 250, d = 198M 1860
+// and 1894, 7 x 500, K = 60 2022 and 2135, 8 x 1000, K = 20, d = 2.6M 165 and 177 (registers).
+template <int WW>
+constexpr int kLaneAhead = WW <= 16 ? 4 : 2;
 constexpr uint32_t kLaneTiles = 2176;          // offset of the tile buffers when lanes keep their cells: behind the head, on a 128-byte boundary
 inline size_t lane_smem_bytes(int T) { return kLaneTiles + 2 * (size_t)(T + kListPadRows) * GW * 4; }
 
@@ -325,11 +331,13 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
         };
         uint32_t next = load_prog(0);
         const uint2 *rec = nullptr, *ent = nullptr;           // of the entries that are asked for
-        uint2 nx[2];
-        // the next two chunks of an item that has `left` steps left
+        constexpr int G = kLaneAhead<WW>;
+        uint2 nx[G];
+        // the next G chunks of an item that has `left` steps left
         auto ask = [&](int left) {
-            if (left > 0) nx[0] = load_u2(ent);
-            if (left > 4) nx[1] = load_u2(ent + kListSlots);
+#pragma unroll
+            for (int q = 0; q < G; ++q)
+                if (left > 4 * q) nx[q] = load_u2(ent + q * kListSlots);
         };
         auto ask_item = [&](uint32_t word) {
             ent = rec + (size_t)(word >> kLaneStepBits) * kListSlots;
@@ -351,14 +359,17 @@ __global__ void __launch_bounds__((PW + WW) * 32, 1) k_local_state_gather(const 
                 if (i >= mine) break;
                 const uint32_t then = i + 1 < LANES ? __shfl_sync(0xffffffffu, words, i + 1) : 0u;
                 unsigned long long a01 = 0ull, a23 = 0ull;
-                for (int left = (int)(word & ((1u << kLaneStepBits) - 1u)); left > 0; left -= 8) {
-                    const uint2 c0 = nx[0], c1 = nx[1];
-                    if (left > 8) {
-                        ent += 2 * kListSlots;
-                        ask(left - 8);
+                for (int left = (int)(word & ((1u << kLaneStepBits) - 1u)); left > 0; left -= 4 * G) {
+                    uint2 ch[G];
+#pragma unroll
+                    for (int q = 0; q < G; ++q) ch[q] = nx[q];
+                    if (left > 4 * G) {
+                        ent += G * kListSlots;
+                        ask(left - 4 * G);
                     } else if (i + 1 < mine) ask_item(then);
                     else ask_tile();
-                    walk_chunks2(c0, c1, left, base, a01, a23);
+#pragma unroll
+                    for (int q = 0; q < G; q += 2) walk_chunks2(ch[q], ch[q + 1], left - 4 * q, base, a01, a23);
                 }
                 asm("add.rn.f32x2 %0, %0, %1;" : "+l"(s01[i]) : "l"(a01));
                 asm("add.rn.f32x2 %0, %0, %1;" : "+l"(s23[i]) : "l"(a23));
