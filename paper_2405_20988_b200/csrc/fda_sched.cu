@@ -42,8 +42,7 @@ constexpr int kBT = 256;                  // threads of a builder block
 constexpr int ML = kListMaxLen;
 constexpr int NRES = kListOct;            // residue classes = lanes per shared-memory pass
 constexpr int kWindow = 64;               // candidates looked at for every place in an octet
-constexpr int kMatchBytes = 288;          // shared memory of the thread that orders an octet's entries
-constexpr int kSpread = 8;                // every kSpread-th thread of the block orders the entries of an octet
+constexpr int kMatchBytes = 288;          // shared memory of the threads that order an octet's entries
 
 struct SchedParams {
     const uint64_t *coeffs;
@@ -59,6 +58,7 @@ struct SchedParams {
     uint32_t *rec_steps;   // [tile] steps of all items; all bits set: a cell has more than one list (k_count_lanes)
     const int2 *lane_rows; // order of the cells of every sketch row (of all parts), or null
     uint32_t *lane_prog;   // see fda_ctx (writing pass)
+    uint16_t *octets;      // [tile * l + row][9 * no_max] lists and steps of the octets, from the counting pass to the writing pass
     const uint64_t *rec_off;   // [tile + 1] byte offsets of the records (writing pass)
     unsigned char *sched;
 };
@@ -74,10 +74,10 @@ struct Carve {
     }
 };
 
-// 32-bit words of the two arrays of hash words, which the matching tables of a row's octets reuse
+// 16-bit words of the two arrays of hash words, which the matching tables of a row's octets reuse
 __host__ __device__ inline size_t hash_words(int T, int ni_row_max)
 {
-    const size_t tables = (size_t)4 * ni_row_max * kMatchBytes / sizeof(uint32_t);
+    const size_t tables = (size_t)4 * ni_row_max * kMatchBytes / sizeof(uint16_t);
     return tables > 2 * (size_t)T ? tables : 2 * (size_t)T;
 }
 
@@ -87,7 +87,7 @@ size_t build_smem(int l, int m, int T, int nl_max, int no_max, int ni_row_max)
     auto a16 = [](size_t b) { return (b + 15) / 16 * 16; };
     size_t s = 0;
     s += a16(sizeof(int) * m) * 3 + a16(sizeof(int) * (m + 1)) * 2;      // cnt, fill, npiece | start, lfirst
-    s += a16(sizeof(uint32_t) * hash_words(T, ni_row_max));               // key, bycell
+    s += a16(sizeof(uint16_t) * hash_words(T, ni_row_max));               // key, bycell
     s += a16(sizeof(uint16_t) * T);                                       // sorted
     s += a16(sizeof(uint16_t) * nl_max) * 4;                              // ls_start, ls_len, ls_cell, order
     s += a16(8 * (size_t)nl_max);                                         // ls_res
@@ -98,10 +98,55 @@ size_t build_smem(int l, int m, int T, int nl_max, int no_max, int ni_row_max)
     return s + 64;
 }
 
-// One block per tile (and part of the sketch rows).  WRITE = false: count the items and entry chunks of the record;
-// WRITE = true: write the record at its offset.
+// Exclusive sum of v over the threads of the block; `warps` holds a word per warp and may be used again after the
+// next barrier.
+__device__ __forceinline__ int block_scan(int v, int *warps)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+    int sum = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, sum, off);
+        if (lane >= off) sum += o;
+    }
+    if (lane == 31) warps[warp] = sum;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < warp; ++w) before += warps[w];
+    return before + sum - v;
+}
+
+// A list that waits for a place in an octet.  info: list number | length << 16 | (cell mod 8) << 23, all bits set
+// when there is none; r0, r1: its indices per residue class, a byte each.
+struct Cand { uint32_t info, r0, r1; };
+
+// The fullest class of an octet, and the sum of the squares of its classes, when the list comes in
+// (cols: two classes to a word; squares: the sum without it)
+__device__ __forceinline__ int fullest_with(const uint32_t (&cols)[NRES / 2], const Cand &x)
+{
+    const uint32_t a = __vmaxu2(cols[0] + __byte_perm(x.r0, 0, 0x4140), cols[1] + __byte_perm(x.r0, 0, 0x4342));
+    const uint32_t b = __vmaxu2(cols[2] + __byte_perm(x.r1, 0, 0x4140), cols[3] + __byte_perm(x.r1, 0, 0x4342));
+    const uint32_t c = __vmaxu2(a, b);
+    return (int)max(c & 0xffffu, c >> 16);
+}
+__device__ __forceinline__ uint32_t squares_with(const uint32_t (&cols)[NRES / 2], uint32_t squares, const Cand &x)
+{
+    uint32_t cross = __dp2a_lo(cols[0], x.r0, 0u);
+    cross = __dp2a_hi(cols[1], x.r0, cross);
+    cross = __dp2a_lo(cols[2], x.r1, cross);
+    cross = __dp2a_hi(cols[3], x.r1, cross);
+    return __dp4a(x.r1, x.r1, __dp4a(x.r0, x.r0, squares + 2u * cross));
+}
+
+// One block per tile (and part of the sketch rows).  WRITE = false: count the items and entry chunks of the record and
+// leave the octets for the writing pass; WRITE = true: write the record at its offset.
+// Bound: latency (serial chains per octet and per warp), so what counts is how many blocks an SM holds and how many
+// threads a chain is shared by: 64 registers and 16-bit hash words for four blocks instead of two, the octets chosen once
+// instead of by both passes, eight threads to the matching of an octet instead of one.  fda_create, both
+// schedules where there are two: 5 x 250, d = 198M 310 -> 165 ms, d = 7M, K = 30 12.7 -> 8.0; 7 x 500, d = 20M, K = 60 74 -> 36;
+// 8 x 1000, d = 2.6M, K = 20 19.0 -> 13.4; 16 x 600, d = 8M 89 -> 45; 5 x 250, d = 61,706 (one schedule) 1.9 -> 1.4.
 template <bool WRITE>
-__global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
+__global__ void __launch_bounds__(kBT, 4) k_build_schedule(const SchedParams p)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -116,8 +161,8 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
     int *npiece = cv.take<int>(m);
     int *start = cv.take<int>(m + 1);
     int *lfirst = cv.take<int>(m + 1);
-    uint32_t *key = cv.take<uint32_t>(hash_words(T, p.ni_row_max));   // by index: cell << 16 | sign << 15 | index
-    uint32_t *bycell = key + T;                    // the same words grouped by cell
+    uint16_t *key = cv.take<uint16_t>(hash_words(T, p.ni_row_max));   // by index: sign << 15 | cell
+    uint16_t *bycell = key + T;                    // the indices grouped by cell
     uint16_t *sorted = cv.take<uint16_t>(T);       // entries (sign << 15 | index), list after list
     uint16_t *ls_start = cv.take<uint16_t>(NL);
     uint16_t *ls_len = cv.take<uint16_t>(NL);
@@ -132,7 +177,7 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
     uint32_t *it_steps = cv.take<uint32_t>((size_t)p.l * p.ni_row_max);
     uint32_t *it_chunk = cv.take<uint32_t>((size_t)p.l * p.ni_row_max);
     uint32_t *it_rank = cv.take<uint32_t>((size_t)p.l * p.ni_row_max);
-    int *tot = cv.take<int>(8);                    // [0] items so far, [1] chunks so far, [2] lists, [3] octets
+    int *tot = cv.take<int>(8);                    // [0] items so far, [1] chunks so far, [2] lists
 
     unsigned char *rec = nullptr;
     uint32_t rec_ni = 0;
@@ -158,7 +203,7 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
             const uint32_t j = (uint32_t)(tile * T + jl);       // below 2^31 + T
             const uint32_t b = fda::bucket_of(c, j, (uint32_t)m, p.magic);
             const uint32_t sg = fda::sign_is_negative(c, j) ? 0x8000u : 0u;
-            key[jl] = (b << 16) | sg | (uint32_t)jl;
+            key[jl] = (uint16_t)(sg | b);
             atomicAdd(&cnt[b], 1);
         }
         __syncthreads();
@@ -173,38 +218,27 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
                 s0 += cnt[t];
                 s1 += np;
             }
-            scan[tid] = s0;
-            __syncthreads();
-            if (tid == 0) { int a = 0; for (int t = 0; t < kBT; ++t) { const int v = scan[t]; scan[t] = a; a += v; } }
-            __syncthreads();
-            int a = scan[tid];
-            for (int t = tid * per; t < min(m, (tid + 1) * per); ++t) { start[t] = a; a += cnt[t]; }
-            if (tid == kBT - 1) start[m] = T;
-            __syncthreads();
-            scan[tid] = s1;
-            __syncthreads();
-            if (tid == 0) { int b = 0; for (int t = 0; t < kBT; ++t) { const int v = scan[t]; scan[t] = b; b += v; } scan[kBT] = b; }
-            __syncthreads();
-            int b = scan[tid];
-            for (int t = tid * per; t < min(m, (tid + 1) * per); ++t) { lfirst[t] = b; b += npiece[t]; }
-            if (tid == 0) { lfirst[m] = scan[kBT]; tot[2] = scan[kBT]; }
+            int a = block_scan(s0, scan), b = block_scan(s1, scan + kBT / 32);
+            for (int t = tid * per; t < min(m, (tid + 1) * per); ++t) {
+                start[t] = a; a += cnt[t];
+                lfirst[t] = b; b += npiece[t];
+            }
+            if (tid == kBT - 1) { start[m] = T; lfirst[m] = b; tot[2] = b; }     // (the last thread's b: all lists)
             __syncthreads();
         }
         const int nl = tot[2];
 
         // ---- group by cell (arrival order), then order every cell's run by index ----
         for (int jl = tid; jl < T; jl += kBT) {
-            const uint32_t k = key[jl];
-            const int b = (int)(k >> 16);
-            bycell[start[b] + atomicAdd(&fill[b], 1)] = k;
+            const int b = key[jl] & 0x7fff;
+            bycell[start[b] + atomicAdd(&fill[b], 1)] = (uint16_t)jl;
         }
         __syncthreads();
         for (int pos = tid; pos < T; pos += kBT) {
-            const uint32_t k = bycell[pos];
-            const int b = (int)(k >> 16);
-            const uint32_t idx = k & 0x1fffu;
+            const uint32_t idx = bycell[pos], k = key[idx];
+            const int b = (int)(k & 0x7fffu);
             int rank = 0;
-            for (int q = start[b]; q < start[b + 1]; ++q) rank += ((bycell[q] & 0x1fffu) < idx) ? 1 : 0;
+            for (int q = start[b]; q < start[b + 1]; ++q) rank += bycell[q] < idx ? 1 : 0;
             sorted[start[b] + rank] = (uint16_t)((k & 0x8000u) | fda_list_row(idx));   // the row the index is stored in
         }
         // ---- lists: a cell's run in pieces of nearly equal length ----
@@ -236,19 +270,36 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
             atomicAdd(&cls[n], 1);
         }
         __syncthreads();
-        // ---- lists by length, longest first, ties by list number ----
-        if (tid == 0 && !p.lane_rows) {
-            int a = 0;
-            for (int len = ML; len >= 1; --len) { const int v = cls[len]; cls[len] = a; a += v; }
+        // ---- lists by length, longest first, ties by list number (one warp, 32 lists at a time) ----
+        const bool choose = !WRITE && !p.lane_rows;
+        if (tid < 32 && choose) {
+            int below = 0;                                           // lists that are longer than 64 - 2 * lane
+            {
+                const int pair = cls[ML - 2 * lane] + cls[ML - 1 - 2 * lane];
+                below = pair;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, below, off);
+                    if (lane >= off) below += v;
+                }
+                below -= pair;
+                const int longer = cls[ML - 2 * lane];
+                cls[ML - 2 * lane] = below;
+                cls[ML - 1 - 2 * lane] = below + longer;
+            }
+            __syncwarp();
+            for (int it0 = 0; it0 < nl; it0 += 32) {
+                const int len = it0 + lane < nl ? (int)ls_len[it0 + lane] : 0;
+                const unsigned peers = __match_any_sync(0xffffffffu, len);
+                const int at = cls[len] + __popc(peers & ((1u << lane) - 1u));
+                __syncwarp();
+                if (len > 0) {
+                    order[at] = (uint16_t)(it0 + lane);
+                    if ((peers >> lane) == 1u) cls[len] = at + 1;       // (the last of them)
+                }
+                __syncwarp();
+            }
         }
-        __syncthreads();
-        if (tid >= 1 && tid <= ML && !p.lane_rows) {
-            int r = cls[tid];
-            for (int it = 0; it < nl; ++it)
-                if (ls_len[it] == tid) order[r++] = (uint16_t)it;
-        }
-        __syncthreads();
-
         // ---- octets (one warp): the longest list left opens an octet; every further place goes
         // to the longest of the next kWindow lists that keeps all residue classes within the
         // opener's length (ties: a cell whose bank group the octet's flush does not use yet,
@@ -275,83 +326,90 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
                 for (int r = 0; r < NRES; ++r) cost = max(cost, cols[r]);
                 oc_cost[o] = (uint16_t)cost;
             }
+        } else if (!choose) {
+            const uint16_t *from = p.octets + (size_t)(rec_no * p.l + i) * 9 * NO;
+            for (int x = tid; x < 9 * no; x += kBT) (x < 8 * no ? oc_list[x] : oc_cost[x - 8 * no]) = from[x];
         } else if (tid < 32) {
-            // order[head ..) are the lists not yet placed, longest first: a list taken from the
-            // window is removed by moving the ones before it up by one, so the order is kept
-            int head = 0;
+            // The next kWindow lists that are not placed yet, longest first, in registers: place s of the window
+            // in lane s % 32 (lo: the first 32, hi: the others).  A list that is taken leaves the window by moving those
+            // behind it up by one; `more` is the list that comes in.
+            // Bound: the one warp's chain of some 200 dependent instructions to a place, three quarters of the
+            // counting pass, which is why the writing pass reads the octets back.
+            auto load = [&](int pos) {
+                Cand x{0xffffffffu, 0u, 0u};
+                if (pos < nl) {
+                    const int li = order[pos];
+                    const uint2 r = *reinterpret_cast<const uint2 *>(ls_res + 8 * li);
+                    x.info = (uint32_t)li | (uint32_t)ls_len[li] << 16 | (uint32_t)(ls_cell[li] & 7) << 23;
+                    x.r0 = r.x; x.r1 = r.y;
+                }
+                return x;
+            };
+            Cand lo = load(lane), hi = load(32 + lane), more = load(kWindow);
+            int next = kWindow + 1;
+            auto from = [&](const Cand &x, int src) {
+                return Cand{__shfl_sync(0xffffffffu, x.info, src), __shfl_sync(0xffffffffu, x.r0, src), __shfl_sync(0xffffffffu, x.r1, src)};
+            };
+            auto take = [&](int w) {
+                const Cand got = from(w < 32 ? lo : hi, w & 31);
+                const Cand l1 = from(lo, (lane + 1) & 31), h1 = from(hi, (lane + 1) & 31);
+                if (lane >= w) lo = lane == 31 ? h1 : l1;
+                if (32 + lane >= w) hi = lane == 31 ? more : h1;
+                more = load(next++);
+                return got;
+            };
             for (int o = 0; o < no; ++o) {
-                const int first = order[head];
-                int cols[NRES];
+                // indices of the octet in the classes 2q, 2q + 1, a half word each, and the sum of their squares
+                uint32_t cols[NRES / 2] = {}, squares = 0;
+                auto add = [&](const Cand &x) {
+                    const uint32_t v[NRES / 2] = {__byte_perm(x.r0, 0, 0x4140), __byte_perm(x.r0, 0, 0x4342),
+                                                  __byte_perm(x.r1, 0, 0x4140), __byte_perm(x.r1, 0, 0x4342)};
+                    squares = squares_with(cols, squares, x);
 #pragma unroll
-                for (int r = 0; r < NRES; ++r) cols[r] = ls_res[8 * first + r];
-                const int L = ls_len[first];
-                unsigned cellmask = 1u << (ls_cell[first] & 7);
-                if (lane == 0) oc_list[8 * o] = (uint16_t)first;
-                ++head;
+                    for (int q = 0; q < NRES / 2; ++q) cols[q] += v[q];
+                };
+                const Cand first = take(0);
+                add(first);
+                const int L = (int)(first.info >> 16 & 127u);
+                unsigned cellmask = 1u << (first.info >> 23);
+                if (lane == 0) oc_list[8 * o] = (uint16_t)first.info;
                 for (int place = 1; place < NRES; ++place) {
                     uint32_t best = 0xffffffffu;
 #pragma unroll
                     for (int half = 0; half < kWindow / 32; ++half) {
-                        const int slot = half * 32 + lane;
-                        const int pos = head + slot;
-                        if (pos < nl) {
-                            const int cand = order[pos];
-                            int mx = 0, sq = 0;
-#pragma unroll
-                            for (int r = 0; r < NRES; ++r) {
-                                const int v = cols[r] + ls_res[8 * cand + r];
-                                mx = max(mx, v);
-                                sq += v * v;
-                            }
-                            uint32_t k;
-                            if (mx <= L) {
-                                const uint32_t conflict = (cellmask >> (ls_cell[cand] & 7)) & 1u;
-                                // a flush conflict (two cells of the octet in one bank group) costs about
-                                // as much as two idle steps of a lane
-                                k = ((uint32_t)(L - ls_len[cand] + 2 * (int)conflict) << 23) |
-                                    ((uint32_t)min(sq, 0xffff) << 6) | (uint32_t)slot;
-                            } else {
-                                k = 0x80000000u | ((uint32_t)min(mx, 0x3ff) << 21) |
-                                    ((uint32_t)min(sq >> 6, 0x7fff) << 6) | (uint32_t)slot;
-                            }
-                            best = min(best, k);
+                        const Cand &x = half ? hi : lo;
+                        const int slot = half * 32 + lane, mx = fullest_with(cols, x), sq = (int)squares_with(cols, squares, x);
+                        uint32_t k;
+                        if (mx <= L) {
+                            const uint32_t conflict = (cellmask >> (x.info >> 23 & 7u)) & 1u;
+                            // a flush conflict (two cells of the octet in one bank group) costs about
+                            // as much as two idle steps of a lane
+                            k = ((uint32_t)(L - (int)(x.info >> 16 & 127u) + 2 * (int)conflict) << 23) |
+                                ((uint32_t)min(sq, 0xffff) << 6) | (uint32_t)slot;
+                        } else {
+                            k = 0x80000000u | ((uint32_t)min(mx, 0x3ff) << 21) |
+                                ((uint32_t)min(sq >> 6, 0x7fff) << 6) | (uint32_t)slot;
                         }
+                        if (x.info != 0xffffffffu) best = min(best, k);
                     }
                     best = __reduce_min_sync(0xffffffffu, best);
                     if (best == 0xffffffffu) {                       // no list left
                         if (lane == 0) oc_list[8 * o + place] = 0xffffu;
                         continue;
                     }
-                    const int w = (int)(best & 63u);
-                    const int cand = order[head + w];
-#pragma unroll
-                    for (int r = 0; r < NRES; ++r) cols[r] += ls_res[8 * cand + r];
-                    cellmask |= 1u << (ls_cell[cand] & 7);
-                    // close the gap: order[head .. head+w) moves up by one, head advances
-                    uint16_t mv[kWindow / 32];
-#pragma unroll
-                    for (int half = 0; half < kWindow / 32; ++half) {
-                        const int slot = half * 32 + lane;
-                        mv[half] = slot < w ? order[head + slot] : (uint16_t)0;
-                    }
-                    __syncwarp();
-#pragma unroll
-                    for (int half = 0; half < kWindow / 32; ++half) {
-                        const int slot = half * 32 + lane;
-                        if (slot < w) order[head + slot + 1] = mv[half];
-                    }
-                    if (lane == 0) oc_list[8 * o + place] = (uint16_t)cand;
-                    ++head;
-                    __syncwarp();
+                    const Cand got = take((int)(best & 63u));
+                    add(got);
+                    cellmask |= 1u << (got.info >> 23);
+                    if (lane == 0) oc_list[8 * o + place] = (uint16_t)got.info;
                 }
-                int cost = L;
-#pragma unroll
-                for (int r = 0; r < NRES; ++r) cost = max(cost, cols[r]);
-                if (lane == 0) oc_cost[o] = (uint16_t)cost;
+                if (lane == 0) oc_cost[o] = (uint16_t)max(L, fullest_with(cols, Cand{0u, 0u, 0u}));
             }
-            if (lane == 0) tot[3] = no;
         }
         __syncthreads();
+        if (choose && p.octets) {
+            uint16_t *to = p.octets + (size_t)(rec_no * p.l + i) * 9 * NO;
+            for (int x = tid; x < 9 * no; x += kBT) to[x] = x < 8 * no ? oc_list[x] : oc_cost[x - 8 * no];
+        }
         // ---- octets by steps (most first, ties by number); four of them make an item ----
         for (int o = tid; o < no; o += kBT) {
             int rank = p.lane_rows ? o : 0;
@@ -390,85 +448,83 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
                 }
                 cells[(size_t)(item0 + q) * kListSlots + ln] = cell;
             }
-            // ---- entries: one thread per octet place of the row's items ----
+            // ---- entries: a warp per item, eight threads per octet, one to each of its lists ----
+            // (with one thread to an octet, four octets to a warp, whose paths differ, an instruction of the
+            // matching served one list where it serves up to 32 here)
             uint16_t *ent = reinterpret_cast<uint16_t *>(rec + ent_off);
-            // (spread over the warps of the block: the matching is serial code on private tables,
-            // and threads of one warp would run its data-dependent paths one after the other)
-            for (int pos = tid / kSpread; (tid % kSpread) == 0 && pos < 4 * ni_row; pos += kBT / kSpread) {
-                const int q = pos / 4, lane0 = (pos % 4) * NRES;
-                const int steps = (int)it_steps[item0 + q];
-                const int padded = (steps + 3) & ~3;
-                uint16_t *dst = ent + (size_t)it_chunk[item0 + q] * (kListSlots * 4);
-                // four steps of the eight lanes, written as one 64-bit word per lane
-                unsigned long long word[NRES];
-                auto write_words = [&](int t) {
-#pragma unroll
-                    for (int s = 0; s < NRES; ++s)
-                        *reinterpret_cast<unsigned long long *>(dst + (size_t)(t >> 2) * (kListSlots * 4) + (lane0 + s) * 4) = word[s];
-                };
-                int delta = 0;
-                if (pos < no) {
-                    const int o = oc_order[pos];
-                    delta = oc_cost[o];
-                    // edge[s * 8 + r]: bits 0..6 the indices of list s in class r, bits 7..16 the padding
-                    // edges that make the graph regular (up to eight full lists in one class: 512), from
-                    // bit 17 on the list's next entry of the class.  The words live in shared memory (the
-                    // hash words of the row are no longer needed), what the search itself works on in
-                    // registers: alive, a bit per edge; match (list -> class), back (class -> list), prev
-                    // and queue, a nibble per entry, 8 for none.  With byte tables in shared memory
-                    // for all of it fda_create took 2.9 instead of 2.3 ms at 5 x 250, d = 200,000, 24.0 instead of
-                    // 22.4 ms at d = 20M.
-                    uint32_t *edge = key + (size_t)pos * (kMatchBytes / 4);
-                    unsigned short *defL = reinterpret_cast<unsigned short *>(edge + NRES * NRES), *defR = defL + NRES;
-                    unsigned long long alive = 0ull;
-                    for (int r = 0; r < NRES; ++r) defR[r] = (unsigned short)delta;
-                    for (int s = 0; s < NRES; ++s) {
-                        const int li = oc_list[8 * o + s];
-                        int a0 = li != 0xffff ? ls_start[li] : 0, len = 0;
-                        for (int r = 0; r < NRES; ++r) {
-                            const int v = li != 0xffff ? ls_res[8 * li + r] : 0;
-                            edge[s * NRES + r] = (uint32_t)v | ((uint32_t)a0 << 17);
-                            if (v) alive |= 1ull << (s * NRES + r);
-                            a0 += v;
-                            len += v;
-                            defR[r] = (unsigned short)(defR[r] - v);
-                        }
-                        defL[s] = (unsigned short)(delta - len);
+            for (int q = tid / 32; q < ni_row; q += kBT / 32) {
+                const int pos = 4 * q + lane / NRES, s = lane % NRES;
+                const int steps = (int)it_steps[item0 + q], padded = (steps + 3) & ~3;
+                uint16_t *dst = ent + (size_t)it_chunk[item0 + q] * (kListSlots * 4) + lane * 4;
+                // edge[r * 8 + s]: bits 0..6 the indices of list s in class r, bits 7..16 the padding
+                // edges that make the graph regular (up to eight full lists in one class: 512), from
+                // bit 17 on the list's next entry of the class.  The words live in shared memory (the
+                // hash words of the row are no longer needed), what the search itself works on in
+                // registers, the same in all eight threads: match (list -> class), back (class -> list), prev
+                // and queue, a nibble per entry, 8 for none; alive, a bit per edge, is put together from the threads' rows.
+                uint32_t *edge = reinterpret_cast<uint32_t *>(key) + (size_t)pos * (kMatchBytes / 4);
+                unsigned short *defL = reinterpret_cast<unsigned short *>(edge + NRES * NRES), *defR = defL + NRES;
+                const int o = pos < no ? oc_order[pos] : 0, delta = pos < no ? oc_cost[o] : 0;
+                const int li = pos < no ? oc_list[8 * o + s] : 0xffff;
+                int a0 = li != 0xffff ? ls_start[li] : 0, len = 0;
+                for (int r = 0; r < NRES; ++r) {
+                    const int v = li != 0xffff ? ls_res[8 * li + r] : 0;
+                    edge[r * NRES + s] = (uint32_t)v | ((uint32_t)a0 << 17);
+                    a0 += v;
+                    len += v;
+                }
+                defL[s] = (unsigned short)(delta - len);
+                __syncwarp();
+                int in_class = 0;
+                for (int x = 0; x < NRES; ++x) in_class += (int)(edge[s * NRES + x] & 0x7fu);
+                defR[s] = (unsigned short)(delta - in_class);
+                __syncwarp();
+                if (s == 0)
+                    for (int x = 0, r = 0; x < NRES && r < NRES;) {
+                        const unsigned dl = defL[x], n = min(dl, (unsigned)defR[r]);
+                        edge[r * NRES + x] += n << 7;
+                        defL[x] = (unsigned short)(dl - n);
+                        defR[r] = (unsigned short)(defR[r] - n);
+                        if (dl == n) ++x; else ++r;
                     }
-                    for (int s = 0, r = 0; s < NRES && r < NRES;) {
-                        const unsigned dl = defL[s], x = min(dl, (unsigned)defR[r]);
-                        if (x) {
-                            edge[s * NRES + r] += x << 7;
-                            alive |= 1ull << (s * NRES + r);
-                        }
-                        defL[s] = (unsigned short)(dl - x);
-                        defR[r] = (unsigned short)(defR[r] - x);
-                        if (dl == x) ++s; else ++r;
-                    }
-                    auto nibble = [](unsigned x, int i) { return (int)((x >> (4 * i)) & 15u); };
-                    auto with = [](unsigned x, int i, int v) { return (x & ~(15u << (4 * i))) | ((unsigned)v << (4 * i)); };
-                    unsigned match = 0x88888888u;
-                    for (int t = 0; t < delta; ++t) {
-                        // keep the edges of the last matching that still exist, complete it with
-                        // augmenting paths (a regular bipartite multigraph has a perfect matching)
-                        unsigned back = 0x88888888u;
+                __syncwarp();
+                unsigned row = 0;                                    // the list's edges that exist
+                for (int r = 0; r < NRES; ++r) row |= (edge[r * NRES + s] & 0x1ffffu) ? 1u << r : 0u;
+
+                auto nibble = [](unsigned x, int i) { return (int)((x >> (4 * i)) & 15u); };
+                auto with = [](unsigned x, int i, int v) { return (x & ~(15u << (4 * i))) | ((unsigned)v << (4 * i)); };
+                unsigned match = 0x88888888u;
+                unsigned long long word = 0ull;
+                for (int t = 0; t < padded; ++t) {
+                    // keep the edges of the last matching that still exist, complete it with
+                    // augmenting paths (a regular bipartite multigraph has a perfect matching)
+                    const int had = nibble(match, s);
+                    const bool keep = had < 8 && ((row >> had) & 1u);
+                    const unsigned kept = (__ballot_sync(0xffffffffu, keep) >> (lane & 24)) & 0xffu;
+                    unsigned back = keep ? (unsigned)(s ^ 8) << (4 * had) : 0u, half = row << (8 * (s & 3));
 #pragma unroll
-                        for (int s = 0; s < NRES; ++s) {
-                            const int r = nibble(match, s);
-                            if (r < 8 && ((alive >> (s * NRES + r)) & 1ull)) back = with(back, r, s); else match = with(match, s, 8);
-                        }
+                    for (int x = 1; x < NRES; x <<= 1) back |= __shfl_xor_sync(0xffffffffu, back, x);
+                    back ^= 0x88888888u;
+                    half |= __shfl_xor_sync(0xffffffffu, half, 1);
+                    half |= __shfl_xor_sync(0xffffffffu, half, 2);
+                    const unsigned other = __shfl_xor_sync(0xffffffffu, half, 4);
+                    const unsigned long long alive = s < 4 ? (unsigned long long)other << 32 | half : (unsigned long long)half << 32 | other;
+                    const bool on = t < delta;
+                    if (on && kept != 0xffu) {
+                        for (int x = 0; x < NRES; ++x)
+                            if (!((kept >> x) & 1u)) match = with(match, x, 8);
                         for (int s0 = 0; s0 < NRES; ++s0) {
                             if (nibble(match, s0) < 8) continue;
                             int qh = 0, qt = 1;
                             unsigned vis = 0, prev = 0, queue = (unsigned)s0;
                             bool done = false;
                             while (qh < qt && !done) {
-                                const int s = nibble(queue, qh++);
-                                unsigned open = (unsigned)(alive >> (s * NRES)) & 0xffu & ~vis;
+                                const int sq = nibble(queue, qh++);
+                                unsigned open = (unsigned)(alive >> (sq * NRES)) & 0xffu & ~vis;
                                 vis |= open;
                                 for (; open && !done; open &= open - 1u) {
                                     const int r = __ffs((int)open) - 1, owner = nibble(back, r);
-                                    prev = with(prev, r, s);
+                                    prev = with(prev, r, sq);
                                     if (owner < 8) {
                                         queue = with(queue, qt++, owner);
                                         continue;
@@ -484,31 +540,27 @@ __global__ void __launch_bounds__(kBT) k_build_schedule(const SchedParams p)
                                 }
                             }
                         }
-                        const int sh = 16 * (t & 3);
-#pragma unroll
-                        for (int s = 0; s < NRES; ++s) {
-                            const int r = nibble(match, s) & 7, at = s * NRES + r;      // (every list is matched)
-                            uint32_t w = edge[at];
-                            uint16_t e;
-                            if (w & 0x7fu) {
-                                e = sorted[w >> 17];
-                                w += (1u << 17) - 1u;
-                            } else {
-                                e = (uint16_t)(T + r);
-                                w -= 1u << 7;
-                            }
-                            edge[at] = w;
-                            if ((w & 0x1ffffu) == 0u) alive &= ~(1ull << at);
-                            word[s] = ((t & 3) ? word[s] : 0ull) | ((unsigned long long)e << sh);
-                        }
-                        if ((t & 3) == 3) write_words(t);
                     }
-                }
-                for (int t = delta; t < padded; ++t) {
-#pragma unroll
-                    for (int s = 0; s < NRES; ++s)
-                        word[s] = ((t & 3) ? word[s] : 0ull) | ((unsigned long long)(uint16_t)(T + s) << (16 * (t & 3)));
-                    if ((t & 3) == 3) write_words(t);
+                    __syncwarp();
+                    uint16_t e = (uint16_t)(T + s);                  // (behind the octet's last step)
+                    if (on) {
+                        const int r = nibble(match, s) & 7;          // (every list is matched)
+                        uint32_t w = edge[r * NRES + s];
+                        if (w & 0x7fu) {
+                            e = sorted[w >> 17];
+                            w += (1u << 17) - 1u;
+                        } else {
+                            e = (uint16_t)(T + r);
+                            w -= 1u << 7;
+                        }
+                        edge[r * NRES + s] = w;
+                        if ((w & 0x1ffffu) == 0u) row &= ~(1u << r);
+                    }
+                    word |= (unsigned long long)e << (16 * (t & 3));
+                    if ((t & 3) == 3) {
+                        *reinterpret_cast<unsigned long long *>(dst + (size_t)(t >> 2) * (kListSlots * 4)) = word;
+                        word = 0ull;
+                    }
                 }
             }
         }
@@ -767,7 +819,12 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
     uint64_t *off = nullptr;
     unsigned char *buf = nullptr;
     auto cleanup = [&]() { cudaFree(items); cudaFree(rows); cudaFree(prog); cudaFree(off); cudaFree(buf); };
-    if (cudaMalloc(&items, sizeof(uint32_t) * (3 * tiles + (size_t)ctx->l * kShifts)) != cudaSuccess ||
+    // one allocation for what only the builder needs (the octets take a twentieth to a fifth of what the schedule does, so without
+    // room for them there is none for the schedule: then it is only counted)
+    const size_t words = 3 * (size_t)tiles + (size_t)ctx->l * kShifts, octet_bytes = lanes ? 0 : sizeof(uint16_t) * 9 * (size_t)tiles * p.l * p.no_max;
+    if (octet_bytes && cudaMalloc(&items, sizeof(uint32_t) * words + octet_bytes) == cudaSuccess) p.octets = reinterpret_cast<uint16_t *>(items + words);
+    else cudaGetLastError();
+    if ((!items && cudaMalloc(&items, sizeof(uint32_t) * words) != cudaSuccess) ||
         cudaMalloc(&rows, sizeof(int2) * ctx->l) != cudaSuccess ||
         cudaMalloc(&off, sizeof(uint64_t) * (tiles + 1)) != cudaSuccess) {
         cudaGetLastError();
@@ -813,7 +870,7 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
     const uint64_t prog_bytes = lanes ? sizeof(uint32_t) * (uint64_t)(lane_items + 1) * tiles : 0;
     const uint64_t all_bytes = total + prog_bytes + ctx->sched_bytes;         // (of both schedules, when this is the second)
     size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || total + prog_bytes > free_b / 3 ||
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || (!lanes && !p.octets) || total + prog_bytes > (free_b + octet_bytes) / 3 ||
         (ctx->sched_limit_bytes > 0 && all_bytes > (uint64_t)ctx->sched_limit_bytes) ||
         cudaMalloc(&buf, total) != cudaSuccess || (lanes && cudaMalloc(&prog, prog_bytes) != cudaSuccess)) {
         cudaGetLastError();

@@ -138,6 +138,12 @@ def test_random_tables(env):
     run(env, 7, 500, rand_coeffs(rng, 7), 300_000, lambda n: [0, n - 1], max_steps_ratio=1.3)
 
 
+# lists that do not fill an octet, a warp or the window that octets are chosen from (64 lists), and one list more
+@pytest.mark.parametrize("l,m", [(1, 1), (2, 7), (3, 33), (2, 63), (1, 64), (2, 65), (16, 33), (3, 700)])
+def test_few_and_many_lists(env, l, m):
+    run(env, l, m, rand_coeffs(np.random.default_rng(34 + m), l), 30_011, lambda n: [0, n - 1])
+
+
 def test_rotating_and_constant_buckets(env):
     l, m = 3, 256
     c = rand_coeffs(np.random.default_rng(32), l)
