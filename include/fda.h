@@ -124,8 +124,9 @@ fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uin
  * What the context holds (the paper has no counterpart).  info (host, 8 values):
  *   [0] device bytes the context owns now   [1] of which: the list schedules (0: none)
  *   [2] 1 when sketch requests run on the list kernel, 0 when on the plain-load kernels
- *   [3] indices per tile of the schedule    [4] bytes of a schedule that was built and dropped
- *       for lack of memory (0: none)        [5] bytes of the lazily built 16-bit hash table
+ *   [3] indices per tile of the first schedule (fda_debug_lane_schedule has the second's)
+ *   [4] bytes of the schedules that were left out for lack of memory or by the caller's cap (0: none)
+ *   [5] bytes of the lazily built 16-bit hash table
  *   [6] microseconds fda_create spent on the schedules  [7] other lazily allocated bytes.
  * Errors: INVALID_ARG (NULL).
  */
@@ -292,6 +293,14 @@ fda_status fda_debug_schedule(const fda_ctx *ctx, int64_t tile, void *record_hos
                               int64_t *info);
 
 /*
+ * The same for the second schedule (see fda_create; the paper has no counterpart): its records have the
+ * same form, no cell has several lists, and an item holds the lists of the same 32 cells in every tile.
+ * Errors: as fda_debug_schedule; UNSUPPORTED when the context has no second schedule.
+ */
+fda_status fda_debug_lane_schedule(const fda_ctx *ctx, int64_t tile, void *record_host, size_t capacity,
+                                   int64_t *info);
+
+/*
  * Name of the kernel that served the context's last fda_local_state or fda_mean_state call (the
  * paper has no counterpart): "k_local_state_gather" (sketch pass over per-cell index lists, in all its
  * forms: every sketch request that a context's list schedule can serve), "k_local_state_linear" (no
@@ -313,6 +322,13 @@ const char *fda_debug_last_kernel(const fda_ctx *ctx);
  * The benchmark uses it to count the launches of a step.
  */
 int fda_debug_last_launches(const fda_ctx *ctx);
+
+/*
+ * Which list schedule the context's last fda_local_state or fda_mean_state call walked (the paper has no
+ * counterpart): 1 the first, 2 the second (the kernel whose lanes keep their cells), 0 none: no sketch was
+ * asked for, or the plain-load kernels served it, or there was no such call, or ctx == NULL.
+ */
+int fda_debug_last_schedule(const fda_ctx *ctx);
 
 /*
  * Local state without a context and without any allocation.  (The paper has no counterpart

@@ -21,7 +21,7 @@ _STATUS = {0: "FDA_OK", 1: "FDA_ERR_INVALID_ARG", 2: "FDA_ERR_UNSUPPORTED", 3: "
            4: "FDA_ERR_NOMEM"}
 
 EXPORTS = ("fda_create", "fda_create_limited", "fda_context_info", "fda_destroy", "fda_state_len", "fda_last_error", "fda_local_state", "fda_mean_state",
-           "fda_combine_estimate", "fda_average_models", "fda_average_models_xi", "fda_round_host", "fda_debug_hash", "fda_debug_read_probe", "fda_debug_last_kernel", "fda_debug_last_launches", "fda_debug_schedule",
+           "fda_combine_estimate", "fda_average_models", "fda_average_models_xi", "fda_round_host", "fda_debug_hash", "fda_debug_read_probe", "fda_debug_last_kernel", "fda_debug_last_launches", "fda_debug_last_schedule", "fda_debug_schedule", "fda_debug_lane_schedule",
            "fda_local_state_linear_noalloc")
 FDA_NOALLOC_MAX_WORKERS = 64
 
@@ -86,6 +86,10 @@ def load_library():
     lib.fda_debug_read_probe.restype = c_int
     lib.fda_debug_schedule.argtypes = [vp, i64, vp, ctypes.c_size_t, vp]
     lib.fda_debug_schedule.restype = c_int
+    lib.fda_debug_lane_schedule.argtypes = [vp, i64, vp, ctypes.c_size_t, vp]
+    lib.fda_debug_lane_schedule.restype = c_int
+    lib.fda_debug_last_schedule.argtypes = [vp]
+    lib.fda_debug_last_schedule.restype = c_int
     lib.fda_debug_last_kernel.argtypes = [vp]
     lib.fda_debug_last_kernel.restype = ctypes.c_char_p
     lib.fda_debug_last_launches.argtypes = [vp]
@@ -276,13 +280,18 @@ class FdaContext:
 
     def fda_debug_schedule(self, tile: int):
         """(record bytes as a numpy uint8 array, info dict) of the list schedule's record of a tile."""
+        return self._record(self._lib.fda_debug_schedule, "fda_debug_schedule", tile)
+
+    def fda_debug_lane_schedule(self, tile: int):
+        """The same for the second schedule, in which every cell stays with one lane."""
+        return self._record(self._lib.fda_debug_lane_schedule, "fda_debug_lane_schedule", tile)
+
+    def _record(self, call, name: str, tile: int):
         info = (ctypes.c_int64 * 8)()
         probe = (ctypes.c_uint8 * 16)()
-        st = self._lib.fda_debug_schedule(self._h, tile, probe, 16, info)
-        self._check(st, "fda_debug_schedule")
+        self._check(call(self._h, tile, probe, 16, info), name)
         buf = np.zeros(int(info[3]), dtype=np.uint8)
-        st = self._lib.fda_debug_schedule(self._h, tile, buf.ctypes.data_as(ctypes.c_void_p), buf.size, info)
-        self._check(st, "fda_debug_schedule")
+        self._check(call(self._h, tile, buf.ctypes.data_as(ctypes.c_void_p), buf.size, info), name)
         keys = ("tile_indices", "slots", "max_len", "record_bytes", "tiles", "pad_rows", "lanes_per_pass",
                 "schedule_bytes")
         return buf, dict(zip(keys, (int(v) for v in info)))
@@ -294,6 +303,10 @@ class FdaContext:
     def fda_debug_last_launches(self) -> int:
         """Kernels that the last fda_local_state call on this context launched."""
         return int(self._lib.fda_debug_last_launches(self._h))
+
+    def fda_debug_last_schedule(self) -> int:
+        """Which list schedule the last state call on this context walked: 0 none, 1 the first, 2 the second."""
+        return int(self._lib.fda_debug_last_schedule(self._h))
 
     @staticmethod
     def new_estimate_buffer(device="cuda"):

@@ -140,6 +140,31 @@ void free_device(fda_ctx *ctx)
     if (ctx->side_stream) cudaStreamDestroy(ctx->side_stream);
 }
 
+// One record of a schedule, and what there is to know about the schedule (fda_debug_schedule)
+fda_status copy_record(const fda_ctx *ctx, const unsigned char *sched, const uint64_t *offsets, int64_t records, int T,
+                       uint64_t bytes, int64_t tile, void *record_host, size_t capacity, int64_t *info)
+{
+    if (tile < 0 || tile >= records) return FDA_ERR_INVALID_ARG;
+    DeviceGuard guard(ctx->device);
+    if (!guard.ok) return FDA_ERR_CUDA;
+    uint64_t off[2] = {0, 0};
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemcpy(off, offsets + tile, sizeof(off), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) { cudaGetLastError(); return FDA_ERR_CUDA; }
+    info[0] = T;
+    info[1] = kListSlots;
+    info[2] = kListMaxLen;
+    info[3] = (int64_t)(off[1] - off[0]);
+    info[4] = records;
+    info[5] = kListPadRows;
+    info[6] = kListOct;
+    info[7] = (int64_t)bytes;
+    const size_t n = capacity < (size_t)info[3] ? capacity : (size_t)info[3];
+    e = cudaMemcpy(record_host, sched + off[0], n, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) { cudaGetLastError(); return FDA_ERR_CUDA; }
+    return FDA_OK;
+}
+
 bool finite_f(float v) { return std::isfinite(v); }
 
 }  // namespace
@@ -252,6 +277,8 @@ const char *fda_last_error(const fda_ctx *ctx) { return ctx ? ctx->err.c_str() :
 const char *fda_debug_last_kernel(const fda_ctx *ctx) { return ctx ? ctx->last_ls_kernel : ""; }
 
 int fda_debug_last_launches(const fda_ctx *ctx) { return ctx ? ctx->last_ls_launches : 0; }
+
+int fda_debug_last_schedule(const fda_ctx *ctx) { return ctx ? ctx->last_schedule : 0; }
 
 fda_status fda_local_state(fda_ctx *ctx, const float *w, int64_t row_stride, int K, int64_t d,
                            const float *w_t0, const float *xi, uint32_t flags, float *states,
@@ -450,25 +477,17 @@ fda_status fda_debug_schedule(const fda_ctx *ctx, int64_t tile, void *record_hos
 {
     if (!ctx || !record_host || !info) return FDA_ERR_INVALID_ARG;
     if (!ctx->sched) return FDA_ERR_UNSUPPORTED;
-    if (tile < 0 || tile >= ctx->sched_tiles * ctx->sched_parts) return FDA_ERR_INVALID_ARG;
-    DeviceGuard guard(ctx->device);
-    if (!guard.ok) return FDA_ERR_CUDA;
-    uint64_t off[2] = {0, 0};
-    cudaError_t e = cudaDeviceSynchronize();
-    if (e == cudaSuccess) e = cudaMemcpy(off, ctx->sched_off + tile, sizeof(off), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) { cudaGetLastError(); return FDA_ERR_CUDA; }
-    info[0] = ctx->sched_T;
-    info[1] = kListSlots;
-    info[2] = kListMaxLen;
-    info[3] = (int64_t)(off[1] - off[0]);
-    info[4] = ctx->sched_tiles * ctx->sched_parts;
-    info[5] = kListPadRows;
-    info[6] = kListOct;
-    info[7] = (int64_t)ctx->sched_bytes;
-    const size_t n = capacity < (size_t)info[3] ? capacity : (size_t)info[3];
-    e = cudaMemcpy(record_host, ctx->sched + off[0], n, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) { cudaGetLastError(); return FDA_ERR_CUDA; }
-    return FDA_OK;
+    return copy_record(ctx, ctx->sched, ctx->sched_off, ctx->sched_tiles * ctx->sched_parts, ctx->sched_T,
+                       ctx->sched_bytes, tile, record_host, capacity, info);
+}
+
+fda_status fda_debug_lane_schedule(const fda_ctx *ctx, int64_t tile, void *record_host, size_t capacity,
+                                   int64_t *info)
+{
+    if (!ctx || !record_host || !info) return FDA_ERR_INVALID_ARG;
+    if (!ctx->lane_sched) return FDA_ERR_UNSUPPORTED;
+    return copy_record(ctx, ctx->lane_sched, ctx->lane_off, ctx->lane_tiles * ctx->lane_parts, ctx->lane_T,
+                       ctx->lane_records, tile, record_host, capacity, info);
 }
 
 fda_status fda_context_info(const fda_ctx *ctx, int64_t *info)
@@ -488,7 +507,7 @@ fda_status fda_context_info(const fda_ctx *ctx, int64_t *info)
     info[1] = sched;
     info[2] = ctx->sched ? 1 : 0;
     info[3] = ctx->sched_T;
-    info[4] = (int64_t)ctx->sched_skipped_bytes;
+    info[4] = (int64_t)(ctx->sched_skipped_bytes + ctx->lane_skipped_bytes);
     info[5] = table;
     info[6] = (int64_t)(ctx->sched_build_ms * 1000.0);
     info[7] = mean + stage;

@@ -77,6 +77,8 @@ struct fda_ctx {
     uint32_t *lane_prog = nullptr;
     int2 *lane_rows = nullptr;
     uint64_t lane_bytes = 0;          // records, offsets and programs
+    uint64_t lane_records = 0;        // bytes of the records
+    uint64_t lane_skipped_bytes = 0;  // size of a second schedule that was not kept (memory limit)
     int lane_T = 0, lane_parts = 1;
     int64_t lane_tiles = 0;
     int lane_items = 0;               // items of a tile (and part of the sketch rows)
@@ -102,6 +104,7 @@ struct fda_ctx {
     uint64_t coeffs_host[6 * FDA_MAX_ROWS] = {0};
     const char *last_ls_kernel = "";   // which kernel served the last fda_local_state / fda_mean_state
     int last_ls_launches = 0;          // kernels the last fda_local_state launched
+    int last_schedule = 0;             // which schedule the last of these calls walked (0: none, 1, 2)
     std::string err;
 };
 

@@ -449,6 +449,7 @@ cudaError_t fda_launch_local_state(fda_ctx *ctx, const float *w, int64_t row_str
                                    int64_t d, const float *w_t0, const float *xi, uint32_t flags,
                                    float *states, cudaStream_t s)
 {
+    ctx->last_schedule = 0;
     {   // sketch requests: the list kernel when the context holds its schedule; requests without a
         // sketch: the streaming kernel; everything else: the plain-load kernels below
         cudaError_t e = fda_launch_local_state_gather(ctx, w, row_stride, K, d, w_t0, xi, flags, states, s);

@@ -457,6 +457,7 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     }
     if (e != cudaSuccess) return e;
     ctx->last_ls_launches = parts.n + 1;
+    ctx->last_schedule = lanes ? 2 : 1;
     const int nb = parts.cpg[0];
     // one worker per lane while all those threads are resident at once (2048 to an SM), four beyond that.  Measured,
     // kernel and finalize back to back, one and four per lane: 5 x 250, K = 10, d = 1.2M (60K threads) 30.0 and 34.3 us;

@@ -359,13 +359,14 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
     // stays in one pass, which allocates nothing.
     // From the averaged drifts that phase 1 below leaves in memory when the sketch is too large for the lane-private
     // bins of k_sketch_vector_rows.
+    ctx->last_schedule = 0;
     const bool lists = sketch && ctx->sched != nullptr, rows_kernel = ctx->columns == 32;
     const int64_t tiles = lists ? (d + ctx->sched_T - 1) / ctx->sched_T : 0;
     const bool one_pass = (vec || K <= std::max(2 * ctx->l, 10)) && tiles >= (vec || !rows_kernel ? 2 : 8) * (int64_t)ctx->n_sm;
     if (lists && one_pass) {
         const cudaError_t e = fda_launch_mean_state_gather(ctx, w, row_stride, K, d, w_t0, xi, flags, mean_state, s);
         if (e != cudaErrorNotSupported) {
-            if (e == cudaSuccess) ctx->last_ls_kernel = "k_mean_state_gather";
+            if (e == cudaSuccess) { ctx->last_ls_kernel = "k_mean_state_gather"; ctx->last_schedule = 1; }
             return e;
         }
     }
@@ -388,7 +389,7 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
     if (lists && !rows_kernel) {
         e = fda_launch_mean_sketch_gather(ctx, ctx->mean_model, K, d, linear, flags, (int)nblk, mean_state, s);
         if (e != cudaErrorNotSupported) {
-            if (e == cudaSuccess) ctx->last_ls_kernel = "k_mean_model + k_mean_state_gather";
+            if (e == cudaSuccess) { ctx->last_ls_kernel = "k_mean_model + k_mean_state_gather"; ctx->last_schedule = 1; }
             return e;
         }
     }

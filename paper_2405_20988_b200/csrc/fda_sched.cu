@@ -875,7 +875,7 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
         cudaMalloc(&buf, total) != cudaSuccess || (lanes && cudaMalloc(&prog, prog_bytes) != cudaSuccess)) {
         cudaGetLastError();
         cleanup();
-        if (!lanes) ctx->sched_skipped_bytes = total;
+        (lanes ? ctx->lane_skipped_bytes : ctx->sched_skipped_bytes) = total + prog_bytes;
         return cudaSuccess;                                                   // leave the memory to the models
     }
     e = cudaMemcpyAsync(off, h_off.data(), sizeof(uint64_t) * (tiles + 1), cudaMemcpyHostToDevice, s);
@@ -889,6 +889,7 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
     cudaFree(items);
     if (lanes) {
         ctx->lane_sched = buf; ctx->lane_off = off; ctx->lane_prog = prog; ctx->lane_rows = rows;
+        ctx->lane_records = total;
         ctx->lane_bytes = total + prog_bytes + sizeof(uint64_t) * (tiles + 1) + sizeof(int2) * ctx->l;
         ctx->lane_T = T; ctx->lane_parts = parts; ctx->lane_tiles = part_tiles;
         ctx->lane_items = lane_items; ctx->lane_walkers = lane_walkers(lane_items);
