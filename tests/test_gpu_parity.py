@@ -422,6 +422,13 @@ def full_round(env, idx):
         torch.cuda.synchronize()
         got = st.cpu().numpy()
         worst = check_states(got, ora, wl.l, wl.m, d, rows=ks)
+        # the same without a projection: on the three long vectors every cell stays with a lane
+        ctx.fda_local_state(w[:, :d], w0, None, 1 | 4, st)
+        assert ctx.fda_debug_last_schedule() == (2 if idx >= 3 else 1)
+        without = ora.copy()
+        without[:, 1] = 0.0
+        worst["without xi"] = check_states(st.cpu().numpy(), without, wl.l, wl.m, d, rows=ks)
+        ctx.fda_local_state(w[:, :d], w0, xg, ALL, st)
         # combine: the oracle runs on the GPU's own fp32 states (isolates this step) ...
         results = {}
         for variant in (F.FDA_VARIANT_LINEAR, F.FDA_VARIANT_SKETCH):
