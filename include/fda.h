@@ -97,7 +97,7 @@ typedef struct {
  *     indices to a block of the sketch kernel at K_max workers: d_max above 11 million for K_max = 8, 1.4
  *     million for 30) whose hash spreads the indices of a tile evenly over the cells: it makes fda_local_state
  *     without a projection a fifth faster and takes half as long to build as the first; it is left out
- *     when it would take more than a third of the memory that is free then;
+ *     when it would take more than a third of the memory that is free then, or on request (fda_create_with);
  *   - lazily, by the first call that needs them: a 16-bit hash table of 2*l bytes per index
  *     (sketch requests on a context without a schedule), d_max floats (fda_mean_state on
  *     short vectors, many unaligned rows, or without a schedule), K_max*d_max floats of staging
@@ -119,6 +119,19 @@ fda_status fda_create(fda_ctx **out, int device, int l, int m, const uint64_t *h
  */
 fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uint64_t *hash_coeffs,
                               int64_t d_max, int K_max, int64_t schedule_limit_bytes);
+
+/* fda_create_with flags */
+enum { FDA_CREATE_ONE_SCHEDULE = 1 };
+
+/*
+ * fda_create_limited with flags (the paper has no counterpart).  FDA_CREATE_ONE_SCHEDULE leaves the second list
+ * schedule out: about half the memory and two thirds of the time that the schedules of a context of long vectors
+ * take, for programs that do not call fda_local_state without a projection on them (LinearFDA, fda_mean_state,
+ * fda_average_models) or would rather have the memory than the fifth of that call's time.
+ * Errors: as fda_create, plus INVALID_ARG for an unknown flag.
+ */
+fda_status fda_create_with(fda_ctx **out, int device, int l, int m, const uint64_t *hash_coeffs,
+                           int64_t d_max, int K_max, int64_t schedule_limit_bytes, uint32_t flags);
 
 /*
  * What the context holds (the paper has no counterpart).  info (host, 8 values):

@@ -16,11 +16,12 @@ FDA_STATE_NORM, FDA_STATE_LINEAR, FDA_STATE_SKETCH = 1, 2, 4
 FDA_VARIANT_LINEAR, FDA_VARIANT_SKETCH = 0, 1
 FDA_AVG_BROADCAST, FDA_AVG_UNCONDITIONAL = 1, 2
 FDA_MAX_ROWS = 16
+FDA_CREATE_ONE_SCHEDULE = 1
 
 _STATUS = {0: "FDA_OK", 1: "FDA_ERR_INVALID_ARG", 2: "FDA_ERR_UNSUPPORTED", 3: "FDA_ERR_CUDA",
            4: "FDA_ERR_NOMEM"}
 
-EXPORTS = ("fda_create", "fda_create_limited", "fda_context_info", "fda_destroy", "fda_state_len", "fda_last_error", "fda_local_state", "fda_mean_state",
+EXPORTS = ("fda_create", "fda_create_limited", "fda_create_with", "fda_context_info", "fda_destroy", "fda_state_len", "fda_last_error", "fda_local_state", "fda_mean_state",
            "fda_combine_estimate", "fda_average_models", "fda_average_models_xi", "fda_round_host", "fda_debug_hash", "fda_debug_read_probe", "fda_debug_last_kernel", "fda_debug_last_launches", "fda_debug_last_schedule", "fda_debug_schedule", "fda_debug_lane_schedule",
            "fda_local_state_linear_noalloc")
 FDA_NOALLOC_MAX_WORKERS = 64
@@ -66,6 +67,8 @@ def load_library():
     lib.fda_create.argtypes = [ctypes.POINTER(vp), c_int, c_int, c_int, vp, i64, c_int]
     lib.fda_create_limited.argtypes = [ctypes.POINTER(vp), c_int, c_int, c_int, vp, i64, c_int, i64]
     lib.fda_create_limited.restype = c_int
+    lib.fda_create_with.argtypes = [ctypes.POINTER(vp), c_int, c_int, c_int, vp, i64, c_int, i64, u32]
+    lib.fda_create_with.restype = c_int
     lib.fda_context_info.argtypes = [vp, vp]
     lib.fda_context_info.restype = c_int
     lib.fda_destroy.argtypes = [vp]
@@ -155,8 +158,9 @@ class FdaContext:
     """Owner of an ``fda_ctx``.  Methods mirror the C entry points one to one."""
 
     def __init__(self, l: int, m: int, hash_coeffs, d_max: int, K_max: int, device: int = 0,
-                 schedule_limit_bytes: int | None = None):
-        """``schedule_limit_bytes``: None calls ``fda_create``; a number calls ``fda_create_limited``."""
+                 schedule_limit_bytes: int | None = None, one_schedule: bool = False):
+        """``schedule_limit_bytes``: None calls ``fda_create``; a number calls ``fda_create_limited``.
+        ``one_schedule``: ``fda_create_with`` and FDA_CREATE_ONE_SCHEDULE."""
         self._lib = load_library()
         self._h = ctypes.c_void_p()
         coeffs = None
@@ -166,7 +170,10 @@ class FdaContext:
                 raise ValueError("hash_coeffs must hold 6*l values")
         self._coeffs = coeffs
         ptr = coeffs.ctypes.data_as(ctypes.c_void_p) if coeffs is not None else None
-        if schedule_limit_bytes is None:
+        if one_schedule:
+            st = self._lib.fda_create_with(ctypes.byref(self._h), device, l, m, ptr, d_max, K_max,
+                                           int(schedule_limit_bytes or 0), FDA_CREATE_ONE_SCHEDULE)
+        elif schedule_limit_bytes is None:
             st = self._lib.fda_create(ctypes.byref(self._h), device, l, m, ptr, d_max, K_max)
         else:
             st = self._lib.fda_create_limited(ctypes.byref(self._h), device, l, m, ptr, d_max, K_max,

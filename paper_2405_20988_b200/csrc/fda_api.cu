@@ -180,8 +180,15 @@ fda_status fda_create(fda_ctx **out, int device, int l, int m, const uint64_t *h
 fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uint64_t *hash_coeffs,
                               int64_t d_max, int K_max, int64_t schedule_limit_bytes)
 {
+    return fda_create_with(out, device, l, m, hash_coeffs, d_max, K_max, schedule_limit_bytes, 0u);
+}
+
+fda_status fda_create_with(fda_ctx **out, int device, int l, int m, const uint64_t *hash_coeffs,
+                           int64_t d_max, int K_max, int64_t schedule_limit_bytes, uint32_t flags)
+{
     if (!out) return FDA_ERR_INVALID_ARG;
     *out = nullptr;
+    if (flags & ~(uint32_t)FDA_CREATE_ONE_SCHEDULE) return FDA_ERR_INVALID_ARG;
     if (l < 0 || l > FDA_MAX_ROWS) return FDA_ERR_INVALID_ARG;
     if (l > 0 && (m < 1 || m > 32768 || !hash_coeffs)) return FDA_ERR_INVALID_ARG;
     if (d_max < 1 || d_max >= (int64_t)1 << 31 || K_max < 1) return FDA_ERR_INVALID_ARG;
@@ -227,7 +234,7 @@ fda_status fda_create_limited(fda_ctx **out, int device, int l, int m, const uin
         if (e == cudaSuccess && schedule_limit_bytes >= 0) {
             const auto t0 = std::chrono::steady_clock::now();
             e = fda_build_list_schedule(ctx, nullptr);
-            if (e == cudaSuccess && ctx->sched) e = fda_build_lane_schedule(ctx, nullptr);
+            if (e == cudaSuccess && ctx->sched && !(flags & FDA_CREATE_ONE_SCHEDULE)) e = fda_build_lane_schedule(ctx, nullptr);
             ctx->sched_build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
         if (e == cudaSuccess) e = cudaMalloc(&ctx->part_sk, sizeof(float) * ctx->part_sk_floats);

@@ -49,6 +49,13 @@ def test_null_and_range_checks_need_no_device(lib):
     assert lib.fda_local_state(None, None, 0, 0, 0, None, None, 0, None, None) == 1
 
 
+def test_unknown_creation_flags_are_refused(lib):
+    h = ctypes.c_void_p()
+    for flags in (2, 3, 0x80000000):
+        assert lib.fda_create_with(ctypes.byref(h), 0, 0, 0, None, 100, 2, 0, flags) == 1 and not h.value
+    assert lib.fda_create_with(None, 0, 0, 0, None, 100, 2, 0, 1) == 1
+
+
 def test_no_cpu_fallback_without_a_device():
     import torch
     if torch.cuda.is_available():

@@ -185,3 +185,32 @@ def test_a_second_schedule_that_does_not_fit_is_reported():
         st = torch.empty((K, ctx.state_len), device="cuda")
         ctx.fda_local_state(torch.ones((K, d), device="cuda"), torch.zeros(d, device="cuda"), None, 5, st)
         assert ctx.fda_debug_last_schedule() == 1
+
+
+def test_the_second_schedule_can_be_left_out():
+    import torch
+    import fda_synth as S
+    import paper_2405_20988_b200 as F
+    l, m, d, K = 5, 250, 800_000, 60
+    coeffs = S.hash_coefficients(3, l)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    w0 = torch.randn(d, device="cuda", generator=gen) * 0.05
+    w = w0 + torch.randn((K, d), device="cuda", generator=gen) * 1e-3
+    xi = torch.randn(d, device="cuda", generator=gen)
+    got = []
+    for one in (True, False):
+        with F.FdaContext(l, m, coeffs, d_max=d, K_max=K, one_schedule=one) as ctx:
+            info = ctx.fda_context_info()
+            assert info["list_kernel"] == 1 and info["schedule_dropped_bytes"] == 0
+            st, xi_st = (torch.empty((K, ctx.state_len), device="cuda") for _ in range(2))
+            mean = torch.empty(ctx.state_len, device="cuda")
+            ctx.fda_local_state(w, w0, None, 5, st)
+            assert ctx.fda_debug_last_schedule() == (1 if one else 2)
+            ctx.fda_local_state(w, w0, xi, 7, xi_st)
+            ctx.fda_mean_state(w, w0, xi, 7, mean)
+            got.append((info["schedule_bytes"], st.cpu().numpy(), xi_st, mean))
+    assert got[0][0] == schedule_bytes(F, l, m, coeffs, d, 4) < got[1][0]
+    check_states(got[0][1], got[1][1].astype(np.float64), l, m, d)
+    assert torch.equal(got[0][2], got[1][2]) and torch.equal(got[0][3], got[1][3])
+    with F.FdaContext(l, m, coeffs, d_max=d, K_max=K, one_schedule=True, schedule_limit_bytes=-1) as ctx:
+        assert ctx.fda_context_info()["list_kernel"] == 0
