@@ -733,17 +733,29 @@ static int list_tile_indices(const fda_ctx *ctx, int rows, int min_len, int *ni_
     return 0;
 }
 
-// Walker warps for `items` items: as many as leave the fewest lanes without a cell, and of those that leave
-// equally many the fewest (every other warp produces).  Measured, K = 8, d = 20M, us with 12 / 20 / 22 / 23 / 24 walkers:
-// 24 items 184 / 196 / 193 / 205 / 211; 40: 303 / 214 / 215 / 226 / 234; 48: 320 / 283 / 289 / 287 / 252; 56: 385 / 286 / 297 /
-// 298 / 312; 64: 484 / 382 / 314 / 317 / 332; 80: 324 / 253 / 244 / 242 / 256; 112: - / 353 / 355 / 314 / 330.
-static int lane_walkers(int items)
+// Walker warps for a block's `items` items of `rows` sketch rows (every other warp of 28 to 32 produces).
+// Up to three rows the producers set the pace: no more than 20 walkers beside 12 of them.  Measured, K = 8, d = 20M, us with
+// 12 / 16 / 20 / 23 / 24 walkers: 3 x 250 (24 items) 158 / 156 / 185 / 204 / 214; 2 x 320 (20) 142 / 142 / 156 / 197 / 197; 3 x 320 (30)
+// 179 / 160 / 164 / 201 / 207; 3 x 500 (48) 187 / 177 / 173 / 207 / 211; 2 x 1000 (64) 203 / 183 / 168 / 199 / 197; 3 x 800 (75) 248 / 216 /
+// 187 / 211 / 209.  From four rows on the walk does: one item to a warp where 12, 16 or 20 warps have that, two up to
+// 32 items, beyond that as many warps as leave the fewest lanes without a cell, and of those that leave equally
+// many the fewest; from 61 items on 20 are too few.  4 x 100 (16 items) 246 / 203 / 209 / 224 / 226; 8 x 64 (16) 373 / 289 / 310 / 299 / 296;
+// 5 x 128 (20) 221 / 239 / 199 / 230 / 231; 8 x 96 (24) 279 / 287 / 373 / 361 / 277; 5 x 160 (25) 244 / 205 / 258 / 249 / 245; 5 x 250 (40) 241 /
+// 232 / 207 / 224 / 229; 6 x 200 (42) 287 / 278 / 300 / 244 / 252; 6 x 250 (48) 254 / 252 / 279 / 275 / 246; 7 x 250 (56) 309 / 310 / 283 /
+// 286 / 297; 5 x 400 (65) 330 / 306 / 273 / 231 / 234; 5 x 500 (80) 299 / 262 / 240 / 227 / 229; 6 x 500 (96) - / 321 / 285 / 273 / 256;
+// 7 x 500 (112) - / 366 / 322 / 290 / 310; 8 x 500 (128) - / - / 394 / 354 / 362.  It misses by up to 6 % at 4 x 350 (44 items, 216 with 23,
+// 205 with 16) and 2 x 640 (40, 168 with 20, 158 with 16).
+static int lane_walkers(int rows, int items)
 {
+    if (rows > 3)
+        for (int w : {12, 16, 20})
+            if (items <= w) return w;
     if (items <= 24) return 12;
     if (items <= 32) return 16;
-    int best = 0;
-    for (int w : {20, 23, 24})
-        if ((items + w - 1) / w <= 7 && (best == 0 || (items + w - 1) / w * w < (items + best - 1) / best * best)) best = w;
+    if (rows <= 3) return 20;
+    int best = items <= 60 ? 20 : 23;
+    for (int w : {23, 24})
+        if ((items + w - 1) / w * w < (items + best - 1) / best * best) best = w;
     return best;
 }
 
@@ -892,7 +904,7 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
         ctx->lane_records = total;
         ctx->lane_bytes = total + prog_bytes + sizeof(uint64_t) * (tiles + 1) + sizeof(int2) * ctx->l;
         ctx->lane_T = T; ctx->lane_parts = parts; ctx->lane_tiles = part_tiles;
-        ctx->lane_items = lane_items; ctx->lane_walkers = lane_walkers(lane_items);
+        ctx->lane_items = lane_items; ctx->lane_walkers = lane_walkers(p.l, lane_items);
         return cudaSuccess;
     }
     cudaFree(rows);

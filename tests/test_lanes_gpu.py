@@ -62,6 +62,18 @@ def test_sketches(l, m, K, d, aligned):
     check(l, m, K, d, S.hash_coefficients(3, l), aligned, l * m + d)
 
 
+# the split of the warps: 12, 16, 20, 23 or 24 walkers with one item each and more (the first hash that is even)
+@pytest.mark.parametrize("l,m", [(4, 64), (4, 96), (4, 128), (5, 128), (3, 200), (7, 96), (5, 160), (4, 288), (6, 200), (6, 250), (3, 500),
+                                 (5, 384), (4, 500), (6, 384), (2, 1000), (3, 800), (5, 500), (6, 500), (8, 480), (4, 1000), (8, 560)])
+@pytest.mark.parametrize("K,d,aligned", [(57, 900_001, False)])
+def test_every_split_of_the_warps(l, m, K, d, aligned):
+    import fda_synth as S
+    import paper_2405_20988_b200 as F
+    few = [schedule_bytes(F, l, m, S.hash_coefficients(s, l), d, k) for s in range(20) for k in (4, K)]
+    seed = next(s for s in range(20) if few[2 * s + 1] > 3 * few[2 * s] // 2)
+    check(l, m, K, d, S.hash_coefficients(seed, l), aligned, l * m + d)
+
+
 @pytest.mark.parametrize("kind,even", [("one bucket", False), ("short period", False), ("index mod m", True)])
 def test_uneven_hashes(kind, even):
     import fda_synth as S
