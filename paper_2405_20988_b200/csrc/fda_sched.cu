@@ -771,9 +771,13 @@ static int lane_geometry(const fda_ctx *ctx, int *parts_out, int *ni_max_out)
     if (T < 10 * m) T += kListBatch;
     while (T > 56 * m && T > 2 * kListBatch) T -= kListBatch;
     if (T < 5 * m || T > 56 * m) return 0;
-    // where a quarter of the lanes would have no cell and the walk is most of the work, the list kernel is as fast
-    // (8 x 100: 380 us, 390 here; 3 x 100: 216 and 193)
-    if (m < 128 && ctx->l >= 6 && (m + kListSlots - 1) / kListSlots * kListSlots * 5 > 6 * m) return 0;
+    // Where a quarter of the lanes would have no cell, or lists that come near their limit leave tiles of two batches, the list
+    // kernel is as fast or faster up to twelve rows.  Measured, K = 8, d = 20M, us, list kernel and this one: of the 96 lanes of
+    // 65 columns 31 idle, 3 x 65 212 and 219, 5 x 65 331 and 350, 8 x 65 387 and 398; 12 x 70 558 and 567; tiles of two batches:
+    // 3 x 48 212 and 231, 8 x 50 420 and 458, 5 x 50 281 and 275; but 16 x 65 777 and 660, 16 x 44 779 and 699.  On the other side of
+    // the line 3 x 72 208 and 206, 8 x 72 373 and 354, 8 x 97 391 and 325, 8 x 100 387 and 328, 3 x 100 206 and 177,
+    // 5 x 56 275 and 238, 8 x 56 400 and 379.
+    if (m < 128 && ctx->l <= 12 && ((m + kListSlots - 1) / kListSlots * kListSlots * 3 > 4 * m || T < 3 * kListBatch)) return 0;
     for (int parts = 1; parts <= 4; parts *= 2) {
         if (ctx->l % parts) break;
         const int rows = ctx->l / parts, items = rows * ((m + kListSlots - 1) / kListSlots);

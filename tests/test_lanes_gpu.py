@@ -74,6 +74,19 @@ def test_every_split_of_the_warps(l, m, K, d, aligned):
     check(l, m, K, d, S.hash_coefficients(seed, l), aligned, l * m + d)
 
 
+# both sides of the line for narrow sketches: lanes without a cell, tiles of two batches, and rows
+@pytest.mark.parametrize("l,m,lanes", [(8, 71, False), (8, 72, True), (5, 54, False), (5, 55, True), (12, 65, False), (13, 65, True), (8, 100, True)])
+def test_narrow_sketches(l, m, lanes):
+    import fda_synth as S
+    import paper_2405_20988_b200 as F
+    K, d = 60, 700_001
+    both = [schedule_bytes(F, l, m, S.hash_coefficients(s, l), d, k) for s in range(20) for k in (4, K)]
+    even = [s for s in range(20) if both[2 * s + 1] > 3 * both[2 * s] // 2]
+    assert (len(even) > 0) == lanes
+    seed = even[0] if lanes else 3
+    check(l, m, K, d, S.hash_coefficients(seed, l), True, l * m, lanes)
+
+
 @pytest.mark.parametrize("kind,even", [("one bucket", False), ("short period", False), ("index mod m", True)])
 def test_uneven_hashes(kind, even):
     import fda_synth as S
