@@ -411,12 +411,16 @@ cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t 
     // shifted pointers: first one block for each of the first `extra` groups, then the other groups
     // on as many blocks each as fit.  The main launch stops at tile t1; all launches write their own
     // slots of the partial sums.  Taken when the second of those launches still has a block per group
-    // and the job is long enough for the gain (tiles / cpg against t1 / cpg tile walks) to show.
+    // and the job is long enough for the gain (tiles / cpg against t1 / cpg tile walks) to show: where a block saves more than two
+    // walks, from 36 tiles a block on with lanes that keep their cells.  Measured, K = 60, one launch and three, by tiles a
+    // block: 3 x 100 32: 133.6 and 134.7 us, 36: 148.0 and 140.8; 5 x 250 40: 186.8 and 185.7, 48: 219.6 and 214.5; 7 x 500 40: 260.4 and
+    // 253.6, 48: 307.8 and 296.5; 8 x 250 40: 271.0 and 257.5; 1 x 250 40: 115.2 and 116.2, 44: 125.4 and 122.4.  The other kernel would
+    // gain from 40 on (5 x 250 221.7 and 214.4, 7 x 500 322.9 and 306.5) but keeps 64 and with it the order of its additions.
     const int extra = ctx->n_sm - blocks;
     const int rest = p.groups - extra;                         // groups of the second tail launch (extra < groups)
     int64_t t1 = p.tiles;
     int cpg_b = 0;
-    if (sched_parts == 1 && extra > 0 && rest > 0 && extra / rest >= 1 && ctx->side_stream && p.tiles >= (lanes ? 48 : 64) * (int64_t)p.cpg) {
+    if (sched_parts == 1 && extra > 0 && rest > 0 && extra / rest >= 1 && ctx->side_stream && p.tiles >= (lanes ? 36 : 64) * (int64_t)p.cpg) {
         cpg_b = extra / rest;
         // tail walks per block: n_tail + n_tail / cpg_b; main walks per block: (tiles - n_tail) / cpg
         const double per_tail = 1.0 + 1.0 / (double)cpg_b;

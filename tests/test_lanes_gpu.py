@@ -128,6 +128,28 @@ def test_calls_below_the_limits_of_the_context(l, m, d, aligned):
             check_states(st[rows].cpu().numpy(), ora, l, m, n)
 
 
+# tiles to a block below the line from which the idle SMs get the last tiles, and behind it
+@pytest.mark.parametrize("tiles,launches", [(35, 2), (40, 4), (41, 4)])
+def test_line_of_the_tail_launches(tiles, launches):
+    import torch
+    import oracle
+    import fda_synth as S
+    import paper_2405_20988_b200 as F
+    l, m, K, coeffs = 5, 250, 60, S.hash_coefficients(3, 5)
+    d = tiles * 9 * 6144 - 3
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    w0 = torch.randn(d, device="cuda", generator=gen) * 0.05
+    w = torch.empty((K, d + 3), device="cuda")[:, :d]
+    w.copy_(w0 + torch.randn((K, d), device="cuda", generator=gen) * 1e-3)
+    with F.FdaContext(l, m, coeffs, d_max=d, K_max=K) as ctx:
+        st = torch.full((K, ctx.state_len), float("nan"), device="cuda")
+        ctx.fda_local_state(w, w0, None, 5, st)
+        assert (ctx.fda_debug_last_schedule(), ctx.fda_debug_last_launches()) == (2, launches)
+        rows = [0, 51, 52, 59]
+        ora = oracle.local_state(w[rows].cpu().numpy(), w0.cpu().numpy(), None, coeffs, l, m, threads=8)
+        check_states(st[rows].cpu().numpy(), ora, l, m, d)
+
+
 # NaN and infinity of one worker show in its norm and in one cell of every row, and nowhere else
 @pytest.mark.parametrize("l,m,K,d", [(5, 250, 60, 900_001), (8, 1000, 57, 600_000)])
 @pytest.mark.parametrize("lanes", [True, False])
