@@ -88,15 +88,17 @@ typedef struct {
  *   - the list schedule of the sketch kernel, when the sketch allows one (tiles of at least 6*m
  *     indices fit the shared memory, or of 5*m with the rows in two or four equal parts).  Per index of d_max
  *     it takes 2.4 * l bytes at m = 250 (2.4 GB for d_max = 2 * 10^8 and l = 5), 2.8 * l at m = 500 and 3.1 to
- *     3.6 * l at m = 1000, and it is built here: per million indices and sketch row in 0.22 ms at m = 250,
- *     0.4 at m = 500 and 0.65 at m = 1000 (5 x 250: 1.1 ms per million indices, 8 x 1000, whose rows are in two
- *     parts: 5.1), about twice that for vectors of a million indices and less.  It is dropped, and sketch
+ *     3.6 * l at m = 1000, and it is built here: per million indices and sketch row in 0.11 to 0.15 ms at
+ *     m = 250, 0.2 at m = 500 and 0.4 at m = 1000 (5 x 250: 0.6 to 0.8 ms per million indices, 8 x 1000, whose rows
+ *     are in two parts: 3.3), two to three times that for vectors of a million indices and less; meanwhile it takes
+ *     another twentieth to seventh of the schedule's size.  It is dropped, and sketch
  *     requests are then served by the slower plain-load kernels, when it would take more than a third of the
  *     free device memory (see fda_create_limited for another cap);
  *   - a second schedule of about the same size for contexts of long vectors (more than twelve tiles of 5120 to 7168
  *     indices to a block of the sketch kernel at K_max workers: d_max above 11 million for K_max = 8, 1.4
- *     million for 30) whose hash spreads the indices of a tile evenly over the cells: it makes fda_local_state
- *     without a projection a fifth faster and takes half as long to build as the first; it is left out
+ *     million for 30) whose hash spreads the indices of a tile evenly over the cells (93 to 98 % of random hashes at
+ *     3 x 100 to 8 x 1000): it makes fda_local_state without a projection about a fifth faster and takes two thirds
+ *     as long to build as the first (a third at 8 x 1000); it is left out
  *     when it would take more than a third of the memory that is free then, or on request (fda_create_with);
  *   - lazily, by the first call that needs them: a 16-bit hash table of 2*l bytes per index
  *     (sketch requests on a context without a schedule), d_max floats (fda_mean_state on
@@ -125,8 +127,8 @@ enum { FDA_CREATE_ONE_SCHEDULE = 1 };
 
 /*
  * fda_create_limited with flags (the paper has no counterpart).  FDA_CREATE_ONE_SCHEDULE leaves the second list
- * schedule out: about half the memory and two thirds of the time that the schedules of a context of long vectors
- * take, for programs that do not call fda_local_state without a projection on them (LinearFDA, fda_mean_state,
+ * schedule out, half the memory and a quarter to two fifths of the time that the schedules of a context of long vectors
+ * take (5 x 250, d = 198M: 4.9 GB and 161 ms with both, 2.5 GB and 102 ms with one), for programs that do not call fda_local_state without a projection on them (LinearFDA, fda_mean_state,
  * fda_average_models) or would rather have the memory than the fifth of that call's time.
  * Errors: as fda_create, plus INVALID_ARG for an unknown flag.
  */
@@ -163,7 +165,10 @@ const char *fda_last_error(const fda_ctx *ctx);
  *   flags       OR of FDA_STATE_*; FDA_STATE_SKETCH needs l > 0
  *   states      out, K x state_len floats
  * Any alignment of w, w_t0, xi is accepted; 16-byte aligned pointers with row_stride a
- * multiple of 4 take the vector path.  Errors: INVALID_ARG (NULL, K < 1 or > K_max, d < 1
+ * multiple of 4 take the vector path.  On a context with a second list schedule a long vector's sketch is a
+ * fifth faster without a projection (xi == NULL or no FDA_STATE_LINEAR) than with one: the call with xi walks the
+ * first schedule, in the same order of additions as on short vectors.  Pass xi only in calls whose projection is used.
+ * Errors: INVALID_ARG (NULL, K < 1 or > K_max, d < 1
  * or > d_max, row_stride < d, unknown flag, SKETCH without a sketch), UNSUPPORTED (a sketch for more
  * workers than the context's partial-sum scratch holds: K above 32 x the SM count, or above 4 x the SM
  * count x the copies of the l*m bins that fit the shared memory when fewer than eight do; nothing is

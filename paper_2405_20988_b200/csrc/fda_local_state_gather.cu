@@ -54,15 +54,19 @@
 // stop between items all at once.  The order of the cells of a row is chosen so that the lists of eight neighbours are
 // copies of one another shifted by an odd number of indices (fda_sched.cu): as long as one another, and spread over
 // the bank groups; steps per entry 1.12 at 5 x 250, 1.19 at 7 x 500 (list kernel 1.16 and 1.23).  Walkers 12 to 24
-// of 28 to 32 warps, so that no lane is without a cell where that can be had; the others produce.  Measured, the
+// of 28 to 32 warps (lane_walkers in fda_sched.cu); the others produce.  Measured, the
 // list kernel and this one: 5 x 250, K = 8, d = 198M 2322 and 1860 us (2500 and 2218 us after half a second, at the
 // power limit); K = 30, d = 7M 347 and 283; 7 x 500, K = 60, d = 20M 2560 and 2022; 8 x 1000, K = 20, d = 2.6M 203 and
-// 166; K = 8, d = 20M: 1 x 250 191 and 128, 8 x 250 343 and 309, 4 x 1000 412 and 240.
+// 166; K = 8, d = 20M: 1 x 250 181 and 128, 3 x 500 218 and 173, 4 x 1000 394 and 241.  The gain depends on the hash (steps
+// per entry) and on the clock: 7 x 500, K = 60 came to 12 to 25 % on different GPUs.
 //
 // Its line: states without a projection, blocks of more than twelve tiles.  Shorter vectors gain little (K = 10,
-// d = 1.2M, four tiles: 33.3 and 31.2 us) for a second schedule in fda_create.  With xi the list kernel stays, although it
-// is slower there too: such a call keeps the order of its additions.  Right after a synchronisation the mean
-// drift is the rounding of the average itself, and the row norms of S-bar then show that order from the fourth digit on.
+// d = 1.2M, four tiles: 33.3 and 31.2 us) for a second schedule in fda_create.  With xi the list kernel stays, a
+// fifth slower on long vectors: what it gives is one order of additions for all sizes, so the digits of a run that projects do
+// not depend on which side of the line its vectors are.  That order shows right after a synchronisation, when the mean
+// drift is the rounding of the average itself: the row norms of S-bar then differ from the fourth digit on.  They are
+// rounding noise on either kernel (the cells are equally far from 64 bits, 1.2e-7 of their norm); runs without a projection
+// took the other order, and the speed.
 //
 // fda_mean_state_gather.cu holds the sibling of this kernel that computes the averaged state of
 // fda_mean_state from the list schedule.
