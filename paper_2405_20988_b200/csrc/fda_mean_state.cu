@@ -357,8 +357,7 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
     //   and 132, K = 16 137 both; 10 x 250, K = 20 3 % and 16 x 250, K = 20 10 % faster in one.
     // Where sketches of many rows lose by it (7 x 250, K = 12 and 16 x 250, K = 32 6 to 8 %, 16 x 100 10 to 15 %) the call
     // stays in one pass, which allocates nothing.
-    // From the averaged drifts that phase 1 below leaves in memory when the sketch is too large for the lane-private
-    // bins of k_sketch_vector_rows.
+    // From the averaged drifts that phase 1 below leaves in memory otherwise.
     ctx->last_schedule = 0;
     const bool lists = sketch && ctx->sched != nullptr, rows_kernel = ctx->columns == 32;
     const int64_t tiles = lists ? (d + ctx->sched_T - 1) / ctx->sched_T : 0;
@@ -386,7 +385,13 @@ cudaError_t fda_launch_mean_state(fda_ctx *ctx, const float *w, int64_t row_stri
     if (e != cudaSuccess) return e;
 
     // phase 2: sketch of u-bar
-    if (lists && !rows_kernel) {
+    // The lists take it from k_sketch_vector_rows, too, where they are short, the rows few and no SM has more than a
+    // tile.  Measured, all kernels, K = 20, d = 60K / 252K / 850K, lane-private bins and lists: 1 x 250 10.5 and 10.1 us / 12.7 and 11.6 /
+    // 21.2 and 17.8; 3 x 500 12.8 and 10.4 / 14.7 and 12.0 / 25.6 and 23.6; 5 x 200 11.1 and 11.0 / 13.6 and 12.5 / 24.6 and 24.4;
+    // 5 x 250, d = 60K 11.8 and 10.7, 500K 18.0 and 15.6; 6 x 250 11.6 and 11.1 / 14.1 and 12.7 / 26.1 and 25.3; but 4 x 100 9.7
+    // and 11.5 / 11.7 and 13.0, 8 x 200 11.2 and 14.1 / 13.7 and 15.7, 16 x 100 11.9 and 15.0.  On longer vectors 5 x 250 would still
+    // gain 3 to 8 %, 4 x 250 lose 4 and 3 x 100 10.
+    if (lists && (!rows_kernel || (ctx->m >= 200 && ctx->l <= 6 && tiles <= ctx->n_sm))) {
         e = fda_launch_mean_sketch_gather(ctx, ctx->mean_model, K, d, linear, flags, (int)nblk, mean_state, s);
         if (e != cudaErrorNotSupported) {
             if (e == cudaSuccess) { ctx->last_ls_kernel = "k_mean_model + k_mean_state_gather"; ctx->last_schedule = 1; }

@@ -21,15 +21,18 @@
 //     with zeros for what lies past the end;
 //   * 8 producer and 24 walker warps at 64 registers.
 //
-// Two callers: the K rows of w (one pass, any number of workers), or the single row of averaged drifts
-// that k_mean_model has left in device memory (no w_t0; the two scalars then come from that
-// kernel's partial sums).  Measured on B200, 5 x 250, K = 8, d = 198M, one pass: 1.50 ms (0.73 of
+// Measured on B200, 5 x 250, K = 8, d = 198M, one pass: 1.50 ms (0.73 of
 // the measured copy bandwidth).  On the way: loads landing in registers four rows at a time with
 // a four-column tile and 12 + 16 warps 2.15 ms; single-column tile 2.07; landing zone with 8 + 20
 // warps 1.73, with 8 + 24 warps 1.67 (6 + 26: 1.86; 12 + 16: 2.01; 4 + 24: 2.12; depth capped at
 // 3 / 2: 1.76 / 1.95); without the L2 prefetch of the next tiles' rows that the per-worker kernel
 // issues, 1.56; with every shared-memory region on a 128-byte boundary, 1.50.  7 x 500, K = 60,
 // d = 20M, where the drifts used to be averaged in a pass of their own first: 0.93 -> 0.82 ms.
+//
+// k_mean_sketch_short, below, walks the same schedule over the single row of averaged drifts that k_mean_model has
+// left in device memory (the two scalars are then that kernel's).
+
+#include <algorithm>
 
 #include "fda_internal.h"
 #include "fda_list_kernel.cuh"
@@ -47,9 +50,7 @@ constexpr int kMaxDepth = 8;
 constexpr int kMaxPiece = 10;                  // rows of a landing-zone slot
 
 struct MeanParams {
-    ListParams q;                    // rows, schedule, partial-sum buffers; q.K = rows that are read
-    int base_zero;                   // the rows are drifts already (no w_t0 to subtract)
-    int sketch_only;                 // leave part_np alone
+    ListParams q;                    // rows, schedule, partial-sum buffers
     int piece;                       // rows of a landing-zone slot: a quad of K rows arrives in K / piece slots
     int depth;                       // slots a producer thread keeps in flight (1 .. kMaxDepth)
 };
@@ -94,6 +95,30 @@ __device__ __forceinline__ void gather1(uint32_t e, uint32_t base, float &a)
     a += __uint_as_float(__float_as_uint(u) ^ ((e & 0x8000u) << 16));
 }
 
+// one chunk of an item: the steps that are left of it, at most four
+__device__ __forceinline__ void gather1_chunk(const uint2 &ch, int left, uint32_t base, float &a)
+{
+    if (left >= 4) {
+        gather1(ch.x & 0xffffu, base, a);
+        gather1(ch.x >> 16, base, a);
+        gather1(ch.y & 0xffffu, base, a);
+        gather1(ch.y >> 16, base, a);
+    } else if (left > 0) {
+        gather1(ch.x & 0xffffu, base, a);
+        if (left > 1) gather1(ch.x >> 16, base, a);
+        if (left > 2) gather1(ch.y & 0xffffu, base, a);
+    }
+}
+// the sum of a lane's list into the bins
+__device__ __forceinline__ void flush1(float *bins, int lm, uint32_t cell, float a)
+{
+    if ((cell & 0x7fffu) < (uint32_t)lm) {
+        float *b = bins + (cell & 0x7fffu);
+        if (cell & 0x8000u) atomicAdd(b, a);                // a cell with several lists
+        else *b += a;
+    }
+}
+
 // Shared-memory offsets: every region starts on a 128-byte boundary (the 16-byte stores and the
 // asynchronous copies need 16; with the landing zone 48 bytes off a 128-byte boundary the pass ran
 // 8 % slower).
@@ -117,7 +142,7 @@ inline size_t mean_smem_fixed(int l, int m, int T, int tab_bytes)
 //   then        the landing zone: depth slots of R rows of kRowPitch bytes
 // (each region on a 128-byte boundary)
 // AHEAD: entry chunks (four steps each) a walker loads before it walks them: eight, or five for the short
-// items of sketches of seven or more rows and of rows in parts (k_local_state_gather has a rule of its own).
+// items of sketches of seven or more rows (k_local_state_gather has a rule of its own).
 // MULTI: the rows of a quad arrive in several slots (more than kMaxPiece rows).
 // VEC: w, w_t0 and xi are 16-byte aligned.
 template <bool LINEAR, int AHEAD, bool MULTI, bool VEC>
@@ -165,7 +190,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
         // Slot s, row r: lz + (s * R + r) * kRowPitch, a thread's 16 bytes of it.  A slot
         // holds up to rp rows of w; the slot of a quad's first rows also w_t0 and xi, behind them.
         const int D = mp.depth, rp = MULTI ? mp.piece : p.K;
-        const int R = rp + (mp.base_zero ? 0 : 1) + (LINEAR ? 1 : 0);
+        const int R = rp + 1 + (LINEAR ? 1 : 0);
         const uint32_t lz = smem_base + lz_off + (uint32_t)pt * 16u;
         int left_i = (int)n_tiles * p.nb;                     // quads of this thread that are still to be asked for,
         int b_i = 0, k_i = 0;                                 // the next one's batch in the tile and first row
@@ -204,8 +229,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
                 copy(dst, p.w + (int64_t)k_i * p.row_stride, MULTI ? min(rp, p.K - k_i) : rp);
                 if (k_i == 0) {
                     dst += (uint32_t)rp * kRowPitch;
-                    if (!mp.base_zero) { copy(dst, p.w_t0, 1); dst += kRowPitch; }
-                    if (LINEAR) copy(dst, p.xi, 1);
+                    copy(dst, p.w_t0, 1);
+                    if (LINEAR) copy(dst + kRowPitch, p.xi, 1);
                 }
                 if (MULTI) k_i += rp;
                 if (!MULTI || k_i >= p.K) {
@@ -229,9 +254,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
                     if (!VEC) __syncwarp();                    // (all lanes' parts of it)
                     const uint32_t src = lz + (uint32_t)(slot * R) * kRowPitch;
                     if (k0 == 0) {
-                        uint32_t q = src + (uint32_t)rp * kRowPitch;
-                        if (!mp.base_zero) { w0 = lds128(q); q += kRowPitch; }
-                        if (LINEAR) x = lds128(q);
+                        const uint32_t q = src + (uint32_t)rp * kRowPitch;
+                        w0 = lds128(q);
+                        if (LINEAR) x = lds128(q + kRowPitch);
                     }
                     const int m = MULTI ? min(rp, p.K - k0) : rp;
 #pragma unroll 4
@@ -324,25 +349,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
                     for (int q = 0; q < AHEAD; ++q)
                         if (c0 + q < nch) ch[q] = __ldg(ent + (size_t)(c0 + q) * kListSlots);
 #pragma unroll
-                    for (int q = 0; q < AHEAD; ++q) {
-                        const int left = steps - 4 * (c0 + q);
-                        if (left >= 4) {
-                            gather1(ch[q].x & 0xffffu, base, a);
-                            gather1(ch[q].x >> 16, base, a);
-                            gather1(ch[q].y & 0xffffu, base, a);
-                            gather1(ch[q].y >> 16, base, a);
-                        } else if (left > 0) {
-                            gather1(ch[q].x & 0xffffu, base, a);
-                            if (left > 1) gather1(ch[q].x >> 16, base, a);
-                            if (left > 2) gather1(ch[q].y & 0xffffu, base, a);
-                        }
-                    }
+                    for (int q = 0; q < AHEAD; ++q) gather1_chunk(ch[q], steps - 4 * (c0 + q), base, a);
                 }
-                if ((cell & 0x7fffu) < (uint32_t)lm) {
-                    float *b = bins + (cell & 0x7fffu);
-                    if (cell & 0x8000u) atomicAdd(b, a);                // a cell with several lists
-                    else *b += a;
-                }
+                flush1(bins, lm, cell, a);
             }
         }
     }
@@ -353,11 +362,109 @@ __global__ void __launch_bounds__(kThreads, 1) k_mean_state_gather(const MeanPar
         float *out = p.part_sk + (size_t)blockIdx.x * (size_t)lm;
         for (int t = tid; t < lm; t += kThreads) out[t] = bins[t];
     }
-    if (tid < 2 && !mp.sketch_only) {
+    if (tid < 2) {
         double t = 0.0;
         for (int q = 0; q < kPW; ++q) t += sums[q * 2 + tid];
         p.part_np[(size_t)blockIdx.x * 2 + tid] = t;
     }
+}
+
+// The sketch of one vector, the averaged drifts: no roles and no second buffer, a block's warps form its tile (24 KB, loaded
+// a tile ahead), then walk.  p.part_tiles blocks share a tile, each walking every p.part_tiles-th item; a block serves one part
+// of the sketch rows.
+// Bound: latency.  A row of the tile is one float, so a tile is formed in one round trip and walked in a few thousand
+// cycles; two small blocks to an SM cover each other's round trips, and a short vector gets more blocks than it has tiles.
+// The first item's entries are asked for in front of fda_grid_wait (the schedule is older than the kernel before this one).
+// Measured, all kernels of the averaged state back to back, K = 20, odd d, against 8 producer and 24 walker warps that served
+// this vector, too: 7 x 500 16.7 -> 12.4 us (d = 60K), 20.3 -> 19.1 (500K), 43.3 -> 38.8 (1.2M), 443 -> 437 (20M); 8 x 1000 in
+// parts, which are one launch now, 26.2 -> 12.4, 29.8 -> 21.1, 62.5 -> 49.9, 256 -> 243 (8M).  16 warps and two blocks to an
+// SM are the best of 8 / 4, 12 / 2, 16 / 1, 16 / 2 and 24 / 1 or within 5 % of it.
+constexpr int kShortWarps = 16, kShortPerSm = 2;
+constexpr int kShortQuads = (kListMaxTile / 4 + kShortWarps * 32 - 1) / (kShortWarps * 32);
+inline size_t mean_short_smem(int lm, int T) { return (size_t)align128((uint32_t)lm * 4u) + (size_t)(T + kListPadRows) * 4; }
+
+__global__ void __launch_bounds__(kShortWarps * 32, kShortPerSm) k_mean_sketch_short(const ListParams p)
+{
+    constexpr int kThreads = kShortWarps * 32, kAhead = 7;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int split = p.part_tiles, T = p.T, lm = p.l * p.m, tiles = (int)p.tiles;
+    // block = (sub * parts + part) * cpg + c: the tiles c, c + cpg, ...
+    const int c = (int)blockIdx.x % p.cpg, part = (int)blockIdx.x / p.cpg % p.groups, sub = (int)blockIdx.x / (p.cpg * p.groups);
+    const uint32_t ut_off = align128((uint32_t)lm * 4u), base = (uint32_t)__cvta_generic_to_shared(smem_raw) + ut_off;
+    float *bins = reinterpret_cast<float *>(smem_raw);
+
+    const uint64_t *sched_off = p.sched_off + (size_t)part * p.nb;
+    const uint32_t *tab = nullptr;
+    const uint16_t *cells = nullptr;
+    const unsigned char *ent0 = nullptr;
+    int it = 0, n_items = 0, steps = 0;
+    uint32_t cell = 0;
+    const uint2 *ent = nullptr;
+    uint2 ch[kAhead];
+    auto ask = [&](int first) {                               // the chunks first .. first + kAhead - 1 of the item
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q)
+            if (4 * (first + q) < steps) ch[q] = __ldg(ent + (size_t)(first + q) * kListSlots);
+    };
+    auto fetch = [&]() {
+        const uint32_t d0 = __ldg(tab + 4 + 2 * it), chunk0 = __ldg(tab + 5 + 2 * it);
+        steps = (int)(d0 & 0xffffu);
+        cell = __ldg(cells + (size_t)(d0 >> 16) * kListSlots + lane);
+        ent = reinterpret_cast<const uint2 *>(ent0 + (size_t)chunk0 * 256) + lane;
+        ask(0);
+    };
+    auto open_tile = [&](int t) {
+        const unsigned char *rec = p.sched + load_u64(sched_off + t);
+        tab = reinterpret_cast<const uint32_t *>(rec);
+        n_items = (int)__ldg(tab);
+        cells = reinterpret_cast<const uint16_t *>(rec + fda_sched_cells_off(n_items));
+        ent0 = rec + fda_sched_entries_off(n_items);
+        it = warp * split + sub;
+        if (it < n_items) fetch();
+    };
+    float4 v[kShortQuads];
+    auto load_tile = [&](int t) {
+#pragma unroll
+        for (int u = 0; u < kShortQuads; ++u) {
+            const int q = tid + u * kThreads;
+            const int64_t j = (int64_t)t * T + 4 * q, left = q < T / 4 ? p.d - j : 0;
+            v[u] = load_quad<false>(p.w + j, left >= 4, left > 0 ? (int)left : 0);
+        }
+    };
+    open_tile(c);
+    for (int t = tid; t < lm; t += kThreads) bins[t] = 0.f;
+    if (tid < kListPadRows) reinterpret_cast<float *>(smem_raw + ut_off)[T + tid] = 0.f;
+    fda_grid_wait();
+    load_tile(c);
+    for (int t = c; t < tiles; t += p.cpg) {
+#pragma unroll
+        for (int u = 0; u < kShortQuads; ++u) {               // row r of the tile at r ^ ((r >> 3) & 3): the quad's floats permuted
+            const int q = tid + u * kThreads, sw = (q >> 1) & 3;
+            if (q < T / 4) store_row(base + 16u * q, comp(v[u], 0 ^ sw), comp(v[u], 1 ^ sw), comp(v[u], 2 ^ sw), comp(v[u], 3 ^ sw));
+        }
+        __syncthreads();
+        const bool more = t + p.cpg < tiles;
+        if (more) load_tile(t + p.cpg);
+        while (it < n_items) {
+            float a = 0.f;
+            for (int c0 = 0;;) {
+#pragma unroll
+                for (int q = 0; q < kAhead; ++q) gather1_chunk(ch[q], steps - 4 * (c0 + q), base, a);
+                c0 += kAhead;
+                if (4 * c0 >= steps) break;
+                ask(c0);
+            }
+            const uint32_t done = cell;
+            it += kShortWarps * split;
+            if (it < n_items) fetch();
+            flush1(bins, lm, done, a);
+        }
+        if (more) open_tile(t + p.cpg);
+        __syncthreads();
+    }
+    float *out = p.part_sk + ((size_t)part * p.cpg * split + sub * p.cpg + c) * lm;
+    for (int t = tid; t < lm; t += kThreads) out[t] = bins[t];
 }
 
 // Averaged state: mean_state[e] = (sum over the blocks of the partials) / divisor, in fp64 and in a
@@ -426,67 +533,17 @@ void (*pick_kernel(bool linear, bool multi, bool vec))(MeanParams)
     return linear ? k_mean_state_gather<true, AHEAD, false, true> : k_mean_state_gather<false, AHEAD, false, true>;
 }
 
-// rows == K: the averaged state of the K rows of w in one pass.  rows == 1 and base_zero: w is the
-// row of averaged drifts; the cells come from it, the two scalars from np_blocks partial pairs that
-// the averaging pass left at the start of ctx->part_np.
-cudaError_t launch_mean(fda_ctx *ctx, const float *w, int64_t row_stride, int rows, bool base_zero, int K, int64_t d,
-                        const float *w_t0, const float *xi, bool have_xi, uint32_t flags, int np_blocks,
-                        float *mean_state, cudaStream_t s)
+// What both passes need of the context and the call (l, m: of a part of the sketch rows)
+ListParams mean_params(const fda_ctx *ctx, const float *w, int64_t row_stride, int K, int64_t d)
 {
-    if (!(flags & FDA_STATE_SKETCH) || ctx->l == 0 || !ctx->sched) return cudaErrorNotSupported;
-    const float *xi_used = (!base_zero && (flags & FDA_STATE_LINEAR)) ? xi : nullptr;
-
-    MeanParams mp{};
-    ListParams &p = mp.q;
-    p.w = w; p.w_t0 = w_t0; p.xi = xi_used; p.row_stride = row_stride;
-    p.K = rows; p.d = d; p.have_xi = xi_used != nullptr;
-    mp.base_zero = base_zero;
-    mp.sketch_only = base_zero;
-    p.vec = ((((uintptr_t)w | (uintptr_t)(base_zero ? w : w_t0) | (uintptr_t)(xi_used ? xi_used : w)) & 15u) == 0) &&
-            (row_stride % 4 == 0);
-    const int parts = ctx->sched_parts;
-    if (parts > 1 && !base_zero) return cudaErrorNotSupported;      // every part would read the K rows again
-    p.l = ctx->l / parts; p.m = ctx->m;
-    const int lm = p.l * p.m;
+    ListParams p{};
+    p.w = w; p.row_stride = row_stride; p.K = K; p.d = d;
+    p.l = ctx->l / ctx->sched_parts; p.m = ctx->m;
     p.T = ctx->sched_T;
     p.sched = ctx->sched; p.sched_off = ctx->sched_off;
     p.part_sk = ctx->part_sk; p.part_np = ctx->part_np;
     p.tiles = (d + p.T - 1) / p.T;
-    p.tab_bytes = fda_list_table_bytes(ctx->sched_ni_max);
-    p.groups = 1;
-    int64_t cpg = ctx->n_sm;
-    if (cpg > p.tiles) cpg = p.tiles;
-    p.cpg = (int)cpg;
-    const int blocks = p.cpg;
-    if ((size_t)blocks * lm * parts > ctx->part_sk_floats || blocks > ctx->max_blocks ||
-        (size_t)blocks * 2 > ctx->part_np_doubles)
-        return cudaErrorNotSupported;
-    if (p.T % kBatch != 0 || kPW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
-    p.nb = p.T / kBatch;
-    // what the single-column tile leaves free becomes the producers' landing zone
-    const size_t fixed = mean_smem_fixed(p.l, p.m, p.T, p.tab_bytes);
-    // (up to kMaxPiece rows arrive in one slot, more of them in several of nearly equal size)
-    const int slots = (rows + kMaxPiece - 1) / kMaxPiece;
-    mp.piece = (rows + slots - 1) / slots;
-    const size_t per_slot = (size_t)kRowPitch * (size_t)(mp.piece + (base_zero ? 0 : 1) + (xi_used ? 1 : 0));
-    const size_t depth = (size_t)ctx->smem_optin > fixed ? ((size_t)ctx->smem_optin - fixed) / per_slot : 0;
-    // too little room to keep three slots per thread in flight: the pass would wait for its loads
-    if (depth < (size_t)(base_zero ? 1 : 3)) return cudaErrorNotSupported;
-    mp.depth = (int)(depth < (size_t)kMaxDepth ? depth : (size_t)kMaxDepth);
-    const size_t smem = fixed + (size_t)mp.depth * per_slot;
-
-    auto kern = p.l >= 7 || parts > 1 ? pick_kernel<5>(xi_used != nullptr, slots > 1, p.vec != 0)
-                                      : pick_kernel<kChunksAhead>(xi_used != nullptr, slots > 1, p.vec != 0);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
-    if (e != cudaSuccess) return e;
-    for (int part = 0; part < parts; ++part) {                       // (the row of averaged drifts is in L2)
-        p.sched_off = ctx->sched_off + (size_t)part * ctx->sched_tiles;
-        p.part_sk = ctx->part_sk + (size_t)part * blocks * lm;
-        e = fda_launch_dependent(kern, blocks, kThreads, smem, s, mp);
-        if (e != cudaSuccess) return e;
-    }
-    return fda_launch_finalize_mean(ctx, blocks, base_zero ? np_blocks : blocks, lm, K, flags, have_xi,
-                                    base_zero ? 1.0 : (double)K, mean_state, s);
+    return p;
 }
 
 }  // namespace
@@ -507,8 +564,41 @@ cudaError_t fda_launch_mean_state_gather(fda_ctx *ctx, const float *w, int64_t r
                                          int64_t d, const float *w_t0, const float *xi,
                                          uint32_t flags, float *mean_state, cudaStream_t s)
 {
-    const bool have_xi = (flags & FDA_STATE_LINEAR) && xi;
-    return launch_mean(ctx, w, row_stride, K, false, K, d, w_t0, xi, have_xi, flags, 0, mean_state, s);
+    if (!(flags & FDA_STATE_SKETCH) || ctx->l == 0 || !ctx->sched) return cudaErrorNotSupported;
+    const float *xi_used = (flags & FDA_STATE_LINEAR) ? xi : nullptr;
+    if (ctx->sched_parts > 1) return cudaErrorNotSupported;         // every part would read the K rows again
+
+    MeanParams mp{};
+    ListParams &p = mp.q;
+    p = mean_params(ctx, w, row_stride, K, d);
+    p.w_t0 = w_t0; p.xi = xi_used; p.have_xi = xi_used != nullptr;
+    p.vec = ((((uintptr_t)w | (uintptr_t)w_t0 | (uintptr_t)(xi_used ? xi_used : w)) & 15u) == 0) && (row_stride % 4 == 0);
+    p.tab_bytes = fda_list_table_bytes(ctx->sched_ni_max);
+    p.groups = 1;
+    p.cpg = (int)std::min((int64_t)ctx->n_sm, p.tiles);
+    const int blocks = p.cpg, lm = ctx->lm;
+    if ((size_t)blocks * lm > ctx->part_sk_floats || blocks > ctx->max_blocks || (size_t)blocks * 2 > ctx->part_np_doubles)
+        return cudaErrorNotSupported;
+    if (p.T % kBatch != 0 || kPW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
+    p.nb = p.T / kBatch;
+    // what the single-column tile leaves free becomes the producers' landing zone
+    const size_t fixed = mean_smem_fixed(p.l, p.m, p.T, p.tab_bytes);
+    // (up to kMaxPiece rows arrive in one slot, more of them in several of nearly equal size)
+    const int slots = (K + kMaxPiece - 1) / kMaxPiece;
+    mp.piece = (K + slots - 1) / slots;
+    const size_t per_slot = (size_t)kRowPitch * (size_t)(mp.piece + 1 + (xi_used ? 1 : 0));
+    const size_t depth = (size_t)ctx->smem_optin > fixed ? ((size_t)ctx->smem_optin - fixed) / per_slot : 0;
+    // too little room to keep three slots per thread in flight: the pass would wait for its loads
+    if (depth < 3) return cudaErrorNotSupported;
+    mp.depth = (int)(depth < (size_t)kMaxDepth ? depth : (size_t)kMaxDepth);
+    const size_t smem = fixed + (size_t)mp.depth * per_slot;
+
+    auto kern = p.l >= 7 ? pick_kernel<5>(xi_used != nullptr, slots > 1, p.vec != 0)
+                         : pick_kernel<kChunksAhead>(xi_used != nullptr, slots > 1, p.vec != 0);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
+    if (e == cudaSuccess) e = fda_launch_dependent(kern, blocks, kThreads, smem, s, mp);
+    if (e != cudaSuccess) return e;
+    return fda_launch_finalize_mean(ctx, blocks, blocks, lm, K, flags, xi_used != nullptr, (double)K, mean_state, s);
 }
 
 // The cells of S-bar from the vector of averaged drifts (d floats, 16-byte aligned), the scalars
@@ -516,6 +606,20 @@ cudaError_t fda_launch_mean_state_gather(fda_ctx *ctx, const float *w, int64_t r
 cudaError_t fda_launch_mean_sketch_gather(fda_ctx *ctx, const float *mean_drift, int K, int64_t d, bool have_xi,
                                           uint32_t flags, int np_blocks, float *mean_state, cudaStream_t s)
 {
-    return launch_mean(ctx, mean_drift, (d + 3) / 4 * 4, 1, true, K, d, nullptr, nullptr, have_xi, flags, np_blocks,
-                       mean_state, s);
+    if (!(flags & FDA_STATE_SKETCH) || ctx->l == 0 || !ctx->sched) return cudaErrorNotSupported;
+    ListParams p = mean_params(ctx, mean_drift, 0, 1, d);
+    const int parts = ctx->sched_parts, lm = p.l * p.m;
+    p.groups = parts;
+    p.nb = (int)ctx->sched_tiles;                                    // records of a part
+    p.cpg = (int)std::max((int64_t)1, std::min((int64_t)ctx->n_sm * kShortPerSm / parts, p.tiles));
+    // up to three blocks to a tile while each has an SM of its own
+    p.part_tiles = (int)std::max((int64_t)1, std::min((int64_t)3, ctx->n_sm / (p.tiles * parts)));
+    const int n = p.cpg * p.part_tiles;                              // partial sketches of a part
+    const size_t smem = mean_short_smem(lm, p.T);
+    if ((size_t)n * lm * parts > ctx->part_sk_floats || p.T > kShortQuads * kShortWarps * 32 * 4 || smem > (size_t)ctx->smem_optin)
+        return cudaErrorNotSupported;
+    cudaError_t e = cudaFuncSetAttribute(k_mean_sketch_short, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
+    if (e == cudaSuccess) e = fda_launch_dependent(k_mean_sketch_short, n * parts, kShortWarps * 32, smem, s, p);
+    if (e != cudaSuccess) return e;
+    return fda_launch_finalize_mean(ctx, n, np_blocks, lm, K, flags, have_xi, 1.0, mean_state, s);
 }
