@@ -94,10 +94,10 @@ typedef struct {
  *     another twentieth to seventh of the schedule's size.  It is dropped, and sketch
  *     requests are then served by the slower plain-load kernels, when it would take more than a third of the
  *     free device memory (see fda_create_limited for another cap);
- *   - a second schedule of about the same size for contexts of long vectors (more than twelve tiles of 5120 to 7168
- *     indices to a block of the sketch kernel at K_max workers: d_max above 11 million for K_max = 8, 1.4
+ *   - a second schedule of about the same size for contexts of long vectors (more than four tiles of 5120 to 7168
+ *     indices to a block of the sketch kernel at K_max workers: d_max above 1.8 million for K_max = 8, 0.45
  *     million for 30) whose hash spreads the indices of a tile evenly over the cells (93 to 98 % of random hashes at
- *     3 x 100 to 8 x 1000): it makes fda_local_state without a projection about a fifth faster and takes two thirds
+ *     3 x 100 to 8 x 1000): it makes fda_local_state without a projection a tenth to a fifth faster and takes two thirds
  *     as long to build as the first (a third at 8 x 1000); it is left out
  *     when it would take more than a third of the memory that is free then, or on request (fda_create_with);
  *   - lazily, by the first call that needs them: a 16-bit hash table of 2*l bytes per index

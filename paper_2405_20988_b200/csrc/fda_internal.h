@@ -108,8 +108,9 @@ struct fda_ctx {
     std::string err;
 };
 
-// Lanes that keep their cells: worth a schedule of their own, and used, when a block has more than twelve tiles.
-inline bool fda_lanes_pay(int64_t tiles, int groups, int n_sm) { return groups <= n_sm && tiles > 12 * (int64_t)(n_sm / groups); }
+// Lanes that keep their cells: worth a schedule of their own, and used, when a block has more than four tiles
+// (fda_local_state_gather.cu has the figures).
+inline bool fda_lanes_pay(int64_t tiles, int groups, int n_sm) { return groups <= n_sm && tiles > 4 * (int64_t)(n_sm / groups); }
 
 // Cell at place `pos` of the order (step, cycle) of a sketch row: the cells 0, step, 2 step, ... (mod m) up to the
 // end of the cycle, then those of the cycle through 1, and so on.

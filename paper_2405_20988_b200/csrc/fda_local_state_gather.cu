@@ -60,8 +60,12 @@
 // 166; K = 8, d = 20M: 1 x 250 181 and 128, 3 x 500 218 and 173, 4 x 1000 394 and 241.  The gain depends on the hash (steps
 // per entry) and on the clock: 7 x 500, K = 60 came to 12 to 25 % on different GPUs.
 //
-// Its line: states without a projection, blocks of more than twelve tiles.  Shorter vectors gain little (K = 10,
-// d = 1.2M, four tiles: 33.3 and 31.2 us) for a second schedule in fda_create.  With xi the list kernel stays, a
+// Its line: states without a projection, blocks of more than four tiles.  Measured with the finalize kernel, list kernel and
+// this one, by tiles a block: 5 x 250, K = 14, d = 1.2M (5.2) 38.2 and 34.9 us, K = 16, d = 1.6M (7) 44.8 and 40.0, K = 30, d = 0.7M
+// (6.3) 43.8 and 39.8; 3 x 100, K = 10, d = 1.5M (6) 28.5 and 25.8; 7 x 500, K = 44, d = 0.6M (7.9) 72.5 and 62.9, K = 20, d = 1M
+// (5.6) 54.7 and 50.8; 4 x 1000, K = 20, d = 1M (4.8) 60.0 and 43.4; 8 x 1000, K = 26, d = 0.3M (4.6) 47.2 and 42.2, K = 44, d = 0.3M
+// (6.8) 63 and 54.  That pays for the second schedule (1.2 to 1.9 ms of fda_create) after some 300 steps.  Shorter vectors gain
+// less (5 x 250, K = 10, d = 1.2M, four tiles: 28.7 and 27.0).  With xi the list kernel stays, a
 // fifth slower on long vectors: what it gives is one order of additions for all sizes, so the digits of a run that projects do
 // not depend on which side of the line its vectors are.  That order shows right after a synchronisation, when the mean
 // drift is the rounding of the average itself: the row norms of S-bar then differ from the fourth digit on.  They are
@@ -300,9 +304,10 @@ cudaError_t launch_lists(ListParams &p, int blocks, size_t smem, bool dependent,
     if (p.T % 128 != 0 || p.T < PW * 128 || PW * 32 * 16 < p.tab_bytes) return cudaErrorNotSupported;
     // all warps form the first tile when a block has at most twelve.  Measured, kernel and finalize back to back:
     // 5 x 250, K = 20, d = 300,000 (two tiles) 18.3 -> 17.4 us, K = 10, d = 1.2M (four) 34.1 -> 32.4 us; 7 x 500, K = 10,
-    // d = 1.2M (five) 46.0 -> 44.5 us; K = 20, d = 2M (twelve) 75.7 -> 75.3 us.
-    const bool first = !PARTS && p.tiles <= 12 * (int64_t)p.cpg;
-    auto kern = first ? pick_kernel<PW, WW, PARTS, !PARTS, 0>(p.have_xi != 0, p.vec != 0)
+    // d = 1.2M (five) 46.0 -> 44.5 us; K = 20, d = 2M (twelve) 75.7 -> 75.3 us.  Rows in parts: 8 x 1000, K = 20, d = 160K
+    // 26.2 -> 25.7 us, K = 40, d = 100K 28.4 -> 27.8 (with xi not: the norms' order of additions stays).
+    const bool first = !(PARTS && p.have_xi) && p.tiles <= 12 * (int64_t)p.cpg;
+    auto kern = first ? pick_kernel<PW, WW, PARTS, true, 0>(p.have_xi != 0, p.vec != 0)
                       : pick_kernel<PW, WW, PARTS, false, 0>(p.have_xi != 0, p.vec != 0);
     if (dependent) return fda_launch_dependent(kern, blocks, (PW + WW) * 32, smem, s, p);
     kern<<<blocks, (PW + WW) * 32, smem, s>>>(p);
@@ -326,7 +331,7 @@ cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx)
         const bool linear = i & 1, vec = i & 2;
         for (auto kern : {pick_kernel<8, 20, false, false, 0>(linear, vec), pick_kernel<5, 23, false, false, 0>(linear, vec),
                           pick_kernel<8, 20, false, true, 0>(linear, vec), pick_kernel<5, 23, false, true, 0>(linear, vec),
-                          pick_kernel<8, 20, true, false, 0>(linear, vec), pick_short(linear, vec)}) {
+                          pick_kernel<8, 20, true, false, 0>(linear, vec), pick_kernel<8, 20, true, true, 0>(false, vec), pick_short(linear, vec)}) {
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin);
             if (e != cudaSuccess) return e;
         }
