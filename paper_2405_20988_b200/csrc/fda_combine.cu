@@ -23,6 +23,10 @@ constexpr int kUnitThreads = kUnitColumns * kUnitSlices;
 // 3.73 (7 x 500, K = 1), 4.25 and 4.08 (3 x 100, K = 27); eleven 7.30 and 4.48 us (8 x 1000, K = 1).  Behind a sketch
 // pass the difference at four trips is lost in the chain (a round with 5 x 250, K = 10, d = 1.2M: 49.8 us with either).
 constexpr int kOneBlockTrips = 3;
+// Partials of a row that the block which takes the median asks for at once, together with the scalars.  Back to back, one after
+// the other and all at once: 5 x 250, K = 14 3.71 and 3.56 us, 7 x 500, K = 20 3.99 and 3.84, 8 x 1000, K = 33 5.00 and 4.83, 3 x 100, K = 30
+// 4.14 and 3.87.  Through shared memory, a thread each: 4.2, 4.3, 4.4, 3.5; the scalars by a block of their own 3.81, 4.07, 4.61, 3.49.
+constexpr int kMeetingBatch = 16;
 constexpr int kBatch = 8;                  // workers whose values of a column are asked for at once
 
 struct CombineParams {
@@ -180,11 +184,18 @@ __global__ void __launch_bounds__(kUnitThreads) k_combine(const CombineParams p)
     __syncthreads();
     if (!last_s || warp != 0) return;
     __threadfence();
+    const double head0 = __ldcg(p.scratch), head1 = __ldcg(p.scratch + 1);
     double row = 0.0;
-    if (lane < p.l)
-        for (int q = 0; q < p.chunks; ++q) row += __ldcg(p.scratch + 2 + lane * p.chunks + q);
+    for (int q0 = 0; q0 < p.chunks; q0 += kMeetingBatch) {
+        double v[kMeetingBatch];
+#pragma unroll
+        for (int q = 0; q < kMeetingBatch; ++q)
+            v[q] = lane < p.l && q0 + q < p.chunks ? __ldcg(p.scratch + 2 + lane * p.chunks + q0 + q) : 0.0;
+#pragma unroll
+        for (int q = 0; q < kMeetingBatch; ++q) row += v[q];
+    }
     if (lane == 0) *p.ticket = 0u;                         // ready for the next launch on this context
-    finish(p, row, __ldcg(p.scratch), __ldcg(p.scratch + 1), lane);
+    finish(p, row, head0, head1, lane);
 }
 
 }  // namespace
