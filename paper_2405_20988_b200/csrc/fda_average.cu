@@ -282,15 +282,30 @@ cudaError_t fda_launch_average(const fda_ctx *ctx, float *w, int64_t row_stride,
     const int broadcast = (flags & FDA_AVG_BROADCAST) ? 1 : 0;
     const int threads = 256;
     // One index per thread on short vectors, up to a number of indices per SM that depends on what the quads cost
-    // there: rows at any alignment pay for windows and shifted stores, many rows for the chain of their batches.
-    // Measured with broadcast, calls back to back, one index per thread and quads.
-    // Aligned: K = 32, d = 84K 4.8 and 6.3 us, 150K 5.9 and 5.8; K = 20, 100K 4.0 and 4.0, 250K 6.9 and 5.9; K = 60, 100K 8.1
-    // and 9.2, 200K 12.5 and 14.1, 300K 18.2 and 15.5, 600K 51 and 37.
-    // Any alignment: K = 4, 100K 3.9 and 3.7, 400K 5.4 and 4.0; K = 16, 150K 4.4 and 7.7, 300K 6.7 and 8.1, 600K 11.3 and 12.3
-    // (without broadcast 3.8 and 4.1, 4.2 and 4.5, 6.7 and 6.1); K = 20, 150K 5.4 and 9.4, without broadcast 200K 4.5 and 5.0, 300K 5.7
-    // and 5.1; K = 44, 75,776 6.4 and 17.9, 450K 21.8 and 23.6; K = 60, 600K 54 and 54, 900K 80 and 91.
-    const int64_t per_sm = K > 32 ? (vec ? 1536 : 4096) : (vec || K < 8 ? 768 : 1536);
-    const bool shrt = d <= (int64_t)ctx->n_sm * per_sm;
+    // there: rows at any alignment pay for windows and shifted stores, many rows for the chain of their batches.  Quads of
+    // one wave (four blocks to an SM, 4096 indices) catch up; a second wave that is less than half full costs as much as a full
+    // one, so behind 4096 indices per SM rows at any alignment go one index per thread once more.  Sixteen rows deep: with 24 or
+    // 32 registers keep too few threads on an SM (K = 30, d = 700K 31.8 us, 40 with either).
+    // Measured, calls back to back, one index per thread and quads, d in thousands.
+    // Aligned, broadcast: K = 12, d = 180 4.3 and 4.5 us; K = 16, 180 5.6 and 6.1; K = 30, 120 6.8 and 10.2, 180 10.2 and 12.6, 260 12.8
+    // and 13.5; K = 20, 180 8.3 and 8.4, 260 10.3 and 9.1; K = 60, 180 18.6 and 22.4, 260 23.9 and 24.9, 380 33.4 and 32.9; K = 8, 260 4.5 and 3.8.
+    // Without: K = 16, 180 4.0 and 4.1; K = 20, 180 5.7 and 5.0; K = 44, 180 8.3 and 9.4.
+    // Any alignment, broadcast: K = 4, 120 3.8 and 3.7, 380 5.4 and 5.3, 520 6.2 and 4.4; K = 6, 260 4.2 and 4.9, 380 5.5 and 5.3; K = 8, 380 6.1 and
+    // 6.6, 520 8.5 and 8.2; K = 12, 380 8.3 and 9.4, 520 10.6 and 11.1, 600 11.9 and 11.7; K = 20, 380 14.0 and 14.1, 520 18.3 and 17.6;
+    // K = 30, 260 13.1 and 17.3, 520 24.1 and 26.2, 600 27.1 and 27.9; in the second wave K = 8, 700 11.1 and 11.9; K = 10, 700 12.6 and 14.9, 900
+    // 15.4 and 16.6; K = 20, 700 23.9 and 26.5, 900 29.8 both; K = 30, 620 28.3 and 37.7, 900 40.5 and 44.5, 1100 50.5 both; K = 60, 700
+    // 63.4 and 78, 900 80.7 and 91, 1100 102 and 99.
+    // Without: K = 8, 200 3.6 and 3.8, 260 3.8 and 3.7; K = 10, 380 5.4 both; K = 20, 260 7.0 and 7.2, 380 8.8 and 8.1; K = 30, 380 9.7 and 11.4;
+    // K = 36, 380 12.7 both, 520 16.5 and 14.5; second wave K = 10, 700 8.2 and 8.5, 900 9.8 and 9.2; K = 20, 620 13.1 both, 700 14.2 and 13.7;
+    // K = 44, 700 23.1 and 28.2, 900 28.1 and 30.9.  With xi_out the lines are older ones.
+    // (17 to 20 workers: a second batch of up to four rows is a round trip for little, so their lines lie lower: K = 20, 450 15.9 and 14.8)
+    const bool many = K >= 10 && !xi_out, rest = K > 16 && K <= 20;
+    int64_t per_sm = vec ? (K > 32 ? 1536 : many && broadcast ? 1300 : 768) : K < 8 ? 768 : 1536;
+    if (!vec && xi_out && K > 32) per_sm = 4096;
+    else if (!vec && many) per_sm = broadcast ? (rest ? 2600 : 3400) : (rest ? 1536 : 2200);
+    else if (!vec && !xi_out && broadcast && K >= 6) per_sm = K >= 8 ? 2600 : 1800;
+    const int64_t quad_wave = (int64_t)ctx->n_sm * 4096, half_wave = (int64_t)ctx->n_sm * (broadcast ? 6400 : 4800);
+    const bool shrt = d <= (int64_t)ctx->n_sm * per_sm || (!vec && many && (broadcast || !rest) && d > quad_wave && d <= half_wave);
     // By ticket when a fixed stride takes every block round many times; four blocks of either kernel fit an SM.
     // Measured, fixed stride and tickets, with broadcast: K = 20, d = 2.6M 71.6 and 72.7 us (two rounds); K = 30,
     // d = 7M 287 and 280 us (six); K = 60, d = 20M 1555 and 1524 us; K = 8, d = 198M 2179 and 2035 us (without broadcast
