@@ -233,15 +233,14 @@ fda_status fda_create_with(fda_ctx **out, int device, int l, int m, const uint64
             e = cudaMemcpy(ctx->coeffs_dev, ctx->coeffs_host, sizeof(uint64_t) * 6 * l, cudaMemcpyHostToDevice);
         if (e == cudaSuccess && schedule_limit_bytes >= 0) {
             const auto t0 = std::chrono::steady_clock::now();
-            e = fda_build_list_schedule(ctx, nullptr);
-            if (e == cudaSuccess && ctx->sched && !(flags & FDA_CREATE_ONE_SCHEDULE)) e = fda_build_lane_schedule(ctx, nullptr);
+            e = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = fda_build_schedules(ctx, !(flags & FDA_CREATE_ONE_SCHEDULE));
             ctx->sched_build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
         }
         if (e == cudaSuccess) e = cudaMalloc(&ctx->part_sk, sizeof(float) * ctx->part_sk_floats);
         if (e == cudaSuccess && ctx->sched) e = fda_setup_local_state_gather(ctx);
         if (e == cudaSuccess && ctx->sched) {
-            e = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
+            e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
         }
     }

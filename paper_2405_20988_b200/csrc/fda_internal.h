@@ -158,8 +158,7 @@ cudaError_t fda_launch_debug_hash(const fda_ctx *ctx, int64_t j0, int64_t n, uin
 cudaError_t fda_launch_local_state(fda_ctx *ctx, const float *w, int64_t row_stride, int K,
                                    int64_t d, const float *w_t0, const float *xi, uint32_t flags,
                                    float *states, cudaStream_t s);
-cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s);   // allocates and fills ctx->sched when it fits
-cudaError_t fda_build_lane_schedule(fda_ctx *ctx, cudaStream_t s);   // the same for ctx->lane_sched, where it pays
+cudaError_t fda_build_schedules(fda_ctx *ctx, bool second);   // allocates and fills ctx->sched when it fits, ctx->lane_sched where it pays
 cudaError_t fda_setup_local_state_gather(const fda_ctx *ctx);
 cudaError_t fda_launch_local_state_gather(fda_ctx *ctx, const float *w, int64_t row_stride, int K,
                                           int64_t d, const float *w_t0, const float *xi,

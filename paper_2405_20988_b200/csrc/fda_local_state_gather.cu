@@ -64,7 +64,7 @@
 // this one, by tiles a block: 5 x 250, K = 14, d = 1.2M (5.2) 38.2 and 34.9 us, K = 16, d = 1.6M (7) 44.8 and 40.0, K = 30, d = 0.7M
 // (6.3) 43.8 and 39.8; 3 x 100, K = 10, d = 1.5M (6) 28.5 and 25.8; 7 x 500, K = 44, d = 0.6M (7.9) 72.5 and 62.9, K = 20, d = 1M
 // (5.6) 54.7 and 50.8; 4 x 1000, K = 20, d = 1M (4.8) 60.0 and 43.4; 8 x 1000, K = 26, d = 0.3M (4.6) 47.2 and 42.2, K = 44, d = 0.3M
-// (6.8) 63 and 54.  That pays for the second schedule (1.2 to 1.9 ms of fda_create) after some 300 steps.  Shorter vectors gain
+// (6.8) 63 and 54.  That pays for the second schedule (0.6 to 1 ms of fda_create) after some 200 steps.  Shorter vectors gain
 // less (5 x 250, K = 10, d = 1.2M, four tiles: 28.7 and 27.0).  With xi the list kernel stays, a
 // fifth slower on long vectors: what it gives is one order of additions for all sizes, so the digits of a run that projects do
 // not depend on which side of the line its vectors are.  That order shows right after a synchronisation, when the mean

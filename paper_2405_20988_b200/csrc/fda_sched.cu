@@ -806,9 +806,16 @@ static int list_geometry(const fda_ctx *ctx, int *parts_out, int *ni_max_out)
     return 0;
 }
 
-// Builds one of the two schedules; none is built (and cudaSuccess returned) for a sketch, a hash, a size or a
-// memory limit that it does not suit.
-static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
+// What the writing pass of a schedule still reads when build_schedule has returned (bytes: also what was
+// pending before, which counts as free memory).
+struct PendingBuild {
+    uint32_t *items = nullptr;
+    size_t bytes = 0;
+};
+
+// Builds one of the two schedules on stream s; none is built (and cudaSuccess returned) for a sketch, a hash, a size or a
+// memory limit that it does not suit.  The writing pass is left running.
+static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s, PendingBuild &pending)
 {
     int ni_max = 0, parts = 1;
     const int T = lanes ? lane_geometry(ctx, &parts, &ni_max) : list_geometry(ctx, &parts, &ni_max);
@@ -841,7 +848,7 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
     if (octet_bytes && cudaMalloc(&items, sizeof(uint32_t) * words + octet_bytes) == cudaSuccess) p.octets = reinterpret_cast<uint16_t *>(items + words);
     else cudaGetLastError();
     if ((!items && cudaMalloc(&items, sizeof(uint32_t) * words) != cudaSuccess) ||
-        cudaMalloc(&rows, sizeof(int2) * ctx->l) != cudaSuccess ||
+        (lanes && cudaMalloc(&rows, sizeof(int2) * ctx->l) != cudaSuccess) ||
         cudaMalloc(&off, sizeof(uint64_t) * (tiles + 1)) != cudaSuccess) {
         cudaGetLastError();
         cleanup();
@@ -886,7 +893,7 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
     const uint64_t prog_bytes = lanes ? sizeof(uint32_t) * (uint64_t)(lane_items + 1) * tiles : 0;
     const uint64_t all_bytes = total + prog_bytes + ctx->sched_bytes;         // (of both schedules, when this is the second)
     size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || (!lanes && !p.octets) || total + prog_bytes > (free_b + octet_bytes) / 3 ||
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || (!lanes && !p.octets) || total + prog_bytes > (free_b + octet_bytes + pending.bytes) / 3 ||
         (ctx->sched_limit_bytes > 0 && all_bytes > (uint64_t)ctx->sched_limit_bytes) ||
         cudaMalloc(&buf, total) != cudaSuccess || (lanes && cudaMalloc(&prog, prog_bytes) != cudaSuccess)) {
         cudaGetLastError();
@@ -900,9 +907,8 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
     p.lane_prog = prog;
     k_build_schedule<true><<<(unsigned)tiles, kBT, bsmem, s>>>(p);
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) { cleanup(); return e; }
-    cudaFree(items);
+    if (e != cudaSuccess) { cudaDeviceSynchronize(); cleanup(); return e; }
+    pending.items = items; pending.bytes = sizeof(uint32_t) * words + octet_bytes;
     if (lanes) {
         ctx->lane_sched = buf; ctx->lane_off = off; ctx->lane_prog = prog; ctx->lane_rows = rows;
         ctx->lane_records = total;
@@ -911,11 +917,22 @@ static cudaError_t build_schedule(fda_ctx *ctx, bool lanes, cudaStream_t s)
         ctx->lane_items = lane_items; ctx->lane_walkers = lane_walkers(p.l, lane_items);
         return cudaSuccess;
     }
-    cudaFree(rows);
     ctx->sched = buf; ctx->sched_off = off; ctx->sched_bytes = total; ctx->sched_T = T;
     ctx->sched_ni_max = ni_max; ctx->sched_tiles = part_tiles; ctx->sched_parts = parts;
     return cudaSuccess;
 }
 
-cudaError_t fda_build_list_schedule(fda_ctx *ctx, cudaStream_t s) { return build_schedule(ctx, false, s); }
-cudaError_t fda_build_lane_schedule(fda_ctx *ctx, cudaStream_t s) { return build_schedule(ctx, true, s); }
+// The second schedule is begun while the first one's writing pass runs: on short vectors, which fill few SMs, both are
+// bound by latency.  fda_create, one after the other and so: 5 x 250, K = 14, d = 1.2M 4.2 and 3.5 ms, 7 x 500, K = 44, d = 0.6M 5.6 and 4.8,
+// 5 x 250, K = 30, d = 7M 8.8 and 8.5, 8 x 1000, K = 20, d = 2.6M 14.3 and 13.9.
+cudaError_t fda_build_schedules(fda_ctx *ctx, bool second)
+{
+    PendingBuild first, last;
+    cudaError_t e = build_schedule(ctx, false, nullptr, first);
+    last.bytes = first.bytes;
+    if (e == cudaSuccess && ctx->sched && second) e = build_schedule(ctx, true, ctx->side_stream, last);
+    const cudaError_t done = cudaDeviceSynchronize();
+    cudaFree(first.items);
+    cudaFree(last.items);
+    return e != cudaSuccess ? e : done;
+}
