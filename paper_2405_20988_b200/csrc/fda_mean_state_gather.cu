@@ -612,8 +612,12 @@ cudaError_t fda_launch_mean_sketch_gather(fda_ctx *ctx, const float *mean_drift,
     p.groups = parts;
     p.nb = (int)ctx->sched_tiles;                                    // records of a part
     p.cpg = (int)std::max((int64_t)1, std::min((int64_t)ctx->n_sm * kShortPerSm / parts, p.tiles));
-    // up to three blocks to a tile while each has an SM of its own
-    p.part_tiles = (int)std::max((int64_t)1, std::min((int64_t)3, ctx->n_sm / (p.tiles * parts)));
+    // up to three blocks to a tile while each has an SM of its own, two to an SM where a warp has six items or more to walk.  Measured, whole
+    // calls, one block to a tile and two, K = 24: 7 x 500 (seven items) d = 400K 21.4 and 21.1 us, 480K 23.8 and 22.7, 612K 31.3 and 29.5, 700K
+    // 34.4 and 32.1; 8 x 1000, K = 20, d = 200K (eight) 18.3 and 16.8, 360K 20.1 and 19.4; but 5 x 250 (three) d = 480K 19.6 and 20.3, K = 8,
+    // d = 800K 17.2 and 18.4; 10 x 250, K = 12, d = 600K (five) 19.3 and 20.1.
+    const bool long_walk = p.l * ((p.m + kListSlots - 1) / kListSlots) >= 6 * kShortWarps && p.tiles * parts > ctx->n_sm / 2;
+    p.part_tiles = (int)std::max((int64_t)1, std::min((int64_t)3, (long_walk ? kShortPerSm : 1) * ctx->n_sm / (p.tiles * parts)));
     const int n = p.cpg * p.part_tiles;                              // partial sketches of a part
     const size_t smem = mean_short_smem(lm, p.T);
     if ((size_t)n * lm * parts > ctx->part_sk_floats || p.T > kShortQuads * kShortWarps * 32 * 4 || smem > (size_t)ctx->smem_optin)
